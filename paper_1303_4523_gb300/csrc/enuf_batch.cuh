@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(1024) kb_bin_scatter(const BinScatterArgs<R>* 
     pdl_enter();
     const int m = cmap[blockIdx.x];
     const BinScatterArgs<R>& a = tab[m >> kBatchShift];
-    k_bin_scatter_body<R>(a.g, a.cnt_blk, a.ctile, a.cpos, a.cfrac, a.cbase, a.boff, a.tstart, a.sq, a.sw, a.sb,
+    k_bin_scatter_body<R>(a.g, a.cnt_blk, a.ctile, a.cpos, a.cfrac, a.cbase, a.boff, a.tstart, a.sq, a.sw, a.sb, nullptr,
                           Blk{m & kBatchLocal, a.nblk});
 }
 
@@ -92,6 +92,8 @@ struct RealArgs {
     const int* tstart;
     const typename V4<R>::T* sq;
     const typename V4<R>::T* sw;
+    const int* sb;
+    const float4* spf;
     R* F;
     double* rpart;
     int nblk;
@@ -101,7 +103,7 @@ __global__ void __launch_bounds__(kRealThreads) kb_real(const RealArgs<R>* __res
     pdl_enter();
     const int m = cmap[blockIdx.x];
     const RealArgs<R>& a = tab[m >> kBatchShift];
-    k_real_body<R>(a.g, a.tstart, a.sq, a.sw, a.F, a.rpart, Blk{m & kBatchLocal, a.nblk});
+    k_real_body<R>(a.g, a.tstart, a.sq, a.sw, a.sb, a.spf, a.F, a.rpart, Blk{m & kBatchLocal, a.nblk});
 }
 
 // the column spreading form of one tile edge T (systems grouped by T)

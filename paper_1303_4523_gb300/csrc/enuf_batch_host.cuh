@@ -16,6 +16,11 @@ inline void append_blocks(std::vector<int>& cmap, int sys, int nblk) {
     for (int b = 0; b < nblk; ++b) cmap.push_back((sys << kBatchShift) | b);
 }
 
+// Real-space blocks of one system of a batch: the batch fills the chip, so a
+// system takes about 4 lanes per charged bead (a tenth of the beads charged)
+// instead of the launch's whole width (the kernel strides over any excess).
+inline int batch_real_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_real, (x.N + 511) / 512)); }
+
 inline int bin_count_smem(const Geo& g) { return (g.ntiles + g.chunk) * (int)sizeof(int); }
 
 }  // namespace batch_detail
@@ -91,9 +96,10 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
         std::vector<int> m;
         for (int s = 0; s < nsys; ++s) {
             const BatchSys& x = sys[s];
-            a[s] = RealArgs<R>{x.g, x.w.tstart, static_cast<const V*>(x.w.sq), static_cast<const V*>(x.w.sw),
-                               static_cast<R*>(x.F), x.w.part + x.w.off_real, x.w.nblk_real};
-            append_blocks(m, s, x.w.nblk_real);
+            const int nb = batch_real_blocks(x);
+            a[s] = RealArgs<R>{x.g, x.w.tstart, static_cast<const V*>(x.w.sq), static_cast<const V*>(x.w.sw), x.w.sb,
+                               x.w.spf, static_cast<R*>(x.F), x.w.part + x.w.off_real, nb};
+            append_blocks(m, s, nb);
         }
         put(L.real, a.data(), a.size() * sizeof(a[0]), m);
         L.real.threads = kRealThreads;
@@ -157,6 +163,7 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
             const Work& w = x.w;
             TotalsArgs t = totals_args(x.g, w, false, 1);
             t.Edev = x.Edev;
+            t.nreal = batch_real_blocks(x);
             // blocks in proportion to the system (a warp per charged bead, <= 1/8 of
             // the beads charged on average; the kernel strides over any excess)
             const int nb = std::max(1, std::min(w.nblk_gather, (x.N + 63) / 64));

@@ -529,6 +529,11 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
         g.kh = P.r_cut / g.kn;
         g.kinv = g.kn / P.r_cut;
     }
+    g.rkd = RealK<double>{g.L, 0.5 * g.L, g.rc * g.rc, g.alpha, g.c2a, g.beta, g.kappa, g.kinv};
+    g.rkf = RealK<float>{(float)g.L, (float)(0.5 * g.L), (float)(g.rc * g.rc), (float)g.alpha, (float)g.c2a,
+                         (float)g.beta, (float)g.kappa, (float)g.kinv};
+    g.slater = P.beta > 0.0 ? 1 : 0;
+    g.r2hi = (float)(g.rc * g.rc) * (1.0f + 1e-4f) + 4e-6f * (float)(g.L * g.rc) + 1e-6f;
     if (P.slater_k) {
         // I'(0) = lim I(r)/r gives the self term
         double i0[3];
@@ -545,7 +550,8 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
     g.rlo = (float)(g.ratio - (double)g.rhi);
 
     Work w{};
-    w.nblk_real = std::min(8 * kSMs, g.ntiles);   // one tile per CTA at most
+    // real space: up to a warp per bead, four CTAs per SM (64 registers a thread)
+    w.nblk_real = std::min(4 * kSMs, (std::max(n_max, 1) + 7) / 8);
     w.nblk_conv = fs.grid_z;
     w.nblk_dpd = 4 * kSMs;
     w.nblk_kin = kSMs;   // one block per SM: its FP64 block sum runs on each SM's few FP64 units once
@@ -571,6 +577,7 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
            o_cpos = take(ncmp * 4 * esz),
            o_cfrac = take(ncmp * 4 * esz), o_cbase = take(ncmp * 4),
            o_sq = take(nm * 4 * esz), o_sw = take(nm * 4 * esz), o_sb = take(nm * 4),
+           o_spf = take(P.prec == ENUF_FP64 ? nm * sizeof(float4) : 0),
            o_wb = take(nm * 3 * 2 * P.p * esz), o_grid = take(n3 * esz),
            o_s1 = take((size_t)n * nc1 * n * csz), o_s2 = take((size_t)nc1 * g.K * n * csz),
            o_s3 = take((size_t)g.nf * n * nc1 * g.K * csz), o_s4 = take((size_t)g.nf * n * n * nc1 * csz),
@@ -593,7 +600,7 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
         w.tstart = (int*)o_tstart; w.ticket = (int*)o_tk; w.check = (unsigned int*)o_ck; w.ctile = (int*)o_ctile;
         w.cpos = (void*)o_cpos; w.cfrac = (void*)o_cfrac;
         w.cbase = (int*)o_cbase;
-        w.sq = (void*)o_sq; w.sw = (void*)o_sw; w.sb = (int*)o_sb; w.wb = (void*)o_wb; w.grid = (void*)o_grid;
+        w.sq = (void*)o_sq; w.sw = (void*)o_sw; w.sb = (int*)o_sb; w.spf = (float4*)o_spf; w.wb = (void*)o_wb; w.grid = (void*)o_grid;
         w.spec1 = (void*)o_s1; w.spec2 = (void*)o_s2; w.spec3 = (void*)o_s3; w.spec4 = (void*)o_s4;
         w.h = (void*)o_h; w.tab = (double*)o_tab; w.tabv = (double*)o_tabv; w.tabr = (void*)o_tabr;
         w.tw = (void*)o_tw; w.part = (double*)o_part; w.Edev = (double*)o_E; w.ktab = (void*)o_ktab;
@@ -611,7 +618,9 @@ void bind(enuf_plan_t p) {
     w.tstart = at(w.tstart); w.ticket = at(w.ticket); w.check = at(w.check); w.ctile = at(w.ctile);
     w.cpos = at(w.cpos); w.cfrac = at(w.cfrac);
     w.cbase = at(w.cbase);
-    w.sq = at(w.sq); w.sw = at(w.sw); w.sb = at(w.sb); w.wb = at(w.wb); w.grid = at(w.grid);
+    w.sq = at(w.sq); w.sw = at(w.sw); w.sb = at(w.sb);
+    w.spf = p->prec == ENUF_FP64 ? at(w.spf) : static_cast<float4*>(w.sq);
+    w.wb = at(w.wb); w.grid = at(w.grid);
     w.spec1 = at(w.spec1); w.spec2 = at(w.spec2); w.spec3 = at(w.spec3); w.spec4 = at(w.spec4);
     w.h = at(w.h); w.tab = at(w.tab); w.tabv = at(w.tabv); w.tabr = at(w.tabr);
     w.tw = at(w.tw); w.part = at(w.part); w.Edev = at(w.Edev); w.ktab = at(w.ktab);

@@ -201,7 +201,7 @@ void enqueue_bin(const Geo& g, const Work& w, int N, const R* pos, const R* q, R
     }
     launch(pdl, true, k_bin_scatter<R>, g.nbin, kBinThreads, g.ntiles * sizeof(int), s, g, (const int*)w.cnt_blk,
            (const int*)w.ctile, static_cast<const V*>(w.cpos), static_cast<const V*>(w.cfrac), (const int*)w.cbase,
-           (const int*)w.boff, (const int*)w.tstart, static_cast<V*>(w.sq), static_cast<V*>(w.sw), w.sb);
+           (const int*)w.boff, (const int*)w.tstart, static_cast<V*>(w.sq), static_cast<V*>(w.sw), w.sb, w.spf);
     if (w.wb)
         launch(pdl, true, k_bin_weights<R>, bin_weight_blocks(g), 256, 0, s, g, (const int*)w.tstart,
                static_cast<const V*>(w.sw), static_cast<R*>(w.wb));
@@ -373,6 +373,7 @@ cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp,
     cudaStreamWaitEvent(s1, evFork, 0);
     rec(ev, 4, true, s1);
     const int real_smem = real_smem_bytes<R>();
+    const float4* spf = w.spf;
     if (dpd) {   // DPD pairs and real-space pairs in one launch
         const DpdDev& d = *dpd;
         launch(false, false, k_pairs<R>, w.nblk_dpd + w.nblk_real, kRealThreads,
@@ -380,10 +381,10 @@ cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp,
                static_cast<const V*>(d.sv), (const int*)d.cstart, static_cast<const R*>(d.atab),
                static_cast<const R*>(d.pos), (const int*)d.bnd, (const uint64_t*)d.step_dev, static_cast<R*>(d.F),
                w.part + w.off_dpd, w.nblk_dpd, g, (const int*)w.tstart, (const V*)sq, (const V*)sw,
-               w.part + w.off_real);
+               (const int*)w.sb, spf, w.part + w.off_real);
     } else {
         launch(false, false, k_real<R>, w.nblk_real, kRealThreads, real_smem, s1, g, (const int*)w.tstart,
-               (const V*)sq, (const V*)sw, F, w.part + w.off_real);
+               (const V*)sq, (const V*)sw, (const int*)w.sb, spf, F, w.part + w.off_real);
     }
     rec(ev, 4, false, s1);
     cudaEventRecord(evJoin, s1);

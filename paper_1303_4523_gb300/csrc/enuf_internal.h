@@ -9,7 +9,6 @@
 
 namespace enuf {
 
-// Geometry and constants every kernel needs, passed by value.
 // Debug builds (-DENUF_CHECK): device-side index checks. ENUF_GUARD(word,
 // cond, bit) is cond, and when cond fails sets bit `bit` of the plan's check
 // word (read by enuf_check_word); the caller skips the access it guards.
@@ -28,6 +27,15 @@ __device__ __forceinline__ bool enuf_guard(unsigned int* word, bool ok, int bit)
 // is a few words; the part allows 227 KB per CTA)
 constexpr int kBinSmem = 224 * 1024;
 
+// Constants of the real-space pair arithmetic in one working precision.
+template <typename R>
+struct RealK {
+    R L, hL, rc2;     // box edge, L / 2, r_c^2
+    R al, c2a, be;    // alpha, 2 alpha / sqrt(pi), beta
+    R kap, kinv;      // kappa, kernel table intervals per unit length
+};
+
+// Geometry and constants every kernel needs, passed by value.
 struct Geo {
     int n;        // oversampled grid per dimension (sigma_s * M)
     int nc;       // kept modes per side, |k_t| <= nc
@@ -60,6 +68,12 @@ struct Geo {
     double kinv;     // kn / r_c
     double kh;       // r_c / kn
     const void* ktab;  // real [kn][kKtStride]: quintic coefficients of J(r) = r u(r) per interval
+    RealK<float> rkf;
+    RealK<double> rkd;
+    int slater;   // beta > 0: the real-space term carries the Slater correction
+    // FP64 cutoff pre-test on float positions: r_c^2 plus a band that covers the float
+    // error (positions and L rounded to float, |r2f - r2| <= ~1.5e-6 L r_c)
+    float r2hi;
     int nmax;          // capacity in beads (sorted charged-bead arrays)
     unsigned int* check;  // debug builds: failure bits of the device index checks
 };
@@ -130,6 +144,7 @@ struct Work {
     void* sq;        // real4 [n_max]  wrapped x, y, z, q (sorted)
     void* sw;        // real4 [n_max]  fractional grid coordinates, original index bits
     int* sb;         // [n_max]  packed base grid index
+    float4* spf;     // [n_max]  float copy of the sorted positions (FP64; FP32: sq itself)
     void* wb;        // real [n_max][3][2p]  window weights psi(u - l) of each sorted bead
     // grids and spectra
     void* grid;      // real [n^3]

@@ -704,7 +704,8 @@ __device__ __forceinline__ void k_bin_scatter_body(Geo g, const int* __restrict_
                                                      const int* __restrict__ cbase, const int* __restrict__ boff,
                                                      const int* __restrict__ tstart,
                                                      typename V4<R>::T* __restrict__ sq,
-                                                     typename V4<R>::T* __restrict__ sw, int* __restrict__ sb, Blk blk) {
+                                                     typename V4<R>::T* __restrict__ sw, int* __restrict__ sb,
+                                                     float4* __restrict__ spf, Blk blk) {
     pdl_enter();
     extern __shared__ int cur[];   // [ntiles] running counts
     const int b = blk.id;
@@ -718,9 +719,12 @@ __device__ __forceinline__ void k_bin_scatter_body(Geo g, const int* __restrict_
         if (!ENUF_GUARD(g.check, (unsigned)t < (unsigned)g.ntiles, 2)) continue;
         const int slot = tstart[t] + boff[b * g.ntiles + t] + atomicAdd(&cur[t], 1);
         if (!ENUF_GUARD(g.check, (unsigned)slot < (unsigned)g.nmax, 2)) continue;
-        sq[slot] = cpos[o];
+        const typename V4<R>::T a = cpos[o];
+        sq[slot] = a;
         sw[slot] = cfrac[o];
         sb[slot] = cbase[o];
+        // FP64: a float copy of the position for the real-space cutoff pre-test
+        if (sizeof(R) == 8 && spf) spf[slot] = make_float4((float)a.x, (float)a.y, (float)a.z, 0.f);
     }
 }
 
@@ -732,8 +736,9 @@ __global__ void __launch_bounds__(1024) k_bin_scatter(Geo g, const int* __restri
                                                      const int* __restrict__ cbase, const int* __restrict__ boff,
                                                      const int* __restrict__ tstart,
                                                      typename V4<R>::T* __restrict__ sq,
-                                                     typename V4<R>::T* __restrict__ sw, int* __restrict__ sb) {
-    k_bin_scatter_body<R>(g, cnt_blk, ctile, cpos, cfrac, cbase, boff, tstart, sq, sw, sb, Blk{(int)blockIdx.x, (int)gridDim.x});
+                                                     typename V4<R>::T* __restrict__ sw, int* __restrict__ sb,
+                                                     float4* __restrict__ spf) {
+    k_bin_scatter_body<R>(g, cnt_blk, ctile, cpos, cfrac, cbase, boff, tstart, sq, sw, sb, spf, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // Window weights of every sorted charged bead (Eq. 14), computed once and
@@ -2012,19 +2017,32 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(Geo g, const int* __r
 
 // ---------------------------------------------------------------------------
 // a7 (electrostatic part): real-space erfc + Slater-correction pairs on the
-// tile bins (Eq. 31, corrected Eq. 32, Eq. 27-28). Warp per charged bead; lanes
-// stride over the candidates of each contiguous run of tiles.
+// tile bins (Eq. 31, corrected Eq. 32, Eq. 27-28).
+//
+// S lanes per charged bead (S a power of 2, chosen per launch), 32 / S
+// consecutive beads of the sorted order per warp. The tiles around a bead's
+// tile form one contiguous run of sorted beads per (y, z) row of tiles; the
+// bead's lanes walk the runs and read the candidates straight from the sorted
+// array (the lanes of beads of one tile read the same lines). What passes the
+// cutoff test goes to shared memory:
+//   FP32: each lane notes its candidates in a list of its own (one predicated
+//     store, no ballot); the lists are evaluated in step, each lane adding
+//     into its own registers, and the S shares of a bead are summed once.
+//     Issue-bound.
+//   FP64: pairs of all the warp's beads go to one ring and are evaluated on
+//     full warps, each pair once, because every FP64 instruction costs the
+//     whole warp's 16 cycles of the SM's few FP64 units; +f and -f go out by
+//     global reductions.
 // ---------------------------------------------------------------------------
 constexpr int kRealThreads = 256;
-constexpr int kRealCap = 2048;     // staged beads (x, y, z, q)
-constexpr int kRealHalo = 1024;    // halo tiles (stencil up to 9 x 9 x 9 + 1 for the prefix)
-constexpr int kRealRound = 8;      // tiles staged together at most
-// FP64 also stages a float copy of the positions for the cutoff pre-test
-template <typename R> __host__ __device__ constexpr int real_cap() { return sizeof(R) == 8 ? 1536 : kRealCap; }
+constexpr int kRealQ = 32;      // FP32: noted candidates per lane
+constexpr int kRealU = 4;       // candidates per lane and iteration (loads in flight)
+constexpr int kRealRing = 256;  // FP64: pair ring per warp (>= 31 + 32 kRealU, a power of 2)
+static_assert(kRealRing >= 31 + 32 * kRealU && (kRealRing & (kRealRing - 1)) == 0, "pair ring");
 template <typename R>
-constexpr int real_smem_bytes() {   // FP64 adds the float copy, the staged slots and the partner queue
-    return (real_cap<R>() + (kRealThreads / 32) * 64) * (int)sizeof(typename V4<R>::T) + (2 * kRealHalo + 1) * 4 +
-           (sizeof(R) == 8 ? real_cap<R>() * ((int)sizeof(float4) + 4) + (kRealThreads / 32) * 64 * 4 : 0);
+constexpr int real_smem_bytes() {
+    return sizeof(R) == 8 ? (kRealThreads / 32) * kRealRing * (int)sizeof(int2)
+                          : kRealThreads * kRealQ * (int)sizeof(int);
 }
 
 // Kernel table: per interval [j h, (j + 1) h] of [0, r_c] the power-basis
@@ -2091,357 +2109,277 @@ __device__ __forceinline__ void real_pair(R r2, R al, R c2a, R be, bool slater, 
     f_r = ff * r;          // virial term r f(r)
 }
 
-// One lane per queued pair (lanes < m).
-// FP64 evaluates each pair once (Newton's third law: +f for bead i in the
-// lane, -f to bead j, original index from its sorted slot, atomically): the
-// pair arithmetic runs on the few FP64 units and halving it pays for the
-// atomics. FP32 evaluates both directions (each bead only adds into its own
-// force), measured faster there.
 template <typename R> __host__ __device__ constexpr bool real_half() { return sizeof(R) == 8; }
 
-template <typename R, typename V>
-__device__ __forceinline__ void real_drain(const Geo& g, const V* qu, const int* quj, int m, int lane, R qi, R kap,
-                                           R al, R c2a, R be, bool slater, const V* __restrict__ sw,
-                                           R* __restrict__ F, R& fx, R& fy, R& fz, R& eacc, R& wacc) {
-    constexpr bool HALF = real_half<R>();
-    if (lane < m) {
-        const V e = qu[lane];
-        const R r2 = dist2(e.x, e.y, e.z);
-        R u, fo, fr;
-        real_pair<R>(r2, al, c2a, be, slater, u, fo, fr, static_cast<const R*>(g.ktab), g.kn, (R)g.kinv);
-        const R qq = kap * qi * e.w;
-        const R gx = qq * fo * e.x, gy = qq * fo * e.y, gz = qq * fo * e.z;
-        fx += gx;
-        fy += gy;
-        fz += gz;
-        if (HALF) {
-            const int j = real_as_int(sw[quj[lane]].w);
-            atomicAdd(&F[3 * j], -gx);
-            atomicAdd(&F[3 * j + 1], -gy);
-            atomicAdd(&F[3 * j + 2], -gz);
-        }
-        const R ws = HALF ? (R)1 : (R)0.5;   // energy and virial per pair
-        eacc += ws * qq * u;
-        wacc += ws * qq * fr;
+// A lane's sums: the force on its bead (FP32), energy and virial.
+template <typename R>
+struct RealSum {
+    R fx, fy, fz, e, w;
+};
+
+// FP32: the pairs (bead pi, noted candidate k of this lane, k < cnt), all lanes in step.
+__device__ __forceinline__ void real_drain(const Geo& g, const float4& pi, const int* list, int cnt,
+                                           const float4* __restrict__ sq, RealSum<float>& a) {
+    const RealK<float>& c = g.rkf;
+    const int m = __reduce_max_sync(0xffffffffu, cnt);
+    for (int k = 0; k < m; ++k) {
+        if (k >= cnt) continue;
+        const float4 pj = sq[list[32 * k]];
+        const float dx = min_image(pi.x, pj.x, c.L, c.hL);
+        const float dy = min_image(pi.y, pj.y, c.L, c.hL);
+        const float dz = min_image(pi.z, pj.z, c.L, c.hL);
+        float u, fo, fr;
+        real_pair<float>(dist2(dx, dy, dz), c.al, c.c2a, c.be, g.slater != 0, u, fo, fr,
+                         static_cast<const float*>(g.ktab), g.kn, c.kinv);
+        const float qq = c.kap * pi.w * pj.w;
+        a.fx += qq * fo * dx;
+        a.fy += qq * fo * dy;
+        a.fz += qq * fo * dz;
+        a.e += 0.5f * qq * u;   // energy and virial per pair and direction
+        a.w += 0.5f * qq * fr;
     }
 }
 
-// Staged FP64: the queue holds the staged index of candidates that passed
-// the float pre-test; the double displacement, the exact cutoff decision and
-// the pair run here, on full warps (the sweep's candidates pass the float
-// test on a few lanes at a time, and every FP64 instruction costs the whole
-// warp's issue on GB300's FP64 units).
-template <typename R, typename V>
-__device__ __forceinline__ void real_drain_staged(const Geo& g, const V& pi, const V* stg, const int* stgslot,
-                                                  const int* quj, int m, int lane, R L, R hL, R rc2, R kap, R al,
-                                                  R c2a, R be, bool slater, const V* __restrict__ sw,
-                                                  R* __restrict__ F, R& fx, R& fy, R& fz, R& eacc, R& wacc) {
-    if (lane < m) {
-        const int f = quj[lane];
-        const V pj = stg[f];
-        const R dx = min_image(pi.x, pj.x, L, hL);
-        const R dy = min_image(pi.y, pj.y, L, hL);
-        const R dz = min_image(pi.z, pj.z, L, hL);
-        const R r2 = dist2(dx, dy, dz);
-        if (r2 < rc2 && r2 > (R)0) {
-            R u, fo, fr;
-            real_pair<R>(r2, al, c2a, be, slater, u, fo, fr, static_cast<const R*>(g.ktab), g.kn, (R)g.kinv);
-            const R qq = kap * pi.w * pj.w;
-            const R gx = qq * fo * dx, gy = qq * fo * dy, gz = qq * fo * dz;
-            fx += gx;
-            fy += gy;
-            fz += gz;
-            const int j = real_as_int(sw[stgslot[f]].w);
-            atomicAdd(&F[3 * j], -gx);
-            atomicAdd(&F[3 * j + 1], -gy);
-            atomicAdd(&F[3 * j + 2], -gz);
-            eacc += qq * u;
-            wacc += qq * fr;
+// FP64: ring entries (bead i, candidate j) with the image in their upper bits
+// (5 bits, 9 z + 3 y + x of 0: -L, 1: none, 2: +L), one per lane. ALL: the
+// displacement is the minimum image instead.
+__device__ __forceinline__ int2 real_entry(int i, int j, int image) {
+    return make_int2(i | (image & 7) << 29, j | (image >> 3) << 29);
+}
+template <bool ALL>
+__device__ __forceinline__ void real_ring(const Geo& g, const int2 e, const double4_32a* __restrict__ sq,
+                                          const double4_32a* __restrict__ sw, double* __restrict__ F,
+                                          RealSum<double>& a) {
+    const RealK<double>& c = g.rkd;
+    const int i = e.x & 0x1fffffff, j = e.y & 0x1fffffff;
+    const double4_32a pi = sq[i], pj = sq[j];
+    double dx, dy, dz;
+    if constexpr (ALL) {
+        dx = min_image(pi.x, pj.x, c.L, c.hL);
+        dy = min_image(pi.y, pj.y, c.L, c.hL);
+        dz = min_image(pi.z, pj.z, c.L, c.hL);
+    } else {
+        dx = pi.x - pj.x;
+        dy = pi.y - pj.y;
+        dz = pi.z - pj.z;
+        const int im = (int)((unsigned)e.x >> 29 | ((unsigned)e.y >> 29) << 3);
+        if (im != 13) {   // across a box face
+            const int iz = im / 9, iy = (im - 9 * iz) / 3, ix = im % 3;
+            if (ix != 1) dx += ix ? c.L : -c.L;
+            if (iy != 1) dy += iy ? c.L : -c.L;
+            if (iz != 1) dz += iz ? c.L : -c.L;
         }
     }
+    const double r2 = dist2(dx, dy, dz);
+    if (!(r2 < c.rc2 && r2 > 0.0)) return;
+    double u, fo, fr;
+    real_pair<double>(r2, c.al, c.c2a, c.be, g.slater != 0, u, fo, fr, static_cast<const double*>(g.ktab), g.kn, c.kinv);
+    const double qq = c.kap * pi.w * pj.w;
+    const double gf = qq * fo;
+    const double gx = gf * dx, gy = gf * dy, gz = gf * dz;
+    double* Fi = F + 3 * (size_t)real_as_int(sw[i].w);
+    double* Fj = F + 3 * (size_t)real_as_int(sw[j].w);
+    atomicAdd(Fi, gx);
+    atomicAdd(Fi + 1, gy);
+    atomicAdd(Fi + 2, gz);
+    atomicAdd(Fj, -gx);
+    atomicAdd(Fj + 1, -gy);
+    atomicAdd(Fj + 2, -gz);
+    a.e = fma(qq, u, a.e);
+    a.w = fma(qq, fr, a.w);
 }
 
-// Halo of a tile: per dimension either the whole periodic row of tiles (when
-// the stencil 2 rs + 1 covers it) or the tiles t - rs .. t + rs.
-__device__ __forceinline__ void halo_dim(int t, int rs, int ntd, int& lo, int& cnt) {
-    if (2 * rs + 1 >= ntd) { lo = 0; cnt = ntd; }
-    else { lo = t - rs; cnt = 2 * rs + 1; }
-}
-
-// Beads [c0, c1) of one tile against the nh-tile halo (total beads), this
-// warp's share being beads c0 + woff, c0 + woff + NW, ... STAGED: candidates
-// from the shared-memory copy; else from global memory through the halo prefix.
-template <typename R, bool STAGED>
-__device__ __forceinline__ void real_beads(const Geo& g, int c0, int c1, int woff, int selfbase, int total, int nh,
-                                           const typename V4<R>::T* stg, const float4* stgf, const int* stgslot,
-                                           const int* hoff, const int* gst, const typename V4<R>::T* __restrict__ sq,
-                                           const typename V4<R>::T* __restrict__ sw, typename V4<R>::T* qu, int* quj,
-                                           R* __restrict__ F, R& eacc, R& wacc) {
+// Beads of this block's share. ALL: the stencil covers whole rows of tiles
+// (few tiles per dimension), every tile is visited once and displacements
+// take the minimum image; else the rows and the x run are wrapped tile by
+// tile, and a run's image shift is one constant (the displacement within r_c
+// is the one of that image: r_c <= rs tiles, 2 rs + 1 <= tiles per dimension).
+template <typename R, bool ALL>
+__device__ __forceinline__ void real_sweep(const Geo& g, int nq, int S, const int* __restrict__ tstart,
+                                           const typename V4<R>::T* __restrict__ sq,
+                                           const typename V4<R>::T* __restrict__ sw, const int* __restrict__ sb,
+                                           const float4* __restrict__ spf, int* list, int2* ring,
+                                           R* __restrict__ F, RealSum<R>& a, Blk blk) {
     using V = typename V4<R>::T;
+    constexpr bool HALF = real_half<R>();
+    constexpr unsigned FULL = 0xffffffffu;
     constexpr int NW = kRealThreads / 32;
-    // FP64: the cutoff test r^2 < r_c^2 runs on the float copy first; candidates
-    // above a band that covers the float error (positions and L rounded to float,
-    // |r2f - r2| <= ~1.5e-6 L r_c) are out, the rest are decided in double
-    constexpr bool PRE = STAGED && sizeof(R) == 8;
-    const float Lf = (float)g.L, hLf = (float)(0.5 * g.L);
-    const float r2hi = (float)(g.rc * g.rc) * (1.0f + 1e-4f) + 4e-6f * (float)(g.L * g.rc) + 1e-6f;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const R L = (R)g.L, hL = (R)(0.5 * g.L);
-    const R rc2 = (R)(g.rc * g.rc);
-    const R al = (R)g.alpha, c2a = (R)g.c2a, be = (R)g.beta, kap = (R)g.kappa;
-    const bool slater = g.beta > 0.0;
-    for (int s = c0 + woff; s < c1; s += NW) {
-        const V pi = sq[s];
-        const float4 pif = make_float4((float)pi.x, (float)pi.y, (float)pi.z, 0.f);
-        const int self = selfbase + (s - c0);   // the bead's own index in the halo order
-        R fx = 0, fy = 0, fz = 0;
-        int cnt = 0;
-        int hseg = 0;
-        const int steps = (total + 31) / 32 + 1;   // the extra step drains the queue
-        for (int it = 0; it < steps; ++it) {
-            const bool last = it == steps - 1;
-            if (!last) {
-                const int f = it * 32 + lane;
-                bool hit = false;
-                R dx = 0, dy = 0, dz = 0, qj = 0;
-                // FP64: each pair once, only candidates with a larger sorted slot;
-                // FP32: every candidate but the bead itself
-                int gs = -1;
-                bool cand;
-                if constexpr (real_half<R>()) {
-                    if (f < total) {
-                        if (STAGED) {
-                            gs = stgslot[f];
-                        } else {
-                            while (hseg + 1 < nh && hoff[hseg + 1] <= f) ++hseg;
-                            gs = gst[hseg] + f - hoff[hseg];
-                        }
+    const int gpw = 32 / S, sub = lane & (S - 1), grp = lane / S;
+    // constants formed on the host: a conversion from double is an instruction on
+    // the part's few FP64 units (16 cycles of them per warp), as is every double
+    // operation of an FP32 kernel
+    const float Lf = g.rkf.L, hLf = g.rkf.hL;
+    // FP64: candidates above a band that covers the float error are out, the rest
+    // are decided in double
+    const float r2hi = HALF ? g.r2hi : g.rkf.rc2;
+    const float rT = 1.0f / (float)g.T;
+    const int ntd = g.ntd, rs = g.rs;
+    int cnt = 0, head = 0;   // noted candidates of this lane (FP32); ring fill and head (FP64)
+    for (int s0 = (blk.id * NW + warp) * gpw; s0 < nq; s0 += blk.n * NW * gpw) {
+        const int s = s0 + grp;
+        const bool own = s < nq;
+        float4 pf;
+        int tx = 0, ty = 0, tz = 0;
+        if (own) {
+            pf = spf[s];
+            const int pb = sb[s];   // grid base of the bead: its tile (base < 1024: the quotient is exact)
+            tx = (int)(((float)(pb & 1023) + 0.5f) * rT);
+            ty = (int)(((float)((pb >> 10) & 1023) + 0.5f) * rT);
+            tz = (int)(((float)((pb >> 20) & 1023) + 0.5f) * rT);
+        }
+        a.fx = a.fy = a.fz = (R)0;
+        // rows of tiles one after the other (uniform over the warp), each as its run
+        // inside the box and its run across the box face (if any bead of the warp
+        // has one), as long as the warp's longest; one more turn empties the lists
+        const int dz0 = ALL ? 0 : (HALF ? 0 : -rs), dz1 = ALL ? ntd - 1 : rs;
+        const int dy0 = ALL ? 0 : -rs, dy1 = ALL ? ntd - 1 : rs;
+        int dz = dz0, dy = HALF && !ALL ? 0 : dy0;
+        bool across = false;   // uniform: the row's part across the box face
+        int w0 = 0, wl = 0;
+        float hx = 0.0f, hy = 0.0f, hz = 0.0f;
+        while (true) {
+            const bool last = dz > dz1;
+            int j0 = 0, len = 0;
+            if (across) {
+                j0 = w0;
+                len = wl;
+            } else if (!last) {
+                int zz = dz, yy = dy;
+                hx = hy = hz = 0.0f;
+                if (!ALL) {
+                    zz += tz;
+                    yy += ty;
+                    if (zz < 0) { zz += ntd; hz = Lf; } else if (zz >= ntd) { zz -= ntd; hz = -Lf; }
+                    if (yy < 0) { yy += ntd; hy = Lf; } else if (yy >= ntd) { yy -= ntd; hy = -Lf; }
+                }
+                const int* ts = tstart + (zz * ntd + yy) * ntd;
+                // FP64, each pair once: the rows after the bead's own, and in its own
+                // row the beads after it
+                const bool home = HALF && !ALL && dz == 0 && dy == 0;
+                const int xa = ALL ? 0 : (home ? tx : tx - rs), xb = ALL ? ntd - 1 : tx + rs;
+                wl = 0;
+                if (own) {
+                    j0 = ts[max(xa, 0)];
+                    if (HALF && (home || ALL)) j0 = max(j0, s + 1);
+                    len = max(0, ts[min(xb, ntd - 1) + 1] - j0);
+                    if (!ALL && (xa < 0 || xb >= ntd)) {
+                        w0 = ts[xa < 0 ? xa + ntd : 0];
+                        wl = ts[xa < 0 ? ntd : xb - ntd + 1] - w0;
                     }
-                    cand = gs > s;
+                }
+            }
+            const int mlen = __reduce_max_sync(FULL, len);
+            const int image = (hz > 0.0f ? 18 : (hz < 0.0f ? 0 : 9)) + (hy > 0.0f ? 6 : (hy < 0.0f ? 0 : 3)) +
+                              (hx > 0.0f ? 2 : (hx < 0.0f ? 0 : 1));
+            for (int t0 = 0;;) {
+                if constexpr (HALF) {
+                    while (cnt >= 32) {
+                        __syncwarp();
+                        real_ring<ALL>(g, ring[(head + lane) & (kRealRing - 1)], sq, sw, F, a);
+                        __syncwarp();
+                        head += 32;
+                        cnt -= 32;
+                    }
                 } else {
-                    cand = f < total && f != self;
-                    if (cand && !STAGED) {
-                        while (hseg + 1 < nh && hoff[hseg + 1] <= f) ++hseg;
-                        gs = gst[hseg] + f - hoff[hseg];
+                    if (last || __any_sync(FULL, cnt > kRealQ - kRealU)) {
+                        real_drain(g, pf, list, cnt, sq, a);
+                        cnt = 0;
                     }
                 }
-                if (PRE && cand) {
-                    const float4 b = stgf[f];
-                    const float rx = min_image(pif.x, b.x, Lf, hLf);
-                    const float ry = min_image(pif.y, b.y, Lf, hLf);
-                    const float rz = min_image(pif.z, b.z, Lf, hLf);
-                    cand = dist2(rx, ry, rz) <= r2hi;
+                if (t0 >= mlen) break;
+                float4 b[kRealU];
+#pragma unroll
+                for (int u = 0; u < kRealU; ++u) {
+                    const int t = t0 + u * S + sub;
+                    if (t < len) b[u] = spf[j0 + t];
                 }
-                if (PRE) {
-                    hit = cand;   // decided exactly in the drain
-                } else if (cand) {
-                    V pj;
-                    pj = STAGED ? stg[f] : sq[gs];
-                    dx = min_image(pi.x, pj.x, L, hL);
-                    dy = min_image(pi.y, pj.y, L, hL);
-                    dz = min_image(pi.z, pj.z, L, hL);
-                    const R r2 = dist2(dx, dy, dz);
-                    hit = r2 < rc2 && r2 > (R)0;
-                    qj = pj.w;
-                }
-                const unsigned m = __ballot_sync(0xffffffffu, hit);
-                if (hit) {
-                    const int at = cnt + __popc(m & ((1u << lane) - 1u));
-                    if (ENUF_GUARD(g.check, at < 64, 7)) {   // the warp's queue holds 64
-                        if (PRE) {
-                            quj[at] = f;
+#pragma unroll
+                for (int u = 0; u < kRealU; ++u) {
+                    const int t = t0 + u * S + sub;
+                    bool hit = false;
+                    if (t < len) {
+                        float ex, ey, ez;
+                        if (ALL) {
+                            ex = min_image(pf.x, b[u].x, Lf, hLf);
+                            ey = min_image(pf.y, b[u].y, Lf, hLf);
+                            ez = min_image(pf.z, b[u].z, Lf, hLf);
                         } else {
-                            V e;
-                            e.x = dx; e.y = dy; e.z = dz; e.w = qj;
-                            qu[at] = e;
-                            if (real_half<R>()) quj[at] = gs;
+                            ex = __fadd_rn(__fsub_rn(pf.x, b[u].x), hx);
+                            ey = __fadd_rn(__fsub_rn(pf.y, b[u].y), hy);
+                            ez = __fadd_rn(__fsub_rn(pf.z, b[u].z), hz);
                         }
+                        const float r2 = dist2(ex, ey, ez);
+                        // FP64 decides exactly in the ring; FP32: the bead itself is at r2 = 0
+                        hit = HALF ? r2 <= r2hi : (r2 < r2hi && r2 > 0.0f);
+                    }
+                    if constexpr (HALF) {
+                        const unsigned m = __ballot_sync(FULL, hit);
+                        const int at = cnt + __popc(m & ((1u << lane) - 1u));
+                        if (hit && ENUF_GUARD(g.check, at < kRealRing, 7))
+                            ring[(head + at) & (kRealRing - 1)] = real_entry(s, j0 + t, image);
+                        cnt += __popc(m);
+                    } else if (hit && ENUF_GUARD(g.check, cnt < kRealQ, 7)) {
+                        list[32 * cnt] = j0 + t;
+                        ++cnt;
                     }
                 }
-                cnt += __popc(m);
+                t0 += kRealU * S;
             }
-            if (cnt >= 32 || (last && cnt > 0)) {
-                const int m = min(cnt, 32);
-                __syncwarp();
-                if constexpr (PRE)
-                    real_drain_staged<R, V>(g, pi, stg, stgslot, quj, m, lane, L, hL, rc2, kap, al, c2a, be, slater,
-                                            sw, F, fx, fy, fz, eacc, wacc);
-                else
-                    real_drain<R, V>(g, qu, quj, m, lane, pi.w, kap, al, c2a, be, slater, sw, F, fx, fy, fz, eacc,
-                                     wacc);
-                __syncwarp();
-                if (lane < cnt - m) {
-                    if (!PRE) qu[lane] = qu[m + lane];
-                    if (real_half<R>()) quj[lane] = quj[m + lane];
-                }
-                __syncwarp();
-                cnt -= m;
+            if (last) break;
+            if (!ALL && !across && __any_sync(FULL, wl > 0)) {
+                across = true;
+                hx = tx - rs < 0 ? Lf : -Lf;   // read by the lanes with wl > 0
+                continue;
+            }
+            across = false;
+            if (++dy > dy1) {
+                dy = dy0;
+                ++dz;
             }
         }
-        if constexpr (sizeof(R) == 8) {   // each lane's share as a global reduction: a warp
-            const int i = real_as_int(sw[s].w);   // sum would run 15 adds on the FP64 units
-            atomicAdd(&F[3 * i], fx);
-            atomicAdd(&F[3 * i + 1], fy);
-            atomicAdd(&F[3 * i + 2], fz);
-        } else {
-        fx = warp_sum_r(fx);
-        fy = warp_sum_r(fy);
-        fz = warp_sum_r(fz);
-        if (lane == 0) {   // a global reduction: other warps (as partners, or the DPD
-            const int i = real_as_int(sw[s].w);   // blocks of a fused pair launch) add into F too
-            atomicAdd(&F[3 * i], fx);
-            atomicAdd(&F[3 * i + 1], fy);
-            atomicAdd(&F[3 * i + 2], fz);
+        if constexpr (!HALF) {
+            for (int o = 1; o < S; o <<= 1) {
+                a.fx += __shfl_xor_sync(FULL, a.fx, o);
+                a.fy += __shfl_xor_sync(FULL, a.fy, o);
+                a.fz += __shfl_xor_sync(FULL, a.fz, o);
+            }
+            if (own && sub == 0) {   // a global reduction: the DPD blocks of a fused pair launch add into F too
+                const int i = real_as_int(sw[s].w);
+                atomicAdd(&F[3 * i], a.fx);
+                atomicAdd(&F[3 * i + 1], a.fy);
+                atomicAdd(&F[3 * i + 2], a.fz);
+            }
         }
-        }
+    }
+    if constexpr (HALF) {   // what is left in the ring (cnt < 32)
+        __syncwarp();
+        if (lane < cnt) real_ring<ALL>(g, ring[(head + lane) & (kRealRing - 1)], sq, sw, F, a);
     }
 }
 
-// Real-space erfc + Slater-correction pairs (Eq. 31, corrected Eq. 32,
-// Eq. 27-28). One CTA per grid tile: the beads of the tiles within r_c (the
-// stencil) are staged in shared memory with coalesced loads; one warp per
-// bead of the central tile runs over the staged candidates; accepted pairs
-// are compacted in a per-warp queue so the pair arithmetic (erfc and exp in
-// FP32, the tabulated kernel in FP64) runs on full warps.
+// spf: positions of the sorted beads in float (FP32: the sorted array itself).
 template <typename R>
 __device__ __forceinline__ void k_real_body(Geo g, const int* __restrict__ tstart,
                                                        const typename V4<R>::T* __restrict__ sq,
                                                        const typename V4<R>::T* __restrict__ sw,
+                                                       const int* __restrict__ sb, const float4* __restrict__ spf,
                                                        R* __restrict__ F, double* __restrict__ rpart, Blk blk) {
     pdl_enter();
-    using V = typename V4<R>::T;
-    constexpr int NW = kRealThreads / 32;
     extern __shared__ __align__(16) unsigned char smraw[];
-    constexpr int CAP = real_cap<R>();
-    V* stg = reinterpret_cast<V*>(smraw);                       // [CAP]
-    V* queue = stg + CAP;                                       // [NW][64]
-    float4* stgf = reinterpret_cast<float4*>(queue + NW * 64);  // [CAP] float positions (FP64 only)
-    int* hoff = reinterpret_cast<int*>(stgf + (sizeof(R) == 8 ? CAP : 0));   // [kRealHalo + 1]
-    int* gst = hoff + kRealHalo + 1;                            // [kRealHalo]
-    int* stgslot = gst + kRealHalo;                             // [CAP] sorted slot of each staged bead (FP64)
-    int* quj = stgslot + CAP;                                   // [NW][64] partner slots (FP64)
-    __shared__ int wtot[NW];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    V* qu = queue + warp * 64;
-    R eacc = 0, wacc = 0;
-    // Rounds of up to kRealRound tiles of this block's sequence whose halos fit
-    // the staging buffer together: each tile's halo is staged into its own
-    // segment, then the warps take the round's beads in turn across the tiles
-    // (a tile holds a few beads at large sizes, fewer than the warps), with no
-    // barrier between tiles. A tile whose halo alone does not fit runs by
-    // itself from global memory.
-    __shared__ int r_c0[kRealRound], r_c1[kRealRound], r_seg[kRealRound], r_self[kRealRound], r_tot[kRealRound];
-    __shared__ int r_cnt, r_used, r_next;
-    int tile = blk.id;
-    while (tile < g.ntiles) {
-        if (tid == 0) {
-            r_cnt = 0;
-            r_used = 0;
-        }
-        __syncthreads();
-        int t = tile;
-        while (t < g.ntiles) {
-            const int tx = t % g.ntd, ty = (t / g.ntd) % g.ntd, tz = t / (g.ntd * g.ntd);
-            int xlo, xc, ylo, yc, zlo, zc;
-            halo_dim(tx, g.rs, g.ntd, xlo, xc);
-            halo_dim(ty, g.rs, g.ntd, ylo, yc);
-            halo_dim(tz, g.rs, g.ntd, zlo, zc);
-            const int nh = xc * yc * zc;   // <= kRealHalo by construction of the plan
-            if (!ENUF_GUARD(g.check, nh <= kRealHalo, 6)) {   // uniform over the block
-                t += blk.n;
-                continue;
-            }
-            // halo tile ranges and their exclusive prefix (block scan, <= 4 per thread)
-            int cnt4[4], sum = 0;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int h = 4 * tid + k;
-                cnt4[k] = 0;
-                if (h < nh) {
-                    const int hx = h % xc, hy = (h / xc) % yc, hz = h / (xc * yc);
-                    const int ax = (xlo + hx + g.ntd) % g.ntd, ay = (ylo + hy + g.ntd) % g.ntd,
-                              az = (zlo + hz + g.ntd) % g.ntd;
-                    const int tt = (az * g.ntd + ay) * g.ntd + ax;
-                    const int st = tstart[tt];
-                    gst[h] = st;
-                    cnt4[k] = tstart[tt + 1] - st;
-                }
-                sum += cnt4[k];
-            }
-            int x = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
-            }
-            if (lane == 31) wtot[warp] = x;
-            __syncthreads();
-            int run = x - sum;
-            for (int w = 0; w < warp; ++w) run += wtot[w];
-            int total = 0;
-            for (int w = 0; w < NW; ++w) total += wtot[w];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int h = 4 * tid + k;
-                if (h < nh) hoff[h] = run;
-                run += cnt4[k];
-            }
-            if (tid == 0) hoff[nh] = total;
-            __syncthreads();
-            const int used = r_used, cnt = r_cnt;
-            const int c0 = tstart[t], c1 = tstart[t + 1];
-            const int hc = (((tz - zlo + g.ntd) % g.ntd) * yc + (ty - ylo + g.ntd) % g.ntd) * xc +
-                           (tx - xlo + g.ntd) % g.ntd;
-            if (total > CAP) {
-                if (cnt == 0) {   // this tile alone, candidates from global memory
-                    real_beads<R, false>(g, c0, c1, warp, hoff[hc], total, nh, stg, stgf, stgslot, hoff, gst, sq,
-                                         sw, qu, quj + warp * 64, F, eacc, wacc);
-                    t += blk.n;
-                }
-                break;   // an oversized halo closes the round
-            }
-            if (used + total > CAP) break;   // staged with the next round
-            for (int f = tid; f < total; f += blockDim.x) {
-                int lo = 0, hi = nh;   // last h with hoff[h] <= f
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if (hoff[mid] <= f) lo = mid; else hi = mid;
-                }
-                const int gsl = gst[lo] + f - hoff[lo];
-                const V v = sq[gsl];
-                stg[used + f] = v;
-                if (real_half<R>()) stgslot[used + f] = gsl;
-                if (sizeof(R) == 8) stgf[used + f] = make_float4((float)v.x, (float)v.y, (float)v.z, 0.f);
-            }
-            if (tid == 0) {
-                r_c0[cnt] = c0;
-                r_c1[cnt] = c1;
-                r_seg[cnt] = used;
-                r_self[cnt] = hoff[hc];
-                r_tot[cnt] = total;
-                r_cnt = cnt + 1;
-                r_used = used + total;
-            }
-            __syncthreads();   // hoff, gst and the counters are read again for the next tile
-            t += blk.n;
-            if (r_cnt == kRealRound) break;
-        }
-        if (tid == 0) r_next = t;
-        __syncthreads();
-        // the round's beads, warps in turn across its tiles
-        const int cnt = r_cnt;
-        int before = 0;
-        for (int k = 0; k < cnt; ++k) {
-            const int c0 = r_c0[k], c1 = r_c1[k], seg = r_seg[k];
-            const int woff = ((warp - before) % NW + NW) % NW;
-            real_beads<R, true>(g, c0, c1, woff, r_self[k], r_tot[k], 0, stg + seg, stgf + seg, stgslot + seg, hoff,
-                                gst, sq, sw, qu, quj + warp * 64, F, eacc, wacc);
-            before += c1 - c0;
-        }
-        tile = r_next;
-        __syncthreads();
-    }
-    double e = (double)eacc, w = (double)wacc;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int* list = reinterpret_cast<int*>(smraw) + warp * 32 * kRealQ + lane;   // FP32: entry k at 32 k
+    int2* ring = reinterpret_cast<int2*>(smraw) + warp * kRealRing;          // FP64
+    const int nq = tstart[g.ntiles];
+    // lanes per bead: as many as give every lane of the launch work
+    int S = 32;
+    while (S > 1 && (long long)nq * S > (long long)blk.n * kRealThreads) S >>= 1;
+    RealSum<R> a{(R)0, (R)0, (R)0, (R)0, (R)0};
+    if (2 * g.rs + 1 >= g.ntd)
+        real_sweep<R, true>(g, nq, S, tstart, sq, sw, sb, spf, list, ring, F, a, blk);
+    else
+        real_sweep<R, false>(g, nq, S, tstart, sq, sw, sb, spf, list, ring, F, a, blk);
+    double e = (double)a.e, w = (double)a.w;
     block_sum2(e, w);
     if (threadIdx.x == 0) {
         rpart[2 * blk.id] = e;
@@ -2450,11 +2388,12 @@ __device__ __forceinline__ void k_real_body(Geo g, const int* __restrict__ tstar
 }
 
 template <typename R>
-__global__ void __launch_bounds__(kRealThreads) k_real(Geo g, const int* __restrict__ tstart,
+__global__ void __launch_bounds__(kRealThreads, sizeof(R) == 4 ? 4 : 2) k_real(Geo g, const int* __restrict__ tstart,
                                                        const typename V4<R>::T* __restrict__ sq,
                                                        const typename V4<R>::T* __restrict__ sw,
+                                                       const int* __restrict__ sb, const float4* __restrict__ spf,
                                                        R* __restrict__ F, double* __restrict__ rpart) {
-    k_real_body<R>(g, tstart, sq, sw, F, rpart, Blk{(int)blockIdx.x, (int)gridDim.x});
+    k_real_body<R>(g, tstart, sq, sw, sb, spf, F, rpart, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // ---------------------------------------------------------------------------
@@ -3086,12 +3025,12 @@ __global__ void __launch_bounds__(kDpdThreads, sizeof(R) == 4 ? 4 : 2)
             const int* __restrict__ bnd, const uint64_t* __restrict__ stepp, R* __restrict__ F,
             double* __restrict__ dpart, int nd, Geo g, const int* __restrict__ tstart,
             const typename V4<R>::T* __restrict__ sq, const typename V4<R>::T* __restrict__ sw,
-            double* __restrict__ rpart) {
+            const int* __restrict__ sb, const float4* __restrict__ spf, double* __restrict__ rpart) {
     static_assert(kDpdThreads == kRealThreads, "one block size for both roles");
     if ((int)blockIdx.x < nd)
         k_dpd_body<R>(d, B, sp, sv, cstart, atab, pos, bnd, stepp, F, dpart, Blk{(int)blockIdx.x, nd});
     else
-        k_real_body<R>(g, tstart, sq, sw, F, rpart, Blk{(int)blockIdx.x - nd, (int)gridDim.x - nd});
+        k_real_body<R>(g, tstart, sq, sw, sb, spf, F, rpart, Blk{(int)blockIdx.x - nd, (int)gridDim.x - nd});
 }
 
 // Table 2 steps 0-2 (m = 1): v0 = v + lambda F dt; v += F dt/2; r += v dt; step += 1.

@@ -1,0 +1,57 @@
+"""The evaluation's kernels at the sizes where their work split can go wrong
+(lists that fill, rows across the box face, few beads, few tiles), against the
+FP64 CPU oracle with the parity tests' bounds."""
+import numpy as np
+import pytest
+
+import oracle as orc  # noqa: F401  (the oracle is built with the library)
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from test_gpu_enuf import TOL, Ref, _bead_max, _gpu, _inputs, _rel_rms, enuf  # noqa: E402,F401
+
+
+def _beads(L, nq, cluster, seed, solvent=37):
+    """nq charged beads, the first `cluster` of them in a unit ball around a box
+    corner (each within r_c of all others, across three faces), the rest
+    uniform, some on the faces; uncharged beads mixed in."""
+    rng = np.random.default_rng(seed)
+    pos = rng.uniform(0.0, L, (nq, 3))
+    pos[:cluster] = rng.uniform(-0.6, 0.6, (cluster, 3)) % L
+    if nq > cluster + 4:
+        pos[cluster] = [0.0, 0.5 * L, np.nextafter(L, 0.0)]
+        pos[cluster + 1] = [-0.25 * L, 1.5 * L, 2.0 * L]      # wrapped inside the library
+    q = np.where(np.arange(nq) % 2 == 0, 1.0, -1.0)
+    pos = np.concatenate([pos, rng.uniform(0.0, L, (solvent, 3))])
+    q = np.concatenate([q, np.zeros(solvent)])
+    order = rng.permutation(len(q))
+    return pos[order], q[order]
+
+
+BASE = dict(alpha=1.0, r_cut=3.0, beta=4.0, kappa=1.1, p=4)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("name,box", [
+    ("stencil_3_of_4", dict(L=12.0, M=20, tile=10)),      # rs = 1, 4 tiles: rows wrapped tile by tile
+    ("stencil_5_of_4", dict(L=9.0, M=16, tile=8)),        # rs = 2, 4 tiles: whole rows, minimum image
+    ("stencil_5_of_8", dict(L=20.0, M=32, tile=8)),       # rs = 2 with room
+    ("stencil_3_of_3", dict(L=9.0, M=18, tile=12)),       # exactly the tiles there are
+])
+@pytest.mark.parametrize("nq,cluster", [(2, 2), (33, 33), (200, 150), (1500, 90)])
+def test_real_space_lists(enuf, prec, name, box, nq, cluster):
+    """Lists that fill several times (150 beads within r_c of one another),
+    lanes per bead from 32 down, beads on and outside the faces: forces and the
+    real-space energy (beads on grid lines may take the other grid base in FP32,
+    which moves E_recip by the window's truncation)."""
+    P = dict(BASE, **box)
+    pos, q = _inputs(prec, *_beads(P["L"], nq, cluster, seed=nq + 7))
+    plan, F, E, Wv = _gpu(enuf, prec, P, pos, q)
+    assert plan.info.tile == P["tile"]
+    ref, t = Ref(P, pos, q), TOL[prec]
+    assert np.all(np.isfinite(F)) and np.all(F[q == 0] == 0.0)
+    assert _rel_rms(F, ref.F) < t["F"] and _bead_max(F, ref.F) < 100 * t["F"]
+    own = max(abs(ref.E[0]), abs(ref.E[2])) if prec == "fp32" else abs(ref.E[0])
+    assert abs(E[0] - ref.E[0]) <= t["E"] * own, (E, ref.E)
+    plan.close()
