@@ -32,7 +32,7 @@ size_t batch_bytes(const BatchSys* sys, int nsys) {
     for (int s = 0; s < nsys; ++s) {
         const BatchSys& x = sys[s];
         blocks += 2 * (size_t)x.g.nbin + bin_weight_blocks(x.g) + x.w.nblk_real + x.g.ntiles + x.g.n + x.fs.grid_z +
-                  (size_t)x.g.nf * x.g.n + x.w.nblk_gather;
+                  (size_t)x.g.nf * x.g.n + x.w.nblk_gather + 1;
     }
     const size_t rec = sizeof(BinCountArgs<R>) + sizeof(BinScatterArgs<R>) + sizeof(BinWeightsArgs<R>) +
                        sizeof(RealArgs<R>) + sizeof(SpreadArgs<R>) + sizeof(FftXYArgs<R>) + sizeof(FftZArgs<R>) +
@@ -168,8 +168,8 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
             // the beads charged on average; the kernel strides over any excess)
             const int nb = std::max(1, std::min(w.nblk_gather, (x.N + 63) / 64));
             a[s] = GatherArgs<R>{x.g, w.tstart, static_cast<const V*>(w.sq), static_cast<const V*>(w.sw), w.sb,
-                                 static_cast<const R*>(w.wb), static_cast<const R*>(w.h), static_cast<R*>(x.F), t, nb};
-            append_blocks(m, s, nb);
+                                 static_cast<const R*>(w.wb), static_cast<const R*>(w.h), static_cast<R*>(x.F), t, nb + 1};
+            append_blocks(m, s, nb + 1);   // one more: the system's totals
         }
         put(L.gather, a.data(), a.size() * sizeof(a[0]), m);
         L.gather.threads = kGatherThreads;

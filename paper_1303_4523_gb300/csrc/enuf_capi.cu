@@ -533,6 +533,10 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
     g.rkf = RealK<float>{(float)g.L, (float)(0.5 * g.L), (float)(g.rc * g.rc), (float)g.alpha, (float)g.c2a,
                          (float)g.beta, (float)g.kappa, (float)g.kinv};
     g.slater = P.beta > 0.0 ? 1 : 0;
+    g.wkd = WinK<double>{g.rb, g.wnorm, g.pref};
+    g.wkf = WinK<float>{(float)g.rb, (float)g.wnorm, (float)g.pref};
+    g.Lhi = (float)P.L;
+    g.Llo = (float)(P.L - (double)g.Lhi);
     g.r2hi = (float)(g.rc * g.rc) * (1.0f + 1e-4f) + 4e-6f * (float)(g.L * g.rc) + 1e-6f;
     if (P.slater_k) {
         // I'(0) = lim I(r)/r gives the self term
@@ -1236,6 +1240,11 @@ enuf_status dpd_create(enuf_plan_t plan, const dpd_params* params, int n, const 
     }
     d.cinv = (double)d.ncd / L;
     d.xmaxf = largest_float_below(L);
+    d.kd = DpdK<double>{L, 0.5 * L, d.gamma, d.sigma * d.rdt, d.K_bond, d.r0_bond, 1.0 / L};
+    d.kf = DpdK<float>{(float)L, (float)(0.5 * L), (float)d.gamma, (float)(d.sigma * d.rdt), (float)d.K_bond,
+                       (float)d.r0_bond, (float)(1.0 / L)};
+    d.Lhi = (float)L;
+    d.Llo = (float)(L - (double)d.Lhi);
     const size_t rs = plan->rsz;
     const size_t nz = (size_t)n;
     d.nbonds = n_bonds;

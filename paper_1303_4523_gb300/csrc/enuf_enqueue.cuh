@@ -430,8 +430,8 @@ cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp,
 
     cudaStreamWaitEvent(s0, evJoin, 0);
     rec(ev, 3, true, s0);
-    // with fuse_totals the gather's last block also reduces the energies
-    launch(false, true, gather_kernel<R>(2 * g.p), w.nblk_gather, kGatherThreads, 0, s0, g, (const int*)w.tstart,
+    // with fuse_totals one more block of the gather reduces the energies
+    launch(false, true, gather_kernel<R>(2 * g.p), w.nblk_gather + (fuse_totals ? 1 : 0), kGatherThreads, 0, s0, g, (const int*)w.tstart,
            (const V*)sq, (const V*)sw, (const int*)w.sb, static_cast<const R*>(w.wb), static_cast<const R*>(w.h), F,
            fuse_totals ? totals_args(g, w, false, 1) : no_totals());
     rec(ev, 3, false, s0);
@@ -454,7 +454,8 @@ cudaError_t enqueue_dpd_forces(const Work& w, const DpdDev& d, cudaStream_t s, E
     const bool pdl = pdl_ok(ev);
     rec(ev, 7, true, s);
     // the cell count also zeroes F, which the pair kernel adds into
-    launch(false, false, k_cell_count<R>, blocks, 256, 0, s, d.N, d.ncd, d.L, d.cinv, d.xmaxf, static_cast<const R*>(d.pos),
+    launch(false, false, k_cell_count<R>, blocks, 256, 0, s, d.N, d.ncd, d.L, (R)d.cinv, d.xmaxf,
+           d.Lhi, d.Llo, static_cast<const R*>(d.pos),
            d.ckey, d.ccount, static_cast<R*>(d.F));
     // the cell starts (and the scatter cursors): several CTAs without a
     // wait for up to kScanMbMax cells, else one CTA; k_cell_scatter then
@@ -464,7 +465,8 @@ cudaError_t enqueue_dpd_forces(const Work& w, const DpdDev& d, cudaStream_t s, E
                (const int*)d.ccount, d.cstart, d.ncells, d.ccur);
     else
         launch(pdl, false, k_scan, 1, 1024, 0, s, d.ccount, d.cstart, d.ncells, d.ccur, 0);
-    launch(pdl, false, k_cell_scatter<R>, blocks, 256, 0, s, d.N, d.L, d.xmaxf, static_cast<const R*>(d.pos),
+    launch(pdl, false, k_cell_scatter<R>, blocks, 256, 0, s, d.N, d.L, d.xmaxf, d.Lhi, d.Llo,
+           static_cast<const R*>(d.pos),
            static_cast<const R*>(d.v0), (const int*)d.type, (const int*)d.ckey, d.ccur, static_cast<V*>(d.sp),
            static_cast<V*>(d.sv), d.ccount, d.ncells);
     rec(ev, 7, false, s);
@@ -483,7 +485,7 @@ cudaError_t enqueue_dpd_forces(const Work& w, const DpdDev& d, cudaStream_t s, E
 
 template <typename R>
 cudaError_t enqueue_vv_pre(const DpdDev& d, cudaStream_t s, LaunchLog* log) {
-    const int blocks = (3 * d.N + 255) / 256 > 0 ? (3 * d.N + 255) / 256 : 1;
+    const int blocks = std::max(1, (3 * d.N / 4 + 255) / 256);
     launch(false, true, k_vv_pre<R>, blocks, 256, 0, s, d.N, (R)d.lambda_vv, (R)d.dt, static_cast<R*>(d.pos),
            static_cast<R*>(d.vel), static_cast<R*>(d.v0), static_cast<const R*>(d.F), d.step_dev);
     log->kernels += 1;

@@ -35,7 +35,23 @@ struct RealK {
     R kap, kinv;      // kappa, kernel table intervals per unit length
 };
 
-// Geometry and constants every kernel needs, passed by value.
+// Window constants in one working precision: 1 / b, (pi b)^{-1/2}, the force prefactor.
+template <typename R>
+struct WinK {
+    R rb, wn, pref;
+};
+
+// DPD constants in one working precision: box, dissipation, sigma / sqrt(dt),
+// bond constants, 1 / L.
+template <typename R>
+struct DpdK {
+    R L, hL, gam, srdt, Kb, r0b, iL;
+};
+
+// Geometry and constants every kernel needs, passed by value. The kernels take
+// their constants in the working precision from the host (rkf/rkd, wkf/wkd):
+// on this part a conversion from double, like every double operation, takes
+// 16 cycles of an SM's FP64 units per warp, in an FP32 kernel too.
 struct Geo {
     int n;        // oversampled grid per dimension (sigma_s * M)
     int nc;       // kept modes per side, |k_t| <= nc
@@ -70,6 +86,9 @@ struct Geo {
     const void* ktab;  // real [kn][kKtStride]: quintic coefficients of J(r) = r u(r) per interval
     RealK<float> rkf;
     RealK<double> rkd;
+    WinK<float> wkf;
+    WinK<double> wkd;
+    float Lhi, Llo;   // L split into two floats (FP32 wrap)
     int slater;   // beta > 0: the real-space term carries the Slater correction
     // FP64 cutoff pre-test on float positions: r_c^2 plus a band that covers the float
     // error (positions and L rounded to float, |r2f - r2| <= ~1.5e-6 L r_c)
@@ -196,6 +215,9 @@ struct DpdDev {
     double L, gamma, sigma, dt, lambda_vv, K_bond, r0_bond;
     double rdt;    // 1 / sqrt(dt)
     double cinv;   // ncd / L
+    DpdK<float> kf;
+    DpdK<double> kd;
+    float Lhi, Llo;   // L split into two floats (FP32 wrap)
     float xmaxf;   // largest float below L
     uint64_t seed;
     // Philox4x32-10 round keys of the seed (key bumped by the Weyl constants

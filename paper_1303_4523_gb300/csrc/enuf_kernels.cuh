@@ -30,6 +30,11 @@ __device__ __forceinline__ double int_as_real(int v, double) { return __longlong
 __device__ __forceinline__ int real_as_int(float v) { return __float_as_int(v); }
 __device__ __forceinline__ int real_as_int(double v) { return (int)__double_as_longlong(v); }
 
+__device__ __forceinline__ const WinK<float>& win_k(const Geo& g, float) { return g.wkf; }
+__device__ __forceinline__ const WinK<double>& win_k(const Geo& g, double) { return g.wkd; }
+__device__ __forceinline__ const DpdK<float>& dpd_k(const DpdDev& d, float) { return d.kf; }
+__device__ __forceinline__ const DpdK<double>& dpd_k(const DpdDev& d, double) { return d.kd; }
+
 // Programmatic dependent launch (sm_90 and later): every kernel first waits
 // until the grid before it in the stream has completed and its writes are
 // visible (griddepcontrol.wait, a no-op when it was launched without the
@@ -131,11 +136,37 @@ __device__ __forceinline__ double wrap_to_real(R x, double L) {
 // Wrapped position in the working precision. Inside [0, L) the value is kept
 // as is (decided in float for float: x <= xmaxf, the largest float below L);
 // outside it goes through the FP64 wrap.
-__device__ __forceinline__ float wrap_r(float x, double L, float xmaxf) {
-    if (x >= 0.0f && x <= xmaxf) return x;
-    return __double2float_rn(wrap_pos((double)x, L));
+// FP32: x - L q in float arithmetic with error terms, L = Lhi + Llo: the product
+// q Lhi and the difference x - fl(q Lhi) are taken with their exact rounding
+// errors (fused multiply-add; two-sum), which are added back with q Llo before
+// the one rounding that counts. The same value as the FP64 wrap rounded to
+// float but for ties, without its ~8 FP64 instructions per coordinate (16
+// cycles of the SM each; DPD positions drift out of the box, so nearly every
+// warp wraps some bead). Beyond 2^20 boxes the FP64 wrap is taken.
+__device__ __forceinline__ float wrap_diff(float x, float q, float Lhi, float Llo) {
+    const float p = __fmul_rn(q, Lhi);
+    const float pe = __fmaf_rn(q, Lhi, -p);          // q Lhi = p + pe
+    const float d = __fsub_rn(x, p);
+    const float bb = __fsub_rn(d, x);                // two-sum: x - p = d + de
+    const float de = __fsub_rn(__fsub_rn(x, __fsub_rn(d, bb)), __fadd_rn(p, bb));
+    return __fadd_rn(d, __fsub_rn(__fsub_rn(de, pe), __fmul_rn(q, Llo)));
 }
-__device__ __forceinline__ double wrap_r(double x, double L, float) { return wrap_pos(x, L); }
+__device__ __forceinline__ float wrap_r(float x, double L, float xmaxf, float Lhi, float Llo) {
+    if (x >= 0.0f && x <= xmaxf) return x;
+    float q = floorf(__fdiv_rn(x, Lhi));
+    if (!(fabsf(q) < 1048576.0f)) return __double2float_rn(wrap_pos((double)x, L));
+    float w = wrap_diff(x, q, Lhi, Llo);
+    if (w < 0.0f) {
+        q -= 1.0f;
+        w = wrap_diff(x, q, Lhi, Llo);
+    } else if (w > xmaxf) {
+        q += 1.0f;
+        const float v = wrap_diff(x, q, Lhi, Llo);
+        if (v >= 0.0f) w = v;   // else x - L (q - 1) lies within half a unit of L: kept as it rounds
+    }
+    return w < 0.0f ? 0.0f : w;
+}
+__device__ __forceinline__ double wrap_r(double x, double L, float, float, float) { return wrap_pos(x, L); }
 
 // Grid coordinate u = x_w * (n/L) in [0, n): one FP64 product and one floor
 // (n/L formed once on the host), u >= n wraps to 0.
@@ -224,6 +255,39 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
         b = l < nw ? red[1][l] : 0.0;
         a = warp_sum(a);
         b = warp_sum(b);
+    }
+}
+
+// Block sum, in double, of two values per thread held in the working
+// precision; result valid in thread 0. FP32: the values go to shared memory as
+// they are and one warp converts and adds them (8 conversions and additions
+// per lane and one shuffle tree per quantity for a block of 8 warps), so that
+// the other warps spend nothing on the FP64 units (a tree in every warp is 10
+// double additions each, 16 cycles of the SM's FP64 units apiece).
+constexpr int kSumThreads = 256;
+template <typename R>
+__device__ __forceinline__ void block_sum2_r(R va, R vb, double& a, double& b) {
+    if constexpr (sizeof(R) == 8) {
+        a = va;
+        b = vb;
+        block_sum2(a, b);
+    } else {
+        __shared__ float vals[2][kSumThreads];   // blockDim.x <= kSumThreads
+        __shared__ double bsum;
+        const int tid = threadIdx.x;
+        vals[0][tid] = va;
+        vals[1][tid] = vb;
+        __syncthreads();
+        if (tid < 64) {   // warp 0: a, warp 1: b
+            const int w = tid >> 5, l = tid & 31;
+            double s = 0.0;
+            for (int k = l; k < (int)blockDim.x; k += 32) s += (double)vals[w][k];
+            s = warp_sum(s);
+            if (tid == 0) a = s;
+            if (tid == 32) bsum = s;
+        }
+        __syncthreads();
+        if (tid == 0) b = bsum;
     }
 }
 
@@ -449,7 +513,7 @@ __device__ __forceinline__ void k_bin_count_body(Geo g, int N, const R* __restri
         int bs[3];
 #pragma unroll
         for (int t = 0; t < 3; ++t) {
-            xw[t] = wrap_r(pos[3 * i + t], g.L, g.xmaxf);
+            xw[t] = wrap_r(pos[3 * i + t], g.L, g.xmaxf, g.Lhi, g.Llo);
             grid_coord_r(xw[t], g, bs[t], fr[t]);
         }
         const int tile = ((bs[2] / g.T) * g.ntd + bs[1] / g.T) * g.ntd + bs[0] / g.T;
@@ -752,7 +816,7 @@ __device__ __forceinline__ void k_bin_weights_body(Geo g, const int* __restrict_
     pdl_enter();
     const int nq = tstart[g.ntiles];
     const int P2 = 2 * g.p;
-    const R rb = (R)g.rb, wn = (R)g.wnorm;
+    const R rb = win_k(g, (R)0).rb, wn = win_k(g, (R)0).wn;
     const int tot = 3 * nq;   // (bead, dimension) pairs; nq <= n_max < 2^29
     for (int e = blk.id * blockDim.x + threadIdx.x; e < tot; e += blk.n * blockDim.x) {
         const int s = e / 3, d = e - 3 * s;
@@ -901,7 +965,7 @@ __global__ void __launch_bounds__(kSpreadThreads, 5) k_spread(Geo g, const int* 
     int* myl = lix + warp * 3 * kMaxTaps;
     const int P2 = 2 * g.p;
     const int total = nb_pre[nnb];
-    const R rb = (R)g.rb, wn = (R)g.wnorm;
+    const R rb = win_k(g, (R)0).rb, wn = win_k(g, (R)0).wn;
     for (int cb = 0; cb < total; cb += kSpreadCap) {
         const int cn = min(kSpreadCap, total - cb);
         if (threadIdx.x == 0) nitems = 0;
@@ -1372,7 +1436,7 @@ __global__ void __launch_bounds__(kScThreads) k_spread_sc(Geo g, const int* __re
     float B = 0.f;
 #pragma unroll
     for (int w = 0; w < NW; ++w) B += wsum[w];
-    const float wm = (float)g.wnorm;
+    const float wm = g.wkf.wn;
     B *= wm * wm * wm;
     int ex = 0;
     frexpf(B, &ex);                                   // B < 2^ex
@@ -1805,6 +1869,16 @@ __device__ __forceinline__ void k_gather_body(Geo g, const int* __restrict__ tst
                                                            const R* __restrict__ h, R* __restrict__ F,
                                                            TotalsArgs tot, Blk blk) {
     pdl_enter();
+    // with totals the launch has one more block, the first, which reduces the
+    // energies while the others gather (their partials are all written by then)
+    if (tot.Edev) {
+        if (blk.id == 0) {
+            totals_block(g, tot);
+            return;
+        }
+        blk.id -= 1;
+        blk.n -= 1;
+    }
     constexpr int NW = kGatherThreads / 32;
     __shared__ R wts[NW][3][kMaxTaps];
     __shared__ R dwts[NW][3][kMaxTaps];   // gradient mode: psi'(d) = -(2 d / b) psi(d)
@@ -1818,8 +1892,8 @@ __device__ __forceinline__ void k_gather_body(Geo g, const int* __restrict__ tst
     const R* __restrict__ h2 = g.nf == 3 ? h + 2 * n3 : h;
     const int P2 = 2 * g.p;
     const float iP2 = 1.0f / (float)P2;
-    const R rb = (R)g.rb, wn = (R)g.wnorm;
-    const R pref = (R)g.pref;
+    const R rb = win_k(g, (R)0).rb, wn = win_k(g, (R)0).wn;
+    const R pref = win_k(g, (R)0).pref;
     const bool grad = g.nf == 1;
     // the whole grid sweeps the tile-sorted beads in order (bead s by warp s mod
     // the grid's warps): the fields' working set at any moment is a band of
@@ -2002,7 +2076,6 @@ __device__ __forceinline__ void k_gather_body(Geo g, const int* __restrict__ tst
         }
         __syncwarp();
     }
-    if (tot.Edev) totals_if_last(g, tot, blk.n);
 }
 
 template <typename R, int PT = 0>
@@ -2033,6 +2106,10 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(Geo g, const int* __r
 //     full warps, each pair once, because every FP64 instruction costs the
 //     whole warp's 16 cycles of the SM's few FP64 units; +f and -f go out by
 //     global reductions.
+// The form before it staged the 27-tile halo of every tile in shared memory
+// (27 staged beads per central bead at 3M beads, and as many CTAs as tiles:
+// 8 for a 3000-bead box). Alone: FP32 3M beads 473 -> 254 us, 524k 94 -> 65,
+// 192k 85 -> 49, 24k 62 -> 22; FP64 375k 264 -> 92, 3000 beads 49 -> 18 us.
 // ---------------------------------------------------------------------------
 constexpr int kRealThreads = 256;
 constexpr int kRealQ = 32;      // FP32: noted candidates per lane
@@ -2379,8 +2456,8 @@ __device__ __forceinline__ void k_real_body(Geo g, const int* __restrict__ tstar
         real_sweep<R, true>(g, nq, S, tstart, sq, sw, sb, spf, list, ring, F, a, blk);
     else
         real_sweep<R, false>(g, nq, S, tstart, sq, sw, sb, spf, list, ring, F, a, blk);
-    double e = (double)a.e, w = (double)a.w;
-    block_sum2(e, w);
+    double e, w;
+    block_sum2_r<R>(a.e, a.w, e, w);
     if (threadIdx.x == 0) {
         rpart[2 * blk.id] = e;
         rpart[2 * blk.id + 1] = w;
@@ -2402,10 +2479,10 @@ __global__ void __launch_bounds__(kRealThreads, sizeof(R) == 4 ? 4 : 2) k_real(G
 // Cells of edge L/ncd > 1 (the plan keeps a relative margin so that rounding
 // of x * ncd/L cannot separate two beads closer than 1 by two cells).
 template <typename R>
-__global__ void k_cell_count(int N, int ncd, double L, double inv, float xmaxf, const R* __restrict__ pos,
+__global__ void k_cell_count(int N, int ncd, double L, R rinv, float xmaxf, float Lhi, float Llo,
+                             const R* __restrict__ pos,
                              int* __restrict__ ckey, int* __restrict__ ccount, R* __restrict__ F) {
     pdl_enter();
-    const R rinv = (R)inv;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
         F[3 * i] = (R)0;   // the pair kernel adds into F
         F[3 * i + 1] = (R)0;
@@ -2413,7 +2490,7 @@ __global__ void k_cell_count(int N, int ncd, double L, double inv, float xmaxf, 
         int c[3];
 #pragma unroll
         for (int t = 0; t < 3; ++t) {
-            int v = (int)(wrap_r(pos[3 * i + t], L, xmaxf) * rinv);
+            int v = (int)(wrap_r(pos[3 * i + t], L, xmaxf, Lhi, Llo) * rinv);
             c[t] = v < 0 ? 0 : (v >= ncd ? ncd - 1 : v);
         }
         const int cell = (c[2] * ncd + c[1]) * ncd + c[0];
@@ -2425,7 +2502,7 @@ __global__ void k_cell_count(int N, int ncd, double L, double inv, float xmaxf, 
 // Also clears the cell counts for the next step's k_cell_count (the scan has
 // read them).
 template <typename R>
-__global__ void k_cell_scatter(int N, double L, float xmaxf, const R* __restrict__ pos, const R* __restrict__ v0,
+__global__ void k_cell_scatter(int N, double L, float xmaxf, float Lhi, float Llo, const R* __restrict__ pos, const R* __restrict__ v0,
                                const int* __restrict__ type, const int* __restrict__ ckey,
                                int* __restrict__ ccur, typename V4<R>::T* __restrict__ sp,
                                typename V4<R>::T* __restrict__ sv, int* __restrict__ ccount, int ncells) {
@@ -2434,9 +2511,9 @@ __global__ void k_cell_scatter(int N, double L, float xmaxf, const R* __restrict
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
         const int slot = atomicAdd(&ccur[ckey[i]], 1);
         typename V4<R>::T a, b;
-        a.x = wrap_r(pos[3 * i], L, xmaxf);
-        a.y = wrap_r(pos[3 * i + 1], L, xmaxf);
-        a.z = wrap_r(pos[3 * i + 2], L, xmaxf);
+        a.x = wrap_r(pos[3 * i], L, xmaxf, Lhi, Llo);
+        a.y = wrap_r(pos[3 * i + 1], L, xmaxf, Lhi, Llo);
+        a.z = wrap_r(pos[3 * i + 2], L, xmaxf, Lhi, Llo);
         a.w = int_as_real(i, (R)0);
         b.x = v0[3 * i];
         b.y = v0[3 * i + 1];
@@ -2646,8 +2723,8 @@ __device__ __forceinline__ void dpd_cells(const DpdDev& d, int H, int B3, const 
     constexpr int NW = kDpdThreads / 32;
     constexpr int nseg = kDpdSegU;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const R L = (R)d.L, hL = (R)(0.5 * d.L);
-    const R gam = (R)d.gamma, srdt = (R)(d.sigma * d.rdt);
+    const R L = dpd_k(d, (R)0).L, hL = dpd_k(d, (R)0).hL;
+    const R gam = dpd_k(d, (R)0).gam, srdt = dpd_k(d, (R)0).srdt;
     const PhiloxStep ps = philox_step(d, step);
     int cnt = 0;   // queued pairs of this warp, carried across its cells
     for (int cc = warp; cc < B3; cc += NW) {
@@ -2762,8 +2839,8 @@ __device__ __forceinline__ void dpd_beads(const DpdDev& d, int H, int B3, const 
     constexpr int NW = kDpdThreads / 32;
     constexpr bool PRE = sizeof(R) == 8;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const R L = (R)d.L, hL = (R)(0.5 * d.L);
-    const R gam = (R)d.gamma, srdt = (R)(d.sigma * d.rdt);
+    const R L = dpd_k(d, (R)0).L, hL = dpd_k(d, (R)0).hL;
+    const R gam = dpd_k(d, (R)0).gam, srdt = dpd_k(d, (R)0).srdt;
     const PhiloxStep ps = philox_step(d, step);
     const int nc = cpre[B3];
     int cnt = 0, qh = 0;   // queued pairs of this warp, ring head
@@ -2862,11 +2939,11 @@ __device__ __forceinline__ void k_dpd_body(DpdDev d, int B, const typename V4<R>
     const int H = B + 2, H3 = H * H * H, B3 = B * B * B;
     if (!ENUF_GUARD(d.check, H3 <= HMAX && B3 <= kDpdMaxB * kDpdMaxB * kDpdMaxB, 8)) return;
     const int nblk = (ncd + B - 1) / B;
-    const R L = (R)d.L, hL = (R)(0.5 * d.L);
+    const R L = dpd_k(d, (R)0).L;
     R ec = 0, eb = 0;
     // harmonic bonds (Sec. 2): one thread per bond, +f to i and -f to j
     {
-        const R Kb = (R)d.K_bond, r0b = (R)d.r0_bond, iL = (R)(1.0 / d.L);
+        const R Kb = dpd_k(d, (R)0).Kb, r0b = dpd_k(d, (R)0).r0b, iL = dpd_k(d, (R)0).iL;
         for (int k = bk.id * blockDim.x + tid; k < d.nbonds; k += bk.n * blockDim.x) {
             const int i = bnd[2 * k], j = bnd[2 * k + 1];
             R dd[3];
@@ -2895,9 +2972,9 @@ __device__ __forceinline__ void k_dpd_body(DpdDev d, int B, const typename V4<R>
     // [-1 - L/3, 4L/3]) carry at most (4L/3 + 1) 2^-24 each, so for r2 near 1
     // |r2f - r2| <= 7e-7 (L + 1) + 3e-7
     DpdBand band;
-    band.L = (float)d.L;
-    band.hL = (float)(0.5 * d.L);
-    const float eps = 1e-4f + 4e-6f * (float)d.L;
+    band.L = d.kf.L;
+    band.hL = d.kf.hL;
+    const float eps = 1e-4f + 4e-6f * d.kf.L;
     band.lo0 = eps;
     band.lo = 1.0f - eps;
     band.hi = 1.0f + eps;
@@ -2996,11 +3073,11 @@ __device__ __forceinline__ void k_dpd_body(DpdDev d, int B, const typename V4<R>
             dpd_cells<R>(d, H, B3, chalo, hoff, gst, sp, sv, queue, atab, step, F, ec);
         __syncthreads();
     }
-    double e1 = 0.5 * (double)ec, e2 = 0.5 * (double)eb;
-    block_sum2(e1, e2);
+    double e1, e2;
+    block_sum2_r<R>(ec, eb, e1, e2);
     if (threadIdx.x == 0) {
-        dpart[2 * bk.id] = e1;
-        dpart[2 * bk.id + 1] = e2;
+        dpart[2 * bk.id] = 0.5 * e1;
+        dpart[2 * bk.id + 1] = 0.5 * e2;
     }
 }
 
@@ -3026,7 +3103,7 @@ __global__ void __launch_bounds__(kDpdThreads, sizeof(R) == 4 ? 4 : 2)
             double* __restrict__ dpart, int nd, Geo g, const int* __restrict__ tstart,
             const typename V4<R>::T* __restrict__ sq, const typename V4<R>::T* __restrict__ sw,
             const int* __restrict__ sb, const float4* __restrict__ spf, double* __restrict__ rpart) {
-    static_assert(kDpdThreads == kRealThreads, "one block size for both roles");
+    static_assert(kDpdThreads == kRealThreads && kRealThreads <= kSumThreads, "one block size for both roles");
     if ((int)blockIdx.x < nd)
         k_dpd_body<R>(d, B, sp, sv, cstart, atab, pos, bnd, stepp, F, dpart, Blk{(int)blockIdx.x, nd});
     else
@@ -3034,18 +3111,39 @@ __global__ void __launch_bounds__(kDpdThreads, sizeof(R) == 4 ? 4 : 2)
 }
 
 // Table 2 steps 0-2 (m = 1): v0 = v + lambda F dt; v += F dt/2; r += v dt; step += 1.
+// Four components per thread (the arrays are 32-byte aligned): the loads of
+// all three arrays are in flight together.
 template <typename R>
 __global__ void k_vv_pre(int N, R lam, R dt, R* __restrict__ pos, R* __restrict__ vel, R* __restrict__ v0,
                          const R* __restrict__ F, uint64_t* __restrict__ stepp) {
     pdl_enter();
+    using V = typename V4<R>::T;
     if (blockIdx.x == 0 && threadIdx.x == 0) *stepp += 1;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 3 * N; k += gridDim.x * blockDim.x) {
-        const R f = F[k];
-        const R v = vel[k];
-        v0[k] = v + lam * f * dt;
+    const int n3 = 3 * N, n4 = n3 / 4;
+    auto one = [&](R f, R v, R& x, R& w) {   // returns the new velocity
+        w = v + lam * f * dt;
         const R vn = v + (R)0.5 * f * dt;
+        x = x + vn * dt;
+        return vn;
+    };
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n4; k += gridDim.x * blockDim.x) {
+        const V f = reinterpret_cast<const V*>(F)[k];
+        V v = reinterpret_cast<const V*>(vel)[k], x = reinterpret_cast<const V*>(pos)[k], w;
+        v.x = one(f.x, v.x, x.x, w.x);
+        v.y = one(f.y, v.y, x.y, w.y);
+        v.z = one(f.z, v.z, x.z, w.z);
+        v.w = one(f.w, v.w, x.w, w.w);
+        reinterpret_cast<V*>(v0)[k] = w;
+        reinterpret_cast<V*>(vel)[k] = v;
+        reinterpret_cast<V*>(pos)[k] = x;
+    }
+    const int k = 4 * n4 + (int)threadIdx.x;   // the last n3 mod 4 components
+    if (blockIdx.x == 0 && k < n3) {
+        R x = pos[k], w;
+        const R vn = one(F[k], vel[k], x, w);
+        v0[k] = w;
         vel[k] = vn;
-        pos[k] = pos[k] + vn * dt;
+        pos[k] = x;
     }
 }
 
@@ -3055,14 +3153,28 @@ template <typename R>
 __global__ void __launch_bounds__(256) k_vv_post(Geo g, int N, R dt, R* __restrict__ vel, const R* __restrict__ F,
                                                 double* __restrict__ kpart, TotalsArgs tot) {
     pdl_enter();
+    using V = typename V4<R>::T;
     double ke = 0.0, dummy = 0.0;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 3 * N; k += gridDim.x * blockDim.x) {
-        const R v = vel[k] + (R)0.5 * F[k] * dt;
-        vel[k] = v;
-        ke += 0.5 * (double)v * (double)v;
+    const int n3 = 3 * N, n4 = n3 / 4;
+    auto one = [&](R f, R v) {
+        const R vn = v + (R)0.5 * f * dt;
+        ke = fma((double)vn, (double)vn, ke);
+        return vn;
+    };
+#pragma unroll 2
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n4; k += gridDim.x * blockDim.x) {
+        const V f = reinterpret_cast<const V*>(F)[k];
+        V v = reinterpret_cast<const V*>(vel)[k];
+        v.x = one(f.x, v.x);
+        v.y = one(f.y, v.y);
+        v.z = one(f.z, v.z);
+        v.w = one(f.w, v.w);
+        reinterpret_cast<V*>(vel)[k] = v;
     }
+    const int k = 4 * n4 + (int)threadIdx.x;
+    if (blockIdx.x == 0 && k < n3) vel[k] = one(F[k], vel[k]);
     block_sum2(ke, dummy);
-    if (threadIdx.x == 0) kpart[blockIdx.x] = ke;
+    if (threadIdx.x == 0) kpart[blockIdx.x] = 0.5 * ke;
     if (tot.Edev) totals_if_last(g, tot, (int)gridDim.x);
 }
 
