@@ -24,50 +24,48 @@ struct BinCountArgs {
     const R* pos;
     const R* q;
     int* cnt_blk;
-    int* bhist;
-    int* ctile;
+    int* tcnt;
+    int* crank;
     typename V4<R>::T* cpos;
     typename V4<R>::T* cfrac;
     int* cbase;
     R* Fzero;
     double* qpart;
-    int* ticket;
-    int* boff;
-    int* tstart;
     int nblk;
 };
 template <typename R>
-__global__ void __launch_bounds__(1024) kb_bin_count(const BinCountArgs<R>* __restrict__ tab, const int* __restrict__ cmap) {
+__global__ void __launch_bounds__(kBinThreads) kb_bin_count(const BinCountArgs<R>* __restrict__ tab, const int* __restrict__ cmap) {
     pdl_enter();
     const int m = cmap[blockIdx.x];
     const BinCountArgs<R>& a = tab[m >> kBatchShift];
-    k_bin_count_body<R>(a.g, a.N, a.pos, a.q, a.cnt_blk, a.bhist, a.ctile, a.cpos, a.cfrac, a.cbase, a.Fzero, a.qpart,
-                        a.ticket, a.boff, a.tstart, Blk{m & kBatchLocal, a.nblk});
+    k_bin_count_body<R>(a.g, a.N, a.pos, a.q, a.cnt_blk, a.tcnt, a.crank, a.cpos, a.cfrac, a.cbase, a.Fzero, a.qpart,
+                        Blk{m & kBatchLocal, a.nblk});
 }
 
 template <typename R>
 struct BinScatterArgs {
     Geo g;
     const int* cnt_blk;
-    const int* ctile;
+    int* tcnt;
+    int* tstart;
+    const int* crank;
     const typename V4<R>::T* cpos;
     const typename V4<R>::T* cfrac;
     const int* cbase;
-    const int* boff;
-    const int* tstart;
     typename V4<R>::T* sq;
     typename V4<R>::T* sw;
     int* sb;
+    int* ticket;
     int nblk;
 };
 template <typename R>
-__global__ void __launch_bounds__(1024) kb_bin_scatter(const BinScatterArgs<R>* __restrict__ tab,
+__global__ void __launch_bounds__(kBinThreads) kb_bin_scatter(const BinScatterArgs<R>* __restrict__ tab,
                                                       const int* __restrict__ cmap) {
     pdl_enter();
     const int m = cmap[blockIdx.x];
     const BinScatterArgs<R>& a = tab[m >> kBatchShift];
-    k_bin_scatter_body<R>(a.g, a.cnt_blk, a.ctile, a.cpos, a.cfrac, a.cbase, a.boff, a.tstart, a.sq, a.sw, a.sb, nullptr,
-                          Blk{m & kBatchLocal, a.nblk});
+    k_bin_scatter_body<R, false>(a.g, a.cnt_blk, a.tcnt, a.tstart, a.crank, a.cpos, a.cfrac, a.cbase, a.sq, a.sw, a.sb,
+                                 nullptr, nullptr, a.ticket, Blk{m & kBatchLocal, a.nblk});
 }
 
 template <typename R>

@@ -21,7 +21,9 @@ inline void append_blocks(std::vector<int>& cmap, int sys, int nblk) {
 // instead of the launch's whole width (the kernel strides over any excess).
 inline int batch_real_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_real, (x.N + 511) / 512)); }
 
-inline int bin_count_smem(const Geo& g) { return (g.ntiles + g.chunk) * (int)sizeof(int); }
+// Window-weight blocks of one system: a thread per (bead, dimension) for a
+// sixth of the beads (the kernel strides over any excess).
+inline int batch_weight_blocks(const BatchSys& x) { return std::max(1, (x.N + 511) / 512); }
 
 }  // namespace batch_detail
 
@@ -31,7 +33,7 @@ size_t batch_bytes(const BatchSys* sys, int nsys) {
     size_t blocks = 0;
     for (int s = 0; s < nsys; ++s) {
         const BatchSys& x = sys[s];
-        blocks += 2 * (size_t)x.g.nbin + bin_weight_blocks(x.g) + x.w.nblk_real + x.g.ntiles + x.g.n + x.fs.grid_z +
+        blocks += 2 * (size_t)x.g.nbin + batch_weight_blocks(x) + x.w.nblk_real + x.g.ntiles + x.g.n + x.fs.grid_z +
                   (size_t)x.g.nf * x.g.n + x.w.nblk_gather + 1;
     }
     const size_t rec = sizeof(BinCountArgs<R>) + sizeof(BinScatterArgs<R>) + sizeof(BinWeightsArgs<R>) +
@@ -70,25 +72,25 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
             const BatchSys& x = sys[s];
             const Geo& g = x.g;
             const Work& w = x.w;
-            a[s] = BinCountArgs<R>{g, x.N, static_cast<const R*>(x.pos), static_cast<const R*>(x.q), w.cnt_blk, w.bhist,
-                                   w.ctile, static_cast<V*>(w.cpos), static_cast<V*>(w.cfrac), w.cbase,
-                                   static_cast<R*>(x.F), w.part + w.off_q, w.ticket, w.boff, w.tstart, g.nbin};
-            b[s] = BinScatterArgs<R>{g, w.cnt_blk, w.ctile, static_cast<const V*>(w.cpos),
-                                     static_cast<const V*>(w.cfrac), w.cbase, w.boff, w.tstart,
-                                     static_cast<V*>(w.sq), static_cast<V*>(w.sw), w.sb, g.nbin};
+            a[s] = BinCountArgs<R>{g, x.N, static_cast<const R*>(x.pos), static_cast<const R*>(x.q), w.cnt_blk, w.tcnt,
+                                   w.crank, static_cast<V*>(w.cpos), static_cast<V*>(w.cfrac), w.cbase,
+                                   static_cast<R*>(x.F), w.part + w.off_q, g.nbin};
+            b[s] = BinScatterArgs<R>{g, w.cnt_blk, w.tcnt, w.tstart, w.crank, static_cast<const V*>(w.cpos),
+                                     static_cast<const V*>(w.cfrac), w.cbase, static_cast<V*>(w.sq),
+                                     static_cast<V*>(w.sw), w.sb, w.ticket, g.nbin};
             c[s] = BinWeightsArgs<R>{g, w.tstart, static_cast<const V*>(w.sw), static_cast<R*>(w.wb),
-                                     bin_weight_blocks(g)};
+                                     batch_weight_blocks(x)};
             append_blocks(ma, s, g.nbin);
             append_blocks(mb, s, g.nbin);
             append_blocks(mc, s, c[s].nblk);
-            L.bin_count.smem = std::max(L.bin_count.smem, bin_count_smem(g));
-            L.bin_scatter.smem = std::max(L.bin_scatter.smem, g.ntiles * (int)sizeof(int));
+            L.bin_count.smem = std::max(L.bin_count.smem, g.chunk * (int)sizeof(int));
+            L.bin_scatter.smem = std::max(L.bin_scatter.smem, (g.ntiles + 1) * (int)sizeof(int));
         }
         put(L.bin_count, a.data(), a.size() * sizeof(a[0]), ma);
         put(L.bin_scatter, b.data(), b.size() * sizeof(b[0]), mb);
         put(L.bin_weights, c.data(), c.size() * sizeof(c[0]), mc);
-        L.bin_count.threads = 1024;
-        L.bin_scatter.threads = 1024;
+        L.bin_count.threads = kBinThreads;
+        L.bin_scatter.threads = kBinThreads;
         L.bin_weights.threads = 256;
     }
     {

@@ -331,21 +331,11 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
         if (hs * hs * hs > 1024)
             return fail(plan, ENUF_ERR_UNSUPPORTED, "real-space stencil of %d^3 tiles too large (r_cut/tile)", hs);
     }
-    // binning blocks: the count kernel holds a chunk-sized list plus the tile
-    // histogram in shared memory (<= kBinSmem), one block per SM: chunks of at
-    // least 2048 beads, as few whole waves of kSMs blocks as the list allows
-    // (a partial second wave doubled the kernel's time at 3M beads)
-    {
-        const int room = kBinSmem / 4 - g.ntiles;   // list entries that fit beside the histogram
-        int waves = 1;
-        // chunks are whole groups of 32 beads (the count kernel deals groups to its blocks)
-        auto chunk_for = [&](int w) { return std::max(2048, ((n_max + w * kSMs - 1) / (w * kSMs) + 31) & ~31); };
-        g.chunk = chunk_for(1);
-        while (g.chunk > room && g.chunk > 2048) g.chunk = chunk_for(++waves);
-    }
+    // binning blocks: up to four per SM, shares of 512 to 8192 beads (whole groups
+    // of 32; the count kernel lists a share's charged beads in shared memory)
+    g.chunk = std::min(8192, std::max(512, ((n_max + 4 * kSMs - 1) / (4 * kSMs) + 31) & ~31));
     g.nbin = std::max(1, (n_max + g.chunk - 1) / g.chunk);
-    // the last binning block walks ntiles x nbin counts: only when that is small
-    g.bin_last = (long long)g.ntiles * g.nbin <= 65536 ? 1 : 0;
+    g.bin_scan = g.ntiles <= kBinScanTiles ? 1 : 0;
     g.kmask = P.kmask;
     g.nf = P.deriv ? 1 : 3;
     g.L = P.L;
@@ -355,6 +345,7 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
     g.rc = P.r_cut;
     g.b = 2.0 * P.sigma_s * P.p / ((2.0 * P.sigma_s - 1.0) * M_PI);
     g.wnorm = 1.0 / std::sqrt(M_PI * g.b);
+    for (int m = 0; m <= P.p; ++m) g.e3[m] = g.wnorm * std::exp(-(double)m * m / g.b);
 
     // FFT passes: enough lines per CTA to keep ~2 CTAs per SM busy, within a
     // 64 KB shared-memory budget; threads ~ one butterfly of radix 4 per line point
@@ -575,9 +566,8 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
     auto take = [&](size_t b) { size_t o = off; off += align256(b); return o; };
     // record offsets in w as integers for now (cast later)
     const size_t ncmp = (size_t)g.nbin * g.chunk;   // compacted-bead slots
-    size_t o_cnt = take((size_t)g.nbin * 4), o_bhist = take((size_t)g.nbin * g.ntiles * 4),
-           o_boff = take((size_t)g.nbin * g.ntiles * 4), o_ttot = take((size_t)g.ntiles * 4),
-           o_tstart = take((size_t)(g.ntiles + 1) * 4), o_tk = take(16), o_ck = take(16), o_ctile = take(ncmp * 4),
+    size_t o_cnt = take((size_t)g.nbin * 4), o_tcnt = take((size_t)g.ntiles * 4),
+           o_tstart = take((size_t)(g.ntiles + 1) * 4), o_tk = take(16), o_ck = take(16), o_crank = take(ncmp * 4),
            o_cpos = take(ncmp * 4 * esz),
            o_cfrac = take(ncmp * 4 * esz), o_cbase = take(ncmp * 4),
            o_sq = take(nm * 4 * esz), o_sw = take(nm * 4 * esz), o_sb = take(nm * 4),
@@ -600,8 +590,8 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
         plan->fs = fs;
         plan->fp = fp;
         // stash offsets; bound to the allocation in bind()
-        w.cnt_blk = (int*)o_cnt; w.bhist = (int*)o_bhist; w.boff = (int*)o_boff; w.ttot = (int*)o_ttot;
-        w.tstart = (int*)o_tstart; w.ticket = (int*)o_tk; w.check = (unsigned int*)o_ck; w.ctile = (int*)o_ctile;
+        w.cnt_blk = (int*)o_cnt; w.tcnt = (int*)o_tcnt;
+        w.tstart = (int*)o_tstart; w.ticket = (int*)o_tk; w.check = (unsigned int*)o_ck; w.crank = (int*)o_crank;
         w.cpos = (void*)o_cpos; w.cfrac = (void*)o_cfrac;
         w.cbase = (int*)o_cbase;
         w.sq = (void*)o_sq; w.sw = (void*)o_sw; w.sb = (int*)o_sb; w.spf = (float4*)o_spf; w.wb = (void*)o_wb; w.grid = (void*)o_grid;
@@ -618,8 +608,8 @@ void bind(enuf_plan_t p) {
     char* b = static_cast<char*>(p->dmem);
     Work& w = p->w;
     auto at = [&](auto ptr) { return reinterpret_cast<decltype(ptr)>(b + reinterpret_cast<size_t>(ptr)); };
-    w.cnt_blk = at(w.cnt_blk); w.bhist = at(w.bhist); w.boff = at(w.boff); w.ttot = at(w.ttot);
-    w.tstart = at(w.tstart); w.ticket = at(w.ticket); w.check = at(w.check); w.ctile = at(w.ctile);
+    w.cnt_blk = at(w.cnt_blk); w.tcnt = at(w.tcnt);
+    w.tstart = at(w.tstart); w.ticket = at(w.ticket); w.check = at(w.check); w.crank = at(w.crank);
     w.cpos = at(w.cpos); w.cfrac = at(w.cfrac);
     w.cbase = at(w.cbase);
     w.sq = at(w.sq); w.sw = at(w.sw); w.sb = at(w.sb);
@@ -1422,7 +1412,7 @@ namespace {
 bool batch_plan_ok(const enuf_plan_s* p) {
     const int T = p->g.T;
     const bool col = T == 8 || T == 10 || T == 12 || T == 16 || T == 20 || T == 24;
-    return p->prec == ENUF_FP32 && p->fs.two && p->fs.fused && p->fs.spread == 1 && col && p->g.bin_last &&
+    return p->prec == ENUF_FP32 && p->fs.two && p->fs.fused && p->fs.spread == 1 && col && p->g.bin_scan &&
            p->w.wb != nullptr;
 }
 
@@ -1653,15 +1643,17 @@ extern "C" enuf_status enuf_spread_noalloc(const enuf_params* params, int n, con
         fprintf(stderr, "enuf_spread_noalloc: %s\n", geo.err);
         return st;
     }
+    // shares of 2048 beads: the binning's scratch must fit the fixed region
+    geo.g.chunk = 2048;
+    geo.g.nbin = std::max(1, (n + 2047) / 2048);
     const Geo& g = geo.g;
     const size_t esz = geo.rsz;
     const size_t nm = (size_t)std::max(n, 1);
     size_t off = 0;
     auto take = [&](size_t b) { size_t o = off; off += align256(b); return o; };
     const size_t ncmp = (size_t)g.nbin * g.chunk;
-    const size_t o_cnt = take((size_t)g.nbin * 4), o_bhist = take((size_t)g.nbin * g.ntiles * 4),
-                 o_boff = take((size_t)g.nbin * g.ntiles * 4), o_ttot = take((size_t)g.ntiles * 4),
-                 o_tstart = take((size_t)(g.ntiles + 1) * 4), o_tk = take(16), o_ctile = take(ncmp * 4),
+    const size_t o_cnt = take((size_t)g.nbin * 4), o_tk = take(16), o_tcnt = take((size_t)g.ntiles * 4),
+                 o_tstart = take((size_t)(g.ntiles + 1) * 4), o_crank = take(ncmp * 4),
                  o_cpos = take(ncmp * 4 * esz), o_cfrac = take(ncmp * 4 * esz), o_cbase = take(ncmp * 4),
                  o_sq = take(nm * 4 * esz), o_sw = take(nm * 4 * esz), o_sb = take(nm * 4),
                  o_part = take((size_t)2 * g.nbin * 8);
@@ -1695,12 +1687,10 @@ extern "C" enuf_status enuf_spread_noalloc(const enuf_params* params, int n, con
     char* b = static_cast<char*>(g_noalloc_addr[dev]);
     Work w{};
     w.cnt_blk = reinterpret_cast<int*>(b + o_cnt);
-    w.bhist = reinterpret_cast<int*>(b + o_bhist);
-    w.boff = reinterpret_cast<int*>(b + o_boff);
-    w.ttot = reinterpret_cast<int*>(b + o_ttot);
+    w.tcnt = reinterpret_cast<int*>(b + o_tcnt);   // cleared below with the ticket
     w.tstart = reinterpret_cast<int*>(b + o_tstart);
     w.ticket = reinterpret_cast<int*>(b + o_tk);   // cleared below, before the binning counts on it
-    w.ctile = reinterpret_cast<int*>(b + o_ctile);
+    w.crank = reinterpret_cast<int*>(b + o_crank);
     w.cpos = b + o_cpos;
     w.cfrac = b + o_cfrac;
     w.cbase = reinterpret_cast<int*>(b + o_cbase);
@@ -1711,9 +1701,10 @@ extern "C" enuf_status enuf_spread_noalloc(const enuf_params* params, int n, con
     w.off_q = 0;
     EvalArgs a{n, pos, q, nullptr, false};
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    // the binning's arrival counter must start at zero: a call that stopped
-    // part way could have left it set (a memset node allocates nothing)
-    e = cudaMemsetAsync(w.ticket, 0, 16, s);
+    // the binning's arrival counter and the tile counters after it must start at
+    // zero: a call that stopped part way could have left them set (a memset node
+    // allocates nothing)
+    e = cudaMemsetAsync(w.ticket, 0, o_tstart - o_tk, s);
     if (e == cudaSuccess)
         e = geo.prec == ENUF_FP32 ? enqueue_spread_only<float>(g, w, a, grid, s)
                                   : enqueue_spread_only<double>(g, w, a, grid, s);

@@ -13,8 +13,6 @@
 
 namespace enuf {
 
-constexpr int kBinThreads = 1024;
-
 inline void rec(Events* ev, int stage, bool start, cudaStream_t s) {
     if (ev && ev->on)
         cudaEventRecordWithFlags(start ? ev->start[stage] : ev->stop[stage], s, cudaEventRecordExternal);
@@ -93,12 +91,6 @@ cudaError_t configure_kernels(int max_smem) {
         cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
         if (r != cudaSuccess) e = r;
     };
-    set((const void*)k_bin_count<R>);
-    // the count kernel may hold a whole SM's shared memory (its chunk list and
-    // the tile histogram; see the plan's chunk rule)
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute((const void*)k_bin_count<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBinSmem);
-    set((const void*)k_bin_scatter<R>);
     set((const void*)k_spread<R>);
     set((const void*)k_fft_x<R>);
     set((const void*)k_fft_y<R>);
@@ -153,11 +145,6 @@ cudaError_t configure_kernels(int max_smem) {
         set((const void*)k_spread_sc<16, 8>);
         set((const void*)k_spread_sc<20, 8>);
         set((const void*)k_spread_sc<24, 8>);
-        set((const void*)kb_bin_count<R>);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute((const void*)kb_bin_count<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kBinSmem);
-        set((const void*)kb_bin_scatter<R>);
         set((const void*)kb_real<R>);
         set((const void*)kb_spread_col<R, 8>);
         set((const void*)kb_spread_col<R, 10>);
@@ -181,34 +168,44 @@ int spread_smem(const Geo& g) {
            (kSpreadThreads / 32) * 3 * kMaxTaps * ((int)sizeof(R) + 4) + kSpreadCap * 4 + kSpreadCap * 8;
 }
 
-// a1: compaction + coordinates + tile histograms, tile offsets, tile scan, scatter.
-// Blocks of the weights kernel: enough words per thread for the plan's capacity,
-// at most four CTAs per SM.
+// Blocks of the weights kernel: a thread per (bead, dimension) were every bead
+// charged, up to a few CTAs per SM. FP64 takes small CTAs (64 threads), so that
+// few beads still spread over all SMs' FP64 units.
+template <typename R>
+constexpr int bin_weight_threads() { return sizeof(R) == 8 ? 64 : 256; }
+template <typename R>
 inline int bin_weight_blocks(const Geo& g) {
-    const long long words = (long long)g.nbin * g.chunk * 6 * g.p;
-    return (int)std::max(1LL, std::min((long long)4 * 152, (words + 255) / 256));
+    const long long rows = (long long)g.nbin * g.chunk * 3;
+    constexpr int T = bin_weight_threads<R>();
+    return (int)std::max(1LL, std::min((long long)(1024 / T) * 152, (rows + T - 1) / T));
 }
 
+// a1: compaction + coordinates + tile ranks, tile starts, scatter; the window
+// weights in the scatter kernel (FP32) or by themselves (FP64: their
+// exponentials need the FP64 units of all SMs).
 template <typename R>
 void enqueue_bin(const Geo& g, const Work& w, int N, const R* pos, const R* q, R* Fzero, cudaStream_t s, bool pdl) {
     using V = typename V4<R>::T;
-    launch(false, true, k_bin_count<R>, g.nbin, kBinThreads, (g.ntiles + g.chunk) * sizeof(int), s, g, N, pos, q,
-           w.cnt_blk, w.bhist, w.ctile, static_cast<V*>(w.cpos), static_cast<V*>(w.cfrac), w.cbase, Fzero,
-           w.part + w.off_q, w.ticket, w.boff, w.tstart);
-    if (!g.bin_last) {
-        launch(pdl, true, k_tile_offsets, (g.ntiles + 255) / 256, 256, 0, s, g, (const int*)w.bhist, w.boff, w.ttot);
-        launch(pdl, true, k_scan, 1, 1024, 0, s, w.ttot, w.tstart, g.ntiles, (int*)nullptr, 0);
-    }
-    launch(pdl, true, k_bin_scatter<R>, g.nbin, kBinThreads, g.ntiles * sizeof(int), s, g, (const int*)w.cnt_blk,
-           (const int*)w.ctile, static_cast<const V*>(w.cpos), static_cast<const V*>(w.cfrac), (const int*)w.cbase,
-           (const int*)w.boff, (const int*)w.tstart, static_cast<V*>(w.sq), static_cast<V*>(w.sw), w.sb, w.spf);
-    if (w.wb)
-        launch(pdl, true, k_bin_weights<R>, bin_weight_blocks(g), 256, 0, s, g, (const int*)w.tstart,
-               static_cast<const V*>(w.sw), static_cast<R*>(w.wb));
+    launch(false, true, k_bin_count<R>, g.nbin, kBinThreads, g.chunk * sizeof(int), s, g, N, pos, q, w.cnt_blk,
+           w.tcnt, w.crank, static_cast<V*>(w.cpos), static_cast<V*>(w.cfrac), w.cbase, Fzero, w.part + w.off_q);
+    if (!g.bin_scan)
+        launch(pdl, true, k_scan_mb, (g.ntiles + kScanMbSpan - 1) / kScanMbSpan, 1024, 0, s, (const int*)w.tcnt,
+               w.tstart, g.ntiles, (int*)nullptr);
+    const bool fused = sizeof(R) == 4 && w.wb;
+    launch(pdl, true, fused ? k_bin_scatter<R, true> : k_bin_scatter<R, false>, g.nbin, kBinThreads,
+           g.bin_scan ? (g.ntiles + 1) * sizeof(int) : 0, s, g, (const int*)w.cnt_blk, w.tcnt, w.tstart,
+           (const int*)w.crank, static_cast<const V*>(w.cpos), static_cast<const V*>(w.cfrac), (const int*)w.cbase,
+           static_cast<V*>(w.sq), static_cast<V*>(w.sw), w.sb, w.spf, static_cast<R*>(w.wb), w.ticket);
+    if (w.wb && !fused)
+        launch(pdl, true, k_bin_weights<R>, bin_weight_blocks<R>(g), bin_weight_threads<R>(), 0, s, g,
+               (const int*)w.tstart, static_cast<const V*>(w.sw), static_cast<R*>(w.wb));
 }
 
 // Kernels enqueue_bin launches.
-inline int bin_kernels(const Geo& g, const Work& w) { return (g.bin_last ? 2 : 4) + (w.wb ? 1 : 0); }
+template <typename R>
+inline int bin_kernels(const Geo& g, const Work& w) {
+    return (g.bin_scan ? 2 : 3) + (w.wb && sizeof(R) == 8 ? 1 : 0);
+}
 
 // Spreading: for the common tile edges the column-stationary kernel (FP32)
 // or its slab form (FP64, where the FP64 instruction count decides), the
@@ -366,7 +363,7 @@ cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp,
     rec(ev, 0, true, s0);
     enqueue_bin<R>(g, w, a.N, pos, q, a.zeroF ? F : nullptr, s0, pdl);
     rec(ev, 0, false, s0);
-    log->kernels += bin_kernels(g, w);
+    log->kernels += bin_kernels<R>(g, w);
 
     // real-space branch
     cudaEventRecord(evFork, s0);

@@ -23,9 +23,10 @@ __device__ __forceinline__ bool enuf_guard(unsigned int* word, bool ok, int bit)
 #define ENUF_GUARD(word, cond, bit) true
 #endif
 
-// dynamic shared memory of the binning count kernel at most (its static share
-// is a few words; the part allows 227 KB per CTA)
-constexpr int kBinSmem = 224 * 1024;
+// Tiles up to which the scatter blocks of the binning scan the counters for
+// themselves (16 KB of shared memory and 16 counters a thread, ~1 us, less than
+// a launch); more go through a scan kernel.
+constexpr int kBinScanTiles = 4096;
 
 // Constants of the real-space pair arithmetic in one working precision.
 template <typename R>
@@ -65,11 +66,12 @@ struct Geo {
     int chunk;    // beads per binning block
     int kmask;
     int nf;       // reciprocal force fields: 3 (ik-differentiation) or 1 (window gradient)
-    int bin_last; // 1: the last binning block computes the tile offsets and starts
-                  //    (ntiles x nbin small); 0: separate offsets and scan kernels
+    int bin_scan; // 1: every scatter block scans the tile counters itself (up to
+                  //    kBinScanTiles tiles); 0: a scan kernel between count and scatter
     double L, alpha, beta, kappa, rc;
     double b;      // Gaussian window parameter 2 sigma p / ((2 sigma - 1) pi)
     double wnorm;  // (pi b)^{-1/2}
+    double e3[9];  // wnorm e^{-m^2/b}, m = 0 .. p
     double ratio;  // n / L: grid coordinate u = x * ratio (one FP64 product)
     double rb;     // 1 / b
     double pref;   // kappa * 2 / L^2 (Eq. 25 prefactor); gradient mode: -kappa n / (pi L^2)
@@ -150,13 +152,11 @@ struct FftShape {
 struct Work {
     // charged binning
     int* cnt_blk;    // [nbin] charged beads of each binning block
-    int* bhist;      // [nbin][ntiles] per-block tile counts
-    int* boff;       // [nbin][ntiles] offset of each block's beads within each tile
-    int* ttot;       // [ntiles] beads per tile
+    int* tcnt;       // [ntiles] tile counters of the binning (0 between evaluations)
     int* tstart;     // [ntiles + 1]
     int* ticket;     // [4] arrival counters of last-block reductions (0 between launches)
     unsigned int* check;  // [1] failure bits of the ENUF_CHECK index checks
-    int* ctile;      // [nbin * chunk] tile of each compacted charged bead
+    int* crank;      // [nbin * chunk] rank of each compacted charged bead in its tile
     void* cpos;      // real4 [nbin * chunk] wrapped x, y, z, q of each compacted charged bead
     void* cfrac;     // real4 [nbin * chunk] fractional grid coordinates, original index bits
     int* cbase;      // [nbin * chunk] packed base grid index

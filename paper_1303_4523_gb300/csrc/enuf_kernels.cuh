@@ -413,21 +413,27 @@ __device__ __forceinline__ void totals_if_last(const Geo& g, const TotalsArgs& t
 // Kahan-compensated accumulator (FP64).
 
 // ---------------------------------------------------------------------------
-// a1: binning of the charged beads into tiles of the oversampled grid.
-// k_bin_count: each block compacts the charged beads of its chunk (warp
-//   ballots into a shared list), computes their grid coordinates in FP64 on
-//   dense warps, histograms their tiles in shared memory and stores each
-//   compacted bead's record.
-//   The last block to finish (arrival counter) walks the per-block counts of
-//   every tile (coalesced), writes each block's offset inside the tile and
-//   scans the tile totals into the tile starts.
-// k_bin_scatter moves the records to their sorted slots; k_bin_weights
-//   computes their window weights. Besides the arrival counter the only
-//   atomics are shared-memory ones.
+// a1: binning of the charged beads into tiles of the oversampled grid, a
+// counting sort in two kernels (three with many tiles):
+// k_bin_count: each block compacts the charged beads of its share (warp
+//   ballots into a shared list), computes their grid coordinates on dense
+//   warps and takes each bead's rank in its tile from the tile's counter (one
+//   global add per charged bead, spread over the tiles).
+// k_bin_scatter: every block scans the tile counters for itself (up to
+//   kBinScanTiles of them; more go through k_scan_mb), moves its records to
+//   their slots (tile start + rank) and, in FP32 single evaluations, computes
+//   their window weights. The last block to have read the counters clears
+//   them for the next evaluation.
+// Per-block tile histograms with a last block that turned them into offsets
+// (the form before) cost that block a walk over tiles x blocks counts, or two
+// more launches. The stage with the window weights, FP32: 81k beads 22.0 ->
+// 15.7 us, 524k 32.5 -> 23.6, 3M 75 -> 51; FP64: 375k 75 -> 55, 3000 28 -> 18.
 // ---------------------------------------------------------------------------
-// Exclusive scan of count ints held in shared memory into out[0..count] (out[count] =
-// total) by the whole block: contiguous chunks per thread, warp and block scans.
-__device__ __forceinline__ void block_exclusive_scan(const int* data, int count, int* __restrict__ out) {
+constexpr int kBinThreads = 256;
+
+// In-place exclusive scan of count ints in shared memory (data[count] = total)
+// by the whole block: contiguous chunks per thread, warp and block scans.
+__device__ __forceinline__ void block_exclusive_scan(int* data, int count) {
     __shared__ int wsum[32];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nwarp = (blockDim.x + 31) >> 5;
     const int per = (count + blockDim.x - 1) / blockDim.x;
@@ -442,39 +448,34 @@ __device__ __forceinline__ void block_exclusive_scan(const int* data, int count,
     }
     if (lane == 31) wsum[w] = x;
     __syncthreads();
-    if (w == 0) {
-        int z = lane < nwarp ? wsum[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, z, o);
-            if (lane >= o) z += y;
-        }
-        wsum[lane] = z;
+    int run = x - sum, total = 0;
+    for (int k = 0; k < nwarp; ++k) {
+        if (k < w) run += wsum[k];
+        total += wsum[k];
     }
-    __syncthreads();
-    int run = (x - sum) + (w > 0 ? wsum[w - 1] : 0);
     for (int i = i0; i < i1; ++i) {
-        out[i] = run;
-        run += data[i];
+        const int v = data[i];
+        data[i] = run;
+        run += v;
     }
-    if (tid == 0) out[count] = wsum[nwarp - 1];
+    if (tid == 0) data[count] = total;
+    __syncthreads();
 }
+
+// Tile coordinate of a grid line: base < 1024, so the float quotient of
+// base + 1/2 is exact.
+__device__ __forceinline__ int tile_of(int base, float rT) { return (int)(((float)base + 0.5f) * rT); }
 
 template <typename R>
 __device__ __forceinline__ void k_bin_count_body(Geo g, int N, const R* __restrict__ pos,
                                                    const R* __restrict__ q, int* __restrict__ cnt_blk,
-                                                   int* __restrict__ bhist, int* __restrict__ ctile,
+                                                   int* __restrict__ tcnt, int* __restrict__ crank,
                                                    typename V4<R>::T* __restrict__ cpos,
                                                    typename V4<R>::T* __restrict__ cfrac, int* __restrict__ cbase,
-                                                   R* __restrict__ Fzero, double* __restrict__ qpart,
-                                                   int* __restrict__ ticket, int* __restrict__ boff,
-                                                   int* __restrict__ tstart, Blk blk) {
+                                                   R* __restrict__ Fzero, double* __restrict__ qpart, Blk blk) {
     pdl_enter();
-    extern __shared__ int sm_bin[];
-    int* hist = sm_bin;                 // [ntiles]
-    int* slist = sm_bin + g.ntiles;     // [chunk]
+    extern __shared__ int slist[];   // [chunk]
     __shared__ int scount;
-    for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) hist[t] = 0;
     if (threadIdx.x == 0) scount = 0;
     __syncthreads();
     const int b = blk.id, lane = threadIdx.x & 31;
@@ -484,28 +485,40 @@ __device__ __forceinline__ void k_bin_count_body(Geo g, int N, const R* __restri
     // are dealt to the blocks round robin: charged beads that sit together in
     // the input order (chains, counterions, salt) are spread over all blocks
     // (at most chunk / 32 groups per block: chunk is a multiple of 32)
+    constexpr int U = 4;   // groups in flight per warp
     const int nwarp = blockDim.x >> 5, warp = threadIdx.x >> 5;
-    const int ngroups = (N + 31) >> 5;
-    for (int gi = b + warp * (int)blk.n; gi < ngroups; gi += nwarp * (int)blk.n) {
-        const int i = gi * 32 + lane;
-        R qi = (R)0;
-        if (i < N) {
-            qi = q[i];
-            if (Fzero) {
-                Fzero[3 * i] = (R)0;
-                Fzero[3 * i + 1] = (R)0;
-                Fzero[3 * i + 2] = (R)0;
+    const int ngroups = (N + 31) >> 5, step = nwarp * blk.n;
+    for (int g0 = b + warp * blk.n; g0 < ngroups; g0 += U * step) {
+        R qv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = (g0 + u * step) * 32 + lane;   // i < N + 32 U step: within an int
+            qv[u] = g0 + u * step < ngroups && i < N ? q[i] : (R)0;
+        }
+        if (Fzero) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int i = (g0 + u * step) * 32 + lane;
+                if (g0 + u * step < ngroups && i < N) {
+                    Fzero[3 * i] = (R)0;
+                    Fzero[3 * i + 1] = (R)0;
+                    Fzero[3 * i + 2] = (R)0;
+                }
             }
         }
-        const bool charged = qi != (R)0;
-        const unsigned m = __ballot_sync(0xffffffffu, charged);
-        int basei = 0;
-        if (lane == 0 && m) basei = atomicAdd(&scount, __popc(m));
-        basei = __shfl_sync(0xffffffffu, basei, 0);
-        if (charged) slist[basei + __popc(m & ((1u << lane) - 1u))] = i;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool charged = qv[u] != (R)0;
+            const unsigned m = __ballot_sync(0xffffffffu, charged);
+            int basei = 0;
+            if (lane == 0 && m) basei = atomicAdd(&scount, __popc(m));
+            basei = __shfl_sync(0xffffffffu, basei, 0);
+            if (charged) slist[basei + __popc(m & ((1u << lane) - 1u))] = (g0 + u * step) * 32 + lane;
+        }
     }
     __syncthreads();
     const int nc = scount;
+    const float rT = 1.0f / (float)g.T;
     for (int k = threadIdx.x; k < nc; k += blockDim.x) {
         if (!ENUF_GUARD(g.check, k < g.chunk, 1)) continue;   // the compacted list holds a chunk
         const int i = slist[k];
@@ -516,18 +529,17 @@ __device__ __forceinline__ void k_bin_count_body(Geo g, int N, const R* __restri
             xw[t] = wrap_r(pos[3 * i + t], g.L, g.xmaxf, g.Lhi, g.Llo);
             grid_coord_r(xw[t], g, bs[t], fr[t]);
         }
-        const int tile = ((bs[2] / g.T) * g.ntd + bs[1] / g.T) * g.ntd + bs[0] / g.T;
+        const int tile = (tile_of(bs[2], rT) * g.ntd + tile_of(bs[1], rT)) * g.ntd + tile_of(bs[0], rT);
         if (!ENUF_GUARD(g.check, (unsigned)tile < (unsigned)g.ntiles, 0)) continue;
-        atomicAdd(&hist[tile], 1);
         const int o = i0 + k;
+        crank[o] = atomicAdd(&tcnt[tile], 1);
         typename V4<R>::T a, c;
         a.x = xw[0]; a.y = xw[1]; a.z = xw[2]; a.w = q[i];
         // charge sums over the compacted beads: only the block's first warps
         // hold nonzero partials, the rest skip the reduction tree
         s1 += (double)a.w;
-        s2 += (double)a.w * (double)a.w;
+        s2 = fma((double)a.w, (double)a.w, s2);
         c.x = fr[0]; c.y = fr[1]; c.z = fr[2]; c.w = int_as_real(i, (R)0);
-        ctile[o] = tile;
         cpos[o] = a;
         cfrac[o] = c;
         cbase[o] = bs[0] | (bs[1] << 10) | (bs[2] << 20);
@@ -538,50 +550,17 @@ __device__ __forceinline__ void k_bin_count_body(Geo g, int N, const R* __restri
         qpart[2 * b] = s1;
         qpart[2 * b + 1] = s2;
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) bhist[b * g.ntiles + t] = hist[t];
-    // the last block to arrive turns the per-block histograms into per-block
-    // offsets within each tile and the tile starts (exclusive scan of the totals)
-    if (!g.bin_last) return;
-    __shared__ int last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1) == (int)blk.n - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
-        int run = 0;
-        for (int b0 = 0; b0 < g.nbin; b0 += 8) {   // eight independent loads in flight
-            int v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = b0 + u < g.nbin ? __ldcg(&bhist[(b0 + u) * g.ntiles + t]) : 0;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                if (b0 + u < g.nbin) boff[(b0 + u) * g.ntiles + t] = run;
-                run += v[u];
-            }
-        }
-        hist[t] = run;   // tile totals
-    }
-    __syncthreads();
-    block_exclusive_scan(hist, g.ntiles, tstart);
-    if (threadIdx.x == 0) *ticket = 0;
 }
 
 template <typename R>
-__global__ void __launch_bounds__(1024) k_bin_count(Geo g, int N, const R* __restrict__ pos,
+__global__ void __launch_bounds__(kBinThreads) k_bin_count(Geo g, int N, const R* __restrict__ pos,
                                                    const R* __restrict__ q, int* __restrict__ cnt_blk,
-                                                   int* __restrict__ bhist, int* __restrict__ ctile,
+                                                   int* __restrict__ tcnt, int* __restrict__ crank,
                                                    typename V4<R>::T* __restrict__ cpos,
                                                    typename V4<R>::T* __restrict__ cfrac, int* __restrict__ cbase,
-                                                   R* __restrict__ Fzero, double* __restrict__ qpart,
-                                                   int* __restrict__ ticket, int* __restrict__ boff,
-                                                   int* __restrict__ tstart) {
-    k_bin_count_body<R>(g, N, pos, q, cnt_blk, bhist, ctile, cpos, cfrac, cbase, Fzero, qpart, ticket, boff, tstart, Blk{(int)blockIdx.x, (int)gridDim.x});
+                                                   R* __restrict__ Fzero, double* __restrict__ qpart) {
+    k_bin_count_body<R>(g, N, pos, q, cnt_blk, tcnt, crank, cpos, cfrac, cbase, Fzero, qpart, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
-
-// One thread per tile: offsets of each block's beads inside the tile, and the tile total.
 
 // Exclusive scan of in[0, count) into out[0, count], out[count] = total; one
 // CTA of 1024 threads, 16 elements per thread and round (four 16-byte loads).
@@ -733,117 +712,138 @@ static __global__ void __launch_bounds__(1024) k_scan_mb(const int* __restrict__
     }
 }
 
-// Separate tile offsets for large tile x block counts: one thread per tile
-// walks the per-block counts (coalesced) and writes each block's offset inside
-// the tile and the tile total (then k_scan gives the tile starts).
-static __global__ void __launch_bounds__(256) k_tile_offsets(Geo g, const int* __restrict__ bhist, int* __restrict__ boff,
-                                                      int* __restrict__ ttot) {
-    pdl_enter();
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= g.ntiles) return;
-    int run = 0;
-    int b = 0;
-    for (; b + 4 <= g.nbin; b += 4) {
-        const int v0 = bhist[b * g.ntiles + t], v1 = bhist[(b + 1) * g.ntiles + t];
-        const int v2 = bhist[(b + 2) * g.ntiles + t], v3 = bhist[(b + 3) * g.ntiles + t];
-        boff[b * g.ntiles + t] = run;
-        boff[(b + 1) * g.ntiles + t] = run + v0;
-        boff[(b + 2) * g.ntiles + t] = run + v0 + v1;
-        boff[(b + 3) * g.ntiles + t] = run + v0 + v1 + v2;
-        run += v0 + v1 + v2 + v3;
+// Window weights of one (bead, dimension) (Eq. 14): out[a] = psi(f + p - 1 - a)
+// for the 2p taps a, f the fractional grid coordinate. FP32: an exponential per
+// tap. FP64: e^{-(f + m)^2/b} = e^{-f^2/b} (e^{-2f/b})^m e^{-m^2/b} (the fast
+// Gaussian gridding of Greengard & Lee, SIAM Rev. 46, 2004): three exponentials
+// and products instead of 2p exponentials on the few FP64 units (375k beads,
+// p = 4: the binning stage 75 -> 55 us with it); |m| <= p <= 8 keeps the
+// products within a few ulp, the rounding that (f + m)^2/b itself brings to the
+// direct form.
+template <typename R>
+__device__ __forceinline__ void window_row(const Geo& g, R f, R* __restrict__ out) {
+    const int p = g.p, P2 = 2 * g.p;
+    if constexpr (sizeof(R) == 8) {
+        const double rb = g.rb;
+        const double e0 = exp(-f * f * rb);
+        const double up = exp(-2.0 * f * rb), dn = exp(2.0 * f * rb);
+        double t = e0;
+        for (int m = 0; m < p; ++m) {   // m = 0 .. p - 1: tap p - 1 - m
+            out[p - 1 - m] = t * g.e3[m];
+            t *= up;
+        }
+        t = e0;
+        for (int m = 1; m <= p; ++m) {   // -m: tap p - 1 + m
+            t *= dn;
+            out[p - 1 + m] = t * g.e3[m];
+        }
+    } else {
+        const float rb = g.wkf.rb, wn = g.wkf.wn;
+        if ((P2 & 3) == 0) {
+            for (int a = 0; a < P2; a += 4) {
+                float w4[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float u = f + (float)(p - 1 - (a + k));
+                    w4[k] = wn * r_exp(-u * u * rb);
+                }
+                *reinterpret_cast<float4*>(out + a) = make_float4(w4[0], w4[1], w4[2], w4[3]);
+            }
+        } else {
+            for (int a = 0; a < P2; ++a) {
+                const float u = f + (float)(p - 1 - a);
+                out[a] = wn * r_exp(-u * u * rb);
+            }
+        }
     }
-    for (; b < g.nbin; ++b) {
-        const int v = bhist[b * g.ntiles + t];
-        boff[b * g.ntiles + t] = run;
-        run += v;
-    }
-    ttot[t] = run;
 }
 
-template <typename R>
-__device__ __forceinline__ void k_bin_scatter_body(Geo g, const int* __restrict__ cnt_blk,
-                                                     const int* __restrict__ ctile,
+// W: the window weights as well, one thread per (bead, dimension).
+template <typename R, bool W>
+__device__ __forceinline__ void k_bin_scatter_body(Geo g, const int* __restrict__ cnt_blk, int* __restrict__ tcnt,
+                                                     int* __restrict__ tstart, const int* __restrict__ crank,
                                                      const typename V4<R>::T* __restrict__ cpos,
                                                      const typename V4<R>::T* __restrict__ cfrac,
-                                                     const int* __restrict__ cbase, const int* __restrict__ boff,
-                                                     const int* __restrict__ tstart,
+                                                     const int* __restrict__ cbase,
                                                      typename V4<R>::T* __restrict__ sq,
                                                      typename V4<R>::T* __restrict__ sw, int* __restrict__ sb,
-                                                     float4* __restrict__ spf, Blk blk) {
+                                                     float4* __restrict__ spf, R* __restrict__ wb,
+                                                     int* __restrict__ ticket, Blk blk) {
     pdl_enter();
-    extern __shared__ int cur[];   // [ntiles] running counts
+    extern __shared__ int pre[];   // [ntiles + 1] tile starts (g.bin_scan)
     const int b = blk.id;
-    for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) cur[t] = 0;
-    __syncthreads();
+    const int* ts = tstart;
+    if (g.bin_scan) {
+        __shared__ int last;
+        for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) pre[t] = __ldcg(&tcnt[t]);
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(ticket, 1) == blk.n - 1;
+        block_exclusive_scan(pre, g.ntiles);   // contains barriers
+        if (last) {   // every block has its copy of the counters
+            for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) tcnt[t] = 0;
+            if (threadIdx.x == 0) *ticket = 0;
+        }
+        if (b == 0)
+            for (int t = threadIdx.x; t <= g.ntiles; t += blockDim.x) tstart[t] = pre[t];
+        ts = pre;
+    } else {   // tstart comes from the scan kernel
+        for (int t = b * blockDim.x + threadIdx.x; t < g.ntiles; t += blk.n * blockDim.x) tcnt[t] = 0;
+    }
     const int nc = cnt_blk[b];
     const int i0 = b * g.chunk;
-    for (int k = threadIdx.x; k < nc; k += blockDim.x) {
+    const float rT = 1.0f / (float)g.T;
+    constexpr int D = W ? 3 : 1;
+    for (int e = threadIdx.x; e < D * nc; e += blockDim.x) {
+        const int k = e / D, d = e - D * k;
         const int o = i0 + k;
-        const int t = ctile[o];
+        const int pb = cbase[o];
+        const int t = (tile_of((pb >> 20) & 1023, rT) * g.ntd + tile_of((pb >> 10) & 1023, rT)) * g.ntd +
+                      tile_of(pb & 1023, rT);
         if (!ENUF_GUARD(g.check, (unsigned)t < (unsigned)g.ntiles, 2)) continue;
-        const int slot = tstart[t] + boff[b * g.ntiles + t] + atomicAdd(&cur[t], 1);
+        const int slot = ts[t] + crank[o];
         if (!ENUF_GUARD(g.check, (unsigned)slot < (unsigned)g.nmax, 2)) continue;
-        const typename V4<R>::T a = cpos[o];
-        sq[slot] = a;
-        sw[slot] = cfrac[o];
-        sb[slot] = cbase[o];
-        // FP64: a float copy of the position for the real-space cutoff pre-test
-        if (sizeof(R) == 8 && spf) spf[slot] = make_float4((float)a.x, (float)a.y, (float)a.z, 0.f);
+        const typename V4<R>::T c = cfrac[o];
+        if (d == 0) {
+            const typename V4<R>::T a = cpos[o];
+            sq[slot] = a;
+            sw[slot] = c;
+            sb[slot] = pb;
+            // FP64: a float copy of the position for the real-space cutoff pre-test
+            if (sizeof(R) == 8 && spf) spf[slot] = make_float4((float)a.x, (float)a.y, (float)a.z, 0.f);
+        }
+        if constexpr (W)
+            window_row<R>(g, d == 0 ? c.x : (d == 1 ? c.y : c.z), wb + ((size_t)slot * 3 + d) * (2 * g.p));
     }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(1024) k_bin_scatter(Geo g, const int* __restrict__ cnt_blk,
-                                                     const int* __restrict__ ctile,
+template <typename R, bool W>
+__global__ void __launch_bounds__(kBinThreads) k_bin_scatter(Geo g, const int* __restrict__ cnt_blk, int* __restrict__ tcnt,
+                                                     int* __restrict__ tstart, const int* __restrict__ crank,
                                                      const typename V4<R>::T* __restrict__ cpos,
                                                      const typename V4<R>::T* __restrict__ cfrac,
-                                                     const int* __restrict__ cbase, const int* __restrict__ boff,
-                                                     const int* __restrict__ tstart,
+                                                     const int* __restrict__ cbase,
                                                      typename V4<R>::T* __restrict__ sq,
                                                      typename V4<R>::T* __restrict__ sw, int* __restrict__ sb,
-                                                     float4* __restrict__ spf) {
-    k_bin_scatter_body<R>(g, cnt_blk, ctile, cpos, cfrac, cbase, boff, tstart, sq, sw, sb, spf, Blk{(int)blockIdx.x, (int)gridDim.x});
+                                                     float4* __restrict__ spf, R* __restrict__ wb,
+                                                     int* __restrict__ ticket) {
+    k_bin_scatter_body<R, W>(g, cnt_blk, tcnt, tstart, crank, cpos, cfrac, cbase, sq, sw, sb, spf, wb, ticket,
+                             Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
-// Window weights of every sorted charged bead (Eq. 14), computed once and
-// read by the spreading and gathering kernels: wb[s][d][a] = psi(u_sd - l_a)
-// for the 2p taps a of dimension d. One thread per (bead, dimension) writes
-// its 2p consecutive weights (16-byte stores when 2p is a multiple of 4 in
-// FP32); all SMs (in FP64 the exponentials run on the FP64 units).
+// Window weights of every sorted charged bead, computed once and read by the
+// spreading and gathering kernels: wb[s][d][a]. One thread per (bead,
+// dimension) writes its 2p consecutive weights; all SMs (in FP64 the
+// exponentials run on the FP64 units).
 template <typename R>
 __device__ __forceinline__ void k_bin_weights_body(Geo g, const int* __restrict__ tstart,
                                                     const typename V4<R>::T* __restrict__ sw, R* __restrict__ wb, Blk blk) {
     pdl_enter();
     const int nq = tstart[g.ntiles];
-    const int P2 = 2 * g.p;
-    const R rb = win_k(g, (R)0).rb, wn = win_k(g, (R)0).wn;
     const int tot = 3 * nq;   // (bead, dimension) pairs; nq <= n_max < 2^29
     for (int e = blk.id * blockDim.x + threadIdx.x; e < tot; e += blk.n * blockDim.x) {
         const int s = e / 3, d = e - 3 * s;
         const typename V4<R>::T fr = sw[s];
-        const R f = d == 0 ? fr.x : (d == 1 ? fr.y : fr.z);
-        R* out = wb + (size_t)e * P2;   // = wb + (s 3 + d) 2p
-        bool done = false;
-        if constexpr (sizeof(R) == 4) {
-            if ((P2 & 3) == 0) {
-                for (int a = 0; a < P2; a += 4) {
-                    float w4[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const R u = f + (R)(g.p - 1 - (a + k));
-                        w4[k] = wn * r_exp(-u * u * rb);
-                    }
-                    *reinterpret_cast<float4*>(out + a) = make_float4(w4[0], w4[1], w4[2], w4[3]);
-                }
-                done = true;
-            }
-        }
-        if (!done) {
-            for (int a = 0; a < P2; ++a) {
-                const R u = f + (R)(g.p - 1 - a);
-                out[a] = wn * r_exp(-u * u * rb);
-            }
-        }
+        window_row<R>(g, d == 0 ? fr.x : (d == 1 ? fr.y : fr.z), wb + (size_t)e * (2 * g.p));
     }
 }
 
@@ -2300,10 +2300,10 @@ __device__ __forceinline__ void real_sweep(const Geo& g, int nq, int S, const in
         int tx = 0, ty = 0, tz = 0;
         if (own) {
             pf = spf[s];
-            const int pb = sb[s];   // grid base of the bead: its tile (base < 1024: the quotient is exact)
-            tx = (int)(((float)(pb & 1023) + 0.5f) * rT);
-            ty = (int)(((float)((pb >> 10) & 1023) + 0.5f) * rT);
-            tz = (int)(((float)((pb >> 20) & 1023) + 0.5f) * rT);
+            const int pb = sb[s];   // grid base of the bead: its tile
+            tx = tile_of(pb & 1023, rT);
+            ty = tile_of((pb >> 10) & 1023, rT);
+            tz = tile_of((pb >> 20) & 1023, rT);
         }
         a.fx = a.fy = a.fz = (R)0;
         // rows of tiles one after the other (uniform over the warp), each as its run
