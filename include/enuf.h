@@ -95,7 +95,9 @@ typedef struct {
                          2 = Stockham stages, the fewest over 2, 3, 4, 5, 8, and for FP32
                          grids from n = 128 on the composite radices 6, 10, 12, 16, 20
                          when that saves a stage. Same result to rounding. */
-    int    spread;    /* spreading kernel (FP32; FP64 always takes 1): 0 = automatic (below);
+    int    spread;    /* spreading kernel (FP32; FP64 takes 0 or 1): 0 = automatic: the
+                         reduction form (a warp per charged bead adds its taps to the cleared
+                         grid by global reductions; batches run it for every value);
                          1 = tile form (one CTA per T^3 tile: column-stationary for
                          T in 8, 10, 12, 16, 20, 24, shared-memory atomics otherwise);
                          2 = footprint form on bricks of whole x rows (or x runs) of
@@ -109,8 +111,8 @@ typedef struct {
                          (scale 2^k with sum over the region's beads of |q| psi(0)^3
                          below 2^30), work on its taps inside the region only (needs
                          p = 4, the region dividing n and n >= 2 (region + T + 8)).
-                         Automatic (0): 4 where admitted and n >= 128, else 1.
-                         Same result to rounding. */
+                         Plans report (enuf_plan_info.spread) 4 for 0 where 4 is admitted
+                         and n >= 128, else 1. Same result to rounding. */
     int    pairs;     /* DPD systems: 1 = two launches, the DPD pairs right after the
                          cell list (before the charged-bead binning is done), then the
                          real-space pairs; 2 = one launch whose blocks take either role,

@@ -31,6 +31,7 @@ struct BinCountArgs {
     int* cbase;
     R* Fzero;
     double* qpart;
+    R* gzero;
     int nblk;
 };
 template <typename R>
@@ -39,7 +40,7 @@ __global__ void __launch_bounds__(kBinThreads) kb_bin_count(const BinCountArgs<R
     const int m = cmap[blockIdx.x];
     const BinCountArgs<R>& a = tab[m >> kBatchShift];
     k_bin_count_body<R>(a.g, a.N, a.pos, a.q, a.cnt_blk, a.tcnt, a.crank, a.cpos, a.cfrac, a.cbase, a.Fzero, a.qpart,
-                        Blk{m & kBatchLocal, a.nblk});
+                        a.gzero, Blk{m & kBatchLocal, a.nblk});
 }
 
 template <typename R>
@@ -104,7 +105,8 @@ __global__ void __launch_bounds__(kRealThreads) kb_real(const RealArgs<R>* __res
     k_real_body<R>(a.g, a.tstart, a.sq, a.sw, a.sb, a.spf, a.F, a.rpart, Blk{m & kBatchLocal, a.nblk});
 }
 
-// the column spreading form of one tile edge T (systems grouped by T)
+// spreading, reduction form (systems grouped by tile edge; PT: the tap count 2p
+// when every system of the group has the same window, else 0)
 template <typename R>
 struct SpreadArgs {
     Geo g;
@@ -115,13 +117,13 @@ struct SpreadArgs {
     R* grid;
     int nblk;
 };
-template <typename R, int T>
-__global__ void __launch_bounds__(col_threads(T)) kb_spread_col(const SpreadArgs<R>* __restrict__ tab,
-                                                               const int* __restrict__ cmap) {
+template <typename R, int PT>
+__global__ void __launch_bounds__(kRedThreads) kb_spread_red(const SpreadArgs<R>* __restrict__ tab,
+                                                             const int* __restrict__ cmap) {
     pdl_enter();
     const int m = cmap[blockIdx.x];
     const SpreadArgs<R>& a = tab[m >> kBatchShift];
-    k_spread_col_body<R, T, false>(a.g, a.tstart, a.sq, a.sb, a.wb, a.grid, Blk{m & kBatchLocal, a.nblk});
+    k_spread_red_body<R, PT>(a.g, a.tstart, a.sq, a.sb, a.wb, a.grid, Blk{m & kBatchLocal, a.nblk});
 }
 
 template <typename R>

@@ -16,10 +16,13 @@ inline void append_blocks(std::vector<int>& cmap, int sys, int nblk) {
     for (int b = 0; b < nblk; ++b) cmap.push_back((sys << kBatchShift) | b);
 }
 
-// Real-space blocks of one system of a batch: the batch fills the chip, so a
-// system takes about 4 lanes per charged bead (a tenth of the beads charged)
-// instead of the launch's whole width (the kernel strides over any excess).
-inline int batch_real_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_real, (x.N + 511) / 512)); }
+// Blocks of one system of a batch in its bead loops. The batch fills the chip,
+// so a system takes few blocks and strides over its beads: real space N / 1024
+// blocks and as many lanes as its beads need (64 systems: 1179 us against 1219
+// with N / 512), gather N / 512 (1171 against 1219 with N / 64), spreading as
+// the gather.
+inline int batch_real_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_real, (x.N + 1023) / 1024)); }
+inline int batch_gather_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_gather, (x.N + 511) / 512)); }
 
 // Window-weight blocks of one system: a thread per (bead, dimension) for a
 // sixth of the beads (the kernel strides over any excess).
@@ -33,7 +36,7 @@ size_t batch_bytes(const BatchSys* sys, int nsys) {
     size_t blocks = 0;
     for (int s = 0; s < nsys; ++s) {
         const BatchSys& x = sys[s];
-        blocks += 2 * (size_t)x.g.nbin + batch_weight_blocks(x) + x.w.nblk_real + x.g.ntiles + x.g.n + x.fs.grid_z +
+        blocks += 2 * (size_t)x.g.nbin + batch_weight_blocks(x) + x.w.nblk_real + x.w.nblk_gather + x.g.n + x.fs.grid_z +
                   (size_t)x.g.nf * x.g.n + x.w.nblk_gather + 1;
     }
     const size_t rec = sizeof(BinCountArgs<R>) + sizeof(BinScatterArgs<R>) + sizeof(BinWeightsArgs<R>) +
@@ -74,7 +77,7 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
             const Work& w = x.w;
             a[s] = BinCountArgs<R>{g, x.N, static_cast<const R*>(x.pos), static_cast<const R*>(x.q), w.cnt_blk, w.tcnt,
                                    w.crank, static_cast<V*>(w.cpos), static_cast<V*>(w.cfrac), w.cbase,
-                                   static_cast<R*>(x.F), w.part + w.off_q, g.nbin};
+                                   static_cast<R*>(x.F), w.part + w.off_q, static_cast<R*>(w.grid), g.nbin};
             b[s] = BinScatterArgs<R>{g, w.cnt_blk, w.tcnt, w.tstart, w.crank, static_cast<const V*>(w.cpos),
                                      static_cast<const V*>(w.cfrac), w.cbase, static_cast<V*>(w.sq),
                                      static_cast<V*>(w.sw), w.sb, w.ticket, g.nbin};
@@ -101,6 +104,7 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
             const int nb = batch_real_blocks(x);
             a[s] = RealArgs<R>{x.g, x.w.tstart, static_cast<const V*>(x.w.sq), static_cast<const V*>(x.w.sw), x.w.sb,
                                x.w.spf, static_cast<R*>(x.F), x.w.part + x.w.off_real, nb};
+            a[s].g.real_lanes = nb * kRealThreads;
             append_blocks(m, s, nb);
         }
         put(L.real, a.data(), a.size() * sizeof(a[0]), m);
@@ -112,20 +116,22 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
         for (int ti = 0; ti < 6; ++ti) {
             std::vector<SpreadArgs<R>> a;
             std::vector<int> m;
+            int taps = -1;   // the group's common tap count, 0: mixed
             for (int s = 0; s < nsys; ++s) {
                 const BatchSys& x = sys[s];
                 if (x.g.T != kT[ti]) continue;
-                const int row = (int)a.size();
+                const int row = (int)a.size(), nb = batch_gather_blocks(x);
+                taps = taps < 0 || taps == 2 * x.g.p ? 2 * x.g.p : 0;
                 a.push_back(SpreadArgs<R>{x.g, x.w.tstart, static_cast<const V*>(x.w.sq), x.w.sb,
-                                          static_cast<const R*>(x.w.wb), static_cast<R*>(x.w.grid), x.g.ntiles});
-                append_blocks(m, row, x.g.ntiles);
+                                          static_cast<const R*>(x.w.wb), static_cast<R*>(x.w.grid), nb});
+                append_blocks(m, row, nb);
             }
             if (a.empty()) continue;
             BatchKernel& k = L.spread[L.nspread++];
             put(k, a.data(), a.size() * sizeof(a[0]), m);
-            k.T = kT[ti];
-            k.threads = col_threads(kT[ti]);
-            k.smem = col_smem<R>(kT[ti], false);
+            k.T = taps;
+            k.threads = kRedThreads;
+            k.smem = 0;
         }
     }
     {
@@ -166,9 +172,7 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
             TotalsArgs t = totals_args(x.g, w, false, 1);
             t.Edev = x.Edev;
             t.nreal = batch_real_blocks(x);
-            // blocks in proportion to the system (a warp per charged bead, <= 1/8 of
-            // the beads charged on average; the kernel strides over any excess)
-            const int nb = std::max(1, std::min(w.nblk_gather, (x.N + 63) / 64));
+            const int nb = batch_gather_blocks(x);
             a[s] = GatherArgs<R>{x.g, w.tstart, static_cast<const V*>(w.sq), static_cast<const V*>(w.sw), w.sb,
                                  static_cast<const R*>(w.wb), static_cast<const R*>(w.h), static_cast<R*>(x.F), t, nb + 1};
             append_blocks(m, s, nb + 1);   // one more: the system's totals
@@ -204,13 +208,11 @@ cudaError_t batch_enqueue(const BatchLaunch& L, cudaStream_t s0, cudaStream_t s1
         const SpreadArgs<R>* tab = (const SpreadArgs<R>*)k.tab;
         const bool pdl = true;   // the predecessor is the binning's last kernel or the previous group
         switch (k.T) {
-            case 8: run(pdl, true, kb_spread_col<R, 8>, k, tab, s0); break;
-            case 10: run(pdl, true, kb_spread_col<R, 10>, k, tab, s0); break;
-            case 12: run(pdl, true, kb_spread_col<R, 12>, k, tab, s0); break;
-            case 16: run(pdl, true, kb_spread_col<R, 16>, k, tab, s0); break;
-            case 20: run(pdl, true, kb_spread_col<R, 20>, k, tab, s0); break;
-            case 24: run(pdl, true, kb_spread_col<R, 24>, k, tab, s0); break;
-            default: return cudaErrorInvalidValue;
+            case 4: run(pdl, true, kb_spread_red<R, 4>, k, tab, s0); break;
+            case 6: run(pdl, true, kb_spread_red<R, 6>, k, tab, s0); break;
+            case 8: run(pdl, true, kb_spread_red<R, 8>, k, tab, s0); break;
+            case 12: run(pdl, true, kb_spread_red<R, 12>, k, tab, s0); break;
+            default: run(pdl, true, kb_spread_red<R, 0>, k, tab, s0); break;
         }
     }
     run(true, true, kb_fft_xy<R>, L.fft_xy, (const FftXYArgs<R>*)L.fft_xy.tab, s0);

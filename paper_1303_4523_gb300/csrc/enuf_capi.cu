@@ -461,10 +461,8 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
         const int scE = T >= 16 ? T : 2 * T, scRT = scE / T;
         const bool sc_ok = 2 * P.p == 8 && (scE == 16 || scE == 20 || scE == 24) && g.ntd % scRT == 0 &&
                            g.ntd >= scRT + 2 && n % 4 == 0 && n >= 2 * (scE + T + 2 * P.p);
-        // automatic: the scatter form where it is admitted and the grid has at least
-        // 128 points per edge (measured faster than the tile form from the 192k-bead
-        // electrolyte, n = 128, to 3M; at n = 96 its 64 regions leave most SMs idle);
-        // the tile form otherwise (faster than forms 2 and 3 at every size measured)
+        // automatic: what the plan reports keeps the tile and scatter forms' sizes (the
+        // scatter form where it is admitted from n = 128 on); the reduction form runs
         int want = P.spread == 0 ? ((sc_ok && n >= 128) ? 4 : 1) : P.spread;
         if (want == 4 && !sc_ok)
             return fail(plan, ENUF_ERR_INVALID, "spread = 4 needs p = 4, a tile edge of 8, 10, 12, 16, 20 or 24 "
@@ -506,6 +504,11 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
     } else if (P.spread > 1) {
         return fail(plan, ENUF_ERR_INVALID, "spread = %d is an FP32 form", P.spread);
     }
+    // the automatic choice runs the reduction form, faster than every other at every
+    // size measured (see k_spread_red); the count kernel clears the grid where that is
+    // at most 16 stores of four values per thread, a memset beside the binning else
+    fs.red = P.spread == 0 ? 1 : 0;
+    if (fs.red) fs.red_zero = (size_t)n * n * n / 4 <= (size_t)g.nbin * 256 * 16 ? 1 : 2;
     g.ratio = (double)n / P.L;
     g.rb = 1.0 / g.b;
     g.pref = P.deriv ? -P.kappa * n / (M_PI * P.L * P.L) : P.kappa * 2.0 / (P.L * P.L);
@@ -545,8 +548,18 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
     g.rlo = (float)(g.ratio - (double)g.rhi);
 
     Work w{};
-    // real space: up to a warp per bead, four CTAs per SM (64 registers a thread)
+    // real space: up to a warp per bead, four CTAs per SM (64 registers a thread). Two
+    // would leave half the registers to the reciprocal chain beside it and gain where
+    // that chain is the longer (3M beads 1292 us against 1305, whole evaluation), but
+    // lose where the pairs are (a quarter of 99000 beads charged: 225 against 158)
     w.nblk_real = std::min(4 * kSMs, (std::max(n_max, 1) + 7) / 8);
+    // S lanes per bead while N_q S stays below this (and two thirds of it for S > 8):
+    // more warps only repeat the walk over a bead's rows, fewer leave its latency
+    // uncovered. Whole evaluations at S = 4 / 8 / 16: 15000 charged of 60000 beads
+    // 158 / 116 / - us, 8100 of 81000 - / 91 / 103; 30000 of 300000 at S = 2 / 4:
+    // 196 / 179. FP64 wants fuller rings, so fewer warps: 2000 of 20000 beads at
+    // S = 16 / 32: 140 / 166
+    g.real_lanes = (P.prec == ENUF_FP32 ? 1024 : 384) * kSMs;
     w.nblk_conv = fs.grid_z;
     w.nblk_dpd = 4 * kSMs;
     w.nblk_kin = kSMs;   // one block per SM: its FP64 block sum runs on each SM's few FP64 units once
@@ -1407,8 +1420,8 @@ struct enuf_batch_s {
 namespace {
 
 // The batched kernels need each system's plan to run the fused-plane
-// two-factor FFT, the column spreading form (tile edges 8..24) and the
-// binning offsets in the last count block.
+// two-factor FFT, a tile edge of the column form (8..24: the systems of one
+// edge spread in one launch) and the tile scan in the scatter kernel.
 bool batch_plan_ok(const enuf_plan_s* p) {
     const int T = p->g.T;
     const bool col = T == 8 || T == 10 || T == 12 || T == 16 || T == 20 || T == 24;

@@ -146,12 +146,6 @@ cudaError_t configure_kernels(int max_smem) {
         set((const void*)k_spread_sc<20, 8>);
         set((const void*)k_spread_sc<24, 8>);
         set((const void*)kb_real<R>);
-        set((const void*)kb_spread_col<R, 8>);
-        set((const void*)kb_spread_col<R, 10>);
-        set((const void*)kb_spread_col<R, 12>);
-        set((const void*)kb_spread_col<R, 16>);
-        set((const void*)kb_spread_col<R, 20>);
-        set((const void*)kb_spread_col<R, 24>);
         set((const void*)kb_fft_xy<R>);
         set((const void*)kb_fft_z<R>);
         set((const void*)kb_fft_yx<R>);
@@ -184,10 +178,12 @@ inline int bin_weight_blocks(const Geo& g) {
 // weights in the scatter kernel (FP32) or by themselves (FP64: their
 // exponentials need the FP64 units of all SMs).
 template <typename R>
-void enqueue_bin(const Geo& g, const Work& w, int N, const R* pos, const R* q, R* Fzero, cudaStream_t s, bool pdl) {
+void enqueue_bin(const Geo& g, const Work& w, int N, const R* pos, const R* q, R* Fzero, R* gzero, cudaStream_t s,
+                 bool pdl) {
     using V = typename V4<R>::T;
     launch(false, true, k_bin_count<R>, g.nbin, kBinThreads, g.chunk * sizeof(int), s, g, N, pos, q, w.cnt_blk,
-           w.tcnt, w.crank, static_cast<V*>(w.cpos), static_cast<V*>(w.cfrac), w.cbase, Fzero, w.part + w.off_q);
+           w.tcnt, w.crank, static_cast<V*>(w.cpos), static_cast<V*>(w.cfrac), w.cbase, Fzero, w.part + w.off_q,
+           gzero);
     if (!g.bin_scan)
         launch(pdl, true, k_scan_mb, (g.ntiles + kScanMbSpan - 1) / kScanMbSpan, 1024, 0, s, (const int*)w.tcnt,
                w.tstart, g.ntiles, (int*)nullptr);
@@ -249,6 +245,23 @@ void enqueue_spread_brick(const Geo& g, const FftShape& fs, const FftPlanDev& fp
     launch(pdl, true, k, fs.brick_grid, fs.brick_threads, fs.brick_smem, s, g, fp, fs.brick_x, (const int*)w.tstart,
            static_cast<const V*>(w.sq), (const int*)w.sb, static_cast<const R*>(w.wb), static_cast<R*>(w.grid),
            static_cast<const C*>(w.tw), static_cast<C*>(w.spec1), fs.brick_lp);
+}
+
+// Reduction-form spreading: a warp per bead for few beads, else four CTAs per SM.
+template <typename R>
+inline void enqueue_spread_red(const Geo& g, const Work& w, int N, cudaStream_t s, bool pdl) {
+    using V = typename V4<R>::T;
+    auto k = k_spread_red<R, 0>;
+    switch (2 * g.p) {
+        case 4: k = k_spread_red<R, 4>; break;
+        case 6: k = k_spread_red<R, 6>; break;
+        case 8: k = k_spread_red<R, 8>; break;
+        case 12: k = k_spread_red<R, 12>; break;
+        default: break;
+    }
+    const int blocks = std::max(1, std::min(8 * 152, (N + 7) / 8));
+    launch(pdl, true, k, blocks, kRedThreads, 0, s, g, (const int*)w.tstart, static_cast<const V*>(w.sq),
+           (const int*)w.sb, static_cast<const R*>(w.wb), static_cast<R*>(w.grid));
 }
 
 // Scatter-form spreading (FP32, spread = 4): one CTA per region of edge sc_E.
@@ -360,11 +373,19 @@ cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp,
     // with per-stage events the two branches run one after the other, so that
     // each stage's events time its kernels alone
     if (ev && ev->on) s1 = s0;
+    if (fs.red_zero == 2) {   // beside the binning; the fork orders the spreading after it
+        cudaEventRecord(evFork, s0);
+        cudaStreamWaitEvent(s1, evFork, 0);
+        cudaMemsetAsync(w.grid, 0, (size_t)g.n * g.n * g.n * sizeof(R), s1);
+        cudaEventRecord(evJoin, s1);
+    }
     rec(ev, 0, true, s0);
-    enqueue_bin<R>(g, w, a.N, pos, q, a.zeroF ? F : nullptr, s0, pdl);
+    enqueue_bin<R>(g, w, a.N, pos, q, a.zeroF ? F : nullptr, fs.red_zero == 1 ? static_cast<R*>(w.grid) : nullptr, s0,
+                   pdl);
     rec(ev, 0, false, s0);
     log->kernels += bin_kernels<R>(g, w);
 
+    if (fs.red_zero == 2) cudaStreamWaitEvent(s0, evJoin, 0);
     // real-space branch
     cudaEventRecord(evFork, s0);
     cudaStreamWaitEvent(s1, evFork, 0);
@@ -389,7 +410,9 @@ cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp,
 
     // reciprocal branch
     rec(ev, 1, true, s0);
-    if constexpr (sizeof(R) == 4) {
+    if (fs.red) {
+        enqueue_spread_red<R>(g, w, a.N, s0, pdl && fs.red_zero == 1);
+    } else if constexpr (sizeof(R) == 4) {
         if (fs.spread == 4)
             enqueue_spread_sc(g, fs, w, s0, pdl);
         else if (fs.spread > 1)
@@ -507,7 +530,7 @@ cudaError_t enqueue_vv_post(const Geo& g, const Work& w, const DpdDev& d, cudaSt
 template <typename R>
 cudaError_t enqueue_spread_only(const Geo& g, const Work& w, const EvalArgs& a, void* grid_out, cudaStream_t s) {
     using V = typename V4<R>::T;
-    enqueue_bin<R>(g, w, a.N, static_cast<const R*>(a.pos), static_cast<const R*>(a.q), nullptr, s, true);
+    enqueue_bin<R>(g, w, a.N, static_cast<const R*>(a.pos), static_cast<const R*>(a.q), nullptr, nullptr, s, true);
     launch(true, true, k_spread<R>, g.ntiles, kSpreadThreads, spread_smem<R>(g), s, g, (const int*)w.tstart,
            static_cast<const V*>(w.sq), static_cast<const V*>(w.sw), (const int*)w.sb, static_cast<R*>(grid_out));
     return cudaGetLastError();

@@ -91,6 +91,7 @@ struct Geo {
     WinK<float> wkf;
     WinK<double> wkd;
     float Lhi, Llo;   // L split into two floats (FP32 wrap)
+    int real_lanes;   // real space: lanes per bead S while N_q S stays below this
     int slater;   // beta > 0: the real-space term carries the Slater correction
     // FP64 cutoff pre-test on float positions: r_c^2 plus a band that covers the float
     // error (positions and L rounded to float, |r2f - r2| <= ~1.5e-6 L r_c)
@@ -144,6 +145,10 @@ struct FftShape {
     // the forward x pass (the x pass kernel is then not launched), 4 scatter form
     // over regions of edge sc_E
     int spread;
+    // automatic choice of the tile or scatter form's sizes: the reduction form runs
+    // (1; plan info keeps reporting `spread`); the grid is cleared by the count kernel
+    // (1) or by a memset beside the binning (2)
+    int red, red_zero;
     int brick_x, brick_threads, brick_smem, brick_grid, brick_lp;
     int sc_E;
 };
@@ -268,7 +273,7 @@ struct BatchKernel {
     void* tab = nullptr;
     int* cmap = nullptr;
     int blocks = 0, threads = 0, smem = 0;
-    int T = 0;   // spreading: the tile edge of this group; gather: the common tap count 2p (0: mixed)
+    int T = 0;   // spreading (per group), gather: the common tap count 2p (0: mixed)
 };
 struct BatchLaunch {
     BatchKernel bin_count, bin_scatter, bin_weights, real, fft_xy, fft_z, fft_yx, gather;

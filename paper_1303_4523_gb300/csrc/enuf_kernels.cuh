@@ -472,7 +472,8 @@ __device__ __forceinline__ void k_bin_count_body(Geo g, int N, const R* __restri
                                                    int* __restrict__ tcnt, int* __restrict__ crank,
                                                    typename V4<R>::T* __restrict__ cpos,
                                                    typename V4<R>::T* __restrict__ cfrac, int* __restrict__ cbase,
-                                                   R* __restrict__ Fzero, double* __restrict__ qpart, Blk blk) {
+                                                   R* __restrict__ Fzero, double* __restrict__ qpart,
+                                                   R* __restrict__ gzero, Blk blk) {
     pdl_enter();
     extern __shared__ int slist[];   // [chunk]
     __shared__ int scount;
@@ -517,6 +518,13 @@ __device__ __forceinline__ void k_bin_count_body(Geo g, int N, const R* __restri
         }
     }
     __syncthreads();
+    if (gzero) {   // clear the grid for the reduction form of the spreading (n even: n^3 is a multiple of 8)
+        const int n4 = g.n * g.n * g.n / 4;
+        typename V4<R>::T z4;
+        z4.x = z4.y = z4.z = z4.w = (R)0;
+        for (int e = b * blockDim.x + threadIdx.x; e < n4; e += blk.n * blockDim.x)
+            reinterpret_cast<typename V4<R>::T*>(gzero)[e] = z4;
+    }
     const int nc = scount;
     const float rT = 1.0f / (float)g.T;
     for (int k = threadIdx.x; k < nc; k += blockDim.x) {
@@ -558,8 +566,9 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(Geo g, int N, const R
                                                    int* __restrict__ tcnt, int* __restrict__ crank,
                                                    typename V4<R>::T* __restrict__ cpos,
                                                    typename V4<R>::T* __restrict__ cfrac, int* __restrict__ cbase,
-                                                   R* __restrict__ Fzero, double* __restrict__ qpart) {
-    k_bin_count_body<R>(g, N, pos, q, cnt_blk, tcnt, crank, cpos, cfrac, cbase, Fzero, qpart, Blk{(int)blockIdx.x, (int)gridDim.x});
+                                                   R* __restrict__ Fzero, double* __restrict__ qpart,
+                                                   R* __restrict__ gzero) {
+    k_bin_count_body<R>(g, N, pos, q, cnt_blk, tcnt, crank, cpos, cfrac, cbase, Fzero, qpart, gzero, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // Exclusive scan of in[0, count) into out[0, count], out[count] = total; one
@@ -1464,6 +1473,80 @@ __global__ void __launch_bounds__(kScThreads) k_spread_sc(Geo g, const int* __re
         *reinterpret_cast<float4*>(grid + ((size_t)(oz + z) * n + (oy + y)) * n + ox + 4 * cq) =
             make_float4((float)v.x * iS, (float)v.y * iS, (float)v.z * iS, (float)v.w * iS);
     }
+}
+
+// ---------------------------------------------------------------------------
+// a2, reduction form: a warp per charged bead adds its (2p)^3 products
+// q w_x w_y w_z to the zeroed grid by global reductions, which the L2 executes;
+// lanes over (x, y) taps (rows of 2p consecutive points), a loop over the z
+// taps. No work on points outside a window, none repeated for neighbouring
+// tiles, and in FP64 the additions do not run on the SM's FP64 units at all
+// (one product per point does). Bound by the L2's reductions (~190 G sectors/s:
+// groups of four points per reduction, half the instructions on 1.4x the
+// sectors, took 44 against 34 us at 524k beads) and, at few beads, by latency.
+// Stage alone against the forms it replaces as the automatic choice (tile form
+// below n = 128, scatter form from there, slab form in FP64): FP32 3000 beads
+// 16.3 -> 6.1 us, 24k 28.6 -> 8.2, 81k 20.5 -> 10.2, 192k 32.7 -> 16.3, 524k
+// 57 -> 34, 3M 208 -> 190; FP64 3000 beads 61 -> 7.9, 375k 190 -> 52. The grid is
+// cleared by the count kernel (up to 16 16- or 32-byte stores a thread) or, when
+// it is large for its beads, by a memset beside the binning.
+// ---------------------------------------------------------------------------
+constexpr int kRedThreads = 256;
+
+// PT = 2p fixed at compile time (unrolled), or 0: any 2p <= 16.
+template <typename R, int PT>
+__device__ __forceinline__ void k_spread_red_body(const Geo& g, const int* __restrict__ tstart,
+                                                  const typename V4<R>::T* __restrict__ sq, const int* __restrict__ sb,
+                                                  const R* __restrict__ wb, R* __restrict__ grid, Blk blk) {
+    pdl_enter();
+    constexpr int NW = kRedThreads / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nq = tstart[g.ntiles], n = g.n, n2 = n * n, P2 = PT ? PT : 2 * g.p, p = P2 / 2;
+    const int rpi = 32 / P2;                    // y taps per round of lanes
+    const int nr = (P2 + rpi - 1) / rpi;        // rounds
+    const int b0 = lane / P2, a = lane - b0 * P2;
+    const bool on = b0 < rpi;
+    for (int s = blk.id * NW + warp; s < nq; s += blk.n * NW) {
+        const int pb = sb[s];
+        const R* w = wb + (size_t)s * 3 * P2;
+        const R wq = on ? sq[s].w * w[a] : (R)0;
+        const R wzl = lane < P2 ? w[2 * P2 + lane] : (R)0;
+        int x = (pb & 1023) - p + 1 + a;
+        x = x < 0 ? x + n : (x >= n ? x - n : x);
+        const int y0 = ((pb >> 10) & 1023) - p + 1;
+        int z = ((pb >> 20) & 1023) - p + 1;
+        z += z < 0 ? n : 0;
+        auto column = [&](int b) {   // the z taps of the lane's column in row b
+            const bool v = on && b < P2;
+            int y = y0 + (v ? b : 0);
+            y = y < 0 ? y + n : (y >= n ? y - n : y);
+            const R wxy = v ? wq * w[P2 + b] : (R)0;
+            R* col = grid + y * n + x;
+            int zz = z;
+#pragma unroll
+            for (int c = 0; c < (PT ? PT : kMaxTaps); ++c) {
+                if (!PT && c >= P2) break;
+                const R wz = __shfl_sync(0xffffffffu, wzl, c);
+                if (v && ENUF_GUARD(g.check, (unsigned)zz < (unsigned)n, 4)) atomicAdd(col + zz * n2, wxy * wz);
+                zz = zz + 1 == n ? 0 : zz + 1;
+            }
+        };
+        if constexpr (PT > 0) {
+            constexpr int RPI = 32 / PT, NR = (PT + RPI - 1) / RPI;
+#pragma unroll
+            for (int r = 0; r < NR; ++r) column(b0 + r * RPI);
+        } else {
+            for (int r = 0; r < nr; ++r) column(b0 + r * rpi);
+        }
+    }
+}
+
+template <typename R, int PT>
+__global__ void __launch_bounds__(kRedThreads) k_spread_red(Geo g, const int* __restrict__ tstart,
+                                                            const typename V4<R>::T* __restrict__ sq,
+                                                            const int* __restrict__ sb, const R* __restrict__ wb,
+                                                            R* __restrict__ grid) {
+    k_spread_red_body<R, PT>(g, tstart, sq, sb, wb, grid, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // ---------------------------------------------------------------------------
@@ -2448,9 +2531,9 @@ __device__ __forceinline__ void k_real_body(Geo g, const int* __restrict__ tstar
     int* list = reinterpret_cast<int*>(smraw) + warp * 32 * kRealQ + lane;   // FP32: entry k at 32 k
     int2* ring = reinterpret_cast<int2*>(smraw) + warp * kRealRing;          // FP64
     const int nq = tstart[g.ntiles];
-    // lanes per bead: as many as give every lane of the launch work
+    // lanes per bead: enough to fill the chip, no more (see the plan's real_lanes)
     int S = 32;
-    while (S > 1 && (long long)nq * S > (long long)blk.n * kRealThreads) S >>= 1;
+    while (S > 1 && (long long)nq * S > (S > 8 ? g.real_lanes / 3 * 2 : g.real_lanes)) S >>= 1;
     RealSum<R> a{(R)0, (R)0, (R)0, (R)0, (R)0};
     if (2 * g.rs + 1 >= g.ntd)
         real_sweep<R, true>(g, nq, S, tstart, sq, sw, sb, spf, list, ring, F, a, blk);

@@ -9,7 +9,7 @@ import oracle as orc  # noqa: F401  (the oracle is built with the library)
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from test_gpu_enuf import TOL, Ref, _bead_max, _gpu, _inputs, _rel_rms, enuf  # noqa: E402,F401
+from test_gpu_enuf import TOL, Ref, _bead_max, _gpu, _inputs, _oparams, _rel_rms, enuf  # noqa: E402,F401
 
 
 def _beads(L, nq, cluster, seed, solvent=37):
@@ -54,4 +54,26 @@ def test_real_space_lists(enuf, prec, name, box, nq, cluster):
     assert _rel_rms(F, ref.F) < t["F"] and _bead_max(F, ref.F) < 100 * t["F"]
     own = max(abs(ref.E[0]), abs(ref.E[2])) if prec == "fp32" else abs(ref.E[0])
     assert abs(E[0] - ref.E[0]) <= t["E"] * own, (E, ref.E)
+    plan.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5, 6, 8])
+@pytest.mark.parametrize("L,M,nq", [(8.0, 12, 300), (9.0, 16, 33), (28.8, 48, 7)])
+def test_reduction_spread_grid(enuf, prec, p, L, M, nq):
+    """The automatic spreading's grid for every window width (unrolled and not),
+    windows across all faces, a grid cleared by the count kernel and one large for
+    its beads (cleared by a memset), and the same again on the used workspace."""
+    P = dict(L=L, M=M, p=p, alpha=1.0, r_cut=3.0, beta=4.0, kappa=1.1)
+    rng = np.random.default_rng(100 * M + p)
+    pos = rng.uniform(-0.02 * L, 1.02 * L, (nq + 20, 3))
+    q = np.where(np.arange(nq + 20) < nq, rng.choice([-1.0, 1.0, 2.0], nq + 20), 0.0)
+    pos, q = _inputs(prec, pos, q)
+    plan, F, E, Wv = _gpu(enuf, prec, P, pos, q)
+    dt = torch.float32 if prec == "fp32" else torch.float64
+    again = torch.empty((nq + 20, 3), dtype=dt, device="cuda")
+    plan.energy_forces(torch.tensor(pos, dtype=dt, device="cuda"), torch.tensor(q, dtype=dt, device="cuda"), again)
+    grid = plan.debug_buffer(enuf.ENUF_BUF_GRID).astype(np.float64)
+    _, _, g_ref, _ = orc.recip_enuf(_oparams(P), pos, q, want_grid=True)
+    assert np.abs(grid - g_ref).max() < TOL[prec]["stage"] * np.abs(g_ref).max()
     plan.close()
