@@ -89,8 +89,10 @@ typedef struct {
                          memory, x+y and y+x fused); 1: always the five line passes x, y, z, y, x */
     int    fft_radix; /* line transforms: 0 = automatic: FP32 grids whose n = f1 f2 with
                          f1, f2 in {4, 5, 6, 8, 10, 12, 16, 20} take the two-factor
-                         kernels (both DFTs in registers, one twiddle pass); other grids
-                         and FP64 the Stockham stages as for 2;
+                         kernels (both DFTs in registers, one twiddle pass), as do, with radices
+                         9, 15 and 18, grids that only then split (n = 108, 180, 216, 288, 300;
+                         enuf_plan_info reports these as for 2); other grids and FP64 the
+                         Stockham stages as for 2;
                          1 = Stockham stages over radices 2, 3, 4, 5, 8 only;
                          2 = Stockham stages, the fewest over 2, 3, 4, 5, 8, and for FP32
                          grids from n = 128 on the composite radices 6, 10, 12, 16, 20

@@ -133,19 +133,29 @@ bool fft_radices(int n, FftPlanDev& fp, bool composite) {
 
 // Two-factor split n = f1 f2 of the FP32 two-factor kernels: both factors in
 // their radix set; the most balanced split, ties to the larger f2 (phase A
-// reads f2 consecutive elements per line and load). False: none.
-bool fft_two_factor(int n, FftPlanDev& fp) {
+// reads f2 consecutive elements per line and load). Lengths without such a
+// split (108, 180, 216, 288, 300, 360, ...) take radices 9, 15 and 18 as well
+// (*ext; plan info then keeps reporting their Stockham schedule): five passes
+// at n = 180 in 172 us against 227 on three Stockham stages. False: none.
+bool fft_two_factor(int n, FftPlanDev& fp, int* ext) {
     static const int kF[] = {4, 5, 6, 8, 10, 12, 16, 20};
+    static const int kFx[] = {4, 5, 6, 8, 9, 10, 12, 15, 16, 18, 20};
     int best1 = 0, best2 = 0;
-    for (int a : kF)
-        for (int b : kF)
-            if (a * b == n) {
+    auto split = [&](const int* f, int cnt) {
+        for (int i = 0; i < cnt; ++i)
+            for (int j = 0; j < cnt; ++j) {
+                const int a = f[i], b = f[j];
+                if (a * b != n) continue;
                 const int m = std::min(a, b), mb = std::min(best1, best2);
                 if (!best1 || m > mb || (m == mb && b > best2)) {
                     best1 = a;
                     best2 = b;
                 }
             }
+    };
+    split(kF, 8);
+    *ext = best1 ? 0 : 1;
+    if (!best1) split(kFx, 11);
     fp.f1 = best1;
     fp.f2 = best2;
     return best1 > 0;
@@ -290,7 +300,8 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
     if (!fft_radices(n, fp, P.prec == ENUF_FP32 && P.fft_radix != 1))
         return fail(plan, ENUF_ERR_UNSUPPORTED, "grid n = %d is not 2^a 3^b 5^c", n);
     fp.f1 = fp.f2 = 0;
-    if (P.prec == ENUF_FP32 && P.fft_radix == 0) fft_two_factor(n, fp);
+    int two_ext = 0;
+    if (P.prec == ENUF_FP32 && P.fft_radix == 0) fft_two_factor(n, fp, &two_ext);
     if (2 * P.p > n) return fail(plan, ENUF_ERR_INVALID, "window 2p = %d wider than the grid", 2 * P.p);
     // tile edge: divides n, >= p, histogram fits in shared memory
     // the spreading kernel holds a T^3 tile of the grid in shared memory: T <= 24
@@ -392,6 +403,7 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
         // two-factor kernels: per line f1 (f2 + 1) phase-A values and n + 1 results;
         // threads: one phase-A or phase-B task per thread (f2 resp. f1 per line)
         fs.two = 1;
+        fs.two_ext = two_ext;
         const int lsa = fft2_lsa(fp.f1, fp.f2), lsb = fft2_lsb(n), per_line = (lsa + lsb) * csz;
         const int fmax = std::max(fp.f1, fp.f2);
         auto shape2 = [&](int total_lines, int mult, int& lines, int& threads, int& grid, int bud) {
@@ -449,7 +461,7 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
         const int stage = brick_stage_bytes<float>();
         // fused: LP line pairs of the x transform after the brick (shared with the staging)
         int lp = 0, fx_smem = 0;
-        const bool fx_ok = fs.two && !fs.fused && T % 2 == 0;
+        const bool fx_ok = fs.two && !fs.two_ext && !fs.fused && T % 2 == 0;
         if (fx_ok) {
             const int per_line = (fft2_lsa(fp.f1, fp.f2) + fft2_lsb(n)) * csz;
             const int acc = T * T * n * rsz;
@@ -936,11 +948,12 @@ static void fill_info(const enuf_plan_s* plan, enuf_plan_info* info) {
     info->n_max = plan->n_max;
     info->fft_kernels = plan->fs.fused ? 3 : (plan->fs.spread == 3 ? 4 : 5);
     info->device_bytes = plan->dbytes;
-    info->fft_two_factor = plan->fp.f1 ? 1 : 0;
+    const bool two = plan->fp.f1 && !plan->fs.two_ext;
+    info->fft_two_factor = two ? 1 : 0;
     info->spread = plan->fs.spread;
     info->brick_x = plan->fs.spread == 2 || plan->fs.spread == 3 ? plan->fs.brick_x : 0;
     info->pairs = pair_launches(plan->P);
-    if (plan->fp.f1) {
+    if (two) {
         info->fft_stages = 2;
         for (int i = 0; i < 8; ++i) info->fft_radix[i] = i == 0 ? plan->fp.f1 : (i == 1 ? plan->fp.f2 : 0);
     } else {
@@ -1425,7 +1438,7 @@ namespace {
 bool batch_plan_ok(const enuf_plan_s* p) {
     const int T = p->g.T;
     const bool col = T == 8 || T == 10 || T == 12 || T == 16 || T == 20 || T == 24;
-    return p->prec == ENUF_FP32 && p->fs.two && p->fs.fused && p->fs.spread == 1 && col && p->g.bin_scan &&
+    return p->prec == ENUF_FP32 && p->fs.two && !p->fs.two_ext && p->fs.fused && p->fs.spread == 1 && col && p->g.bin_scan &&
            p->w.wb != nullptr;
 }
 

@@ -127,19 +127,33 @@ cudaError_t configure_kernels(int max_smem) {
     };
     if constexpr (sizeof(R) == 4) {
         carve((const void*)k2_fft_x<R>);
+        carve((const void*)k2_fft_x<R, true>);
         carve((const void*)k2_fft_y<R>);
+        carve((const void*)k2_fft_y<R, true>);
         carve((const void*)k2_fft_z<R>);
+        carve((const void*)k2_fft_z<R, true>);
         carve((const void*)k2_fft_zp<R>);
+        carve((const void*)k2_fft_zp<R, true>);
         carve((const void*)k2_fft_iy<R>);
+        carve((const void*)k2_fft_iy<R, true>);
         carve((const void*)k2_fft_ix<R>);
+        carve((const void*)k2_fft_ix<R, true>);
         set((const void*)k2_fft_x<R>);
+        set((const void*)k2_fft_x<R, true>);
         set((const void*)k2_fft_y<R>);
+        set((const void*)k2_fft_y<R, true>);
         set((const void*)k2_fft_z<R>);
+        set((const void*)k2_fft_z<R, true>);
         set((const void*)k2_fft_zp<R>);
+        set((const void*)k2_fft_zp<R, true>);
         set((const void*)k2_fft_iy<R>);
+        set((const void*)k2_fft_iy<R, true>);
         set((const void*)k2_fft_ix<R>);
+        set((const void*)k2_fft_ix<R, true>);
         set((const void*)k2_fft_xy<R>);
+        set((const void*)k2_fft_xy<R, true>);
         set((const void*)k2_fft_yx<R>);
+        set((const void*)k2_fft_yx<R, true>);
         set((const void*)k_spread_brick<R, false>);
         set((const void*)k_spread_brick<R, true>);
         set((const void*)k_spread_sc<16, 8>);
@@ -278,36 +292,36 @@ inline void enqueue_spread_sc(const Geo& g, const FftShape& fs, const Work& w, c
 // evZ (or nullptr) is recorded right after the z pass, whose blocks write the
 // reciprocal energy and virial partials (the kernel after it then launches
 // without programmatic dependent launch: its stream predecessor is the record).
-template <typename R>
+template <typename R, bool EXT>
 void enqueue_fft2(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0, bool pdl,
                   LaunchLog* log, cudaEvent_t evZ) {
     using C = typename Cx<R>::T;
     const C* tw = static_cast<const C*>(w.tw);
     if (fs.fused) {
-        launch(pdl, true, k2_fft_xy<R>, g.n, fs.t_xy, fs.smem_xy, s0, g, fp, static_cast<const R*>(w.grid), tw,
+        launch(pdl, true, k2_fft_xy<R, EXT>, g.n, fs.t_xy, fs.smem_xy, s0, g, fp, static_cast<const R*>(w.grid), tw,
                static_cast<C*>(w.spec2));
-        launch(pdl, true, k2_fft_z<R>, fs.grid_z, fs.tz, fs.smem_z, s0, g, fp, static_cast<const C*>(w.spec2), tw,
+        launch(pdl, true, k2_fft_z<R, EXT>, fs.grid_z, fs.tz, fs.smem_z, s0, g, fp, static_cast<const C*>(w.spec2), tw,
                (const double*)w.tab, (const double*)w.tabv, static_cast<const R*>(w.tabr), static_cast<C*>(w.spec3),
                w.part + w.off_recip, fs.lz, 1);
         if (evZ) cudaEventRecord(evZ, s0);
-        launch(pdl && !evZ, true, k2_fft_yx<R>, g.nf * g.n, fs.t_yx, fs.smem_yx, s0, g, fp,
+        launch(pdl && !evZ, true, k2_fft_yx<R, EXT>, g.nf * g.n, fs.t_yx, fs.smem_yx, s0, g, fp,
                static_cast<const C*>(w.spec3), tw, static_cast<R*>(w.h));
         log->kernels += 4;
     } else {
         if (fs.spread != 3) {
-            launch(pdl, true, k2_fft_x<R>, fs.grid_x, fs.tx, fs.smem_x, s0, g, fp, static_cast<const R*>(w.grid), tw,
+            launch(pdl, true, k2_fft_x<R, EXT>, fs.grid_x, fs.tx, fs.smem_x, s0, g, fp, static_cast<const R*>(w.grid), tw,
                    static_cast<C*>(w.spec1), fs.lx);
             log->kernels += 1;
         }
-        launch(pdl, true, k2_fft_y<R>, dim3(g.nc + 1, fs.grid_y_z), fs.ty, fs.smem_y, s0, g, fp,
+        launch(pdl, true, k2_fft_y<R, EXT>, dim3(g.nc + 1, fs.grid_y_z), fs.ty, fs.smem_y, s0, g, fp,
                static_cast<const C*>(w.spec1), tw, static_cast<C*>(w.spec2), fs.ly);
-        launch(pdl, true, k2_fft_zp<R>, fs.grid_z, fs.tz, fs.smem_z, s0, g, fp, static_cast<const C*>(w.spec2), tw,
+        launch(pdl, true, k2_fft_zp<R, EXT>, fs.grid_z, fs.tz, fs.smem_z, s0, g, fp, static_cast<const C*>(w.spec2), tw,
                (const double*)w.tab, (const double*)w.tabv, static_cast<const R*>(w.tabr), static_cast<C*>(w.spec3),
                w.part + w.off_recip, fs.lz);
         if (evZ) cudaEventRecord(evZ, s0);
-        launch(pdl && !evZ, true, k2_fft_iy<R>, fs.grid_iy, fs.tiy, fs.smem_iy, s0, g, fp,
+        launch(pdl && !evZ, true, k2_fft_iy<R, EXT>, fs.grid_iy, fs.tiy, fs.smem_iy, s0, g, fp,
                static_cast<const C*>(w.spec3), tw, static_cast<C*>(w.spec4), fs.liy);
-        launch(pdl, true, k2_fft_ix<R>, fs.grid_ix, fs.tix, fs.smem_ix, s0, g, fp, static_cast<const C*>(w.spec4),
+        launch(pdl, true, k2_fft_ix<R, EXT>, fs.grid_ix, fs.tix, fs.smem_ix, s0, g, fp, static_cast<const C*>(w.spec4),
                tw, static_cast<R*>(w.h), fs.lix);
         log->kernels += 5;   // the spreading kernel and four passes
     }
@@ -428,8 +442,10 @@ cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp,
     // step's energies but the kinetic one while the last FFT pass and the gather run
     const cudaEvent_t ez = evZ && evT ? evZ : nullptr;
     if constexpr (sizeof(R) == 4) {
-        if (fs.two)
-            enqueue_fft2<R>(g, fs, fp, w, s0, pdl, log, ez);
+        if (fs.two_ext)
+            enqueue_fft2<R, true>(g, fs, fp, w, s0, pdl, log, ez);
+        else if (fs.two)
+            enqueue_fft2<R, false>(g, fs, fp, w, s0, pdl, log, ez);
         else if (fs.composite)
             enqueue_fft<R, true>(g, fs, fp, w, s0, pdl, log, ez);
         else

@@ -9,7 +9,8 @@
 // w = e^{-+2 pi i/n}), does an R-point DFT and writes the results to
 // (j - k) R + k + m Ns. After the last stage the line is in natural order.
 // Radices 2, 3, 4, 5, 8 and the composites 6, 10, 12, 16, 20 (two small DFTs
-// in registers with compile-time twiddles), so most lengths take two stages.
+// in registers with compile-time twiddles), so most lengths take two stages
+// (9, 15 and 18 serve the two-factor transform below only).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -254,9 +255,12 @@ struct CompositeDft {
     }
 };
 template <typename R, bool INV> struct SmallDft<R, 6, INV> : CompositeDft<R, 2, 3, INV> {};
+template <typename R, bool INV> struct SmallDft<R, 9, INV> : CompositeDft<R, 3, 3, INV> {};
 template <typename R, bool INV> struct SmallDft<R, 10, INV> : CompositeDft<R, 2, 5, INV> {};
 template <typename R, bool INV> struct SmallDft<R, 12, INV> : CompositeDft<R, 4, 3, INV> {};
+template <typename R, bool INV> struct SmallDft<R, 15, INV> : CompositeDft<R, 3, 5, INV> {};
 template <typename R, bool INV> struct SmallDft<R, 16, INV> : CompositeDft<R, 4, 4, INV> {};
+template <typename R, bool INV> struct SmallDft<R, 18, INV> : CompositeDft<R, 2, 9, INV> {};
 template <typename R, bool INV> struct SmallDft<R, 20, INV> : CompositeDft<R, 4, 5, INV> {};
 
 // One Stockham stage over nlines lines (line l at offset l*ls, swizzled inside).
@@ -426,7 +430,9 @@ __host__ __device__ constexpr int fft2_lsb(int n) { return n + 1; }
 // fft2_twiddles fills. buf holds nlines rows
 // of fft2_lsa(f1, f2) values. Contains __syncthreads (call from all threads);
 // the caller synchronises before reading what store wrote to shared memory.
-template <typename R, bool INV, typename Load, typename Store>
+// EXT: radices 9, 15 and 18 are compiled in as well (instances of their own:
+// in the common kernels the larger switch cost 0.7-1.2 us a launch at n = 96).
+template <typename R, bool INV, bool EXT, typename Load, typename Store>
 __device__ __forceinline__ void fft2_lines(typename Cx<R>::T* __restrict__ buf, const typename Cx<R>::T* tw,
                                            const FftPlanDev& fp, int nlines, Load&& load, Store&& store) {
     const int f1 = fp.f1, f2 = fp.f2, lsa = fft2_lsa(f1, f2);
@@ -439,7 +445,13 @@ __device__ __forceinline__ void fft2_lines(typename Cx<R>::T* __restrict__ buf, 
         case 12: fft2_phase_a<R, 12, INV>(buf, lsa, nlines, f2, tw, load); break;
         case 16: fft2_phase_a<R, 16, INV>(buf, lsa, nlines, f2, tw, load); break;
         case 20: fft2_phase_a<R, 20, INV>(buf, lsa, nlines, f2, tw, load); break;
-        default: break;
+        default:
+            if constexpr (EXT) {
+                if (f1 == 9) fft2_phase_a<R, 9, INV>(buf, lsa, nlines, f2, tw, load);
+                else if (f1 == 15) fft2_phase_a<R, 15, INV>(buf, lsa, nlines, f2, tw, load);
+                else if (f1 == 18) fft2_phase_a<R, 18, INV>(buf, lsa, nlines, f2, tw, load);
+            }
+            break;
     }
     __syncthreads();
     switch (f2) {
@@ -451,7 +463,13 @@ __device__ __forceinline__ void fft2_lines(typename Cx<R>::T* __restrict__ buf, 
         case 12: fft2_phase_b<R, 12, INV>(buf, lsa, nlines, f1, store); break;
         case 16: fft2_phase_b<R, 16, INV>(buf, lsa, nlines, f1, store); break;
         case 20: fft2_phase_b<R, 20, INV>(buf, lsa, nlines, f1, store); break;
-        default: break;
+        default:
+            if constexpr (EXT) {
+                if (f2 == 9) fft2_phase_b<R, 9, INV>(buf, lsa, nlines, f1, store);
+                else if (f2 == 15) fft2_phase_b<R, 15, INV>(buf, lsa, nlines, f1, store);
+                else if (f2 == 18) fft2_phase_b<R, 18, INV>(buf, lsa, nlines, f1, store);
+            }
+            break;
     }
 }
 

@@ -27,7 +27,7 @@ namespace enuf {
 // Persistent CTAs over groups of LP line pairs (2 LP consecutive real rows,
 // one contiguous run of the grid), the next group's rows copied into shared
 // memory asynchronously while the current group is transformed.
-template <typename R>
+template <typename R, bool EXT = false>
 __global__ void __launch_bounds__(512) k2_fft_x(Geo g, FftPlanDev fp, const R* __restrict__ grid,
                                                const typename Cx<R>::T* __restrict__ twg,
                                                typename Cx<R>::T* __restrict__ spec1, int LP) {
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(512) k2_fft_x(Geo g, FftPlanDev fp, const R* _
         const R* src = In + buf * per;
         const int row0 = grp * 2 * LP;   // first real row (z n + y), y even
         const int nl = min(LP, npairs - grp * LP);
-        fft2_lines<R, false>(
+        fft2_lines<R, false, EXT>(
             A, tw, fp, nl,
             [&](int c, int x) {
                 C v;
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(512) k2_fft_x(Geo g, FftPlanDev fp, const R* _
 }
 
 // forward y for lines (z, kx): spec1[z][kx][y] -> spec2[kx][ky][z], |ky| <= nc
-template <typename R>
+template <typename R, bool EXT = false>
 __global__ void __launch_bounds__(512) k2_fft_y(Geo g, FftPlanDev fp, const typename Cx<R>::T* __restrict__ spec1,
                                                const typename Cx<R>::T* __restrict__ twg,
                                                typename Cx<R>::T* __restrict__ spec2, int LB) {
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(512) k2_fft_y(Geo g, FftPlanDev fp, const type
     const int z0 = blockIdx.y * LB;
     const int nl = min(LB, n - z0);
     __syncthreads();
-    fft2_lines<R, false>(
+    fft2_lines<R, false, EXT>(
         A, tw, fp, nl, [&](int c, int y) { return spec1[((size_t)(z0 + c) * nc1 + kx) * n + y]; },
         [&](int c, int k, C v) {
             if (k <= nc || k >= n - nc) B[c * lsb + k] = v;
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(512) k2_fft_y(Geo g, FftPlanDev fp, const type
 // transform of the lines (elements from load(c, z)), the energy and virial
 // sums of their kept modes added to se, sv, the inverse transforms, and the
 // fields written to spec3. Contains __syncthreads (call from all threads).
-template <typename R, typename Load>
+template <typename R, bool EXT, typename Load>
 __device__ __forceinline__ void k2_z_lines(const Geo& g, const FftPlanDev& fp, const typename Cx<R>::T* tw,
                                            typename Cx<R>::T* A, typename Cx<R>::T* B, int l0, int nl, Load&& load,
                                            const double* __restrict__ tab, const double* __restrict__ tabv,
@@ -143,7 +143,7 @@ __device__ __forceinline__ void k2_z_lines(const Geo& g, const FftPlanDev& fp, c
     const int n = g.n, nc = g.nc, K = g.K, nf = g.nf, lsb = fft2_lsb(n);
     const int NL = (nc + 1) * K;
     const int ni = nf == 3 ? 2 : 1;   // inverse transforms per line
-    fft2_lines<R, false>(A, tw, fp, nl, load, [&](int c, int k, C v) {
+    fft2_lines<R, false, EXT>(A, tw, fp, nl, load, [&](int c, int k, C v) {
         if (k <= nc || k >= n - nc) B[c * lsb + k] = v;
     });
     __syncthreads();
@@ -164,7 +164,7 @@ __device__ __forceinline__ void k2_z_lines(const Geo& g, const FftPlanDev& fp, c
     }
     // inverse transforms of every line: line b nl + c of the batch (b = 0: G,
     // or D F in gradient mode; b = 1: Gz)
-    fft2_lines<R, true>(
+    fft2_lines<R, true, EXT>(
         A, tw, fp, ni * nl,
         [&](int line, int m) {
             const int b = line >= nl ? 1 : 0;
@@ -207,7 +207,7 @@ __device__ __forceinline__ void k2_z_lines(const Geo& g, const FftPlanDev& fp, c
     }
 }
 
-template <typename R>
+template <typename R, bool EXT = false>
 __device__ __forceinline__ void k2_fft_z_body(Geo g, FftPlanDev fp, const typename Cx<R>::T* __restrict__ spec2,
                                                const typename Cx<R>::T* __restrict__ twg,
                                                const double* __restrict__ tab, const double* __restrict__ tabv,
@@ -227,10 +227,10 @@ __device__ __forceinline__ void k2_fft_z_body(Geo g, FftPlanDev fp, const typena
     __syncthreads();
     double se = 0.0, sv = 0.0;
     if (plane_major)   // spec2[z][l]: lines gathered across planes
-        k2_z_lines<R>(g, fp, tw, A, B, l0, nl, [&](int c, int z) { return spec2[(size_t)z * NL + l0 + c]; }, tab,
+        k2_z_lines<R, EXT>(g, fp, tw, A, B, l0, nl, [&](int c, int z) { return spec2[(size_t)z * NL + l0 + c]; }, tab,
                       tabv, tabr, spec3, se, sv);
     else               // spec2[l][z]: lines contiguous
-        k2_z_lines<R>(g, fp, tw, A, B, l0, nl, [&](int c, int z) { return spec2[(size_t)(l0 + c) * n + z]; }, tab,
+        k2_z_lines<R, EXT>(g, fp, tw, A, B, l0, nl, [&](int c, int z) { return spec2[(size_t)(l0 + c) * n + z]; }, tab,
                       tabv, tabr, spec3, se, sv);
     block_sum2(se, sv);
     if (threadIdx.x == 0) {
@@ -239,20 +239,20 @@ __device__ __forceinline__ void k2_fft_z_body(Geo g, FftPlanDev fp, const typena
     }
 }
 
-template <typename R>
+template <typename R, bool EXT = false>
 __global__ void __launch_bounds__(512) k2_fft_z(Geo g, FftPlanDev fp, const typename Cx<R>::T* __restrict__ spec2,
                                                const typename Cx<R>::T* __restrict__ twg,
                                                const double* __restrict__ tab, const double* __restrict__ tabv,
                                                const R* __restrict__ tabr, typename Cx<R>::T* __restrict__ spec3,
                                                double* __restrict__ epart, int LB, int plane_major) {
-    k2_fft_z_body<R>(g, fp, spec2, twg, tab, tabv, tabr, spec3, epart, LB, plane_major, Blk{(int)blockIdx.x, (int)gridDim.x});
+    k2_fft_z_body<R, EXT>(g, fp, spec2, twg, tab, tabv, tabr, spec3, epart, LB, plane_major, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // The z pass over lines contiguous in spec2 ([l][z], the five-pass layout) with
 // persistent CTAs: groups of LB lines, the next group's lines copied into
 // shared memory asynchronously while this one is transformed; one energy
 // partial per CTA.
-template <typename R>
+template <typename R, bool EXT = false>
 __global__ void __launch_bounds__(512) k2_fft_zp(Geo g, FftPlanDev fp, const typename Cx<R>::T* __restrict__ spec2,
                                                 const typename Cx<R>::T* __restrict__ twg,
                                                 const double* __restrict__ tab, const double* __restrict__ tabv,
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(512) k2_fft_zp(Geo g, FftPlanDev fp, const typ
         __syncthreads();
         const C* Ig = In + buf * per;
         const int l0 = grp * LB, nl = min(LB, NL - l0);
-        k2_z_lines<R>(g, fp, tw, A, B, l0, nl, [&](int c, int z) { return Ig[c * n + z]; }, tab, tabv, tabr, spec3,
+        k2_z_lines<R, EXT>(g, fp, tw, A, B, l0, nl, [&](int c, int z) { return Ig[c * n + z]; }, tab, tabv, tabr, spec3,
                       se, sv);
         __syncthreads();
     }
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(512) k2_fft_zp(Geo g, FftPlanDev fp, const typ
 }
 
 // inverse y for lines (a, z, kx): K inputs zero-padded to n; output spec4[a][z][y][kx]
-template <typename R>
+template <typename R, bool EXT = false>
 __global__ void __launch_bounds__(512) k2_fft_iy(Geo g, FftPlanDev fp, const typename Cx<R>::T* __restrict__ spec3,
                                                 const typename Cx<R>::T* __restrict__ twg,
                                                 typename Cx<R>::T* __restrict__ spec4, int LB) {
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(512) k2_fft_iy(Geo g, FftPlanDev fp, const typ
     const int l0 = blockIdx.x * LB;
     const int nl = min(LB, NLT - l0);
     __syncthreads();
-    fft2_lines<R, true>(
+    fft2_lines<R, true, EXT>(
         A, tw, fp, nl,
         [&](int c, int m) {
             const int ky = m <= n / 2 ? m : m - n;
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(512) k2_fft_iy(Geo g, FftPlanDev fp, const typ
 // 16-byte offset), copied into shared memory with asynchronous 16-byte copies
 // one group ahead, so a group's transform runs while the next group's rows are
 // in flight (the pass was bound by the latency of its loads).
-template <typename R>
+template <typename R, bool EXT = false>
 __global__ void __launch_bounds__(512) k2_fft_ix(Geo g, FftPlanDev fp, const typename Cx<R>::T* __restrict__ spec4,
                                                 const typename Cx<R>::T* __restrict__ twg, R* __restrict__ h,
                                                 int LP) {
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(512) k2_fft_ix(Geo g, FftPlanDev fp, const typ
         const C* Ig = In + buf * per;
         const int row0 = grp * 2 * LP;
         const int nl = min(LP, npairs - grp * LP);
-        fft2_lines<R, true>(
+        fft2_lines<R, true, EXT>(
             A, tw, fp, nl,
             [&](int c, int m) {
                 const C* ra = Ig + 2 * c * nc1;
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(512) k2_fft_ix(Geo g, FftPlanDev fp, const typ
 // rows as n/2 complex lines, x transforms split into the half spectra
 // kx = 0..nc (the y columns), y transforms of the nc + 1 columns, keep
 // |ky| <= nc; output spec2[z][kx][ky] (plane-major).
-template <typename R>
+template <typename R, bool EXT = false>
 __device__ __forceinline__ void k2_fft_xy_body(Geo g, FftPlanDev fp, const R* __restrict__ grid,
                                                 const typename Cx<R>::T* __restrict__ twg,
                                                 typename Cx<R>::T* __restrict__ spec2, Blk blk) {
@@ -437,7 +437,7 @@ __device__ __forceinline__ void k2_fft_xy_body(Geo g, FftPlanDev fp, const R* __
     const int z = blk.id;
     const R* gz = grid + (size_t)z * n * n;
     __syncthreads();
-    fft2_lines<R, false>(
+    fft2_lines<R, false, EXT>(
         A, tw, fp, h,
         [&](int c, int x) {
             C v;
@@ -465,7 +465,7 @@ __device__ __forceinline__ void k2_fft_xy_body(Geo g, FftPlanDev fp, const R* __
     }
     __syncthreads();
     C* out = spec2 + (size_t)z * nc1 * K;
-    fft2_lines<R, false>(
+    fft2_lines<R, false, EXT>(
         B, tw, fp, nc1, [&](int kx, int y) { return P[kx * n + y]; },
         [&](int kx, int k, C v) {
             if (k <= nc) out[kx * K + k + nc] = v;
@@ -473,18 +473,18 @@ __device__ __forceinline__ void k2_fft_xy_body(Geo g, FftPlanDev fp, const R* __
         });
 }
 
-template <typename R>
+template <typename R, bool EXT = false>
 __global__ void __launch_bounds__(512) k2_fft_xy(Geo g, FftPlanDev fp, const R* __restrict__ grid,
                                                 const typename Cx<R>::T* __restrict__ twg,
                                                 typename Cx<R>::T* __restrict__ spec2) {
-    k2_fft_xy_body<R>(g, fp, grid, twg, spec2, Blk{(int)blockIdx.x, (int)gridDim.x});
+    k2_fft_xy_body<R, EXT>(g, fp, grid, twg, spec2, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // Inverse y and x of one (field, z-plane) in shared memory (small grids):
 // the plane spec3[a][z][kx][ky] zero-padded to n along y, inverse y of the
 // nc + 1 columns, then two Hermitian rows per complex line (C2R) inverse
 // along x; output h[a][z][y][x].
-template <typename R>
+template <typename R, bool EXT = false>
 __device__ __forceinline__ void k2_fft_yx_body(Geo g, FftPlanDev fp, const typename Cx<R>::T* __restrict__ spec3,
                                                 const typename Cx<R>::T* __restrict__ twg, R* __restrict__ h, Blk blk) {
     pdl_enter();
@@ -498,7 +498,7 @@ __device__ __forceinline__ void k2_fft_yx_body(Geo g, FftPlanDev fp, const typen
     const int az = blk.id;   // a * n + z
     const C* in = spec3 + (size_t)az * nc1 * K;
     __syncthreads();
-    fft2_lines<R, true>(
+    fft2_lines<R, true, EXT>(
         A, tw, fp, nc1,
         [&](int kx, int m) {
             const int ky = m <= n / 2 ? m : m - n;
@@ -511,7 +511,7 @@ __device__ __forceinline__ void k2_fft_yx_body(Geo g, FftPlanDev fp, const typen
         [&](int kx, int y, C v) { Yc[kx * lsb + y] = v; });
     __syncthreads();
     R* out = h + (size_t)az * n * n;
-    fft2_lines<R, true>(
+    fft2_lines<R, true, EXT>(
         A, tw, fp, hn,
         [&](int c, int m) {
             C a, b;
@@ -539,10 +539,10 @@ __device__ __forceinline__ void k2_fft_yx_body(Geo g, FftPlanDev fp, const typen
         });
 }
 
-template <typename R>
+template <typename R, bool EXT = false>
 __global__ void __launch_bounds__(512) k2_fft_yx(Geo g, FftPlanDev fp, const typename Cx<R>::T* __restrict__ spec3,
                                                 const typename Cx<R>::T* __restrict__ twg, R* __restrict__ h) {
-    k2_fft_yx_body<R>(g, fp, spec3, twg, h, Blk{(int)blockIdx.x, (int)gridDim.x});
+    k2_fft_yx_body<R, EXT>(g, fp, spec3, twg, h, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 }  // namespace enuf
@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(768) k_spread_brick(Geo g, FftPlanDev fp, int 
         for (int c0 = 0; c0 < npair; c0 += LP) {
             const int nl = min(LP, npair - c0);
             __syncthreads();
-            fft2_lines<R, false>(
+            fft2_lines<R, false, false>(
                 A, tw, fp, nl,
                 [&](int c, int x) {
                     C v;

@@ -141,6 +141,7 @@ struct FftShape {
     int t_xy, t_yx, smem_xy, smem_yx;
     int composite;   // the radix plan uses 6, 10, 12, 16 or 20 (FP32): the CR kernel instances
     int two;         // FP32 two-factor kernels (FftPlanDev::f1, f2), same shapes and layouts
+    int two_ext;     // their split uses radix 9, 15 or 18 (reported as the Stockham schedule)
     // spreading: 1 tile form, 2 footprint bricks into the grid, 3 bricks fused with
     // the forward x pass (the x pass kernel is then not launched), 4 scatter form
     // over regions of edge sc_E

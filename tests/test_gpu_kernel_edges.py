@@ -9,7 +9,7 @@ import oracle as orc  # noqa: F401  (the oracle is built with the library)
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from test_gpu_enuf import TOL, Ref, _bead_max, _gpu, _inputs, _oparams, _rel_rms, enuf  # noqa: E402,F401
+from test_gpu_enuf import TOL, Ref, _bead_max, _check, _gpu, _inputs, _oparams, _rel_rms, enuf  # noqa: E402,F401
 
 
 def _beads(L, nq, cluster, seed, solvent=37):
@@ -77,3 +77,28 @@ def test_reduction_spread_grid(enuf, prec, p, L, M, nq):
     _, _, g_ref, _ = orc.recip_enuf(_oparams(P), pos, q, want_grid=True)
     assert np.abs(grid - g_ref).max() < TOL[prec]["stage"] * np.abs(g_ref).max()
     plan.close()
+
+
+@pytest.mark.parametrize("deriv", [0, 1])
+@pytest.mark.parametrize("n,fft_path", [(108, 0), (108, 1), (180, 0), (216, 0), (288, 0), (300, 0), (360, 0)])
+def test_fft_radices_9_15_18(enuf, n, fft_path, deriv):
+    """FP32 grids that split into two register radices only with 9, 15 or 18: the
+    fields against the Stockham stages' on the same beads (FP32 FFT rounding,
+    ~1e-6 of the largest value), forces and energies against the oracle's up to
+    n = 216 (its plain DFTs take n^4 steps)."""
+    L = n / 5.0
+    P = dict(L=L, M=n // 2, p=4, alpha=1.0, r_cut=3.0, beta=4.0, kappa=1.1, fft_path=fft_path, deriv=deriv)
+    rng = np.random.default_rng(n)
+    pos = rng.uniform(0.0, L, (300, 3))
+    q = np.where(np.arange(300) % 2 == 0, 1.0, -1.0)
+    pos, q = _inputs("fp32", pos, q)
+    plan, F, E, Wv = _gpu(enuf, "fp32", P, pos, q)
+    other, F2, E2, _ = _gpu(enuf, "fp32", dict(P, fft_radix=2), pos, q)
+    assert plan.info.fft_two_factor == 0 and plan.info.fft_kernels == other.info.fft_kernels
+    h, h2 = (x.debug_buffer(enuf.ENUF_BUF_FIELD).astype(np.float64) for x in (plan, other))
+    assert np.abs(h - h2).max() < TOL["fp32"]["stage"] * np.abs(h2).max()
+    assert _rel_rms(F, F2) < TOL["fp32"]["F"] and abs(E[1] - E2[1]) < TOL["fp32"]["E"] * abs(E2[1])
+    if n <= 216:
+        _check("fp32", F, E, Wv, Ref(P, pos, q))
+    plan.close()
+    other.close()
