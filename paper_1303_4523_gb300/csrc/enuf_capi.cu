@@ -1149,6 +1149,9 @@ enuf_status initial_force(dpd_system_t sys) {
                        plan->stream));
     enuf_status st = enqueue_force_eval(sys, plan->stream, plan->aux, nullptr, &log);
     if (st != ENUF_OK) return st;
+    cudaError_t e = plan->prec == ENUF_FP32 ? enqueue_dpd_add<float>(sys->d, plan->stream, &log, true)
+                                            : enqueue_dpd_add<double>(sys->d, plan->stream, &log, true);
+    if (e != cudaSuccess) return fail(plan, ENUF_ERR_CUDA, "dpd forces: %s", cudaGetErrorString(e));
     st = enqueue_tot(plan, true, plan->stream, &log);
     if (st != ENUF_OK) return st;
     CU(cudaMemcpyAsync(plan->hE, plan->w.Edev, 16 * sizeof(double), cudaMemcpyDeviceToHost, plan->stream));
@@ -1245,16 +1248,11 @@ enuf_status dpd_create(enuf_plan_t plan, const dpd_params* params, int n, const 
         d.rk1[r] = (uint32_t)(d.seed >> 32) + (uint32_t)r * 0xBB67AE85u;
     }
     d.rdt = 1.0 / std::sqrt(params->dt);
-    // cell blocks of B^3 cells: the largest B <= 4 (and <= ncd - 2, so the
-    // (B + 2)^3 halo holds distinct cells) whose mean halo population stays
-    // below 85% of the staging capacity (density 3: B = 4; density 4: B = 3)
-    d.B = std::max(1, std::min(4, d.ncd - 2));
-    {
-        const double cell = L / d.ncd;
-        const double per_cell = (double)n / (L * L * L) * cell * cell * cell;
-        while (d.B > 1 && (d.B + 2) * (d.B + 2) * (d.B + 2) * per_cell > 0.85 * kDpdCap) --d.B;
-    }
+    // pair sweep: S lanes per bead while N S stays below this (4 steps of 20000 / 40000 /
+    // 81000 beads: 232 / 285 / 377 us at 300 per SM, 264 / 306 / 404 at 1100)
+    d.lanes = 512 * kSMs;
     d.cinv = (double)d.ncd / L;
+    d.cinvf = (float)d.cinv;
     d.xmaxf = largest_float_below(L);
     d.kd = DpdK<double>{L, 0.5 * L, d.gamma, d.sigma * d.rdt, d.K_bond, d.r0_bond, 1.0 / L};
     d.kf = DpdK<float>{(float)L, (float)(0.5 * L), (float)d.gamma, (float)(d.sigma * d.rdt), (float)d.K_bond,
@@ -1271,7 +1269,7 @@ enuf_status dpd_create(enuf_plan_t plan, const dpd_params* params, int n, const 
                  o_atab = take((size_t)d.ntypes * d.ntypes * rs), o_bnd = take(std::max<size_t>(1, (size_t)n_bonds) * 8),
                  o_ckey = take(nz * 4),
                  o_ccount = take((size_t)d.ncells * 4), o_cstart = take(((size_t)d.ncells + 1) * 4),
-                 o_ccur = take(((size_t)d.ncells + 1) * 4), o_sp = take(nz * 4 * rs), o_sv = take(nz * 4 * rs),
+                 o_ccur = take(((size_t)d.ncells + 1) * 4), o_sp = take(nz * 4 * rs), o_sv = take(nz * 4 * rs), o_df = take(nz * sizeof(float4)),
                  o_step = take(8);
     cudaError_t e = dev_alloc(&sys->dmem, off);
     if (e != cudaSuccess) {
@@ -1285,7 +1283,8 @@ enuf_status dpd_create(enuf_plan_t plan, const dpd_params* params, int n, const 
     d.bnd = reinterpret_cast<int*>(b + o_bnd);
     d.ckey = reinterpret_cast<int*>(b + o_ckey); d.ccount = reinterpret_cast<int*>(b + o_ccount);
     d.cstart = reinterpret_cast<int*>(b + o_cstart); d.ccur = reinterpret_cast<int*>(b + o_ccur);
-    d.sp = b + o_sp; d.sv = b + o_sv; d.step_dev = reinterpret_cast<uint64_t*>(b + o_step);
+    d.sp = b + o_sp; d.sv = b + o_sv; d.df = reinterpret_cast<float4*>(b + o_df);
+    d.step_dev = reinterpret_cast<uint64_t*>(b + o_step);
     auto bail = [&](enuf_status s) { dpd_destroy(sys); return s; };
     if (cudaMemset(sys->dmem, 0, off) != cudaSuccess) return bail(fail(plan, ENUF_ERR_CUDA, "memset failed"));
     std::vector<char> at((size_t)d.ntypes * d.ntypes * rs);

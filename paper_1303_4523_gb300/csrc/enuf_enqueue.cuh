@@ -371,6 +371,12 @@ auto gather_kernel(int taps) {
     }
 }
 
+// Float positions of the cell-sorted beads.
+template <typename R>
+inline const float4* dpd_spf(const DpdDev& d) {
+    return sizeof(R) == 8 ? d.df : static_cast<const float4*>(d.sp);
+}
+
 template <typename R>
 cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w,
                          const EvalArgs& a, cudaStream_t s0, cudaStream_t s1, cudaEvent_t evFork,
@@ -409,10 +415,10 @@ cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp,
     if (dpd) {   // DPD pairs and real-space pairs in one launch
         const DpdDev& d = *dpd;
         launch(false, false, k_pairs<R>, w.nblk_dpd + w.nblk_real, kRealThreads,
-               std::max(real_smem, dpd_smem_bytes<R>()), s1, d, d.B, static_cast<const V*>(d.sp),
-               static_cast<const V*>(d.sv), (const int*)d.cstart, static_cast<const R*>(d.atab),
-               static_cast<const R*>(d.pos), (const int*)d.bnd, (const uint64_t*)d.step_dev, static_cast<R*>(d.F),
-               w.part + w.off_dpd, w.nblk_dpd, g, (const int*)w.tstart, (const V*)sq, (const V*)sw,
+               std::max(real_smem, dpd_smem_bytes<R>()), s1, d, static_cast<const V*>(d.sp),
+               static_cast<const V*>(d.sv), dpd_spf<R>(d), (const int*)d.cstart, static_cast<const R*>(d.atab),
+               static_cast<const R*>(d.pos), (const int*)d.bnd, (const uint64_t*)d.step_dev, d.df,
+               static_cast<R*>(d.F), w.part + w.off_dpd, w.nblk_dpd, g, (const int*)w.tstart, (const V*)sq, (const V*)sw,
                (const int*)w.sb, spf, w.part + w.off_real);
     } else {
         launch(false, false, k_real<R>, w.nblk_real, kRealThreads, real_smem, s1, g, (const int*)w.tstart,
@@ -503,16 +509,16 @@ cudaError_t enqueue_dpd_forces(const Work& w, const DpdDev& d, cudaStream_t s, E
         launch(pdl, false, k_scan, 1, 1024, 0, s, d.ccount, d.cstart, d.ncells, d.ccur, 0);
     launch(pdl, false, k_cell_scatter<R>, blocks, 256, 0, s, d.N, d.L, d.xmaxf, d.Lhi, d.Llo,
            static_cast<const R*>(d.pos),
-           static_cast<const R*>(d.v0), (const int*)d.type, (const int*)d.ckey, d.ccur, static_cast<V*>(d.sp),
-           static_cast<V*>(d.sv), d.ccount, d.ncells);
+           static_cast<const R*>(d.v0), (const int*)d.type, d.ckey, d.ccur, static_cast<V*>(d.sp),
+           static_cast<V*>(d.sv), d.df, d.ccount, d.ncells);
     rec(ev, 7, false, s);
     log->kernels += 3;
     if (!pair_kernel) return cudaGetLastError();   // the pairs run in k_pairs with the real space
     rec(ev, 5, true, s);
     const int dpd_smem = dpd_smem_bytes<R>();
-    launch(pdl, false, k_dpd<R>, w.nblk_dpd, kDpdThreads, dpd_smem, s, d, d.B, static_cast<const V*>(d.sp),
-           static_cast<const V*>(d.sv), (const int*)d.cstart, static_cast<const R*>(d.atab),
-           static_cast<const R*>(d.pos), (const int*)d.bnd, (const uint64_t*)d.step_dev, static_cast<R*>(d.F),
+    launch(pdl, false, k_dpd<R>, w.nblk_dpd, kDpdThreads, dpd_smem, s, d, static_cast<const V*>(d.sp),
+           static_cast<const V*>(d.sv), dpd_spf<R>(d), (const int*)d.cstart, static_cast<const R*>(d.atab),
+           static_cast<const R*>(d.pos), (const int*)d.bnd, (const uint64_t*)d.step_dev, d.df, static_cast<R*>(d.F),
            w.part + w.off_dpd);
     rec(ev, 5, false, s);
     log->kernels += 1;
@@ -536,8 +542,19 @@ cudaError_t enqueue_vv_post(const Geo& g, const Work& w, const DpdDev& d, cudaSt
     TotalsArgs t = totals_args(g, w, true, 2);
     if (pre) t.pre = w.part + w.off_pre;
     launch(pdl, true, k_vv_post<R>, w.nblk_kin, 256, 0, s, g, d.N, (R)d.dt, static_cast<R*>(d.vel),
-           static_cast<const R*>(d.F), w.part + w.off_kin, t);
+           static_cast<R*>(d.F), (const float4*)d.df, (const int*)d.ckey, w.part + w.off_kin, t);
     log->kernels += 1;
+    return cudaGetLastError();
+}
+
+// FP32: the DPD pair forces into F, after a force evaluation outside a step.
+template <typename R>
+cudaError_t enqueue_dpd_add(const DpdDev& d, cudaStream_t s, LaunchLog* log, bool pdl) {
+    if constexpr (sizeof(R) == 4) {
+        launch(pdl, true, k_dpd_add, std::max(1, std::min(4 * 152, (d.N + 255) / 256)), 256, 0, s, d.N,
+               static_cast<float*>(d.F), (const float4*)d.df, (const int*)d.ckey);
+        log->kernels += 1;
+    }
     return cudaGetLastError();
 }
 
@@ -571,6 +588,7 @@ namespace enuf {
     template cudaError_t enqueue_vv_pre<R>(const DpdDev&, cudaStream_t, LaunchLog*);                         \
     template cudaError_t enqueue_vv_post<R>(const Geo&, const Work&, const DpdDev&, cudaStream_t, LaunchLog*,  \
                                             bool, bool);                                                     \
+    template cudaError_t enqueue_dpd_add<R>(const DpdDev&, cudaStream_t, LaunchLog*, bool);                   \
     template cudaError_t enqueue_spread_only<R>(const Geo&, const Work&, const EvalArgs&, void*, cudaStream_t);
 
 }  // namespace enuf

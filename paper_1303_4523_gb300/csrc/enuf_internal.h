@@ -100,10 +100,6 @@ struct Geo {
     unsigned int* check;  // debug builds: failure bits of the device index checks
 };
 
-// Beads of one DPD cell block plus its halo that the pair kernel stages in
-// shared memory (blocks with more take the unstaged path).
-constexpr int kDpdCap = 896;
-
 // Footprint spreading on bricks (k_spread_brick): staging capacities and the
 // shared memory of a brick of T x T rows of BX points (fx_bytes: the fused x
 // pass's twiddles and line buffers, which reuse the staging region).
@@ -217,10 +213,11 @@ struct TotalsArgs {
 struct DpdDev {
     unsigned int* check;   // the plan's check word (debug builds)
     int N, ntypes, ncd, ncells;
-    int B;             // cells per block edge of the DPD kernel (<= 4, B + 2 <= ncd)
+    int lanes;         // pair sweep: lanes per bead S while N S stays below this
     double L, gamma, sigma, dt, lambda_vv, K_bond, r0_bond;
     double rdt;    // 1 / sqrt(dt)
     double cinv;   // ncd / L
+    float cinvf;
     DpdK<float> kf;
     DpdK<double> kd;
     float Lhi, Llo;   // L split into two floats (FP32 wrap)
@@ -237,6 +234,9 @@ struct DpdDev {
     int* bnd;                // bond pairs [nbonds][2]
     int* ckey; int* ccount; int* cstart; int* ccur;
     void* sp; void* sv;      // real4 [N] sorted: (x, y, z, orig) and (v0, type)
+    // float4 [N], sorted order: FP32 the DPD force accumulators (ckey then holds every
+    // bead's slot), FP64 a float copy of the positions
+    float4* df;
     uint64_t* step_dev;      // device copy of the step counter
 };
 
@@ -304,6 +304,8 @@ cudaError_t enqueue_vv_pre(const DpdDev& d, cudaStream_t s, LaunchLog* log);
 template <typename R>
 cudaError_t enqueue_vv_post(const Geo& g, const Work& w, const DpdDev& d, cudaStream_t s, LaunchLog* log, bool pdl,
                             bool pre = false);
+template <typename R>
+cudaError_t enqueue_dpd_add(const DpdDev& d, cudaStream_t s, LaunchLog* log, bool pdl);
 template <typename R>
 cudaError_t enqueue_spread_only(const Geo& g, const Work& w, const EvalArgs& a, void* grid_out, cudaStream_t s);
 // Batched launch sequence (FP32): a system qualifies when its plan runs the

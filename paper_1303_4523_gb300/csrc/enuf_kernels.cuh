@@ -34,6 +34,8 @@ __device__ __forceinline__ const WinK<float>& win_k(const Geo& g, float) { retur
 __device__ __forceinline__ const WinK<double>& win_k(const Geo& g, double) { return g.wkd; }
 __device__ __forceinline__ const DpdK<float>& dpd_k(const DpdDev& d, float) { return d.kf; }
 __device__ __forceinline__ const DpdK<double>& dpd_k(const DpdDev& d, double) { return d.kd; }
+__device__ __forceinline__ float dpd_cinv(const DpdDev& d, float) { return d.cinvf; }
+__device__ __forceinline__ double dpd_cinv(const DpdDev& d, double) { return d.cinv; }
 
 // Programmatic dependent launch (sm_90 and later): every kernel first waits
 // until the grid before it in the stream has completed and its writes are
@@ -2583,12 +2585,14 @@ __global__ void k_cell_count(int N, int ncd, double L, R rinv, float xmaxf, floa
 }
 
 // Also clears the cell counts for the next step's k_cell_count (the scan has
-// read them).
+// read them). FP32: clears the force accumulators of the sorted beads (df) and
+// leaves every bead's slot in ckey; FP64: a float copy of the positions (spf).
 template <typename R>
-__global__ void k_cell_scatter(int N, double L, float xmaxf, float Lhi, float Llo, const R* __restrict__ pos, const R* __restrict__ v0,
-                               const int* __restrict__ type, const int* __restrict__ ckey,
+__global__ void k_cell_scatter(int N, double L, float xmaxf, float Lhi, float Llo, const R* __restrict__ pos,
+                               const R* __restrict__ v0, const int* __restrict__ type, int* __restrict__ ckey,
                                int* __restrict__ ccur, typename V4<R>::T* __restrict__ sp,
-                               typename V4<R>::T* __restrict__ sv, int* __restrict__ ccount, int ncells) {
+                               typename V4<R>::T* __restrict__ sv, float4* __restrict__ df, int* __restrict__ ccount,
+                               int ncells) {
     pdl_enter();
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) ccount[c] = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
@@ -2604,6 +2608,12 @@ __global__ void k_cell_scatter(int N, double L, float xmaxf, float Lhi, float Ll
         b.w = int_as_real(type[i], (R)0);
         sp[slot] = a;
         sv[slot] = b;
+        if constexpr (sizeof(R) == 4) {
+            df[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
+            ckey[i] = slot;
+        } else {
+            df[slot] = make_float4((float)a.x, (float)a.y, (float)a.z, 0.f);
+        }
     }
 }
 
@@ -2659,369 +2669,126 @@ __device__ __forceinline__ R dpd_theta(const PhiloxStep& ps, const DpdDev& d, in
                (R)(1.7320508075688772935 * (2.3283064365386962890625e-10 - 1.0)));
 }
 
-// DPD pair forces (Eq. 2-7, R_c = 1) + bonds (Sec. 2), added into F (which
-// the caller zeroes): F[i] += F^C + F^D + F^R/sqrt(dt) + F^S. One CTA per B^3
-// block of cells; the beads of the (B+2)^3 halo cells are staged in shared
-// memory in halo-cell order (a warp per halo row: the H cells of a row along
-// x are one contiguous run of the staged order). Every pair is evaluated once
-// (Newton's third law; theta_ij is symmetric): a bead's partners are the
-// beads of its forward half shell -- the beads after it in its own cell and
-// the 13 neighbouring cells lexicographically after it, which in the staged
-// copy are 5 contiguous runs of slots. One lane per central bead walks its
-// runs (dpd_beads); the pairs within r = 1 go to a per-warp ring of pairs and
-// the pair arithmetic (Philox draw, weights, dissipation) runs on full warps.
-// The forces go out by global reductions, +f to i and -f to j (executed in
-// L2: shared-memory float adds are compare-and-swap loops on this part, and
-// in FP64 each of their iterations costs an add on the few FP64 units). The
-// harmonic bonds run as one thread per bond into F. A block whose halo holds
-// more beads than the staging capacity sweeps the global cell list instead,
-// one warp per central cell (dpd_cells).
+// DPD pair forces (Eq. 2-7, R_c = 1): F^C + F^D + F^R/sqrt(dt) on every pair
+// closer than 1, each pair once (Newton's third law; theta_ij is symmetric),
+// and the bonds (Sec. 2), one thread per bond, into F (zeroed by the caller).
 //
-// The staged copies are unwrapped: the halo cells that lie across a box
-// face are shifted by L, so the plain difference of two staged positions is
-// the minimum image of every pair within r = 1 (cell edge >= 1) and no pair
-// needs the wrap test. FP64: the cutoff test r^2 < 1 is taken on a float copy
-// of the staged positions first and redone in double only inside a band
-// around 1 (and near 0) that covers the float error, so the decision is the
-// double one.
+// S lanes per bead of the cell-sorted order, 32 / S consecutive beads per warp,
+// as in the real-space sweep: a bead's partners are the beads of its forward
+// half shell -- those after it in its own cell, the next cell along x, the
+// cells x-1..x+1 of the row (0, +1) and of the rows (+1, -1..1) -- which are 5
+// contiguous runs of sorted beads (and their parts across the box face), read
+// straight from the sorted arrays. Cells have an edge > 1 and there are at
+// least 3 per dimension, so a run's image shift is one constant.
+//   FP32: each lane notes its pairs in a list of its own and evaluates the
+//     lists in step; the force on its bead stays in registers, -f goes to bead
+//     j's accumulator by one 16-byte reduction (df, sorted order, cleared by
+//     k_cell_scatter; the closing kick adds it to F).
+//   FP64: the cutoff is tested on a float copy, the pairs go to a ring per warp
+//     and are decided and evaluated on full warps (every FP64 instruction costs
+//     the whole warp); +f and -f go to F by global reductions.
+// The form before staged 4^3-cell blocks with their halo in shared memory: 512
+// blocks of uneven size at 81k beads, six 4-byte reductions per pair. The one
+// launch of both pair sums at 81k beads 49 -> 39 us (FP32), the step 101 -> 94;
+// steps of 3000 beads 56 -> 44; FP64 steps 374 -> 357 (bound by the FP64
+// instructions of the pairs in either form).
 constexpr int kDpdThreads = 256;
-// kDpdCap (staged beads per block) is in enuf_internal.h: the host sizes the
-// cell blocks against it
-constexpr int kDpdMaxB = 4;      // cells per block edge
-constexpr int kDpdSegU = 14;     // unstaged half shell: single cells
-constexpr int kDpdU = 4;         // bead sweep: candidates per lane and iteration
-constexpr int kDpdQ = 256;       // bead sweep: pair ring per warp (>= 31 + 32 kDpdU, a power of 2)
-static_assert(kDpdQ >= 31 + 32 * kDpdU && (kDpdQ & (kDpdQ - 1)) == 0, "pair ring");
-
 template <typename R>
-constexpr int dpd_smem_bytes() {
-    return 2 * kDpdCap * (int)sizeof(typename V4<R>::T) + (sizeof(R) == 8 ? kDpdCap * (int)sizeof(float4) : 0) +
-           (kDpdThreads / 32) * kDpdQ * 8;
+constexpr int dpd_smem_bytes() { return real_smem_bytes<R>(); }
+
+// Four consecutive floats by one reduction (16-byte aligned).
+__device__ __forceinline__ void red_add4(float4* p, float a, float b, float c, float d) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
-// One warp-wide batch of up to 32 queued pairs (valid lanes) of the global
-// cell list (wrapped positions: minimum image), all lanes call. The queue
-// holds runs of one i (dpd_cells loops over i inside a candidate chunk): in
-// FP32 the +f of a run is summed in the warp first, then added once; in FP64
-// it goes per pair (the segmented sum would run on the few FP64 units).
-template <typename R, typename V>
-__device__ __forceinline__ void dpd_pairs(const bool valid, const int2 e, const V* __restrict__ P,
-                                          const V* __restrict__ Pv, R* __restrict__ F,
-                                          const R* __restrict__ atab, int ntypes, R L, R hL, R gam, R srdt,
-                                          const PhiloxStep& ps, const DpdDev& d, R& ec) {
-    const int lane = threadIdx.x & 31;
-    R fx = 0, fy = 0, fz = 0;
-    int key = -1, oi = 0;
-    if (valid) {
-        const V pi = P[e.x], vi = Pv[e.x];
-        const V pj = P[e.y], vj = Pv[e.y];
-        const R rx = min_image(pi.x, pj.x, L, hL);
-        const R ry = min_image(pi.y, pj.y, L, hL);
-        const R rz = min_image(pi.z, pj.z, L, hL);
-        const R r2 = dist2(rx, ry, rz);
-        const R ir = r_rsqrt(r2);
-        const R r = r2 * ir;
-        const R w = (R)1 - r;
-        const int i = real_as_int(pi.w), j = real_as_int(pj.w);
-        const int ti = real_as_int(vi.w), tj = real_as_int(vj.w);
-        const R a = atab[ti * ntypes + tj];
-        const R vd = (vi.x - vj.x) * rx + (vi.y - vj.y) * ry + (vi.z - vj.z) * rz;   // r_ij . v_ij
-        const R th = dpd_theta<R>(ps, d, i, j);
-        // Eq. 3-5 with w^D = (w^R)^2 = w^2: |F| = w (a - gamma w (r.v)/r + sigma theta/sqrt(dt))
-        const R wi = w * ir;
-        const R fm = wi * fma(-gam * wi, vd, fma(srdt, th, a));
-        fx = fm * rx;
-        fy = fm * ry;
-        fz = fm * rz;
-        // -f to bead j: a global reduction (executed in L2, no compare-and-swap loop)
-        atomicAdd(&F[3 * j], -fx);
-        atomicAdd(&F[3 * j + 1], -fy);
-        atomicAdd(&F[3 * j + 2], -fz);
-        ec = fma(a * w, w, ec);   // a w^2; halved once per block
-        key = e.x;
-        oi = i;
-    }
-    if constexpr (sizeof(R) == 8) {
-        // FP64: +f to bead i per pair as well (the segmented sum below would
-        // run its adds and double shuffles on the few FP64 units)
-        if (key >= 0) {
-            atomicAdd(&F[3 * oi], fx);
-            atomicAdd(&F[3 * oi + 1], fy);
-            atomicAdd(&F[3 * oi + 2], fz);
-        }
-        (void)lane;
-        return;
-    }
-    // runs of equal i: sum each run into its first lane (segmented suffix sums)
-    const int prev = __shfl_up_sync(0xffffffffu, key, 1);
-    const bool head = lane == 0 || prev != key;
-    const unsigned heads = __ballot_sync(0xffffffffu, head);
-    const unsigned after = lane == 31 ? 0u : heads & (0xffffffffu << (lane + 1));
-    const int end = after ? __ffs(after) - 1 : 32;
-    // levels up to the longest run of the batch (typically 2-3 of 5)
-    const int longest = __reduce_max_sync(0xffffffffu, head ? end - lane : 0);
-    for (int o = 1; o < longest; o <<= 1) {
-        const R ax = __shfl_down_sync(0xffffffffu, fx, o);
-        const R ay = __shfl_down_sync(0xffffffffu, fy, o);
-        const R az = __shfl_down_sync(0xffffffffu, fz, o);
-        if (lane + o < end) {
-            fx += ax;
-            fy += ay;
-            fz += az;
-        }
-    }
-    if (head && key >= 0) {
-        atomicAdd(&F[3 * oi], fx);
-        atomicAdd(&F[3 * oi + 1], fy);
-        atomicAdd(&F[3 * oi + 2], fz);
-    }
-}
-
-// The exact cutoff decision 0 < r^2 < 1 in the working precision (WRAP:
-// minimum image of wrapped positions; else the unwrapped staged frame).
-template <typename R, typename V, bool WRAP>
-__device__ __forceinline__ bool dpd_within(const V& pi, const V& pj, R L, R hL) {
-    const R rx = WRAP ? min_image(pi.x, pj.x, L, hL) : pi.x - pj.x;
-    const R ry = WRAP ? min_image(pi.y, pj.y, L, hL) : pi.y - pj.y;
-    const R rz = WRAP ? min_image(pi.z, pj.z, L, hL) : pi.z - pj.z;
-    const R r2 = dist2(rx, ry, rz);
-    return r2 < (R)1 && r2 > (R)0;
-}
-
-struct DpdBand {   // float pre-test of the FP64 path: r2f > hi: out; lo0 < r2f < lo: in; else exact
-    float L, hL, lo0, lo, hi;
-};
-
-// All central cells of one block on the global cell list (a block whose halo
-// overflows the staging capacity), one warp per cell: lanes over the
-// candidates of the cell's half shell (its own cell, the next along x and the
-// 12 cells of the rows after it, each looked up wrapped), a loop over the
-// cell's beads; positions are wrapped, so pairs take the minimum image.
+// |F| / r of a pair at squared distance r2 (Eq. 3-5 with w^D = (w^R)^2 = w^2):
+// w (a - gamma w (r.v)/r + sigma theta/sqrt(dt)) / r; adds a w^2 to ec.
 template <typename R>
-__device__ __forceinline__ void dpd_cells(const DpdDev& d, int H, int B3, const int* chalo, const int* hoff,
-                                          const int* gst, const typename V4<R>::T* __restrict__ P,
-                                          const typename V4<R>::T* __restrict__ Pv, int2* queue,
-                                          const R* __restrict__ atab, uint64_t step, R* __restrict__ F, R& ec) {
-    using V = typename V4<R>::T;
-    constexpr int NW = kDpdThreads / 32;
-    constexpr int nseg = kDpdSegU;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const R L = dpd_k(d, (R)0).L, hL = dpd_k(d, (R)0).hL;
-    const R gam = dpd_k(d, (R)0).gam, srdt = dpd_k(d, (R)0).srdt;
-    const PhiloxStep ps = philox_step(d, step);
-    int cnt = 0;   // queued pairs of this warp, carried across its cells
-    for (int cc = warp; cc < B3; cc += NW) {
-        const int h = chalo[cc];
-        if (h < 0) continue;
-        const int cb = gst[h];
-        const int nself = hoff[h + 1] - hoff[h];
-        if (nself == 0) continue;
-        // lane s < nseg: cell s of the half shell as (start slot, length)
-        int sst = 0, sln = 0;
-        if (lane < nseg) {
-            int hc;
-            if (lane == 0) hc = h;
-            else if (lane == 1) hc = h + 1;
-            else if (lane < 5) hc = h + H + (lane - 3);
-            else hc = h + H * H + ((lane - 5) / 3 - 1) * H + ((lane - 5) % 3 - 1);
-            sst = gst[hc];
-            sln = hoff[hc + 1] - hoff[hc];
-        }
-        int x = sln;   // inclusive prefix of the cell counts
-#pragma unroll
-        for (int o = 1; o < 16; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        const int soff = x - sln;          // cell s starts at map position soff
-        const int delta = sst - soff;      // slot = map position + delta
-        const int mc = __shfl_sync(0xffffffffu, x, nseg - 1);
-        // lanes over the map (one candidate j per lane per chunk), loop over the
-        // cell's beads i (broadcast loads); queue runs are then runs of one i
-        for (int jb = 0; jb < mc; jb += 32) {
-            const int jf = jb + lane;
-            int s = 0;
-            for (int k = 1; k < nseg; ++k) s += jf >= __shfl_sync(0xffffffffu, soff, k) ? 1 : 0;
-            const int j = jf + __shfl_sync(0xffffffffu, delta, s);
-            const bool vj = jf < mc;
-            V pj;
-            if (vj) pj = P[j];
-            for (int ii = 0; ii < nself; ++ii) {
-                const int me = cb + ii;
-                // forward only within the cell itself (run 0)
-                bool hit = false;
-                if (vj && (s != 0 || j > me)) hit = dpd_within<R, V, true>(P[me], pj, L, hL);
-                const unsigned m = __ballot_sync(0xffffffffu, hit);
-                if (hit && ENUF_GUARD(d.check, cnt + __popc(m & ((1u << lane) - 1u)) < 64, 9))
-                    queue[cnt + __popc(m & ((1u << lane) - 1u))] = make_int2(me, j);
-                cnt += __popc(m);
-                if (cnt >= 32) {
-                    __syncwarp();
-                    dpd_pairs<R, V>(true, queue[lane], P, Pv, F, atab, d.ntypes, L, hL, gam, srdt, ps, d, ec);
-                    __syncwarp();
-                    if (lane < cnt - 32) queue[lane] = queue[32 + lane];
-                    __syncwarp();
-                    cnt -= 32;
-                }
-            }
-        }
-    }
-    __syncwarp();
-    if (cnt > 0) dpd_pairs<R, V>(lane < cnt, queue[lane], P, Pv, F, atab, d.ntypes, L, hL, gam, srdt, ps, d, ec);
-}
-
-// One warp-wide batch of up to 32 queued pairs (i, j) whose i are mostly
-// distinct (the bead sweep below queues one pair per lane and candidate):
-// +f to i and -f to j, each by one global reduction per component.
-template <typename R, typename V>
-__device__ __forceinline__ void dpd_pairs_red(const bool valid, const int2 e, const V* __restrict__ P,
-                                              const V* __restrict__ Pv, R* __restrict__ F,
-                                              const R* __restrict__ atab, int ntypes, R gam, R srdt,
-                                              const PhiloxStep& ps, const DpdDev& d, R& ec) {
-    if (!valid) return;
-    const V pi = P[e.x], vi = Pv[e.x];
-    const V pj = P[e.y], vj = Pv[e.y];
-    const R rx = pi.x - pj.x, ry = pi.y - pj.y, rz = pi.z - pj.z;   // unwrapped staged frame
-    const R r2 = dist2(rx, ry, rz);
+__device__ __forceinline__ R dpd_force(const DpdDev& d, const PhiloxStep& ps, R r2, R vd, R a, int i, int j, R& ec) {
     const R ir = r_rsqrt(r2);
     const R w = (R)1 - r2 * ir;
-    const int i = real_as_int(pi.w), j = real_as_int(pj.w);
-    const R a = atab[real_as_int(vi.w) * ntypes + real_as_int(vj.w)];
-    const R vd = (vi.x - vj.x) * rx + (vi.y - vj.y) * ry + (vi.z - vj.z) * rz;   // r_ij . v_ij
     const R th = dpd_theta<R>(ps, d, i, j);
-    // Eq. 3-5 with w^D = (w^R)^2 = w^2: |F| = w (a - gamma w (r.v)/r + sigma theta/sqrt(dt))
     const R wi = w * ir;
-    const R fm = wi * fma(-gam * wi, vd, fma(srdt, th, a));
-    const R fx = fm * rx, fy = fm * ry, fz = fm * rz;
-    atomicAdd(&F[3 * i], fx);
-    atomicAdd(&F[3 * i + 1], fy);
-    atomicAdd(&F[3 * i + 2], fz);
-    atomicAdd(&F[3 * j], -fx);
-    atomicAdd(&F[3 * j + 1], -fy);
-    atomicAdd(&F[3 * j + 2], -fz);
-    ec = fma(a * w, w, ec);   // a w^2; halved once per block
+    ec = fma(a * w, w, ec);   // halved once per block
+    return wi * fma(-dpd_k(d, (R)0).gam * wi, vd, fma(dpd_k(d, (R)0).srdt, th, a));
 }
 
-// The staged pair sweep with one lane per central bead: lane f of the block's
-// central beads (cpre: prefix of the central cells' counts) walks the forward
-// half shell of its cell -- the rest of its own cell and the next cell along
-// x (run 0: slots after its own), the row (0, +1, -1..1) (run 1) and the
-// three rows (+1, -1..1, -1..1) (runs 2-4), each a contiguous run of staged
-// slots -- one candidate per iteration. A warp tests 32 beads' candidates at
-// once; the pairs within r = 1 go to the warp's queue and are evaluated on
-// full warps. Against one warp per cell (lanes over candidates, a loop over
-// the cell's beads) this has no per-cell prefix of run lengths, no chunk
-// remainders and one test per candidate.
-template <typename R>
-__device__ __forceinline__ void dpd_beads(const DpdDev& d, int H, int B3, const int* chalo, const int* cpre,
-                                          const int* hoff, const typename V4<R>::T* __restrict__ P,
-                                          const typename V4<R>::T* __restrict__ Pv, const float4* Pf,
-                                          const DpdBand band, int2* queue, const R* __restrict__ atab,
-                                          uint64_t step, R* __restrict__ F, R& ec) {
-    using V = typename V4<R>::T;
-    constexpr int NW = kDpdThreads / 32;
-    constexpr bool PRE = sizeof(R) == 8;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const R L = dpd_k(d, (R)0).L, hL = dpd_k(d, (R)0).hL;
-    const R gam = dpd_k(d, (R)0).gam, srdt = dpd_k(d, (R)0).srdt;
-    const PhiloxStep ps = philox_step(d, step);
-    const int nc = cpre[B3];
-    int cnt = 0, qh = 0;   // queued pairs of this warp, ring head
-    for (int base = warp * 32; base < nc; base += NW * 32) {
-        const int f = base + lane;
-        const bool own = f < nc;
-        int i = 0, h = 0;
-        if (own) {
-            int lo = 0, hi = B3;   // the central cell holding bead f
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (cpre[mid] <= f) lo = mid; else hi = mid;
-            }
-            h = chalo[lo];
-            i = hoff[h] + f - cpre[lo];
-        }
-        V pi;
-        float4 pif;
-        if (own) {
-            pi = P[i];
-            if constexpr (PRE) pif = Pf[i];
-        }
-        // the five runs one after the other (uniform over the warp); within a
-        // run, lane-local candidate t of the run, as long as the warp's longest
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            int j0 = 0, len = 0;
-            if (own) {
-                const int o = k == 0 ? 0 : (k == 1 ? H - 1 : H * H + (k - 3) * H - 1);
-                j0 = k == 0 ? i + 1 : hoff[h + o];
-                len = hoff[h + o + (k == 0 ? 2 : 3)] - j0;
-            }
-            const int mlen = __reduce_max_sync(0xffffffffu, len);
-            // kDpdU candidates per lane and iteration: their loads and tests
-            // are independent, then one ballot and append each
-            for (int t = 0; t < mlen; t += kDpdU) {
-                bool hit[kDpdU];
-#pragma unroll
-                for (int u = 0; u < kDpdU; ++u) {
-                    hit[u] = false;
-                    if (t + u < len) {
-                        const int j = j0 + t + u;
-                        if constexpr (PRE) {
-                            const float4 b = Pf[j];
-                            const float r2 = dist2(pif.x - b.x, pif.y - b.y, pif.z - b.z);
-                            if (r2 <= band.hi)
-                                hit[u] = (r2 < band.lo && r2 > band.lo0) || dpd_within<R, V, false>(pi, P[j], L, hL);
-                        } else {
-                            hit[u] = dpd_within<R, V, false>(pi, P[j], L, hL);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < kDpdU; ++u) {
-                    const unsigned m = __ballot_sync(0xffffffffu, hit[u]);
-                    if (hit[u]) queue[(qh + cnt + __popc(m & ((1u << lane) - 1u))) & (kDpdQ - 1)] = make_int2(i, j0 + t + u);
-                    cnt += __popc(m);
-                }
-                while (cnt >= 32) {
-                    __syncwarp();
-                    dpd_pairs_red<R, V>(true, queue[(qh + lane) & (kDpdQ - 1)], P, Pv, F, atab, d.ntypes, gam, srdt,
-                                        ps, d, ec);
-                    qh += 32;
-                    cnt -= 32;
-                }
-            }
-        }
+// FP32: the noted pairs of this lane's bead (pi, vi), all lanes in step.
+__device__ __forceinline__ void dpd_drain(const DpdDev& d, const PhiloxStep& ps, const float4& pi, const float4& vi,
+                                          const int* list, int cnt, const float4* __restrict__ sp,
+                                          const float4* __restrict__ sv, const float* __restrict__ atab,
+                                          float4* __restrict__ df, float& fx, float& fy, float& fz, float& ec) {
+    const float L = d.kf.L, hL = d.kf.hL;
+    const float* arow = atab + __float_as_int(vi.w) * d.ntypes;
+    const int m = __reduce_max_sync(0xffffffffu, cnt);
+    for (int k = 0; k < m; ++k) {
+        if (k >= cnt) continue;
+        const int j = list[32 * k];
+        const float4 pj = sp[j], vj = sv[j];
+        const float rx = min_image(pi.x, pj.x, L, hL);
+        const float ry = min_image(pi.y, pj.y, L, hL);
+        const float rz = min_image(pi.z, pj.z, L, hL);
+        const float vd = (vi.x - vj.x) * rx + (vi.y - vj.y) * ry + (vi.z - vj.z) * rz;   // r_ij . v_ij
+        const float fm = dpd_force<float>(d, ps, dist2(rx, ry, rz), vd, arow[__float_as_int(vj.w)],
+                                          __float_as_int(pi.w), __float_as_int(pj.w), ec);
+        const float gx = fm * rx, gy = fm * ry, gz = fm * rz;
+        fx += gx;
+        fy += gy;
+        fz += gz;
+        red_add4(df + j, -gx, -gy, -gz, 0.f);
     }
-    __syncwarp();
-    if (cnt > 0)
-        dpd_pairs_red<R, V>(lane < cnt, queue[(qh + lane) & (kDpdQ - 1)], P, Pv, F, atab, d.ntypes, gam, srdt, ps, d,
-                            ec);
 }
 
+// FP64: one ring entry (bead i, candidate j, image as in real_entry) per lane.
+__device__ __forceinline__ void dpd_ring(const DpdDev& d, const PhiloxStep& ps, const int2 e,
+                                         const double4_32a* __restrict__ sp, const double4_32a* __restrict__ sv,
+                                         const double* __restrict__ atab, double* __restrict__ F, double& ec) {
+    const int i = e.x & 0x1fffffff, j = e.y & 0x1fffffff;
+    const double4_32a pi = sp[i], pj = sp[j];
+    double rx = pi.x - pj.x, ry = pi.y - pj.y, rz = pi.z - pj.z;
+    const int im = (int)((unsigned)e.x >> 29 | ((unsigned)e.y >> 29) << 3);
+    if (im != 13) {   // across a box face
+        const double L = d.kd.L;
+        const int iz = im / 9, iy = (im - 9 * iz) / 3, ix = im % 3;
+        if (ix != 1) rx += ix ? L : -L;
+        if (iy != 1) ry += iy ? L : -L;
+        if (iz != 1) rz += iz ? L : -L;
+    }
+    const double r2 = dist2(rx, ry, rz);
+    if (!(r2 < 1.0 && r2 > 0.0)) return;
+    const double4_32a vi = sv[i], vj = sv[j];
+    const int oi = real_as_int(pi.w), oj = real_as_int(pj.w);
+    const double vd = (vi.x - vj.x) * rx + (vi.y - vj.y) * ry + (vi.z - vj.z) * rz;
+    const double fm = dpd_force<double>(d, ps, r2, vd, atab[real_as_int(vi.w) * d.ntypes + real_as_int(vj.w)], oi, oj,
+                                        ec);
+    const double gx = fm * rx, gy = fm * ry, gz = fm * rz;
+    atomicAdd(&F[3 * oi], gx);
+    atomicAdd(&F[3 * oi + 1], gy);
+    atomicAdd(&F[3 * oi + 2], gz);
+    atomicAdd(&F[3 * oj], -gx);
+    atomicAdd(&F[3 * oj + 1], -gy);
+    atomicAdd(&F[3 * oj + 2], -gz);
+}
+
+// spf: float positions of the sorted beads (FP32: sp itself).
 template <typename R>
-__device__ __forceinline__ void k_dpd_body(DpdDev d, int B, const typename V4<R>::T* __restrict__ sp, const typename V4<R>::T* __restrict__ sv,
-          const int* __restrict__ cstart, const R* __restrict__ atab, const R* __restrict__ pos,
-          const int* __restrict__ bnd, const uint64_t* __restrict__ stepp, R* __restrict__ F,
-          double* __restrict__ dpart, Blk bk) {
+__device__ __forceinline__ void k_dpd_body(const DpdDev& d, const typename V4<R>::T* __restrict__ sp,
+                                           const typename V4<R>::T* __restrict__ sv,
+                                           const float4* __restrict__ spf, const int* __restrict__ cstart,
+                                           const R* __restrict__ atab, const R* __restrict__ pos,
+                                           const int* __restrict__ bnd, const uint64_t* __restrict__ stepp,
+                                           float4* __restrict__ df, R* __restrict__ F, double* __restrict__ dpart,
+                                           Blk bk) {
     pdl_enter();
     using V = typename V4<R>::T;
     constexpr bool F64 = sizeof(R) == 8;
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int NW = kDpdThreads / 32;
     extern __shared__ __align__(16) unsigned char smraw[];
-    V* spos = reinterpret_cast<V*>(smraw);                                  // [kDpdCap]
-    V* svel = spos + kDpdCap;                                               // [kDpdCap]
-    float4* spf = reinterpret_cast<float4*>(svel + kDpdCap);                // [kDpdCap] (FP64 only)
-    int2* queues = reinterpret_cast<int2*>(spf + (F64 ? kDpdCap : 0));      // [NW][kDpdQ]
-    constexpr int HMAX = (kDpdMaxB + 2) * (kDpdMaxB + 2) * (kDpdMaxB + 2);
-    __shared__ int hoff[HMAX + 1], gst[HMAX];
-    __shared__ int chalo[kDpdMaxB * kDpdMaxB * kDpdMaxB];
-    __shared__ int cpre[kDpdMaxB * kDpdMaxB * kDpdMaxB + 1];   // prefix of the central cells' counts
-    __shared__ unsigned char hsh[HMAX];   // per halo cell: 2 bits per axis, 1: -L, 2: +L
-    const uint64_t step = *stepp;
-    const int ncd = d.ncd, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int2* queue = queues + warp * kDpdQ;
-    const int H = B + 2, H3 = H * H * H, B3 = B * B * B;
-    if (!ENUF_GUARD(d.check, H3 <= HMAX && B3 <= kDpdMaxB * kDpdMaxB * kDpdMaxB, 8)) return;
-    const int nblk = (ncd + B - 1) / B;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int* list = reinterpret_cast<int*>(smraw) + warp * 32 * kRealQ + lane;   // FP32: entry k at 32 k
+    int2* ring = reinterpret_cast<int2*>(smraw) + warp * kRealRing;          // FP64
+    const PhiloxStep ps = philox_step(d, *stepp);
     const R L = dpd_k(d, (R)0).L;
     R ec = 0, eb = 0;
     // harmonic bonds (Sec. 2): one thread per bond, +f to i and -f to j
@@ -3051,126 +2818,145 @@ __device__ __forceinline__ void k_dpd_body(DpdDev d, int B, const typename V4<R>
             }
         }
     }
-    // float band of the FP64 cutoff test: the staged float positions (in
-    // [-1 - L/3, 4L/3]) carry at most (4L/3 + 1) 2^-24 each, so for r2 near 1
-    // |r2f - r2| <= 7e-7 (L + 1) + 3e-7
-    DpdBand band;
-    band.L = d.kf.L;
-    band.hL = d.kf.hL;
-    const float eps = 1e-4f + 4e-6f * d.kf.L;
-    band.lo0 = eps;
-    band.lo = 1.0f - eps;
-    band.hi = 1.0f + eps;
-    for (int blk = bk.id; blk < nblk * nblk * nblk; blk += bk.n) {
-        const int bx = blk % nblk, by = (blk / nblk) % nblk, bz = blk / (nblk * nblk);
-        const int c0x = bx * B, c0y = by * B, c0z = bz * B;
-        if (tid < H3) {   // halo cell ranges (H^3 <= 216 cells)
-            const int hx = tid % H, hy = (tid / H) % H, hz = tid / (H * H);
-            const int ux = c0x - 1 + hx, uy = c0y - 1 + hy, uz = c0z - 1 + hz;   // unwrapped
-            const int cx = (ux + ncd) % ncd, cy = (uy + ncd) % ncd, cz = (uz + ncd) % ncd;
-            const int c = (cz * ncd + cy) * ncd + cx;
-            const int st = cstart[c];
-            gst[tid] = st;
-            hoff[tid] = cstart[c + 1] - st;
-            auto code = [&](int u) { return u < 0 ? 1 : (u >= ncd ? 2 : 0); };
-            hsh[tid] = (unsigned char)(code(ux) | code(uy) << 2 | code(uz) << 4);
+    // FP64: float positions carry at most L 2^-24 each, so for r2 near 1
+    // |r2f - r2| <= 7e-7 (L + 1)
+    const float Lf = d.kf.L, hi = F64 ? 1.0f + 1e-4f + 4e-6f * Lf : 1.0f;
+    const int ncd = d.ncd;
+    int S = 32;
+    while (S > 1 && (long long)d.N * S > d.lanes) S >>= 1;
+    const int gpw = 32 / S, sub = lane & (S - 1), grp = lane / S;
+    int cnt = 0, head = 0;   // noted pairs of this lane (FP32); ring fill and head (FP64)
+    for (int s0 = (bk.id * NW + warp) * gpw; s0 < d.N; s0 += bk.n * NW * gpw) {
+        const int s = s0 + grp;
+        const bool own = s < d.N;
+        float4 pf;
+        V vi;
+        int cx = 0, cy = 0, cz = 0;
+        if (own) {
+            pf = spf[s];
+            if constexpr (!F64) vi = sv[s];
+            const V pw = sp[s];   // the cell as k_cell_count decided it, in the working precision
+            const R ri = dpd_cinv(d, (R)0);
+            cx = min((int)(pw.x * ri), ncd - 1);
+            cy = min((int)(pw.y * ri), ncd - 1);
+            cz = min((int)(pw.z * ri), ncd - 1);
         }
-        if (tid < B3) {   // central cells of this block (clipped at the box edge)
-            const int ix = tid % B, iy = (tid / B) % B, iz = tid / (B * B);
-            const bool ok = c0x + ix < ncd && c0y + iy < ncd && c0z + iz < ncd;
-            chalo[tid] = ok ? ((iz + 1) * H + (iy + 1)) * H + (ix + 1) : -1;
-        }
-        __syncthreads();
-        if (warp == 0) {   // exclusive prefix of the halo counts (<= 7 per lane)
-            const int per = (H3 + 31) / 32;
-            int v[7], sum = 0;
-#pragma unroll
-            for (int k = 0; k < 7; ++k) {
-                const int h = lane * per + k;
-                v[k] = (k < per && h < H3) ? hoff[h] : 0;
-                sum += v[k];
-            }
-            int x = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
-            }
-            int run = x - sum;
-#pragma unroll
-            for (int k = 0; k < 7; ++k) {
-                const int h = lane * per + k;
-                if (k < per && h < H3) hoff[h] = run;
-                run += v[k];
-            }
-            if (lane == 31) hoff[H3] = x;
-        }
-        __syncthreads();
-        const int total = hoff[H3];
-        const bool staged = total <= kDpdCap;
-        if (staged && warp == 0) {   // central cells' bead counts, exclusive prefix (B3 <= 64)
-            const int c0 = 2 * lane, c1 = 2 * lane + 1;
-            const int h0 = c0 < B3 ? chalo[c0] : -1, h1 = c1 < B3 ? chalo[c1] : -1;
-            const int n0 = h0 >= 0 ? hoff[h0 + 1] - hoff[h0] : 0;
-            const int n1 = h1 >= 0 ? hoff[h1 + 1] - hoff[h1] : 0;
-            int x = n0 + n1;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
-            }
-            const int ex = x - n0 - n1;
-            if (c0 < B3) cpre[c0] = ex;
-            if (c1 < B3) cpre[c1] = ex + n0;
-            if (lane == 31) cpre[B3] = x;
-        }
-        if (staged) {
-            // a warp per halo row (H cells along x, contiguous in the staged
-            // order); a lane finds its bead's cell among the row's H
-            for (int r = warp; r < H * H; r += kDpdThreads / 32)
-            for (int f = hoff[r * H] + lane; f < hoff[r * H + H]; f += 32) {
-                int lo = r * H;
-#pragma unroll
-                for (int q = 1; q < kDpdMaxB + 2; ++q) lo += (q < H && f >= hoff[r * H + q]) ? 1 : 0;
-                const int j = gst[lo] + f - hoff[lo];
-                V p = sp[j];
-                // the halo is H <= ncd distinct cells: shift the cells across
-                // the box faces into one frame (cell edge >= 1, so beads of
-                // adjacent halo cells are within r = 1 only as this image)
-                const int sc = hsh[lo];
-                if (sc) {
-                    auto sh = [&](int c) { return c == 1 ? -L : (c == 2 ? L : (R)0); };
-                    p.x += sh(sc & 3);
-                    p.y += sh((sc >> 2) & 3);
-                    p.z += sh(sc >> 4);
+        float fx = 0.f, fy = 0.f, fz = 0.f;
+        // the half shell's rows (uniform over the warp), each as its run inside the box
+        // and its run across the box face; one more turn empties the lists
+        int row = 0;
+        bool across = false;
+        int w0 = 0, wl = 0;
+        float hx = 0.0f, hy = 0.0f, hz = 0.0f;
+        while (true) {
+            const bool last = row == 5;
+            int j0 = 0, len = 0;
+            if (across) {
+                j0 = w0;
+                len = wl;
+            } else if (!last) {
+                const int dz = row >= 2 ? 1 : 0, dy = row >= 2 ? row - 3 : row;
+                int zz = cz + dz, yy = cy + dy;
+                hx = hy = hz = 0.0f;
+                if (zz >= ncd) { zz -= ncd; hz = -Lf; }
+                if (yy < 0) { yy += ncd; hy = Lf; } else if (yy >= ncd) { yy -= ncd; hy = -Lf; }
+                const int* cs = cstart + (zz * ncd + yy) * ncd;
+                const int xa = row == 0 ? cx : cx - 1, xb = cx + 1;
+                wl = 0;
+                if (own) {
+                    j0 = row == 0 ? s + 1 : cs[max(xa, 0)];
+                    len = cs[min(xb, ncd - 1) + 1] - j0;
+                    if (xa < 0 || xb >= ncd) {
+                        w0 = cs[xa < 0 ? ncd - 1 : 0];
+                        wl = cs[xa < 0 ? ncd : 1] - w0;
+                    }
                 }
-                spos[f] = p;
-                svel[f] = sv[j];
-                if (F64) spf[f] = make_float4((float)p.x, (float)p.y, (float)p.z, 0.f);
             }
+            const int mlen = __reduce_max_sync(FULL, len);
+            const int image = (hz < 0.0f ? 0 : 9) + (hy > 0.0f ? 6 : (hy < 0.0f ? 0 : 3)) +
+                              (hx > 0.0f ? 2 : (hx < 0.0f ? 0 : 1));
+            for (int t0 = 0;;) {
+                if constexpr (F64) {
+                    while (cnt >= 32) {
+                        __syncwarp();
+                        dpd_ring(d, ps, ring[(head + lane) & (kRealRing - 1)], sp, sv, atab, F, ec);
+                        __syncwarp();
+                        head += 32;
+                        cnt -= 32;
+                    }
+                } else {
+                    if (last || __any_sync(FULL, cnt > kRealQ - kRealU)) {
+                        dpd_drain(d, ps, pf, vi, list, cnt, sp, sv, atab, df, fx, fy, fz, ec);
+                        cnt = 0;
+                    }
+                }
+                if (t0 >= mlen) break;
+                float4 b[kRealU];
+#pragma unroll
+                for (int u = 0; u < kRealU; ++u) {
+                    const int t = t0 + u * S + sub;
+                    if (t < len) b[u] = spf[j0 + t];
+                }
+#pragma unroll
+                for (int u = 0; u < kRealU; ++u) {
+                    const int t = t0 + u * S + sub;
+                    bool hit = false;
+                    if (t < len) {
+                        const float r2 = dist2(__fadd_rn(__fsub_rn(pf.x, b[u].x), hx),
+                                               __fadd_rn(__fsub_rn(pf.y, b[u].y), hy),
+                                               __fadd_rn(__fsub_rn(pf.z, b[u].z), hz));
+                        hit = F64 ? r2 <= hi : (r2 < hi && r2 > 0.0f);   // FP64 decides in the ring
+                    }
+                    if constexpr (F64) {
+                        const unsigned m = __ballot_sync(FULL, hit);
+                        const int at = cnt + __popc(m & ((1u << lane) - 1u));
+                        if (hit && ENUF_GUARD(d.check, at < kRealRing, 8))
+                            ring[(head + at) & (kRealRing - 1)] = real_entry(s, j0 + t, image);
+                        cnt += __popc(m);
+                    } else if (hit && ENUF_GUARD(d.check, cnt < kRealQ, 8)) {
+                        list[32 * cnt] = j0 + t;
+                        ++cnt;
+                    }
+                }
+                t0 += kRealU * S;
+            }
+            if (last) break;
+            if (!across && __any_sync(FULL, wl > 0)) {
+                across = true;
+                hx = row > 0 && cx == 0 ? Lf : -Lf;   // read by the lanes with wl > 0
+                continue;
+            }
+            across = false;
+            ++row;
         }
-        __syncthreads();
-        if (staged)
-            dpd_beads<R>(d, H, B3, chalo, cpre, hoff, spos, svel, spf, band, queue, atab, step, F, ec);
-        else
-            dpd_cells<R>(d, H, B3, chalo, hoff, gst, sp, sv, queue, atab, step, F, ec);
-        __syncthreads();
+        if constexpr (!F64) {
+            for (int o = 1; o < S; o <<= 1) {
+                fx += __shfl_xor_sync(FULL, fx, o);
+                fy += __shfl_xor_sync(FULL, fy, o);
+                fz += __shfl_xor_sync(FULL, fz, o);
+            }
+            if (own && sub == 0) red_add4(df + s, fx, fy, fz, 0.f);
+        }
+    }
+    if constexpr (F64) {   // what is left in the ring (cnt < 32)
+        __syncwarp();
+        if (lane < cnt) dpd_ring(d, ps, ring[(head + lane) & (kRealRing - 1)], sp, sv, atab, F, ec);
     }
     double e1, e2;
     block_sum2_r<R>(ec, eb, e1, e2);
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         dpart[2 * bk.id] = 0.5 * e1;
         dpart[2 * bk.id + 1] = 0.5 * e2;
     }
 }
 
 template <typename R>
-__global__ void __launch_bounds__(kDpdThreads, sizeof(R) == 4 ? 4 : 2)
-    k_dpd(DpdDev d, int B, const typename V4<R>::T* __restrict__ sp, const typename V4<R>::T* __restrict__ sv,
-          const int* __restrict__ cstart, const R* __restrict__ atab, const R* __restrict__ pos,
-          const int* __restrict__ bnd, const uint64_t* __restrict__ stepp, R* __restrict__ F,
-          double* __restrict__ dpart) {
-    k_dpd_body<R>(d, B, sp, sv, cstart, atab, pos, bnd, stepp, F, dpart, Blk{(int)blockIdx.x, (int)gridDim.x});
+__global__ void __launch_bounds__(kDpdThreads, sizeof(R) == 4 ? 4 : 3)
+    k_dpd(DpdDev d, const typename V4<R>::T* __restrict__ sp, const typename V4<R>::T* __restrict__ sv,
+          const float4* __restrict__ spf, const int* __restrict__ cstart, const R* __restrict__ atab,
+          const R* __restrict__ pos, const int* __restrict__ bnd, const uint64_t* __restrict__ stepp,
+          float4* __restrict__ df, R* __restrict__ F, double* __restrict__ dpart) {
+    k_dpd_body<R>(d, sp, sv, spf, cstart, atab, pos, bnd, stepp, df, F, dpart, Blk{(int)blockIdx.x, (int)gridDim.x});
 }
 
 // The DPD pair forces and the real-space electrostatic pairs in one launch
@@ -3180,17 +2966,18 @@ __global__ void __launch_bounds__(kDpdThreads, sizeof(R) == 4 ? 4 : 2)
 // partials; launched once both cell structures exist.
 template <typename R>
 __global__ void __launch_bounds__(kDpdThreads, sizeof(R) == 4 ? 4 : 2)
-    k_pairs(DpdDev d, int B, const typename V4<R>::T* __restrict__ sp, const typename V4<R>::T* __restrict__ sv,
-            const int* __restrict__ cstart, const R* __restrict__ atab, const R* __restrict__ pos,
-            const int* __restrict__ bnd, const uint64_t* __restrict__ stepp, R* __restrict__ F,
-            double* __restrict__ dpart, int nd, Geo g, const int* __restrict__ tstart,
-            const typename V4<R>::T* __restrict__ sq, const typename V4<R>::T* __restrict__ sw,
-            const int* __restrict__ sb, const float4* __restrict__ spf, double* __restrict__ rpart) {
+    k_pairs(DpdDev d, const typename V4<R>::T* __restrict__ sp, const typename V4<R>::T* __restrict__ sv,
+            const float4* __restrict__ spf, const int* __restrict__ cstart, const R* __restrict__ atab,
+            const R* __restrict__ pos, const int* __restrict__ bnd, const uint64_t* __restrict__ stepp,
+            float4* __restrict__ df, R* __restrict__ F, double* __restrict__ dpart, int nd, Geo g,
+            const int* __restrict__ tstart, const typename V4<R>::T* __restrict__ sq,
+            const typename V4<R>::T* __restrict__ sw, const int* __restrict__ sb, const float4* __restrict__ sqf,
+            double* __restrict__ rpart) {
     static_assert(kDpdThreads == kRealThreads && kRealThreads <= kSumThreads, "one block size for both roles");
     if ((int)blockIdx.x < nd)
-        k_dpd_body<R>(d, B, sp, sv, cstart, atab, pos, bnd, stepp, F, dpart, Blk{(int)blockIdx.x, nd});
+        k_dpd_body<R>(d, sp, sv, spf, cstart, atab, pos, bnd, stepp, df, F, dpart, Blk{(int)blockIdx.x, nd});
     else
-        k_real_body<R>(g, tstart, sq, sw, sb, spf, F, rpart, Blk{(int)blockIdx.x - nd, (int)gridDim.x - nd});
+        k_real_body<R>(g, tstart, sq, sw, sb, sqf, F, rpart, Blk{(int)blockIdx.x - nd, (int)gridDim.x - nd});
 }
 
 // Table 2 steps 0-2 (m = 1): v0 = v + lambda F dt; v += F dt/2; r += v dt; step += 1.
@@ -3230,32 +3017,63 @@ __global__ void k_vv_pre(int N, R lam, R dt, R* __restrict__ pos, R* __restrict_
     }
 }
 
-// Table 2 step 6: v += F dt/2; kinetic energy partials.
-// The last block then reduces all energies of the step (totals).
+// FP32: adds the DPD pair forces (df, in the cell-sorted order; slot: each
+// bead's place in it) to F. The closing kick does it in a step; this kernel in
+// force evaluations outside one.
+static __global__ void __launch_bounds__(256) k_dpd_add(int N, float* __restrict__ F, const float4* __restrict__ df,
+                                                        const int* __restrict__ slot) {
+    pdl_enter();
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        const float4 a = df[slot[i]];
+        F[3 * i] += a.x;
+        F[3 * i + 1] += a.y;
+        F[3 * i + 2] += a.z;
+    }
+}
+
+// Table 2 step 6: v += F dt/2 (FP32: after adding the DPD pair forces to F);
+// kinetic energy partials. The last block then reduces all energies of the
+// step (totals).
 template <typename R>
-__global__ void __launch_bounds__(256) k_vv_post(Geo g, int N, R dt, R* __restrict__ vel, const R* __restrict__ F,
+__global__ void __launch_bounds__(256) k_vv_post(Geo g, int N, R dt, R* __restrict__ vel, R* __restrict__ F,
+                                                const float4* __restrict__ df, const int* __restrict__ slot,
                                                 double* __restrict__ kpart, TotalsArgs tot) {
     pdl_enter();
-    using V = typename V4<R>::T;
     double ke = 0.0, dummy = 0.0;
-    const int n3 = 3 * N, n4 = n3 / 4;
     auto one = [&](R f, R v) {
         const R vn = v + (R)0.5 * f * dt;
         ke = fma((double)vn, (double)vn, ke);
         return vn;
     };
+    if constexpr (sizeof(R) == 4) {
 #pragma unroll 2
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n4; k += gridDim.x * blockDim.x) {
-        const V f = reinterpret_cast<const V*>(F)[k];
-        V v = reinterpret_cast<const V*>(vel)[k];
-        v.x = one(f.x, v.x);
-        v.y = one(f.y, v.y);
-        v.z = one(f.z, v.z);
-        v.w = one(f.w, v.w);
-        reinterpret_cast<V*>(vel)[k] = v;
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+            const float4 a = df[slot[i]];
+            const float f0 = F[3 * i] + a.x, f1 = F[3 * i + 1] + a.y, f2 = F[3 * i + 2] + a.z;
+            const float v0 = vel[3 * i], v1 = vel[3 * i + 1], v2 = vel[3 * i + 2];
+            F[3 * i] = f0;
+            F[3 * i + 1] = f1;
+            F[3 * i + 2] = f2;
+            vel[3 * i] = one(f0, v0);
+            vel[3 * i + 1] = one(f1, v1);
+            vel[3 * i + 2] = one(f2, v2);
+        }
+    } else {
+        using V = typename V4<R>::T;
+        const int n3 = 3 * N, n4 = n3 / 4;
+#pragma unroll 2
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n4; k += gridDim.x * blockDim.x) {
+            const V f = reinterpret_cast<const V*>(F)[k];
+            V v = reinterpret_cast<const V*>(vel)[k];
+            v.x = one(f.x, v.x);
+            v.y = one(f.y, v.y);
+            v.z = one(f.z, v.z);
+            v.w = one(f.w, v.w);
+            reinterpret_cast<V*>(vel)[k] = v;
+        }
+        const int k = 4 * n4 + (int)threadIdx.x;
+        if (blockIdx.x == 0 && k < n3) vel[k] = one(F[k], vel[k]);
     }
-    const int k = 4 * n4 + (int)threadIdx.x;
-    if (blockIdx.x == 0 && k < n3) vel[k] = one(F[k], vel[k]);
     block_sum2(ke, dummy);
     if (threadIdx.x == 0) kpart[blockIdx.x] = 0.5 * ke;
     if (tot.Edev) totals_if_last(g, tot, (int)gridDim.x);

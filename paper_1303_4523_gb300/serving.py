@@ -241,7 +241,7 @@ class GpuBackend:
         if req.kind == "force":
             return plan_bytes + s.N * 7 * esz
         ncells = int(math.floor(s.L / (1 + 1e-5))) ** 3
-        return plan_bytes + s.N * (21 * esz + 16) + ncells * 16 + 4096
+        return plan_bytes + s.N * (21 * esz + 32) + ncells * 16 + 4096
 
     def launch(self, key: str, req: Request):
         torch, enuf = self.torch, self.enuf
