@@ -1,7 +1,7 @@
 """In-tree build of libenuf.so (sm_103a) with nvcc; no cmake, no torch extension.
 
-The three translation units (C ABI, FP32 kernels, FP64 kernels) compile in
-parallel; the shared library links the CUDA runtime statically so it loads
+The translation units (C ABI, FP32 kernels, FP64 kernels, the FP32 FFT passes
+of single lengths) compile in parallel; the shared library links the CUDA runtime statically so it loads
 next to any PyTorch build. build(check=True) makes the debug build
 libenuf_check.so (-DENUF_CHECK: device index checks that record failure
 bits, see enuf_check_word).
@@ -20,7 +20,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libenuf.so")
 BUILD_CHECK = os.path.join(HERE, "_build_check")
 LIB_CHECK = os.path.join(HERE, "libenuf_check.so")
-SOURCES = ["enuf_capi.cu", "enuf_k32.cu", "enuf_k64.cu"]
+SOURCES = ["enuf_capi.cu", "enuf_k32.cu", "enuf_k64.cu", *(f"enuf_fft32_{c}.cu" for c in "abcdefgh"), "enuf_batch32.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "nvcc")
 

@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(512, 2) kb_fft_xy(const FftXYArgs<R>* __restri
     pdl_enter();
     const int m = cmap[blockIdx.x];
     const FftXYArgs<R>& a = tab[m >> kBatchShift];
-    k2_fft_xy_body<R>(a.g, a.fp, a.grid, a.twg, a.spec2, Blk{m & kBatchLocal, a.nblk});
+    k2_fft_xy_body<R, 0, 0>(a.g, a.fp, a.grid, a.twg, a.spec2, Blk{m & kBatchLocal, a.nblk});
 }
 
 template <typename R>
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(512) kb_fft_z(const FftZArgs<R>* __restrict__ 
     pdl_enter();
     const int m = cmap[blockIdx.x];
     const FftZArgs<R>& a = tab[m >> kBatchShift];
-    k2_fft_z_body<R>(a.g, a.fp, a.spec2, a.twg, a.tab, a.tabv, a.tabr, a.spec3, a.epart, a.LB, 1,
+    k2_fft_z_body<R, 0, 0>(a.g, a.fp, a.spec2, a.twg, a.tab, a.tabv, a.tabr, a.spec3, a.epart, a.LB,
                      Blk{m & kBatchLocal, a.nblk});
 }
 
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(512, 2) kb_fft_yx(const FftYXArgs<R>* __restri
     pdl_enter();
     const int m = cmap[blockIdx.x];
     const FftYXArgs<R>& a = tab[m >> kBatchShift];
-    k2_fft_yx_body<R>(a.g, a.fp, a.spec3, a.twg, a.h, Blk{m & kBatchLocal, a.nblk});
+    k2_fft_yx_body<R, 0, 0>(a.g, a.fp, a.spec3, a.twg, a.h, Blk{m & kBatchLocal, a.nblk});
 }
 
 template <typename R>

@@ -190,6 +190,13 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
 }
 
 template <typename R>
+cudaError_t configure_batch(int max_smem) {
+    return first_error({set_smem((const void*)kb_real<R>, max_smem, false), set_smem((const void*)kb_fft_xy<R>, max_smem, false),
+                        set_smem((const void*)kb_fft_z<R>, max_smem, false),
+                        set_smem((const void*)kb_fft_yx<R>, max_smem, false)});
+}
+
+template <typename R>
 cudaError_t batch_enqueue(const BatchLaunch& L, cudaStream_t s0, cudaStream_t s1, cudaEvent_t evFork, cudaEvent_t evJoin,
                           LaunchLog* log) {
     auto run = [&](bool pdl, bool critical, auto kern, const BatchKernel& k, auto* tab, cudaStream_t s) {
@@ -221,6 +228,7 @@ cudaError_t batch_enqueue(const BatchLaunch& L, cudaStream_t s0, cudaStream_t s1
     cudaStreamWaitEvent(s0, evJoin, 0);
     const GatherArgs<R>* gtab = (const GatherArgs<R>*)L.gather.tab;
     switch (L.gather.T) {
+        case 4: run(false, true, kb_gather<R, 4>, L.gather, gtab, s0); break;
         case 6: run(false, true, kb_gather<R, 6>, L.gather, gtab, s0); break;
         case 8: run(false, true, kb_gather<R, 8>, L.gather, gtab, s0); break;
         case 10: run(false, true, kb_gather<R, 10>, L.gather, gtab, s0); break;

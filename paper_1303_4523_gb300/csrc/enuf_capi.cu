@@ -41,6 +41,7 @@ cudaError_t ensure_configured(int prec) {
     std::lock_guard<std::mutex> lock(g_config_mu);
     if (g_configured[dev][pi]) return cudaSuccess;
     e = prec == ENUF_FP32 ? configure_kernels<float>(kMaxSmem) : configure_kernels<double>(kMaxSmem);
+    if (e == cudaSuccess && prec == ENUF_FP32) e = configure_batch<float>(kMaxSmem);
     if (e == cudaSuccess) g_configured[dev][pi] = true;
     return e;
 }
@@ -412,43 +413,49 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
             grid = (total_lines + lines - 1) / lines;
             threads = std::min(512, std::max(64, ((mult * lines * fmax + 31) / 32) * 32));
         };
-        // persistent passes (x, inverse y, inverse x): the next group's input (extra
-        // bytes per line) double-buffered in shared memory; ~72 KB keeps three CTAs
-        // per SM, the grid is what stays resident
-        auto pipe_shape = [&](int total_lines, int extra, int& lines, int& threads, int& grid, int& smem) {
-            lines = std::max(1, std::min(64, (72 * 1024 - n * csz - 16) / (per_line + extra)));
-            threads = std::min(512, std::max(64, ((lines * fmax + 31) / 32) * 32));
-            smem = n * csz + lines * (per_line + extra) + 16;   // + alignment of the input buffers
-            const int groups = (total_lines + lines - 1) / lines;
+        // persistent passes (x, z, inverse x): ~72 KB keeps three CTAs per SM, the grid is
+        // what stays resident; the lines per CTA are the kernels' own (compile-time for
+        // the lengths with instances of their own)
+        auto threads_for = [&](int lines) { return std::min(512, std::max(64, (lines * fmax + 31) / 32 * 32)); };
+        auto resident = [&](int groups, int smem, int threads) {
             const int by_smem = (228 * 1024) / (smem + 1024), by_threads = 2048 / threads;
             const int by_regs = 65536 / (64 * threads);
             const int per_sm = std::max(1, std::min(std::min(by_smem, by_threads), std::min(by_regs, 32)));
-            grid = std::min(groups, per_sm * kSMs);
+            return std::min(groups, per_sm * kSMs);
         };
-        shape2(n * nc1, 1, fs.ly, fs.ty, gyz, budget);
-        fs.grid_y_z = (n + fs.ly - 1) / fs.ly;
-        // the z pass holds one inverse line per line, two with three fields (and
-        // ~83 registers a thread): a smaller budget keeps several CTAs per SM
+        // the z pass holds one inverse line per line, two with three fields
         const int zmul = g.nf == 3 ? 2 : 1;
-        shape2(nc1 * g.K, zmul, fs.lz, fs.tz, fs.grid_z, 56 * 1024);
-        fs.smem_z = n * csz + zmul * fs.lz * per_line;
-        pipe_shape(n * n / 2, 4 * n * (int)sizeof(float), fs.lx, fs.tx, fs.grid_x, fs.smem_x);
-        // inverse y: one CTA per group (its input lines are contiguous already; the
-        // persistent form measured slower, 123 against 106 us at n = 320)
-        shape2(g.nf * n * nc1, 1, fs.liy, fs.tiy, fs.grid_iy, budget);
-        fs.smem_iy = n * csz + fs.liy * per_line;
-        pipe_shape(g.nf * n * n / 2, 4 * nc1 * csz, fs.lix, fs.tix, fs.grid_ix, fs.smem_ix);
-        fs.smem_y = n * csz + fs.ly * per_line;
         fs.smem_xy = (n + (n / 2) * (lsa + lsb)) * csz;
         fs.smem_yx = (n + (n / 2) * lsa + nc1 * lsb) * csz;
         fs.fused = (fs.smem_xy <= 100 * 1024 && P.fft_path == 0) ? 1 : 0;
         fs.composite = 0;
-        // five passes: the z pass persistent as well (lines contiguous in spec2);
-        // the fused plane path keeps one CTA per line group (spec2 plane-major)
-        if (!fs.fused) {
-            pipe_shape(nc1 * g.K, (zmul - 1) * per_line + 2 * n * csz, fs.lz, fs.tz, fs.grid_z, fs.smem_z);
-            fs.tz = std::min(512, std::max(64, ((zmul * fs.lz * fmax + 31) / 32) * 32));
+        if (fs.fused) {
+            // the z pass keeps one CTA per line group (spec2 plane-major); a smaller
+            // budget keeps several CTAs per SM
+            shape2(nc1 * g.K, zmul, fs.lz, fs.tz, fs.grid_z, 56 * 1024);
+            fs.smem_z = n * csz + zmul * fs.lz * per_line;
+        } else {
+            const int f1 = fp.f1, f2 = fp.f2;
+            fs.lx = fft2_lx(f1, f2);
+            fs.tx = threads_for(fs.lx);
+            fs.smem_x = n * csz + fs.lx * (per_line + 4 * n * (int)sizeof(float)) + 16;   // + alignment of the input
+            fs.grid_x = resident((n * n / 2 + fs.lx - 1) / fs.lx, fs.smem_x, fs.tx);
+            fs.ly = fs.liy = fft2_ly(f1, f2);
+            fs.ty = fs.tiy = threads_for(fs.ly);
+            fs.smem_y = fs.smem_iy = n * csz + fs.ly * per_line;
+            fs.grid_y_z = (n + fs.ly - 1) / fs.ly;
+            fs.grid_iy = (g.nf * n * nc1 + fs.liy - 1) / fs.liy;
+            fs.lz = fft2_lz(f1, f2, zmul);
+            fs.tz = threads_for(zmul * fs.lz);
+            fs.smem_z = n * csz + fs.lz * (zmul * per_line + 2 * n * csz) + 16;
+            fs.grid_z = resident((nc1 * g.K + fs.lz - 1) / fs.lz, fs.smem_z, fs.tz);
+            fs.lix = fft2_lix(f1, f2, g.nf);   // row pairs, of every field
+            fs.tix = threads_for(g.nf * fs.lix);
+            fs.smem_ix = n * csz + g.nf * fs.lix * (per_line + 4 * nc1 * csz) + 16;
+            fs.grid_ix = resident((n * n / 2 + fs.lix - 1) / fs.lix, fs.smem_ix, fs.tix);
         }
+        // the five passes leave three fields interleaved
+        g.h4 = !fs.fused && g.nf == 3 ? 1 : 0;
     }
     // spreading form (FP32): bricks of whole x rows fused with the x pass where the
     // two-factor five-pass FFT runs and the brick fits; footprint bricks into the
@@ -600,7 +607,7 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
            o_wb = take(nm * 3 * 2 * P.p * esz), o_grid = take(n3 * esz),
            o_s1 = take((size_t)n * nc1 * n * csz), o_s2 = take((size_t)nc1 * g.K * n * csz),
            o_s3 = take((size_t)g.nf * n * nc1 * g.K * csz), o_s4 = take((size_t)g.nf * n * n * nc1 * csz),
-           o_h = take(g.nf * n3 * esz), o_tab = take(ntab * 8), o_tabv = take(ntab * 8), o_tabr = take(ntab * esz),
+           o_h = take((g.h4 ? 4 : g.nf) * n3 * esz), o_tab = take(ntab * 8), o_tabv = take(ntab * 8), o_tabr = take(ntab * esz),
            o_tw = take((size_t)n * csz), o_part = take((size_t)npart * 8), o_E = take(16 * 8),
            o_ktab = take((size_t)g.kn * (P.prec == ENUF_FP64 ? kKtStride64 : kKtStride32) * esz);
     if (bytes) *bytes = off;
@@ -899,6 +906,7 @@ enuf_status enuf_plan(const enuf_params* params, int n_max, void* cuda_stream, e
     };
     {
         cudaError_t e = ensure_configured(plan->prec);
+        if (e == cudaSuccess && plan->fs.two) e = configure_fft2(plan->fs, plan->fp, kMaxSmem);
         if (e != cudaSuccess) return bail(fail(plan, ENUF_ERR_CUDA, "configure: %s", cudaGetErrorString(e)));
     }
     if (cuda_stream) {
@@ -1065,6 +1073,14 @@ enuf_status enuf_debug_buffer(enuf_plan_t plan, int which, void* host, size_t by
     else return fail(plan, ENUF_ERR_INVALID, "unknown buffer %d", which);
     if (bytes != need) return fail(plan, ENUF_ERR_INVALID, "buffer needs %zu bytes, got %zu", need, bytes);
     CU(cudaStreamSynchronize(plan->stream));
+    if (which == ENUF_BUF_FIELD && plan->g.h4) {   // float4 (h_x, h_y, h_z, 0) per point on the device
+        std::vector<float> h4(4 * n3);
+        CU(cudaMemcpy(h4.data(), src, 4 * n3 * sizeof(float), cudaMemcpyDeviceToHost));
+        float* out = static_cast<float*>(host);
+        for (size_t e = 0; e < n3; ++e)
+            for (int f = 0; f < 3; ++f) out[f * n3 + e] = h4[4 * e + f];
+        return ENUF_OK;
+    }
     CU(cudaMemcpy(host, src, need, cudaMemcpyDeviceToHost));
     return ENUF_OK;
 }

@@ -5,6 +5,7 @@
 // Every sequence is stream-ordered and capturable into a CUDA graph.
 #pragma once
 #include <algorithm>
+#include <initializer_list>
 #include <utility>
 
 #include "enuf_batch.cuh"
@@ -84,6 +85,66 @@ inline TotalsArgs no_totals() {
     return t;
 }
 
+// The Stockham passes of one evaluation (fused plane passes or five line
+// passes); CR selects the kernels compiled with the composite radices. The FP32
+// instances are compiled in a translation unit of their own.
+inline cudaError_t set_smem(const void* f, int max_smem, bool carve) {
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+    // the two-factor passes prefer the largest shared-memory carve-out (several CTAs per SM)
+    if (e == cudaSuccess && carve) e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    return e;
+}
+inline cudaError_t first_error(std::initializer_list<cudaError_t> l) {
+    for (cudaError_t e : l)
+        if (e != cudaSuccess) return e;
+    return cudaSuccess;
+}
+template <typename R, bool CR>
+struct StockhamPasses {   // members defined out of class: an extern instance is then not compiled here
+    static cudaError_t configure(int ms);
+    static void enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0, bool pdl,
+                        LaunchLog* log, cudaEvent_t evZ);
+};
+template <typename R, bool CR>
+cudaError_t StockhamPasses<R, CR>::configure(int ms) {
+    return first_error({set_smem((const void*)k_fft_x<R, CR>, ms, false), set_smem((const void*)k_fft_y<R, CR>, ms, false),
+                        set_smem((const void*)k_fft_z<R, CR>, ms, false), set_smem((const void*)k_fft_iy<R, CR>, ms, false),
+                        set_smem((const void*)k_fft_ix<R, CR>, ms, false), set_smem((const void*)k_fft_xy<R, CR>, ms, false),
+                        set_smem((const void*)k_fft_yx<R, CR>, ms, false)});
+}
+template <typename R, bool CR>
+void StockhamPasses<R, CR>::enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0, bool pdl, LaunchLog* log, cudaEvent_t evZ) {
+    using C = typename Cx<R>::T;
+    const C* tw = static_cast<const C*>(w.tw);
+    if (fs.fused) {   // whole z-planes in shared memory: x+y, z (+convolve), y+x
+        launch(pdl, true, k_fft_xy<R, CR>, g.n, fs.t_xy, fs.smem_xy, s0, g, fp, static_cast<const R*>(w.grid),
+               tw, static_cast<C*>(w.spec2));
+        launch(pdl, true, k_fft_z<R, CR>, fs.grid_z, fs.tz, fs.smem_z, s0, g, fp, static_cast<const C*>(w.spec2),
+               tw, (const double*)w.tab, (const double*)w.tabv, static_cast<const R*>(w.tabr),
+               static_cast<C*>(w.spec3), w.part + w.off_recip, fs.lz, 1);
+        if (evZ) cudaEventRecord(evZ, s0);
+        launch(pdl && !evZ, true, k_fft_yx<R, CR>, g.nf * g.n, fs.t_yx, fs.smem_yx, s0, g, fp,
+               static_cast<const C*>(w.spec3), tw, static_cast<R*>(w.h));
+        log->kernels += 4;
+    } else {
+        launch(pdl, true, k_fft_x<R, CR>, fs.grid_x, fs.tx, fs.smem_x, s0, g, fp, static_cast<const R*>(w.grid),
+               tw, static_cast<C*>(w.spec1), fs.lx);
+        launch(pdl, true, k_fft_y<R, CR>, dim3(g.nc + 1, fs.grid_y_z), fs.ty, fs.smem_y, s0, g, fp,
+               static_cast<const C*>(w.spec1), tw, static_cast<C*>(w.spec2), fs.ly);
+        launch(pdl, true, k_fft_z<R, CR>, fs.grid_z, fs.tz, fs.smem_z, s0, g, fp, static_cast<const C*>(w.spec2),
+               tw, (const double*)w.tab, (const double*)w.tabv, static_cast<const R*>(w.tabr),
+               static_cast<C*>(w.spec3), w.part + w.off_recip, fs.lz, 0);
+        if (evZ) cudaEventRecord(evZ, s0);
+        launch(pdl && !evZ, true, k_fft_iy<R, CR>, fs.grid_iy, fs.tiy, fs.smem_iy, s0, g, fp,
+               static_cast<const C*>(w.spec3), tw, static_cast<C*>(w.spec4), fs.liy);
+        launch(pdl, true, k_fft_ix<R, CR>, fs.grid_ix, fs.tix, fs.smem_ix, s0, g, fp, static_cast<const C*>(w.spec4),
+               tw, static_cast<R*>(w.h), fs.lix);
+        log->kernels += 6;
+    }
+}
+extern template struct StockhamPasses<float, false>;
+extern template struct StockhamPasses<float, true>;
+
 template <typename R>
 cudaError_t configure_kernels(int max_smem) {
     cudaError_t e = cudaSuccess;
@@ -92,20 +153,6 @@ cudaError_t configure_kernels(int max_smem) {
         if (r != cudaSuccess) e = r;
     };
     set((const void*)k_spread<R>);
-    set((const void*)k_fft_x<R>);
-    set((const void*)k_fft_y<R>);
-    set((const void*)k_fft_z<R>);
-    set((const void*)k_fft_iy<R>);
-    set((const void*)k_fft_ix<R>);
-    if constexpr (sizeof(R) == 4) {
-        set((const void*)k_fft_x<R, true>);
-        set((const void*)k_fft_y<R, true>);
-        set((const void*)k_fft_z<R, true>);
-        set((const void*)k_fft_iy<R, true>);
-        set((const void*)k_fft_ix<R, true>);
-        set((const void*)k_fft_xy<R, true>);
-        set((const void*)k_fft_yx<R, true>);
-    }
     set((const void*)k_spread_col<R, 8, false>);
     set((const void*)k_spread_col<R, 8, true>);
     set((const void*)k_spread_col<R, 10, false>);
@@ -118,55 +165,20 @@ cudaError_t configure_kernels(int max_smem) {
     set((const void*)k_spread_col<R, 20, true>);
     set((const void*)k_spread_col<R, 24, false>);
     set((const void*)k_spread_col<R, 24, true>);
-    set((const void*)k_fft_xy<R>);
-    set((const void*)k_fft_yx<R>);
-    // the FFT passes prefer the largest shared-memory carve-out (several CTAs per SM)
-    auto carve = [&](const void* f) {
-        cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        if (r != cudaSuccess) e = r;
-    };
     if constexpr (sizeof(R) == 4) {
-        carve((const void*)k2_fft_x<R>);
-        carve((const void*)k2_fft_x<R, true>);
-        carve((const void*)k2_fft_y<R>);
-        carve((const void*)k2_fft_y<R, true>);
-        carve((const void*)k2_fft_z<R>);
-        carve((const void*)k2_fft_z<R, true>);
-        carve((const void*)k2_fft_zp<R>);
-        carve((const void*)k2_fft_zp<R, true>);
-        carve((const void*)k2_fft_iy<R>);
-        carve((const void*)k2_fft_iy<R, true>);
-        carve((const void*)k2_fft_ix<R>);
-        carve((const void*)k2_fft_ix<R, true>);
-        set((const void*)k2_fft_x<R>);
-        set((const void*)k2_fft_x<R, true>);
-        set((const void*)k2_fft_y<R>);
-        set((const void*)k2_fft_y<R, true>);
-        set((const void*)k2_fft_z<R>);
-        set((const void*)k2_fft_z<R, true>);
-        set((const void*)k2_fft_zp<R>);
-        set((const void*)k2_fft_zp<R, true>);
-        set((const void*)k2_fft_iy<R>);
-        set((const void*)k2_fft_iy<R, true>);
-        set((const void*)k2_fft_ix<R>);
-        set((const void*)k2_fft_ix<R, true>);
-        set((const void*)k2_fft_xy<R>);
-        set((const void*)k2_fft_xy<R, true>);
-        set((const void*)k2_fft_yx<R>);
-        set((const void*)k2_fft_yx<R, true>);
         set((const void*)k_spread_brick<R, false>);
         set((const void*)k_spread_brick<R, true>);
         set((const void*)k_spread_sc<16, 8>);
         set((const void*)k_spread_sc<20, 8>);
         set((const void*)k_spread_sc<24, 8>);
-        set((const void*)kb_real<R>);
-        set((const void*)kb_fft_xy<R>);
-        set((const void*)kb_fft_z<R>);
-        set((const void*)kb_fft_yx<R>);
     }
     set((const void*)k_real<R>);
     set((const void*)k_dpd<R>);
     set((const void*)k_pairs<R>);
+    if (e == cudaSuccess) e = StockhamPasses<R, false>::configure(max_smem);
+    if constexpr (sizeof(R) == 4) {
+        if (e == cudaSuccess) e = StockhamPasses<R, true>::configure(max_smem);
+    }
     return e;
 }
 
@@ -246,8 +258,6 @@ inline void enqueue_spread(const Geo& g, const Work& w, R* grid, cudaStream_t s,
            static_cast<const V*>(w.sq), static_cast<const V*>(w.sw), (const int*)w.sb, grid);
 }
 
-// The FFT passes of one evaluation (fused plane passes or five line passes);
-// CR selects the kernels compiled with the composite radices.
 // Footprint spreading on bricks (FP32): into the grid (spread = 2), or fused
 // with the forward x pass into spec1 (spread = 3).
 template <typename R>
@@ -287,82 +297,117 @@ inline void enqueue_spread_sc(const Geo& g, const FftShape& fs, const Work& w, c
            static_cast<float*>(w.grid));
 }
 
-// The same passes on the two-factor kernels (FP32 grids with n = f1 f2); with
-// the spreading fused with the x pass (spread = 3) the x pass is already done.
-// evZ (or nullptr) is recorded right after the z pass, whose blocks write the
+// The same passes on the two-factor kernels (FP32 grids with n = f1 f2): the
+// plane passes and the five passes of one length, or of any (<0, 0>). With the
+// spreading fused with the x pass (spread = 3) the x pass is already done. evZ
+// (or nullptr) is recorded right after the z pass, whose blocks write the
 // reciprocal energy and virial partials (the kernel after it then launches
 // without programmatic dependent launch: its stream predecessor is the record).
-template <typename R, bool EXT>
-void enqueue_fft2(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0, bool pdl,
-                  LaunchLog* log, cudaEvent_t evZ) {
-    using C = typename Cx<R>::T;
-    const C* tw = static_cast<const C*>(w.tw);
-    if (fs.fused) {
-        launch(pdl, true, k2_fft_xy<R, EXT>, g.n, fs.t_xy, fs.smem_xy, s0, g, fp, static_cast<const R*>(w.grid), tw,
-               static_cast<C*>(w.spec2));
-        launch(pdl, true, k2_fft_z<R, EXT>, fs.grid_z, fs.tz, fs.smem_z, s0, g, fp, static_cast<const C*>(w.spec2), tw,
-               (const double*)w.tab, (const double*)w.tabv, static_cast<const R*>(w.tabr), static_cast<C*>(w.spec3),
-               w.part + w.off_recip, fs.lz, 1);
-        if (evZ) cudaEventRecord(evZ, s0);
-        launch(pdl && !evZ, true, k2_fft_yx<R, EXT>, g.nf * g.n, fs.t_yx, fs.smem_yx, s0, g, fp,
-               static_cast<const C*>(w.spec3), tw, static_cast<R*>(w.h));
-        log->kernels += 4;
-    } else {
-        if (fs.spread != 3) {
-            launch(pdl, true, k2_fft_x<R, EXT>, fs.grid_x, fs.tx, fs.smem_x, s0, g, fp, static_cast<const R*>(w.grid), tw,
-                   static_cast<C*>(w.spec1), fs.lx);
-            log->kernels += 1;
-        }
-        launch(pdl, true, k2_fft_y<R, EXT>, dim3(g.nc + 1, fs.grid_y_z), fs.ty, fs.smem_y, s0, g, fp,
-               static_cast<const C*>(w.spec1), tw, static_cast<C*>(w.spec2), fs.ly);
-        launch(pdl, true, k2_fft_zp<R, EXT>, fs.grid_z, fs.tz, fs.smem_z, s0, g, fp, static_cast<const C*>(w.spec2), tw,
-               (const double*)w.tab, (const double*)w.tabv, static_cast<const R*>(w.tabr), static_cast<C*>(w.spec3),
-               w.part + w.off_recip, fs.lz);
-        if (evZ) cudaEventRecord(evZ, s0);
-        launch(pdl && !evZ, true, k2_fft_iy<R, EXT>, fs.grid_iy, fs.tiy, fs.smem_iy, s0, g, fp,
-               static_cast<const C*>(w.spec3), tw, static_cast<C*>(w.spec4), fs.liy);
-        launch(pdl, true, k2_fft_ix<R, EXT>, fs.grid_ix, fs.tix, fs.smem_ix, s0, g, fp, static_cast<const C*>(w.spec4),
-               tw, static_cast<R*>(w.h), fs.lix);
-        log->kernels += 5;   // the spreading kernel and four passes
+// The instances are compiled in translation units of their own (enuf_fft32_*.cu).
+template <int F1, int F2>
+struct Fft2Planes {   // members defined out of class: an extern instance is then not compiled here
+    static cudaError_t configure(int ms);
+    static void enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0,
+                        bool pdl, LaunchLog* log, cudaEvent_t evZ);
+};
+template <int F1, int F2>
+cudaError_t Fft2Planes<F1, F2>::configure(int ms) {
+    return first_error({set_smem((const void*)k2_fft_xy<float, F1, F2>, ms, true),
+                        set_smem((const void*)k2_fft_z<float, F1, F2>, ms, true),
+                        set_smem((const void*)k2_fft_yx<float, F1, F2>, ms, true)});
+}
+template <int F1, int F2>
+void Fft2Planes<F1, F2>::enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0, bool pdl, LaunchLog* log, cudaEvent_t evZ) {
+    const float2* tw = static_cast<const float2*>(w.tw);
+    launch(pdl, true, k2_fft_xy<float, F1, F2>, g.n, fs.t_xy, fs.smem_xy, s0, g, fp,
+           static_cast<const float*>(w.grid), tw, static_cast<float2*>(w.spec2));
+    launch(pdl, true, k2_fft_z<float, F1, F2>, fs.grid_z, fs.tz, fs.smem_z, s0, g, fp,
+           static_cast<const float2*>(w.spec2), tw, (const double*)w.tab, (const double*)w.tabv,
+           static_cast<const float*>(w.tabr), static_cast<float2*>(w.spec3), w.part + w.off_recip, fs.lz);
+    if (evZ) cudaEventRecord(evZ, s0);
+    launch(pdl && !evZ, true, k2_fft_yx<float, F1, F2>, g.nf * g.n, fs.t_yx, fs.smem_yx, s0, g, fp,
+           static_cast<const float2*>(w.spec3), tw, static_cast<float*>(w.h));
+    log->kernels += 4;   // with the spreading kernel
+}
+template <int F1, int F2>
+struct Fft2Lines {   // members defined out of class: an extern instance is then not compiled here
+    static cudaError_t configure(int ms);
+    static void enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0,
+                        bool pdl, LaunchLog* log, cudaEvent_t evZ);
+};
+template <int F1, int F2>
+cudaError_t Fft2Lines<F1, F2>::configure(int ms) {
+    return first_error({set_smem((const void*)k2_fft_x<float, F1, F2>, ms, true),
+                        set_smem((const void*)k2_fft_y<float, F1, F2>, ms, true),
+                        set_smem((const void*)k2_fft_zp<float, F1, F2, 3>, ms, true),
+                        set_smem((const void*)k2_fft_zp<float, F1, F2, 1>, ms, true),
+                        set_smem((const void*)k2_fft_iy<float, F1, F2>, ms, true),
+                        set_smem((const void*)k2_fft_ix<float, F1, F2, 3>, ms, true),
+                        set_smem((const void*)k2_fft_ix<float, F1, F2, 1>, ms, true)});
+}
+template <int F1, int F2>
+void Fft2Lines<F1, F2>::enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0, bool pdl, LaunchLog* log, cudaEvent_t evZ) {
+    const float2* tw = static_cast<const float2*>(w.tw);
+    if (fs.spread != 3 || fs.red) {
+        launch(pdl, true, k2_fft_x<float, F1, F2>, fs.grid_x, fs.tx, fs.smem_x, s0, g, fp,
+               static_cast<const float*>(w.grid), tw, static_cast<float2*>(w.spec1), fs.lx);
+        log->kernels += 1;
     }
+    launch(pdl, true, k2_fft_y<float, F1, F2>, dim3(g.nc + 1, fs.grid_y_z), fs.ty, fs.smem_y, s0, g, fp,
+           static_cast<const float2*>(w.spec1), tw, static_cast<float2*>(w.spec2), fs.ly);
+    launch(pdl, true, g.nf == 3 ? k2_fft_zp<float, F1, F2, 3> : k2_fft_zp<float, F1, F2, 1>, fs.grid_z, fs.tz,
+           fs.smem_z, s0, g, fp, static_cast<const float2*>(w.spec2), tw, (const double*)w.tab,
+           (const double*)w.tabv, static_cast<const float*>(w.tabr), static_cast<float2*>(w.spec3),
+           w.part + w.off_recip, fs.lz);
+    if (evZ) cudaEventRecord(evZ, s0);
+    launch(pdl && !evZ, true, k2_fft_iy<float, F1, F2>, fs.grid_iy, fs.tiy, fs.smem_iy, s0, g, fp,
+           static_cast<const float2*>(w.spec3), tw, static_cast<float2*>(w.spec4), fs.liy);
+    launch(pdl, true, g.nf == 3 ? k2_fft_ix<float, F1, F2, 3> : k2_fft_ix<float, F1, F2, 1>, fs.grid_ix, fs.tix,
+           fs.smem_ix, s0, g, fp, static_cast<const float2*>(w.spec4), tw, static_cast<float*>(w.h), fs.lix);
+    log->kernels += 5;   // the spreading kernel and four passes
 }
 
-template <typename R, bool CR>
-void enqueue_fft(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0, bool pdl,
-                 LaunchLog* log, cudaEvent_t evZ) {
-    using C = typename Cx<R>::T;
-    const C* tw = static_cast<const C*>(w.tw);
-    if (fs.fused) {   // whole z-planes in shared memory: x+y, z (+convolve), y+x
-        launch(pdl, true, k_fft_xy<R, CR>, g.n, fs.t_xy, fs.smem_xy, s0, g, fp, static_cast<const R*>(w.grid),
-               tw, static_cast<C*>(w.spec2));
-        launch(pdl, true, k_fft_z<R, CR>, fs.grid_z, fs.tz, fs.smem_z, s0, g, fp, static_cast<const C*>(w.spec2),
-               tw, (const double*)w.tab, (const double*)w.tabv, static_cast<const R*>(w.tabr),
-               static_cast<C*>(w.spec3), w.part + w.off_recip, fs.lz, 1);
-        if (evZ) cudaEventRecord(evZ, s0);
-        launch(pdl && !evZ, true, k_fft_yx<R, CR>, g.nf * g.n, fs.t_yx, fs.smem_yx, s0, g, fp,
-               static_cast<const C*>(w.spec3), tw, static_cast<R*>(w.h));
-        log->kernels += 4;
-    } else {
-        launch(pdl, true, k_fft_x<R, CR>, fs.grid_x, fs.tx, fs.smem_x, s0, g, fp, static_cast<const R*>(w.grid),
-               tw, static_cast<C*>(w.spec1), fs.lx);
-        launch(pdl, true, k_fft_y<R, CR>, dim3(g.nc + 1, fs.grid_y_z), fs.ty, fs.smem_y, s0, g, fp,
-               static_cast<const C*>(w.spec1), tw, static_cast<C*>(w.spec2), fs.ly);
-        launch(pdl, true, k_fft_z<R, CR>, fs.grid_z, fs.tz, fs.smem_z, s0, g, fp, static_cast<const C*>(w.spec2),
-               tw, (const double*)w.tab, (const double*)w.tabv, static_cast<const R*>(w.tabr),
-               static_cast<C*>(w.spec3), w.part + w.off_recip, fs.lz, 0);
-        if (evZ) cudaEventRecord(evZ, s0);
-        launch(pdl && !evZ, true, k_fft_iy<R, CR>, fs.grid_iy, fs.tiy, fs.smem_iy, s0, g, fp,
-               static_cast<const C*>(w.spec3), tw, static_cast<C*>(w.spec4), fs.liy);
-        launch(pdl, true, k_fft_ix<R, CR>, fs.grid_ix, fs.tix, fs.smem_ix, s0, g, fp, static_cast<const C*>(w.spec4),
-               tw, static_cast<R*>(w.h), fs.lix);
-        log->kernels += 6;
+// Lengths with instances of their own: every n <= 112 of two radices (plane
+// passes), every larger one up to 400, and 108 in both forms.
+#define ENUF_FFT2_PLANES_A(X) X(4, 4) X(4, 5) X(4, 6) X(4, 8) X(6, 6) X(5, 8) X(6, 8)
+#define ENUF_FFT2_PLANES_B(X) X(6, 10) X(8, 8) X(6, 12) X(8, 10) X(8, 12) X(10, 10) X(9, 12)
+#define ENUF_FFT2_LINES_A(X) X(9, 12) X(10, 12) X(8, 16) X(12, 12) X(10, 16)
+#define ENUF_FFT2_LINES_B(X) X(12, 15) X(12, 16) X(10, 20) X(12, 18)
+#define ENUF_FFT2_LINES_C(X) X(12, 20) X(16, 16) X(16, 18) X(15, 20)
+#define ENUF_FFT2_LINES_D(X) X(16, 20) X(18, 18) X(18, 20) X(20, 20)
+extern template struct Fft2Planes<0, 0>;
+extern template struct Fft2Lines<0, 0>;
+#define ENUF_FFT2_PLANES(X) ENUF_FFT2_PLANES_A(X) ENUF_FFT2_PLANES_B(X)
+#define ENUF_FFT2_LINES(X) ENUF_FFT2_LINES_A(X) ENUF_FFT2_LINES_B(X) ENUF_FFT2_LINES_C(X) ENUF_FFT2_LINES_D(X)
+#define ENUF_EXTERN(a, b) extern template struct Fft2Planes<a, b>;
+ENUF_FFT2_PLANES(ENUF_EXTERN)
+#undef ENUF_EXTERN
+#define ENUF_EXTERN(a, b) extern template struct Fft2Lines<a, b>;
+ENUF_FFT2_LINES(ENUF_EXTERN)
+#undef ENUF_EXTERN
+
+// f.template operator()<F1, F2>() for the plan's split, <0, 0> without an instance
+template <typename Planes, typename Lines>
+inline auto fft2_dispatch(const FftShape& fs, const FftPlanDev& fp, Planes&& planes, Lines&& lines) {
+#define ENUF_CASE(a, b) \
+    if (fp.f1 == a && fp.f2 == b) return planes(Fft2Planes<a, b>{});
+    if (fs.fused) {
+        ENUF_FFT2_PLANES(ENUF_CASE)
+        return planes(Fft2Planes<0, 0>{});
     }
+#undef ENUF_CASE
+#define ENUF_CASE(a, b) \
+    if (fp.f1 == a && fp.f2 == b) return lines(Fft2Lines<a, b>{});
+    ENUF_FFT2_LINES(ENUF_CASE)
+#undef ENUF_CASE
+    return lines(Fft2Lines<0, 0>{});
 }
 
 // the gather with its tap loops unrolled for the common window widths
 template <typename R>
 auto gather_kernel(int taps) {
     switch (taps) {
+        case 4: return k_gather<R, 4>;
         case 6: return k_gather<R, 6>;
         case 8: return k_gather<R, 8>;
         case 10: return k_gather<R, 10>;
@@ -448,16 +493,15 @@ cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp,
     // step's energies but the kinetic one while the last FFT pass and the gather run
     const cudaEvent_t ez = evZ && evT ? evZ : nullptr;
     if constexpr (sizeof(R) == 4) {
-        if (fs.two_ext)
-            enqueue_fft2<R, true>(g, fs, fp, w, s0, pdl, log, ez);
-        else if (fs.two)
-            enqueue_fft2<R, false>(g, fs, fp, w, s0, pdl, log, ez);
-        else if (fs.composite)
-            enqueue_fft<R, true>(g, fs, fp, w, s0, pdl, log, ez);
+        if (fs.two) {
+            auto run = [&](auto passes) { passes.enqueue(g, fs, fp, w, s0, pdl, log, ez); };
+            fft2_dispatch(fs, fp, run, run);
+        } else if (fs.composite)
+            StockhamPasses<R, true>::enqueue(g, fs, fp, w, s0, pdl, log, ez);
         else
-            enqueue_fft<R, false>(g, fs, fp, w, s0, pdl, log, ez);
+            StockhamPasses<R, false>::enqueue(g, fs, fp, w, s0, pdl, log, ez);
     } else {
-        enqueue_fft<R, false>(g, fs, fp, w, s0, pdl, log, ez);
+        StockhamPasses<R, false>::enqueue(g, fs, fp, w, s0, pdl, log, ez);
     }
     rec(ev, 2, false, s0);
 

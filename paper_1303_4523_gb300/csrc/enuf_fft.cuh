@@ -363,14 +363,51 @@ namespace enuf {
 // shared-memory accesses, against the runtime-radix Stockham stages'
 // per-stage quotients, swizzles and twiddle indices.
 // ---------------------------------------------------------------------------
-template <typename R, int F1, bool INV, typename Load>
-__device__ __forceinline__ void fft2_phase_a(typename Cx<R>::T* __restrict__ buf, int lsa, int nlines, int f2,
+// Row stride of a phase-A line buffer, and of a buffer of natural-order
+// results. A two-factor pass with L lines per CTA holds the twiddle table (n
+// values), L phase-A rows and L result rows in shared memory.
+__host__ __device__ constexpr int fft2_lsa(int f1, int f2) { return f1 * (f2 + 1); }
+__host__ __device__ constexpr int fft2_lsb(int n) { return n + 1; }
+
+// The lengths a two-factor kernel works with. FftLen<F1, F2>: compile-time, so
+// that every offset, quotient and loop bound of a pass is a constant (the
+// runtime form spends two thirds of its instructions on them: ~95 per complex
+// point in the inverse x pass at n = 320, of which ~30 are the transform);
+// FftLen<0, 0>: from the plan, for lengths without an instance of their own and
+// for batches of mixed sizes.
+template <int F1, int F2>
+struct FftLen {
+    static constexpr int kF1 = F1, kF2 = F2;
+    static constexpr int n = F1 * F2, f1 = F1, f2 = F2, nc = n / 4 - 1, nc1 = nc + 1, K = 2 * nc + 1;
+    static constexpr int lsa = fft2_lsa(F1, F2), lsb = fft2_lsb(n);
+    __device__ __forceinline__ FftLen(int, int, int) {}
+    static __device__ __forceinline__ int by_n(int a) { return (int)((unsigned)a / (unsigned)n); }
+    static __device__ __forceinline__ int by_f1(int a) { return (int)((unsigned)a / (unsigned)F1); }
+    static __device__ __forceinline__ int by_f2(int a) { return (int)((unsigned)a / (unsigned)F2); }
+    static __device__ __forceinline__ int by_K(int a) { return (int)((unsigned)a / (unsigned)K); }
+    static __device__ __forceinline__ int by_nc1(int a) { return (int)((unsigned)a / (unsigned)nc1); }
+};
+template <>
+struct FftLen<0, 0> {
+    static constexpr int kF1 = 0, kF2 = 0;
+    int n, f1, f2, nc, nc1, K, lsa, lsb;
+    __device__ __forceinline__ FftLen(int f1_, int f2_, int nc_)
+        : n(f1_ * f2_), f1(f1_), f2(f2_), nc(nc_), nc1(nc_ + 1), K(2 * nc_ + 1), lsa(fft2_lsa(f1_, f2_)),
+          lsb(fft2_lsb(f1_ * f2_)) {}
+    __device__ __forceinline__ int by_n(int a) const { return qdiv(a, n, 1.0f / (float)n); }
+    __device__ __forceinline__ int by_f1(int a) const { return qdiv(a, f1, 1.0f / (float)f1); }
+    __device__ __forceinline__ int by_f2(int a) const { return qdiv(a, f2, 1.0f / (float)f2); }
+    __device__ __forceinline__ int by_K(int a) const { return qdiv(a, K, 1.0f / (float)K); }
+    __device__ __forceinline__ int by_nc1(int a) const { return qdiv(a, nc1, 1.0f / (float)nc1); }
+};
+
+template <typename R, int F1, bool INV, typename Len, typename Load>
+__device__ __forceinline__ void fft2_phase_a(typename Cx<R>::T* __restrict__ buf, const Len& L, int nlines,
                                              const typename Cx<R>::T* __restrict__ tw, Load& load) {
     using C = typename Cx<R>::T;
-    const int total = nlines * f2;
-    const float rf2 = 1.0f / (float)f2;
+    const int f2 = L.f2, total = nlines * f2;
     for (int task = threadIdx.x; task < total; task += blockDim.x) {
-        const int line = qdiv(task, f2, rf2), t = task - line * f2;
+        const int line = L.by_f2(task), t = task - line * f2;
         C v[F1];
 #pragma unroll
         for (int j = 0; j < F1; ++j) v[j] = load(line, t + f2 * j);
@@ -381,21 +418,20 @@ __device__ __forceinline__ void fft2_phase_a(typename Cx<R>::T* __restrict__ buf
             if (INV) w.y = -w.y;
             v[k] = cmul(v[k], w);
         }
-        C* d = buf + line * lsa + t;
+        C* d = buf + line * L.lsa + t;
 #pragma unroll
         for (int k = 0; k < F1; ++k) d[k * (f2 + 1)] = v[k];
     }
 }
 
-template <typename R, int F2, bool INV, typename Store>
-__device__ __forceinline__ void fft2_phase_b(const typename Cx<R>::T* __restrict__ buf, int lsa, int nlines, int f1,
+template <typename R, int F2, bool INV, typename Len, typename Store>
+__device__ __forceinline__ void fft2_phase_b(const typename Cx<R>::T* __restrict__ buf, const Len& L, int nlines,
                                              Store& store) {
     using C = typename Cx<R>::T;
-    const int total = nlines * f1;
-    const float rf1 = 1.0f / (float)f1;
+    const int f1 = L.f1, total = nlines * f1;
     for (int task = threadIdx.x; task < total; task += blockDim.x) {
-        const int line = qdiv(task, f1, rf1), k1 = task - line * f1;
-        const C* s = buf + line * lsa + k1 * (F2 + 1);
+        const int line = L.by_f1(task), k1 = task - line * f1;
+        const C* s = buf + line * L.lsa + k1 * (F2 + 1);
         C u[F2];
 #pragma unroll
         for (int t = 0; t < F2; ++t) u[t] = s[t];
@@ -409,68 +445,78 @@ __device__ __forceinline__ void fft2_phase_b(const typename Cx<R>::T* __restrict
 // (t < f2, k < f1; forward sign), from the table twg[m] = w_n^m: the lanes of
 // a phase-A step read consecutive values (the natural table, read at t k,
 // puts lanes of an even k on few banks).
-template <typename C>
-__device__ __forceinline__ void fft2_twiddles(C* __restrict__ tw, const C* __restrict__ twg, const FftPlanDev& fp) {
-    const int f2 = fp.f2, n = fp.f1 * fp.f2;
-    const float rf2 = 1.0f / (float)f2;
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-        const int k = qdiv(e, f2, rf2), t = e - k * f2;
+template <typename C, typename Len>
+__device__ __forceinline__ void fft2_twiddles(C* __restrict__ tw, const C* __restrict__ twg, const Len& L) {
+    for (int e = threadIdx.x; e < L.n; e += blockDim.x) {
+        const int k = L.by_f2(e), t = e - k * L.f2;
         tw[e] = twg[t * k];
     }
 }
 
-// Row stride of a phase-A line buffer, and of a buffer of natural-order
-// results. A two-factor pass with L lines per CTA holds the twiddle table (n
-// values), L phase-A rows and L result rows in shared memory.
-__host__ __device__ constexpr int fft2_lsa(int f1, int f2) { return f1 * (f2 + 1); }
-__host__ __device__ constexpr int fft2_lsb(int n) { return n + 1; }
-
 // The whole two-factor transform of nlines lines: load(line, m) gives element
 // m of a line, store(line, k, X_k) takes the results; tw is the table that
-// fft2_twiddles fills. buf holds nlines rows
-// of fft2_lsa(f1, f2) values. Contains __syncthreads (call from all threads);
-// the caller synchronises before reading what store wrote to shared memory.
-// EXT: radices 9, 15 and 18 are compiled in as well (instances of their own:
-// in the common kernels the larger switch cost 0.7-1.2 us a launch at n = 96).
-template <typename R, bool INV, bool EXT, typename Load, typename Store>
+// fft2_twiddles fills. buf holds nlines rows of L.lsa values. Contains
+// __syncthreads (call from all threads); the caller synchronises before
+// reading what store wrote to shared memory.
+template <typename R, bool INV, typename Len, typename Load, typename Store>
 __device__ __forceinline__ void fft2_lines(typename Cx<R>::T* __restrict__ buf, const typename Cx<R>::T* tw,
-                                           const FftPlanDev& fp, int nlines, Load&& load, Store&& store) {
-    const int f1 = fp.f1, f2 = fp.f2, lsa = fft2_lsa(f1, f2);
-    switch (f1) {
-        case 4: fft2_phase_a<R, 4, INV>(buf, lsa, nlines, f2, tw, load); break;
-        case 5: fft2_phase_a<R, 5, INV>(buf, lsa, nlines, f2, tw, load); break;
-        case 6: fft2_phase_a<R, 6, INV>(buf, lsa, nlines, f2, tw, load); break;
-        case 8: fft2_phase_a<R, 8, INV>(buf, lsa, nlines, f2, tw, load); break;
-        case 10: fft2_phase_a<R, 10, INV>(buf, lsa, nlines, f2, tw, load); break;
-        case 12: fft2_phase_a<R, 12, INV>(buf, lsa, nlines, f2, tw, load); break;
-        case 16: fft2_phase_a<R, 16, INV>(buf, lsa, nlines, f2, tw, load); break;
-        case 20: fft2_phase_a<R, 20, INV>(buf, lsa, nlines, f2, tw, load); break;
-        default:
-            if constexpr (EXT) {
-                if (f1 == 9) fft2_phase_a<R, 9, INV>(buf, lsa, nlines, f2, tw, load);
-                else if (f1 == 15) fft2_phase_a<R, 15, INV>(buf, lsa, nlines, f2, tw, load);
-                else if (f1 == 18) fft2_phase_a<R, 18, INV>(buf, lsa, nlines, f2, tw, load);
-            }
-            break;
+                                           const Len& L, int nlines, Load&& load, Store&& store) {
+    if constexpr (Len::kF1 > 0) {
+        fft2_phase_a<R, Len::kF1, INV>(buf, L, nlines, tw, load);
+        __syncthreads();
+        fft2_phase_b<R, Len::kF2, INV>(buf, L, nlines, store);
+    } else {
+        switch (L.f1) {
+            case 4: fft2_phase_a<R, 4, INV>(buf, L, nlines, tw, load); break;
+            case 5: fft2_phase_a<R, 5, INV>(buf, L, nlines, tw, load); break;
+            case 6: fft2_phase_a<R, 6, INV>(buf, L, nlines, tw, load); break;
+            case 8: fft2_phase_a<R, 8, INV>(buf, L, nlines, tw, load); break;
+            case 10: fft2_phase_a<R, 10, INV>(buf, L, nlines, tw, load); break;
+            case 12: fft2_phase_a<R, 12, INV>(buf, L, nlines, tw, load); break;
+            case 16: fft2_phase_a<R, 16, INV>(buf, L, nlines, tw, load); break;
+            case 20: fft2_phase_a<R, 20, INV>(buf, L, nlines, tw, load); break;
+            default: break;
+        }
+        __syncthreads();
+        switch (L.f2) {
+            case 4: fft2_phase_b<R, 4, INV>(buf, L, nlines, store); break;
+            case 5: fft2_phase_b<R, 5, INV>(buf, L, nlines, store); break;
+            case 6: fft2_phase_b<R, 6, INV>(buf, L, nlines, store); break;
+            case 8: fft2_phase_b<R, 8, INV>(buf, L, nlines, store); break;
+            case 10: fft2_phase_b<R, 10, INV>(buf, L, nlines, store); break;
+            case 12: fft2_phase_b<R, 12, INV>(buf, L, nlines, store); break;
+            case 16: fft2_phase_b<R, 16, INV>(buf, L, nlines, store); break;
+            case 20: fft2_phase_b<R, 20, INV>(buf, L, nlines, store); break;
+            default: break;
+        }
     }
-    __syncthreads();
-    switch (f2) {
-        case 4: fft2_phase_b<R, 4, INV>(buf, lsa, nlines, f1, store); break;
-        case 5: fft2_phase_b<R, 5, INV>(buf, lsa, nlines, f1, store); break;
-        case 6: fft2_phase_b<R, 6, INV>(buf, lsa, nlines, f1, store); break;
-        case 8: fft2_phase_b<R, 8, INV>(buf, lsa, nlines, f1, store); break;
-        case 10: fft2_phase_b<R, 10, INV>(buf, lsa, nlines, f1, store); break;
-        case 12: fft2_phase_b<R, 12, INV>(buf, lsa, nlines, f1, store); break;
-        case 16: fft2_phase_b<R, 16, INV>(buf, lsa, nlines, f1, store); break;
-        case 20: fft2_phase_b<R, 20, INV>(buf, lsa, nlines, f1, store); break;
-        default:
-            if constexpr (EXT) {
-                if (f2 == 9) fft2_phase_b<R, 9, INV>(buf, lsa, nlines, f1, store);
-                else if (f2 == 15) fft2_phase_b<R, 15, INV>(buf, lsa, nlines, f1, store);
-                else if (f2 == 18) fft2_phase_b<R, 18, INV>(buf, lsa, nlines, f1, store);
-            }
-            break;
-    }
+}
+
+// Lines per CTA of the passes: what fits a shared-memory budget beside the
+// twiddle table. ab: transforms held per line (phase-A and result rows);
+// extra: further bytes per line (input buffers of the persistent passes).
+__host__ __device__ constexpr int fft2_lines_for(int f1, int f2, int csz, int ab, int extra, int budget, int cap) {
+    const int n = f1 * f2, per = ab * (fft2_lsa(f1, f2) + fft2_lsb(n)) * csz + extra;
+    const int l = (budget - n * csz - 16) / per;
+    return l < 1 ? 1 : (l > cap ? cap : l);
+}
+constexpr int kFftPipe = 72 * 1024;   // persistent passes: three CTAs per SM
+constexpr int kFftLine = 64 * 1024;
+// x: input rows double buffered; inverse x: LP line pairs of each of nf fields,
+// Hermitian rows double buffered
+__host__ __device__ constexpr int fft2_lx(int f1, int f2) { return fft2_lines_for(f1, f2, 8, 1, 16 * f1 * f2, kFftPipe, 64); }
+__host__ __device__ constexpr int fft2_lz(int f1, int f2, int ni) {
+    return fft2_lines_for(f1, f2, 8, ni, 16 * f1 * f2, kFftPipe, 64);
+}
+__host__ __device__ constexpr int fft2_lix(int f1, int f2, int nf) {
+    return fft2_lines_for(f1, f2, 8, nf, nf * 32 * (f1 * f2 / 4), kFftPipe, 64);
+}
+
+// Lines per CTA of the y passes: runs of a multiple of 4 values (32-byte
+// sectors) in the transposed output.
+__host__ __device__ constexpr int fft2_ly(int f1, int f2) {
+    const int l = fft2_lines_for(f1, f2, 8, 1, 0, kFftLine, 16);
+    return l >= 4 ? l / 4 * 4 : l;
 }
 
 }  // namespace enuf

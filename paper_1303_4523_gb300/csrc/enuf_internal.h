@@ -66,6 +66,7 @@ struct Geo {
     int chunk;    // beads per binning block
     int kmask;
     int nf;       // reciprocal force fields: 3 (ik-differentiation) or 1 (window gradient)
+    int h4;       // FP32: the fields interleaved, float4 (h_x, h_y, h_z, 0) per point
     int bin_scan; // 1: every scatter block scans the tile counters itself (up to
                   //    kBinScanTiles tiles); 0: a scan kernel between count and scatter
     double L, alpha, beta, kappa, rc;
@@ -127,7 +128,7 @@ struct FftShape {
     int ly;    // lines per CTA, forward y
     int lz;    // lines per CTA, z pass (forward + convolve + 3 inverses)
     int liy;   // lines per CTA, inverse y
-    int lix;   // complex lines per CTA, inverse x
+    int lix;   // complex lines per CTA, inverse x (two-factor: row pairs, of every field)
     int tx, ty, tz, tiy, tix;   // threads per CTA of each pass
     int smem_x, smem_y, smem_z, smem_iy, smem_ix;   // dynamic smem bytes
     int grid_x, grid_y_z, grid_z, grid_iy, grid_ix; // CTAs (grid_y_z: z-chunks of the y pass)
@@ -171,9 +172,9 @@ struct Work {
     void* grid;      // real [n^3]
     void* spec1;     // cplx [n][nc+1][n]      after forward x   ([z][kx][y])
     void* spec2;     // cplx [nc+1][K][n]      after forward y   ([kx][ky][z])
-    void* spec3;     // cplx [3][n][nc+1][K]   after z pass      ([a][z][kx][ky])
+    void* spec3;     // cplx [3][n][nc+1][K]   after z pass      ([a][z][kx][ky]; two-factor: G and Gz)
     void* spec4;     // cplx [3][n][n][nc+1]   after inverse y   ([a][z][y][kx])
-    void* h;         // real [3][n^3]          conjugated-NFFT fields
+    void* h;         // real [3][n^3]          conjugated-NFFT fields (Geo::h4: real [n^3][4])
     double* tab;     // [nc+1][K][K] influence/deconvolution table D(k) (0 outside the mode set)
     double* tabv;    // [nc+1][K][K] D(k) times the virial weight 1 - 2 pi^2 k^2/(alpha L)^2
     void* tabr;      // real copy of tab
@@ -283,6 +284,8 @@ struct BatchLaunch {
 };
 
 template <typename R> cudaError_t configure_kernels(int max_smem);
+// Attributes of the two-factor FFT kernels a plan runs (those of one length).
+cudaError_t configure_fft2(const FftShape& fs, const FftPlanDev& fp, int max_smem);
 template <typename R> int spread_smem(const Geo& g);
 // dpd (a DPD step with fused pair kernels, or nullptr): the real-space launch
 // also runs the DPD pair forces (k_pairs), which enqueue_dpd_forces then leaves out.
@@ -314,7 +317,7 @@ cudaError_t enqueue_spread_only(const Geo& g, const Work& w, const EvalArgs& a, 
 // them (argument tables and block maps) into dbuf and fills the launch
 // parameters; batch_enqueue launches the sequence (fork/join on s1 for the
 // real-space pairs).
-bool batch_eligible(const BatchSys& s);
+template <typename R> cudaError_t configure_batch(int max_smem);
 template <typename R> size_t batch_bytes(const BatchSys* sys, int nsys);
 template <typename R>
 cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* out);

@@ -2019,7 +2019,37 @@ __device__ __forceinline__ void k_gather_body(Geo g, const int* __restrict__ tst
                 dz[c] = grad ? dwts[warp][2][c] : (R)0;
                 oz[c] = lix[warp][2][c];
             }
-            if (!grad && NRD <= 2) {
+            if (sizeof(R) == 4 && g.h4) {
+                // interleaved fields: a point's three values by one 16-byte load, a round's
+                // 2p loads issued before the sums (planar fields cost three loads of 32-byte
+                // rows each: twice the L1 lookups)
+                const float4* __restrict__ h4 = reinterpret_cast<const float4*>(h);
+#pragma unroll
+                for (int r = 0; r < NRD; ++r) {
+                    const int ab = lane + 32 * r;
+                    const bool on = NAB % 32 == 0 || ab < NAB;
+                    const int b = on ? ab / PT : 0, a = on ? ab - b * PT : 0;
+                    const int rowo = lix[warp][1][b] * n + lix[warp][0][a];
+                    float4 v[PT];
+#pragma unroll
+                    for (int c = 0; c < PT; ++c) {
+                        int off = oz[c] + rowo;
+                        if (!ENUF_GUARD(g.check, (size_t)off < n3, 5)) off = 0;
+                        v[c] = h4[off];
+                    }
+                    R s0 = 0, s1 = 0, s2 = 0;
+#pragma unroll
+                    for (int c = 0; c < PT; ++c) {
+                        s0 = fma(wz[c], (R)v[c].x, s0);
+                        s1 = fma(wz[c], (R)v[c].y, s1);
+                        s2 = fma(wz[c], (R)v[c].z, s2);
+                    }
+                    const R wab = on ? wts[warp][0][a] * wts[warp][1][b] : (R)0;
+                    ax = fma(wab, s0, ax);
+                    ay = fma(wab, s1, ay);
+                    az = fma(wab, s2, az);
+                }
+            } else if (!grad && NRD <= 2) {
                 // three fields, at most two rounds: every round's loads issued before
                 // the sums (6 p loads in flight per lane)
                 R hv[NRD][3][PT];
@@ -2131,6 +2161,13 @@ __device__ __forceinline__ void k_gather_body(Geo g, const int* __restrict__ tst
                     const R w = wts[warp][2][c];
                     const int off = lix[warp][2][c] + rowo;   // z index pre-scaled by n^2
                     if (!ENUF_GUARD(g.check, (size_t)off < n3, 5)) continue;
+                    if (sizeof(R) == 4 && g.h4) {
+                        const float4 v = reinterpret_cast<const float4*>(h)[off];
+                        s0 = fma(w, (R)v.x, s0);
+                        s1 = fma(w, (R)v.y, s1);
+                        s2 = fma(w, (R)v.z, s2);
+                        continue;
+                    }
                     s0 = fma(w, h0[off], s0);
                     s1 = fma(w, h1[off], s1);
                     s2 = fma(w, h2[off], s2);
