@@ -191,9 +191,9 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
 
 template <typename R>
 cudaError_t configure_batch(int max_smem) {
-    return first_error({set_smem((const void*)kb_real<R>, max_smem, false), set_smem((const void*)kb_fft_xy<R>, max_smem, false),
-                        set_smem((const void*)kb_fft_z<R>, max_smem, false),
-                        set_smem((const void*)kb_fft_yx<R>, max_smem, false)});
+    return first_error({set_smem((const void*)kb_real<R>, max_smem), set_smem((const void*)kb_fft_xy<R>, max_smem),
+                        set_smem((const void*)kb_fft_z<R>, max_smem),
+                        set_smem((const void*)kb_fft_yx<R>, max_smem)});
 }
 
 template <typename R>

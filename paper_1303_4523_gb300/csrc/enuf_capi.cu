@@ -583,6 +583,14 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
     w.nblk_dpd = 4 * kSMs;
     w.nblk_kin = kSMs;   // one block per SM: its FP64 block sum runs on each SM's few FP64 units once
     w.nblk_gather = 4 * kSMs;
+    // The pair kernels and the spreading run beside the FFT passes and take their
+    // shared-memory split: without one split per plan the branches mostly waited for
+    // each other's SMs to empty (whole: 81k beads 91 -> 84 us, 4 steps of them 400 ->
+    // 351, 3M 1111 -> 1074, FP64 4 steps 1430 -> 1340; the FP32 step with its small
+    // kernels on the split as well 413, the gather on a split of 100 loses its L1:
+    // 524k 267 -> 307)
+    w.carve = P.prec == ENUF_FP64 ? 75 : (fs.two && !fs.fused ? kCarveLines : kCarvePlanes);
+    w.carve_b = P.prec == ENUF_FP64 ? 75 : 0;
     w.off_q = 0;
     w.off_real = w.off_q + 2 * g.nbin;
     w.off_recip = w.off_real + 2 * w.nblk_real;
@@ -1185,8 +1193,8 @@ enuf_status capture_step(dpd_system_t sys) {
     LaunchLog log;
     Events* ev = plan->ev.on ? &plan->ev : nullptr;
     if (ev) cudaEventRecordWithFlags(ev->start[6], plan->stream, cudaEventRecordExternal);
-    cudaError_t e = plan->prec == ENUF_FP32 ? enqueue_vv_pre<float>(sys->d, plan->stream, &log)
-                                            : enqueue_vv_pre<double>(sys->d, plan->stream, &log);
+    cudaError_t e = plan->prec == ENUF_FP32 ? enqueue_vv_pre<float>(plan->w, sys->d, plan->stream, &log)
+                                            : enqueue_vv_pre<double>(plan->w, sys->d, plan->stream, &log);
     enuf_status st = e == cudaSuccess ? ENUF_OK : fail(plan, ENUF_ERR_CUDA, "vv_pre: %s", cudaGetErrorString(e));
     if (st == ENUF_OK) st = enqueue_force_eval(sys, plan->stream, plan->aux, ev, &log, true);
     if (st == ENUF_OK) {

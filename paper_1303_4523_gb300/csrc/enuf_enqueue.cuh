@@ -39,22 +39,37 @@ inline int launch_priority(bool critical) {
     return critical ? greatest : 0;
 }
 
+// carve (percent, 0: the driver's choice): shared memory's preferred share of the
+// SM's L1. Kernels of the two branches only share an SM under one split, and a
+// change of split waits until the SM is empty (see the plan's carve).
 template <typename... P, typename... A>
-inline void launch(bool pdl, bool critical, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                   A&&... args) {
+inline void launch_carved(int carve, bool pdl, bool critical, void (*k)(P...), dim3 grid, dim3 block, size_t smem,
+                          cudaStream_t s, A&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributePriority;
-    at[0].val.priority = launch_priority(critical);
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[3];
+    unsigned int n = 0;
+    at[n].id = cudaLaunchAttributePriority;
+    at[n++].val.priority = launch_priority(critical);
+    if (pdl) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (carve) {
+        at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        at[n++].val.sharedMemCarveout = (unsigned int)carve;
+    }
     cfg.attrs = at;
-    cfg.numAttrs = pdl ? 2 : 1;
+    cfg.numAttrs = n;
     cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
+}
+template <typename... P, typename... A>
+inline void launch(bool pdl, bool critical, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                   A&&... args) {
+    launch_carved(0, pdl, critical, k, grid, block, smem, s, std::forward<A>(args)...);
 }
 
 inline bool pdl_ok(const Events* ev) { return !(ev && ev->on); }
@@ -88,10 +103,9 @@ inline TotalsArgs no_totals() {
 // The Stockham passes of one evaluation (fused plane passes or five line
 // passes); CR selects the kernels compiled with the composite radices. The FP32
 // instances are compiled in a translation unit of their own.
-inline cudaError_t set_smem(const void* f, int max_smem, bool carve) {
+inline cudaError_t set_smem(const void* f, int max_smem, int carve = 0) {
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
-    // the two-factor passes prefer the largest shared-memory carve-out (several CTAs per SM)
-    if (e == cudaSuccess && carve) e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e == cudaSuccess && carve) e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
     return e;
 }
 inline cudaError_t first_error(std::initializer_list<cudaError_t> l) {
@@ -107,13 +121,14 @@ struct StockhamPasses {   // members defined out of class: an extern instance is
 };
 template <typename R, bool CR>
 cudaError_t StockhamPasses<R, CR>::configure(int ms) {
-    return first_error({set_smem((const void*)k_fft_x<R, CR>, ms, false), set_smem((const void*)k_fft_y<R, CR>, ms, false),
-                        set_smem((const void*)k_fft_z<R, CR>, ms, false), set_smem((const void*)k_fft_iy<R, CR>, ms, false),
-                        set_smem((const void*)k_fft_ix<R, CR>, ms, false), set_smem((const void*)k_fft_xy<R, CR>, ms, false),
-                        set_smem((const void*)k_fft_yx<R, CR>, ms, false)});
+    return first_error({set_smem((const void*)k_fft_x<R, CR>, ms), set_smem((const void*)k_fft_y<R, CR>, ms),
+                        set_smem((const void*)k_fft_z<R, CR>, ms), set_smem((const void*)k_fft_iy<R, CR>, ms),
+                        set_smem((const void*)k_fft_ix<R, CR>, ms), set_smem((const void*)k_fft_xy<R, CR>, ms),
+                        set_smem((const void*)k_fft_yx<R, CR>, ms)});
 }
 template <typename R, bool CR>
-void StockhamPasses<R, CR>::enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0, bool pdl, LaunchLog* log, cudaEvent_t evZ) {
+void StockhamPasses<R, CR>::enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w,
+        cudaStream_t s0, bool pdl, LaunchLog* log, cudaEvent_t evZ) {
     using C = typename Cx<R>::T;
     const C* tw = static_cast<const C*>(w.tw);
     if (fs.fused) {   // whole z-planes in shared memory: x+y, z (+convolve), y+x
@@ -207,19 +222,19 @@ template <typename R>
 void enqueue_bin(const Geo& g, const Work& w, int N, const R* pos, const R* q, R* Fzero, R* gzero, cudaStream_t s,
                  bool pdl) {
     using V = typename V4<R>::T;
-    launch(false, true, k_bin_count<R>, g.nbin, kBinThreads, g.chunk * sizeof(int), s, g, N, pos, q, w.cnt_blk,
+    launch_carved(w.carve_b, false, true, k_bin_count<R>, g.nbin, kBinThreads, g.chunk * sizeof(int), s, g, N, pos, q, w.cnt_blk,
            w.tcnt, w.crank, static_cast<V*>(w.cpos), static_cast<V*>(w.cfrac), w.cbase, Fzero, w.part + w.off_q,
            gzero);
     if (!g.bin_scan)
-        launch(pdl, true, k_scan_mb, (g.ntiles + kScanMbSpan - 1) / kScanMbSpan, 1024, 0, s, (const int*)w.tcnt,
+        launch_carved(w.carve_b, pdl, true, k_scan_mb, (g.ntiles + kScanMbSpan - 1) / kScanMbSpan, 1024, 0, s, (const int*)w.tcnt,
                w.tstart, g.ntiles, (int*)nullptr);
     const bool fused = sizeof(R) == 4 && w.wb;
-    launch(pdl, true, fused ? k_bin_scatter<R, true> : k_bin_scatter<R, false>, g.nbin, kBinThreads,
+    launch_carved(w.carve_b, pdl, true, fused ? k_bin_scatter<R, true> : k_bin_scatter<R, false>, g.nbin, kBinThreads,
            g.bin_scan ? (g.ntiles + 1) * sizeof(int) : 0, s, g, (const int*)w.cnt_blk, w.tcnt, w.tstart,
            (const int*)w.crank, static_cast<const V*>(w.cpos), static_cast<const V*>(w.cfrac), (const int*)w.cbase,
            static_cast<V*>(w.sq), static_cast<V*>(w.sw), w.sb, w.spf, static_cast<R*>(w.wb), w.ticket);
     if (w.wb && !fused)
-        launch(pdl, true, k_bin_weights<R>, bin_weight_blocks<R>(g), bin_weight_threads<R>(), 0, s, g,
+        launch_carved(w.carve_b, pdl, true, k_bin_weights<R>, bin_weight_blocks<R>(g), bin_weight_threads<R>(), 0, s, g,
                (const int*)w.tstart, static_cast<const V*>(w.sw), static_cast<R*>(w.wb));
 }
 
@@ -284,7 +299,7 @@ inline void enqueue_spread_red(const Geo& g, const Work& w, int N, cudaStream_t 
         default: break;
     }
     const int blocks = std::max(1, std::min(8 * 152, (N + 7) / 8));
-    launch(pdl, true, k, blocks, kRedThreads, 0, s, g, (const int*)w.tstart, static_cast<const V*>(w.sq),
+    launch_carved(w.carve, pdl, true, k, blocks, kRedThreads, 0, s, g, (const int*)w.tstart, static_cast<const V*>(w.sq),
            (const int*)w.sb, static_cast<const R*>(w.wb), static_cast<R*>(w.grid));
 }
 
@@ -312,12 +327,13 @@ struct Fft2Planes {   // members defined out of class: an extern instance is the
 };
 template <int F1, int F2>
 cudaError_t Fft2Planes<F1, F2>::configure(int ms) {
-    return first_error({set_smem((const void*)k2_fft_xy<float, F1, F2>, ms, true),
-                        set_smem((const void*)k2_fft_z<float, F1, F2>, ms, true),
-                        set_smem((const void*)k2_fft_yx<float, F1, F2>, ms, true)});
+    return first_error({set_smem((const void*)k2_fft_xy<float, F1, F2>, ms, kCarvePlanes),
+                        set_smem((const void*)k2_fft_z<float, F1, F2>, ms, kCarvePlanes),
+                        set_smem((const void*)k2_fft_yx<float, F1, F2>, ms, kCarvePlanes)});
 }
 template <int F1, int F2>
-void Fft2Planes<F1, F2>::enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0, bool pdl, LaunchLog* log, cudaEvent_t evZ) {
+void Fft2Planes<F1, F2>::enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w,
+        cudaStream_t s0, bool pdl, LaunchLog* log, cudaEvent_t evZ) {
     const float2* tw = static_cast<const float2*>(w.tw);
     launch(pdl, true, k2_fft_xy<float, F1, F2>, g.n, fs.t_xy, fs.smem_xy, s0, g, fp,
            static_cast<const float*>(w.grid), tw, static_cast<float2*>(w.spec2));
@@ -337,16 +353,17 @@ struct Fft2Lines {   // members defined out of class: an extern instance is then
 };
 template <int F1, int F2>
 cudaError_t Fft2Lines<F1, F2>::configure(int ms) {
-    return first_error({set_smem((const void*)k2_fft_x<float, F1, F2>, ms, true),
-                        set_smem((const void*)k2_fft_y<float, F1, F2>, ms, true),
-                        set_smem((const void*)k2_fft_zp<float, F1, F2, 3>, ms, true),
-                        set_smem((const void*)k2_fft_zp<float, F1, F2, 1>, ms, true),
-                        set_smem((const void*)k2_fft_iy<float, F1, F2>, ms, true),
-                        set_smem((const void*)k2_fft_ix<float, F1, F2, 3>, ms, true),
-                        set_smem((const void*)k2_fft_ix<float, F1, F2, 1>, ms, true)});
+    return first_error({set_smem((const void*)k2_fft_x<float, F1, F2>, ms, kCarveLines),
+                        set_smem((const void*)k2_fft_y<float, F1, F2>, ms, kCarveLines),
+                        set_smem((const void*)k2_fft_zp<float, F1, F2, 3>, ms, kCarveLines),
+                        set_smem((const void*)k2_fft_zp<float, F1, F2, 1>, ms, kCarveLines),
+                        set_smem((const void*)k2_fft_iy<float, F1, F2>, ms, kCarveLines),
+                        set_smem((const void*)k2_fft_ix<float, F1, F2, 3>, ms, kCarveLines),
+                        set_smem((const void*)k2_fft_ix<float, F1, F2, 1>, ms, kCarveLines)});
 }
 template <int F1, int F2>
-void Fft2Lines<F1, F2>::enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w, cudaStream_t s0, bool pdl, LaunchLog* log, cudaEvent_t evZ) {
+void Fft2Lines<F1, F2>::enqueue(const Geo& g, const FftShape& fs, const FftPlanDev& fp, const Work& w,
+        cudaStream_t s0, bool pdl, LaunchLog* log, cudaEvent_t evZ) {
     const float2* tw = static_cast<const float2*>(w.tw);
     if (fs.spread != 3 || fs.red) {
         launch(pdl, true, k2_fft_x<float, F1, F2>, fs.grid_x, fs.tx, fs.smem_x, s0, g, fp,
@@ -459,14 +476,14 @@ cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp,
     const float4* spf = w.spf;
     if (dpd) {   // DPD pairs and real-space pairs in one launch
         const DpdDev& d = *dpd;
-        launch(false, false, k_pairs<R>, w.nblk_dpd + w.nblk_real, kRealThreads,
+        launch_carved(w.carve, false, false, k_pairs<R>, w.nblk_dpd + w.nblk_real, kRealThreads,
                std::max(real_smem, dpd_smem_bytes<R>()), s1, d, static_cast<const V*>(d.sp),
                static_cast<const V*>(d.sv), dpd_spf<R>(d), (const int*)d.cstart, static_cast<const R*>(d.atab),
                static_cast<const R*>(d.pos), (const int*)d.bnd, (const uint64_t*)d.step_dev, d.df,
                static_cast<R*>(d.F), w.part + w.off_dpd, w.nblk_dpd, g, (const int*)w.tstart, (const V*)sq, (const V*)sw,
                (const int*)w.sb, spf, w.part + w.off_real);
     } else {
-        launch(false, false, k_real<R>, w.nblk_real, kRealThreads, real_smem, s1, g, (const int*)w.tstart,
+        launch_carved(w.carve, false, false, k_real<R>, w.nblk_real, kRealThreads, real_smem, s1, g, (const int*)w.tstart,
                (const V*)sq, (const V*)sw, (const int*)w.sb, spf, F, w.part + w.off_real);
     }
     rec(ev, 4, false, s1);
@@ -509,7 +526,7 @@ cudaError_t enqueue_enuf(const Geo& g, const FftShape& fs, const FftPlanDev& fp,
         cudaStreamWaitEvent(s1, evZ, 0);
         TotalsArgs t = totals_args(g, w, true, 0);
         t.pre = w.part + w.off_pre;
-        launch(false, false, k_totals_pre, 8, 256, 0, s1, t);
+        launch_carved(w.carve_b, false, false, k_totals_pre, 8, 256, 0, s1, t);
         cudaEventRecord(evT, s1);
         log->kernels += 1;
     }
@@ -540,18 +557,18 @@ cudaError_t enqueue_dpd_forces(const Work& w, const DpdDev& d, cudaStream_t s, E
     const bool pdl = pdl_ok(ev);
     rec(ev, 7, true, s);
     // the cell count also zeroes F, which the pair kernel adds into
-    launch(false, false, k_cell_count<R>, blocks, 256, 0, s, d.N, d.ncd, d.L, (R)d.cinv, d.xmaxf,
+    launch_carved(w.carve_b, false, false, k_cell_count<R>, blocks, 256, 0, s, d.N, d.ncd, d.L, (R)d.cinv, d.xmaxf,
            d.Lhi, d.Llo, static_cast<const R*>(d.pos),
            d.ckey, d.ccount, static_cast<R*>(d.F));
     // the cell starts (and the scatter cursors): several CTAs without a
     // wait for up to kScanMbMax cells, else one CTA; k_cell_scatter then
     // clears the counts
     if (d.ncells <= kScanMbMax)
-        launch(pdl, false, k_scan_mb, (d.ncells + kScanMbSpan - 1) / kScanMbSpan, 1024, 0, s,
+        launch_carved(w.carve_b, pdl, false, k_scan_mb, (d.ncells + kScanMbSpan - 1) / kScanMbSpan, 1024, 0, s,
                (const int*)d.ccount, d.cstart, d.ncells, d.ccur);
     else
         launch(pdl, false, k_scan, 1, 1024, 0, s, d.ccount, d.cstart, d.ncells, d.ccur, 0);
-    launch(pdl, false, k_cell_scatter<R>, blocks, 256, 0, s, d.N, d.L, d.xmaxf, d.Lhi, d.Llo,
+    launch_carved(w.carve_b, pdl, false, k_cell_scatter<R>, blocks, 256, 0, s, d.N, d.L, d.xmaxf, d.Lhi, d.Llo,
            static_cast<const R*>(d.pos),
            static_cast<const R*>(d.v0), (const int*)d.type, d.ckey, d.ccur, static_cast<V*>(d.sp),
            static_cast<V*>(d.sv), d.df, d.ccount, d.ncells);
@@ -560,7 +577,7 @@ cudaError_t enqueue_dpd_forces(const Work& w, const DpdDev& d, cudaStream_t s, E
     if (!pair_kernel) return cudaGetLastError();   // the pairs run in k_pairs with the real space
     rec(ev, 5, true, s);
     const int dpd_smem = dpd_smem_bytes<R>();
-    launch(pdl, false, k_dpd<R>, w.nblk_dpd, kDpdThreads, dpd_smem, s, d, static_cast<const V*>(d.sp),
+    launch_carved(w.carve, pdl, false, k_dpd<R>, w.nblk_dpd, kDpdThreads, dpd_smem, s, d, static_cast<const V*>(d.sp),
            static_cast<const V*>(d.sv), dpd_spf<R>(d), (const int*)d.cstart, static_cast<const R*>(d.atab),
            static_cast<const R*>(d.pos), (const int*)d.bnd, (const uint64_t*)d.step_dev, d.df, static_cast<R*>(d.F),
            w.part + w.off_dpd);
@@ -570,9 +587,9 @@ cudaError_t enqueue_dpd_forces(const Work& w, const DpdDev& d, cudaStream_t s, E
 }
 
 template <typename R>
-cudaError_t enqueue_vv_pre(const DpdDev& d, cudaStream_t s, LaunchLog* log) {
+cudaError_t enqueue_vv_pre(const Work& w, const DpdDev& d, cudaStream_t s, LaunchLog* log) {
     const int blocks = std::max(1, (3 * d.N / 4 + 255) / 256);
-    launch(false, true, k_vv_pre<R>, blocks, 256, 0, s, d.N, (R)d.lambda_vv, (R)d.dt, static_cast<R*>(d.pos),
+    launch_carved(w.carve_b, false, true, k_vv_pre<R>, blocks, 256, 0, s, d.N, (R)d.lambda_vv, (R)d.dt, static_cast<R*>(d.pos),
            static_cast<R*>(d.vel), static_cast<R*>(d.v0), static_cast<const R*>(d.F), d.step_dev);
     log->kernels += 1;
     return cudaGetLastError();
@@ -585,7 +602,7 @@ cudaError_t enqueue_vv_post(const Geo& g, const Work& w, const DpdDev& d, cudaSt
                             bool pre) {
     TotalsArgs t = totals_args(g, w, true, 2);
     if (pre) t.pre = w.part + w.off_pre;
-    launch(pdl, true, k_vv_post<R>, w.nblk_kin, 256, 0, s, g, d.N, (R)d.dt, static_cast<R*>(d.vel),
+    launch_carved(w.carve_b, pdl, true, k_vv_post<R>, w.nblk_kin, 256, 0, s, g, d.N, (R)d.dt, static_cast<R*>(d.vel),
            static_cast<R*>(d.F), (const float4*)d.df, (const int*)d.ckey, w.part + w.off_kin, t);
     log->kernels += 1;
     return cudaGetLastError();
@@ -629,7 +646,7 @@ namespace enuf {
     template cudaError_t enqueue_totals<R>(const Geo&, const Work&, bool, cudaStream_t, LaunchLog*, bool);   \
     template cudaError_t enqueue_dpd_forces<R>(const Work&, const DpdDev&, cudaStream_t, Events*,            \
                                                LaunchLog*, bool);                                            \
-    template cudaError_t enqueue_vv_pre<R>(const DpdDev&, cudaStream_t, LaunchLog*);                         \
+    template cudaError_t enqueue_vv_pre<R>(const Work&, const DpdDev&, cudaStream_t, LaunchLog*);                       \
     template cudaError_t enqueue_vv_post<R>(const Geo&, const Work&, const DpdDev&, cudaStream_t, LaunchLog*,  \
                                             bool, bool);                                                     \
     template cudaError_t enqueue_dpd_add<R>(const DpdDev&, cudaStream_t, LaunchLog*, bool);                   \

@@ -118,6 +118,11 @@ __host__ __device__ constexpr int brick_smem(int T, int BX, int fx_bytes) {
     return T * T * BX * (int)sizeof(R) + (brick_stage_bytes<R>() > fx_bytes ? brick_stage_bytes<R>() : fx_bytes);
 }
 
+// Preferred shared-memory split of the two-factor FFT kernels (percent): the plane
+// passes share SMs with the pair kernels, the persistent line passes want three
+// CTAs of 72 KB.
+constexpr int kCarvePlanes = 60, kCarveLines = 100;
+
 // Row length of the real-space kernel table (16-byte aligned rows).
 constexpr int kKtStride64 = 6;   // c_0..c_5 in double
 constexpr int kKtStride32 = 8;   // c_0..c_5 in float, 2 padding
@@ -185,6 +190,9 @@ struct Work {
     // partial-sum segments (offsets into part, in doubles)
     int off_q, off_real, off_recip, off_dpd, off_kin;
     int nblk_real, nblk_conv, nblk_dpd, nblk_kin, nblk_gather;
+    // preferred shared-memory split (percent, 0: none) of the pair and spreading kernels,
+    // and of the binning, cell list and integrator
+    int carve, carve_b;
     int off_pre;   // 8 doubles: the step's quantities 0-7 reduced beside the gather
 };
 
@@ -303,7 +311,7 @@ template <typename R>
 cudaError_t enqueue_dpd_forces(const Work& w, const DpdDev& d, cudaStream_t s, Events* ev, LaunchLog* log,
                                bool pair_kernel = true);
 template <typename R>
-cudaError_t enqueue_vv_pre(const DpdDev& d, cudaStream_t s, LaunchLog* log);
+cudaError_t enqueue_vv_pre(const Work& w, const DpdDev& d, cudaStream_t s, LaunchLog* log);
 template <typename R>
 cudaError_t enqueue_vv_post(const Geo& g, const Work& w, const DpdDev& d, cudaStream_t s, LaunchLog* log, bool pdl,
                             bool pre = false);
