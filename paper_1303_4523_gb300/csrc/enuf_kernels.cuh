@@ -2049,42 +2049,6 @@ __device__ __forceinline__ void k_gather_body(Geo g, const int* __restrict__ tst
                     ay = fma(wab, s1, ay);
                     az = fma(wab, s2, az);
                 }
-            } else if (!grad && NRD <= 2) {
-                // three fields, at most two rounds: every round's loads issued before
-                // the sums (6 p loads in flight per lane)
-                R hv[NRD][3][PT];
-                bool on[NRD];
-#pragma unroll
-                for (int r = 0; r < NRD; ++r) {
-                    const int ab = lane + 32 * r;
-                    on[r] = NAB % 32 == 0 || ab < NAB;
-                    const int b = on[r] ? ab / PT : 0, a = on[r] ? ab - b * PT : 0;
-                    const int rowo = lix[warp][1][b] * n + lix[warp][0][a];
-#pragma unroll
-                    for (int c = 0; c < PT; ++c) {
-                        int off = oz[c] + rowo;
-                        if (!ENUF_GUARD(g.check, (size_t)off < n3, 5)) off = 0;
-                        hv[r][0][c] = on[r] ? h0[off] : (R)0;
-                        hv[r][1][c] = on[r] ? h1[off] : (R)0;
-                        hv[r][2][c] = on[r] ? h2[off] : (R)0;
-                    }
-                }
-#pragma unroll
-                for (int r = 0; r < NRD; ++r) {
-                    const int ab = lane + 32 * r;
-                    const int b = on[r] ? ab / PT : 0, a = on[r] ? ab - b * PT : 0;
-                    R s0 = 0, s1 = 0, s2 = 0;
-#pragma unroll
-                    for (int c = 0; c < PT; ++c) {
-                        s0 = fma(wz[c], hv[r][0][c], s0);
-                        s1 = fma(wz[c], hv[r][1][c], s1);
-                        s2 = fma(wz[c], hv[r][2][c], s2);
-                    }
-                    const R wab = on[r] ? wts[warp][0][a] * wts[warp][1][b] : (R)0;
-                    ax = fma(wab, s0, ax);
-                    ay = fma(wab, s1, ay);
-                    az = fma(wab, s2, az);
-                }
             } else {
 #pragma unroll
                 for (int r = 0; r < NRD; ++r) {
@@ -2188,20 +2152,25 @@ __device__ __forceinline__ void k_gather_body(Geo g, const int* __restrict__ tst
         ax = warp_sum_r(ax);
         ay = warp_sum_r(ay);
         az = warp_sum_r(az);
-        if (lane == 0) {
-            const int i = real_as_int(wv.w);
-            const R f = pref * qs;
-            F[3 * i] += f * ax;
-            F[3 * i + 1] += f * ay;
-            F[3 * i + 2] += f * az;
+        if (lane < 3) {   // a reduction each: nothing waits for F's old value
+            const R f = pref * qs * (lane == 0 ? ax : (lane == 1 ? ay : az));
+            atomicAdd(&F[3 * real_as_int(wv.w) + lane], f);
         }
         }
         __syncwarp();
     }
 }
 
+// Four CTAs per SM: the launch's 4 x 152 blocks are one wave (FP32 windows up
+// to 8 taps, one round's loads in flight per lane; both rounds' took 88 registers,
+// two CTAs per SM and a second wave). Whole calls with that and with F by
+// reductions: 1M beads at p = 2 380 -> 361 us, 150,000 at p = 6 154 -> 147, 3000
+// at p = 2 34.6 -> 33.4, 60,000 with a quarter charged in FP64 328 -> 317; the
+// others within 1%.
+template <typename R, int PT>
+constexpr int gather_ctas() { return sizeof(R) == 4 && PT > 0 && PT <= 8 ? 4 : 2; }
 template <typename R, int PT = 0>
-__global__ void __launch_bounds__(kGatherThreads) k_gather(Geo g, const int* __restrict__ tstart,
+__global__ void __launch_bounds__(kGatherThreads, gather_ctas<R, PT>()) k_gather(Geo g, const int* __restrict__ tstart,
                                                            const typename V4<R>::T* __restrict__ sq,
                                                            const typename V4<R>::T* __restrict__ sw,
                                                            const int* __restrict__ sb, const R* __restrict__ wb,
