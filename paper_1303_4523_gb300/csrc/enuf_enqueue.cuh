@@ -384,18 +384,8 @@ void Fft2Lines<F1, F2>::enqueue(const Geo& g, const FftShape& fs, const FftPlanD
     log->kernels += 5;   // the spreading kernel and four passes
 }
 
-// Lengths with instances of their own: every n <= 112 of two radices (plane
-// passes), every larger one up to 400, and 108 in both forms.
-#define ENUF_FFT2_PLANES_A(X) X(4, 4) X(4, 5) X(4, 6) X(4, 8) X(6, 6) X(5, 8) X(6, 8)
-#define ENUF_FFT2_PLANES_B(X) X(6, 10) X(8, 8) X(6, 12) X(8, 10) X(8, 12) X(10, 10) X(9, 12)
-#define ENUF_FFT2_LINES_A(X) X(9, 12) X(10, 12) X(8, 16) X(12, 12) X(10, 16)
-#define ENUF_FFT2_LINES_B(X) X(12, 15) X(12, 16) X(10, 20) X(12, 18)
-#define ENUF_FFT2_LINES_C(X) X(12, 20) X(16, 16) X(16, 18) X(15, 20)
-#define ENUF_FFT2_LINES_D(X) X(16, 20) X(18, 18) X(18, 20) X(20, 20)
 extern template struct Fft2Planes<0, 0>;
 extern template struct Fft2Lines<0, 0>;
-#define ENUF_FFT2_PLANES(X) ENUF_FFT2_PLANES_A(X) ENUF_FFT2_PLANES_B(X)
-#define ENUF_FFT2_LINES(X) ENUF_FFT2_LINES_A(X) ENUF_FFT2_LINES_B(X) ENUF_FFT2_LINES_C(X) ENUF_FFT2_LINES_D(X)
 #define ENUF_EXTERN(a, b) extern template struct Fft2Planes<a, b>;
 ENUF_FFT2_PLANES(ENUF_EXTERN)
 #undef ENUF_EXTERN

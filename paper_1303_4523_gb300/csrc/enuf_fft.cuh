@@ -519,4 +519,28 @@ __host__ __device__ constexpr int fft2_ly(int f1, int f2) {
     return l >= 4 ? l / 4 * 4 : l;
 }
 
+// Lengths with instances of their own: every n <= 112 of two radices (plane
+// passes), every larger one up to 400, and 108 in both forms.
+#define ENUF_FFT2_PLANES_A(X) X(4, 4) X(4, 5) X(4, 6) X(4, 8) X(6, 6) X(5, 8) X(6, 8)
+#define ENUF_FFT2_PLANES_B(X) X(6, 10) X(8, 8) X(6, 12) X(8, 10) X(8, 12) X(10, 10) X(9, 12)
+#define ENUF_FFT2_LINES_A(X) X(9, 12) X(10, 12) X(8, 16) X(12, 12) X(10, 16)
+#define ENUF_FFT2_LINES_B(X) X(12, 15) X(12, 16) X(10, 20) X(12, 18)
+#define ENUF_FFT2_LINES_C(X) X(12, 20) X(16, 16) X(16, 18) X(15, 20)
+#define ENUF_FFT2_LINES_D(X) X(16, 20) X(18, 18) X(18, 20) X(20, 20)
+#define ENUF_FFT2_PLANES(X) ENUF_FFT2_PLANES_A(X) ENUF_FFT2_PLANES_B(X)
+#define ENUF_FFT2_LINES(X) ENUF_FFT2_LINES_A(X) ENUF_FFT2_LINES_B(X) ENUF_FFT2_LINES_C(X) ENUF_FFT2_LINES_D(X)
+
+// body(f1, f2) with the split of fp as constants where the plane passes have
+// kernels of that length, (0, 0) otherwise.
+template <typename Body>
+__device__ __forceinline__ void fft2_by_length(const FftPlanDev& fp, Body body) {
+    switch (32 * fp.f1 + fp.f2) {
+#define ENUF_CASE(a, b) \
+    case 32 * a + b: body(std::integral_constant<int, a>{}, std::integral_constant<int, b>{}); break;
+        ENUF_FFT2_PLANES(ENUF_CASE)
+#undef ENUF_CASE
+        default: body(std::integral_constant<int, 0>{}, std::integral_constant<int, 0>{});
+    }
+}
+
 }  // namespace enuf
