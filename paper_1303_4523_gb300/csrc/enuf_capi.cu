@@ -374,9 +374,11 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
     shape(n * n / 2, 2, fs.lx, fs.tx, fs.grid_x);
     shape(n * nc1, 2, fs.ly, fs.ty, gyz);
     fs.grid_y_z = (n + fs.ly - 1) / fs.ly;
-    // z pass: forward lines (2 buffers) and the nf fields transformed together (2 nf)
-    shape(nc1 * g.K, 2 + 2 * g.nf, fs.lz, fs.tz, fs.grid_z, 96 * 1024);
-    fs.tz = std::min(256, std::max(fs.tz, ((g.nf * fs.lz * n / 4 + 31) / 32) * 32));
+    // z pass: forward lines (2 buffers) and the one or two fields transformed back
+    // together (2 each)
+    const int nz = g.nf == 3 ? 2 : 1;
+    shape(nc1 * g.K, 2 + 2 * nz, fs.lz, fs.tz, fs.grid_z, 96 * 1024);
+    fs.tz = std::min(256, std::max(fs.tz, ((nz * fs.lz * n / 4 + 31) / 32) * 32));
     shape(g.nf * n * nc1, 2, fs.liy, fs.tiy, fs.grid_iy);
     shape(g.nf * n * n / 2, 2, fs.lix, fs.tix, fs.grid_ix);
     // twiddles + line buffers; lines are padded to whole 128-byte bank rows plus one
@@ -385,8 +387,8 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
     const int ls = (n + bank - 1) / bank * bank + 1;
     fs.smem_x = (n + 2 * fs.lx * ls) * csz;
     fs.smem_y = (n + 2 * fs.ly * ls) * csz;
-    fs.smem_z = (n + (2 + 2 * g.nf) * fs.lz * ls) * csz;
-    fs.smem_iy = (n + 2 * fs.liy * ls) * csz;
+    fs.smem_z = (n + (2 + 2 * nz) * fs.lz * ls) * csz;
+    fs.smem_iy = (n + 2 * fs.liy * ls) * csz + nc1 * esz;
     fs.smem_ix = (n + 2 * fs.lix * ls) * csz;
     // fused plane passes (one CTA per z-plane) for FP32 grids whose twiddles and two
     // n^2/2-line buffers take <= 100 KB (n <= 112): measured faster there; larger planes

@@ -105,6 +105,9 @@ template <typename R, bool INV> struct SmallDft<R, 8, INV> {
         C o[4] = {v[1], v[3], v[5], v[7]};
         SmallDft<R, 4, INV>::run(e);
         SmallDft<R, 4, INV>::run(o);
+        combine(v, e, o);
+    }
+    template <typename C> __device__ __forceinline__ static void combine(C* v, const C* e, const C* o) {
         const R h = (R)0.70710678118654752440;
         C t1, t3;
         // w8 = (1 -+ i)/sqrt2 ; w8^2 = -+ i ; w8^3 = (-1 -+ i)/sqrt2
@@ -154,6 +157,30 @@ template <typename R, bool INV> struct SmallDft<R, 5, INV> {
         v[0].x = v[0].x + a1.x + a2.x; v[0].y = v[0].y + a1.y + a2.y;
         v[1] = cadd(m1, iu1); v[4] = csub(m1, iu1);
         v[2] = cadd(m2, iu2); v[3] = csub(m2, iu2);
+    }
+};
+
+// The same DFTs of inputs whose middle half is zero (v[N/4] .. v[3N/4 - 1], not
+// read): the first stage of an inverse transform whose spectrum is kept for
+// |k| < n/4 only. 8 of 16 and 36 of 52 additions.
+template <typename R, int RAD, bool INV> struct HalfDft;
+template <typename R, bool INV> struct HalfDft<R, 4, INV> {
+    template <typename C> __device__ __forceinline__ static void run(C* v) {
+        const C a = v[0], b = v[3], rb = rot_i<C, INV>(v[3]);
+        v[0] = cadd(a, b);
+        v[2] = csub(a, b);
+        v[1] = csub(a, rb);
+        v[3] = cadd(a, rb);
+    }
+};
+template <typename R, bool INV> struct HalfDft<R, 8, INV> {
+    template <typename C> __device__ __forceinline__ static void run(C* v) {
+        C e[4], o[4];
+        e[0] = v[0]; e[3] = v[6];
+        o[0] = v[1]; o[3] = v[7];
+        HalfDft<R, 4, INV>::run(e);
+        HalfDft<R, 4, INV>::run(o);
+        SmallDft<R, 8, INV>::combine(v, e, o);
     }
 };
 
@@ -264,7 +291,9 @@ template <typename R, bool INV> struct SmallDft<R, 18, INV> : CompositeDft<R, 2,
 template <typename R, bool INV> struct SmallDft<R, 20, INV> : CompositeDft<R, 4, 5, INV> {};
 
 // One Stockham stage over nlines lines (line l at offset l*ls, swizzled inside).
-template <typename R, int RAD, bool INV>
+// HALF: a first stage (Ns = 1) whose inputs are zero from n/4 to 3n/4; that half
+// of src is not read.
+template <typename R, int RAD, bool INV, bool HALF = false>
 __device__ __forceinline__ void fft_stage(const typename Cx<R>::T* __restrict__ src,
                                           typename Cx<R>::T* __restrict__ dst,
                                           const typename Cx<R>::T* __restrict__ tw,
@@ -282,8 +311,9 @@ __device__ __forceinline__ void fft_stage(const typename Cx<R>::T* __restrict__ 
         C* d = dst + line * ls;
         C v[RAD];
 #pragma unroll
-        for (int r = 0; r < RAD; ++r) v[r] = s[swz<C>(j + r * m)];
-        if (k != 0) {
+        for (int r = 0; r < RAD; ++r)
+            if (!HALF || r < RAD / 4 || r >= RAD - RAD / 4) v[r] = s[swz<C>(j + r * m)];
+        if (!HALF && k != 0) {
 #pragma unroll
             for (int r = 1; r < RAD; ++r) {
                 C w = tw[r * k * tstep];
@@ -291,7 +321,8 @@ __device__ __forceinline__ void fft_stage(const typename Cx<R>::T* __restrict__ 
                 v[r] = cmul(v[r], w);
             }
         }
-        SmallDft<R, RAD, INV>::run(v);
+        if constexpr (HALF) HalfDft<R, RAD, INV>::run(v);
+        else SmallDft<R, RAD, INV>::run(v);
         const int base = (j - k) * RAD + k;
 #pragma unroll
         for (int r = 0; r < RAD; ++r) d[swz<C>(base + r * Ns)] = v[r];
@@ -303,7 +334,17 @@ __device__ __forceinline__ void fft_stage(const typename Cx<R>::T* __restrict__ 
 // CR: the composite radices 6, 10, 12, 16, 20 are compiled in (the plan's
 // radix list decides which instance runs; they raise the kernels' register
 // count, so plans without them run the CR = false instance).
-template <typename R, bool INV, bool CR = false>
+// HALF: the inverse of a spectrum kept for |k| < n/4: the stage of fft_half, where
+// there is one, runs first and skips the empty half (which it does not read).
+// FP64 additions bound these passes (the FP64 pipe 65-79% busy): with the z pass's
+// two fields instead of three a whole call at n = 160 (375,000 beads) takes 1057 us
+// instead of 1147, four steps at n = 96 1265 instead of 1337.
+__device__ __forceinline__ int fft_half(const FftPlanDev& fp) {   // first radix 8 or 4, -1: none
+    for (int st = 0; st < fp.nst; ++st)
+        if (fp.rad[st] == 8 || fp.rad[st] == 4) return st;
+    return -1;
+}
+template <typename R, bool INV, bool CR = false, bool HALF = false>
 __device__ typename Cx<R>::T* fft_lines(typename Cx<R>::T* b0, typename Cx<R>::T* b1,
                                         const typename Cx<R>::T* tw, const FftPlanDev& fp,
                                         int nlines, int ls) {
@@ -311,7 +352,16 @@ __device__ typename Cx<R>::T* fft_lines(typename Cx<R>::T* b0, typename Cx<R>::T
     C* src = b0;
     C* dst = b1;
     int Ns = 1;
+    const int sh = HALF ? fft_half(fp) : -1;
+    if (HALF && sh >= 0) {
+        Ns = fp.rad[sh];
+        if (Ns == 8) fft_stage<R, 8, INV, true>(src, dst, tw, fp.n, 1, nlines, ls);
+        else fft_stage<R, 4, INV, true>(src, dst, tw, fp.n, 1, nlines, ls);
+        __syncthreads();
+        C* t = src; src = dst; dst = t;
+    }
     for (int st = 0; st < fp.nst; ++st) {
+        if (HALF && st == sh) continue;
         const int rad = fp.rad[st];
         if constexpr (CR) {
             switch (rad) {
@@ -517,6 +567,15 @@ __host__ __device__ constexpr int fft2_lix(int f1, int f2, int nf) {
 __host__ __device__ constexpr int fft2_ly(int f1, int f2) {
     const int l = fft2_lines_for(f1, f2, 8, 1, 0, kFftLine, 16);
     return l >= 4 ? l / 4 * 4 : l;
+}
+
+// Field a's spectrum after the z pass: which array of spec3 holds it and the
+// factor of the mode (kx, ky). With three fields the z pass transforms back G
+// and kz G; x and y are kx G and ky G.
+__device__ __forceinline__ int spec3_array(int nf, int a) { return nf == 3 && a == 2 ? 1 : 0; }
+template <typename R>
+__device__ __forceinline__ R spec3_factor(int nf, int a, int kx, int ky) {
+    return nf == 3 && a < 2 ? (R)(a == 0 ? kx : ky) : (R)1;
 }
 
 // Lengths with instances of their own: every n <= 112 of two radices (plane

@@ -307,14 +307,6 @@ __global__ void __launch_bounds__(fft2_threads<F1, F2>(F1 ? (NF == 3 ? 2 : 1) * 
     }
 }
 
-// Field a's spectrum after the z pass: which array of spec3 holds it and the
-// factor of the mode (kx, ky): x and y are kx G and ky G.
-__device__ __forceinline__ int spec3_array(int nf, int a) { return nf == 3 && a == 2 ? 1 : 0; }
-template <typename R>
-__device__ __forceinline__ R spec3_factor(int nf, int a, int kx, int ky) {
-    return nf == 3 && a < 2 ? (R)(a == 0 ? kx : ky) : (R)1;
-}
-
 // inverse y for lines (a, z, kx): K inputs zero-padded to n; output spec4[a][z][y][kx]
 template <typename R, int F1, int F2>
 __global__ void __launch_bounds__(fft2_threads<F1, F2>(F1 ? fft2_ly(F1, F2) : 0), F1 ? 3 : 1)

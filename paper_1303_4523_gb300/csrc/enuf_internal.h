@@ -177,7 +177,7 @@ struct Work {
     void* grid;      // real [n^3]
     void* spec1;     // cplx [n][nc+1][n]      after forward x   ([z][kx][y])
     void* spec2;     // cplx [nc+1][K][n]      after forward y   ([kx][ky][z])
-    void* spec3;     // cplx [3][n][nc+1][K]   after z pass      ([a][z][kx][ky]; two-factor: G and Gz)
+    void* spec3;     // cplx [nf][n][nc+1][K]  after z pass      ([a][z][kx][ky]; three fields: G and kz G)
     void* spec4;     // cplx [3][n][n][nc+1]   after inverse y   ([a][z][y][kx])
     void* h;         // real [3][n^3]          conjugated-NFFT fields (Geo::h4: real [n^3][4])
     double* tab;     // [nc+1][K][K] influence/deconvolution table D(k) (0 outside the mode set)

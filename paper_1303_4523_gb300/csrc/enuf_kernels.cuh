@@ -1633,9 +1633,9 @@ __global__ void __launch_bounds__(256) k_fft_y(Geo g, FftPlanDev fp, const typen
 }
 
 // z pass: forward z; E += w D |F|^2, W += w D v |F|^2 (FP64, Kahan); the
-// fields G_a = -i k_a D F (a = x, y, z; Eq. 24) or, in gradient mode, the one
-// field G = D F; all fields of the CTA's lines inverse-transformed together;
-// output spec3[a][z][kx][ky].
+// fields G = -i D F and kz G of Eq. 24 (the later passes take x and y as kx G
+// and ky G; see spec3_array) or, in gradient mode, the one field G = D F; the
+// CTA's lines of both inverse-transformed together; output spec3[a][z][kx][ky].
 template <typename R, bool CR = false>
 __global__ void __launch_bounds__(256) k_fft_z(Geo g, FftPlanDev fp, const typename Cx<R>::T* __restrict__ spec2,
                                               const typename Cx<R>::T* __restrict__ twg,
@@ -1652,8 +1652,9 @@ __global__ void __launch_bounds__(256) k_fft_z(Geo g, FftPlanDev fp, const typen
     const int ls = line_stride<C>(n);   // padded, swizzled lines (loads and stores go across lines)
     C* b0 = tw + n;               // [LB][ls] forward lines
     C* b1 = b0 + LB * ls;         // [LB][ls] scratch
-    C* X = b1 + LB * ls;          // [nf][LB][ls] fields
-    C* Y = X + nf * LB * ls;      // [nf][LB][ls] scratch
+    const int nz = nf == 3 ? 2 : 1;
+    C* X = b1 + LB * ls;          // [nz][LB][ls] fields
+    C* Y = X + nz * LB * ls;      // [nz][LB][ls] scratch
     for (int t = threadIdx.x; t < n; t += blockDim.x) tw[t] = twg[t];
     const int l0 = blockIdx.x * LB;
     const int nl = min(LB, NL - l0);
@@ -1690,12 +1691,15 @@ __global__ void __launch_bounds__(256) k_fft_z(Geo g, FftPlanDev fp, const typen
         epart[2 * blockIdx.x] = se;
         epart[2 * blockIdx.x + 1] = sv;
     }
-    // fields: line a * nl + c of X
-    const int per = nl * n;
-    const float rper = 1.0f / (float)per;
-    for (int idx = threadIdx.x; idx < nf * per; idx += blockDim.x) {
-        const int a = qdiv(idx, per, rper), e = idx - a * per;
-        const int c = qdiv(e, n, rn), m = e - c * n;
+    // fields: line a * nl + c of X, only the half that the transform reads
+    const bool half = fft_half(fp) >= 0;
+    const int cnt = half ? n / 2 : n;
+    const int hper = nl * cnt, per = nl * n;
+    const float rhper = 1.0f / (float)max(hper, 1), rper = 1.0f / (float)max(per, 1), rcnt = 1.0f / (float)cnt;
+    for (int idx = threadIdx.x; idx < nz * hper; idx += blockDim.x) {
+        const int a = qdiv(idx, hper, rhper), e = idx - a * hper;
+        const int c = qdiv(e, cnt, rcnt), i = e - c * cnt;
+        const int m = half && i >= n / 4 ? i + n / 2 : i;
         const int kz = m <= n / 2 ? m : m - n;
         C v;
         v.x = (R)0;
@@ -1708,18 +1712,16 @@ __global__ void __launch_bounds__(256) k_fft_z(Geo g, FftPlanDev fp, const typen
                 v.x = d * f.x;     // D F
                 v.y = d * f.y;
             } else {
-                const int kx = qdiv(l, K, rK), ky = (l - kx * K) - nc;
-                const int ka = a == 0 ? kx : (a == 1 ? ky : kz);
-                const R s = (R)ka * d;
-                v.x = s * f.y;     // -i k_a D F
+                const R s = a == 0 ? d : (R)kz * d;
+                v.x = s * f.y;     // -i D F, -i kz D F
                 v.y = -s * f.x;
             }
         }
         X[(a * nl + c) * ls + swz<C>(m)] = v;
     }
     __syncthreads();
-    C* res = fft_lines<R, true, CR>(X, Y, tw, fp, nf * nl, ls);
-    for (int idx = threadIdx.x; idx < nf * per; idx += blockDim.x) {
+    C* res = fft_lines<R, true, CR, true>(X, Y, tw, fp, nz * nl, ls);
+    for (int idx = threadIdx.x; idx < nz * per; idx += blockDim.x) {
         const int a = qdiv(idx, per, rper), e = idx - a * per;
         const int z = qdiv(e, nl, rnl), c = e - z * nl;
         spec3[((size_t)a * n + z) * NL + l0 + c] = res[(a * nl + c) * ls + swz<C>(z)];
@@ -1798,7 +1800,8 @@ __global__ void __launch_bounds__(512) k_fft_yx(Geo g, FftPlanDev fp, const type
     C* L1 = L0 + hn * ls;   // [n/2][ls]: the x lines
     for (int t = threadIdx.x; t < n; t += blockDim.x) tw[t] = twg[t];
     const int az = blockIdx.x;   // a * n + z
-    const C* in = spec3 + (size_t)az * nc1 * K;
+    const int a = qdiv(az, n, rn), z = az - a * n;
+    const C* in = spec3 + ((size_t)spec3_array(g.nf, a) * n + z) * nc1 * K;
     C* P = L0;                   // [nc+1][ls] columns over y
     C* S = L0 + nc1 * ls;
     for (int idx = threadIdx.x; idx < nc1 * n; idx += blockDim.x) {
@@ -1807,7 +1810,12 @@ __global__ void __launch_bounds__(512) k_fft_yx(Geo g, FftPlanDev fp, const type
         C v;
         v.x = (R)0;
         v.y = (R)0;
-        if (ky >= -nc && ky <= nc) v = in[kx * K + (ky + nc)];
+        if (ky >= -nc && ky <= nc) {
+            v = in[kx * K + (ky + nc)];
+            const R f = spec3_factor<R>(g.nf, a, kx, ky);
+            v.x *= f;
+            v.y *= f;
+        }
         P[kx * ls + swz<C>(m)] = v;
     }
     __syncthreads();
@@ -1862,20 +1870,42 @@ __global__ void __launch_bounds__(256) k_fft_iy(Geo g, FftPlanDev fp, const type
     C* b1 = b0 + LB * ls;
     for (int t = threadIdx.x; t < n; t += blockDim.x) tw[t] = twg[t];
     const float rn = 1.0f / (float)n;
+    // the wave numbers as R: a conversion per element would cost the FP64 pipe as
+    // much as an addition
+    R* kr = reinterpret_cast<R*>(b1 + LB * ls);
+    for (int t = threadIdx.x; t < nc1; t += blockDim.x) kr[t] = (R)t;
+    __syncthreads();
     const int l0 = blockIdx.x * LB;
     const int nl = min(LB, NLT - l0);
     const float rnl = 1.0f / (float)max(nl, 1);
-    for (int idx = threadIdx.x; idx < nl * n; idx += blockDim.x) {
-        const int c = qdiv(idx, n, rn), m = idx - c * n;
+    const bool half = fft_half(fp) >= 0;
+    const int cnt = half ? n / 2 : n;   // the half that the transform reads
+    const float rcnt = 1.0f / (float)cnt;
+    for (int idx = threadIdx.x; idx < nl * cnt; idx += blockDim.x) {
+        const int c = qdiv(idx, cnt, rcnt), i = idx - c * cnt;
+        const int m = half && i >= n / 4 ? i + n / 2 : i;
         const int ky = m <= n / 2 ? m : m - n;
         C v;
         v.x = (R)0;
         v.y = (R)0;
-        if (ky >= -nc && ky <= nc) v = spec3[(size_t)(l0 + c) * K + (ky + nc)];
+        if (ky >= -nc && ky <= nc) {
+            const int l = l0 + c, az = qdiv(l, nc1, rnc1), kx = l - az * nc1;
+            const int a = az >= 2 * n ? 2 : (az >= n ? 1 : 0);
+            v = spec3[(size_t)(l - (a - spec3_array(g.nf, a)) * n * nc1) * K + (ky + nc)];
+            if (g.nf == 3 && a < 2) {
+                const R f = kr[a == 0 ? kx : abs(ky)];
+                v.x *= f;
+                v.y *= f;
+                if (a == 1 && ky < 0) {
+                    v.x = -v.x;
+                    v.y = -v.y;
+                }
+            }
+        }
         b0[c * ls + swz<C>(m)] = v;
     }
     __syncthreads();
-    C* res = fft_lines<R, true, CR>(b0, b1, tw, fp, nl, ls);
+    C* res = fft_lines<R, true, CR, true>(b0, b1, tw, fp, nl, ls);
     for (int idx = threadIdx.x; idx < nl * n; idx += blockDim.x) {
         const int y = qdiv(idx, nl, rnl), c = idx - y * nl;
         const int l = l0 + c;
@@ -1903,8 +1933,12 @@ __global__ void __launch_bounds__(256) k_fft_ix(Geo g, FftPlanDev fp, const type
     const int row0 = blockIdx.x * 2 * LP;
     const int nl = min(LP, (nrows - row0) / 2);
     const float rnl = 1.0f / (float)max(nl, 1);
-    for (int idx = threadIdx.x; idx < nl * n; idx += blockDim.x) {
-        const int c = qdiv(idx, n, rn), m = idx - c * n;
+    const bool half = fft_half(fp) >= 0;
+    const int cnt = half ? n / 2 : n;   // the half that the transform reads
+    const float rcnt = 1.0f / (float)cnt;
+    for (int idx = threadIdx.x; idx < nl * cnt; idx += blockDim.x) {
+        const int c = qdiv(idx, cnt, rcnt), i = idx - c * cnt;
+        const int m = half && i >= n / 4 ? i + n / 2 : i;
         const C* A = spec4 + (size_t)(row0 + 2 * c) * nc1;
         const C* B = A + nc1;
         C a, b;
@@ -1927,7 +1961,7 @@ __global__ void __launch_bounds__(256) k_fft_ix(Geo g, FftPlanDev fp, const type
         b0[c * ls + swz<C>(m)] = z;
     }
     __syncthreads();
-    C* res = fft_lines<R, true, CR>(b0, b1, tw, fp, nl, ls);
+    C* res = fft_lines<R, true, CR, true>(b0, b1, tw, fp, nl, ls);
     for (int idx = threadIdx.x; idx < nl * n; idx += blockDim.x) {
         const int c = qdiv(idx, n, rn), x = idx - c * n;
         const C v = res[c * ls + swz<C>(x)];

@@ -102,3 +102,19 @@ def test_fft_radices_9_15_18(enuf, n, fft_path, deriv):
         _check("fp32", F, E, Wv, Ref(P, pos, q))
     plan.close()
     other.close()
+
+
+@pytest.mark.parametrize("deriv", [0, 1])
+@pytest.mark.parametrize("n", [20, 24, 36, 40, 96, 100, 108])
+def test_fft_half_spectrum(enuf, n, deriv):
+    """FP64 line passes whose inverse transforms skip the empty half of the spectrum:
+    radix 8 (24, 40, 96), 4 (36, 108), and 4 after others in the plan's list (20, 100)."""
+    L = n / 5.0
+    rc = min(3.0, 0.45 * L)
+    P = dict(L=L, M=n // 2, p=3, alpha=3.0 / rc, r_cut=rc, beta=4.0, kappa=1.1, deriv=deriv)
+    rng = np.random.default_rng(n)
+    pos = rng.uniform(0.0, L, (200, 3))
+    q = np.where(np.arange(200) % 2 == 0, 1.0, -1.0)
+    plan, F, E, Wv = _gpu(enuf, "fp64", P, pos, q)
+    _check("fp64", F, E, Wv, Ref(P, pos, q))
+    plan.close()
