@@ -97,8 +97,8 @@ struct RealArgs {
     double* rpart;
     int nblk;
 };
-template <typename R>
-__global__ void __launch_bounds__(kRealThreads) kb_real(const RealArgs<R>* __restrict__ tab, const int* __restrict__ cmap) {
+template <typename R, int CTAS>
+__global__ void __launch_bounds__(kRealThreads, CTAS) kb_real(const RealArgs<R>* __restrict__ tab, const int* __restrict__ cmap) {
     pdl_enter();
     const int m = cmap[blockIdx.x];
     const RealArgs<R>& a = tab[m >> kBatchShift];
@@ -207,8 +207,9 @@ struct GatherArgs {
     int nblk;
 };
 // PT: the tap count 2p when every system of the batch has the same window, else 0
+// (above 8 taps four CTAs per SM would spill 120 to 168 bytes)
 template <typename R, int PT>
-__global__ void __launch_bounds__(kGatherThreads, 4) kb_gather(const GatherArgs<R>* __restrict__ tab,
+__global__ void __launch_bounds__(kGatherThreads, PT > 8 ? 2 : 4) kb_gather(const GatherArgs<R>* __restrict__ tab,
                                                             const int* __restrict__ cmap) {
     pdl_enter();
     const int m = cmap[blockIdx.x];

@@ -19,9 +19,11 @@ inline void append_blocks(std::vector<int>& cmap, int sys, int nblk) {
 // Blocks of one system of a batch in its bead loops. The batch fills the chip,
 // so a system takes few blocks and strides over its beads: real space N / 1024
 // blocks and as many lanes as its beads need (64 systems: 1179 us against 1219
-// with N / 512), gather N / 512 (1171 against 1219 with N / 64), spreading as
-// the gather.
+// with N / 512), gather N / 512 (1171 against 1219 with N / 64), spreading
+// N / 256 (its launches, one per tile edge, follow each other: 40 systems of
+// 3000 to 20,000 beads 345 -> 333 us against N / 512 with the next rule).
 inline int batch_real_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_real, (x.N + 1023) / 1024)); }
+inline int batch_spread_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_gather, (x.N + 255) / 256)); }
 inline int batch_gather_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_gather, (x.N + 511) / 512)); }
 
 // Window-weight blocks of one system: a thread per (bead, dimension) for a
@@ -120,7 +122,7 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
             for (int s = 0; s < nsys; ++s) {
                 const BatchSys& x = sys[s];
                 if (x.g.T != kT[ti]) continue;
-                const int row = (int)a.size(), nb = batch_gather_blocks(x);
+                const int row = (int)a.size(), nb = batch_spread_blocks(x);
                 taps = taps < 0 || taps == 2 * x.g.p ? 2 * x.g.p : 0;
                 a.push_back(SpreadArgs<R>{x.g, x.w.tstart, static_cast<const V*>(x.w.sq), x.w.sb,
                                           static_cast<const R*>(x.w.wb), static_cast<R*>(x.w.grid), nb});
@@ -191,7 +193,7 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
 
 template <typename R>
 cudaError_t configure_batch(int max_smem) {
-    return first_error({set_smem((const void*)kb_real<R>, max_smem), set_smem((const void*)kb_fft_xy<R>, max_smem),
+    return first_error({set_smem((const void*)kb_real<R, 2>, max_smem), set_smem((const void*)kb_real<R, 4>, max_smem), set_smem((const void*)kb_fft_xy<R>, max_smem),
                         set_smem((const void*)kb_fft_z<R>, max_smem),
                         set_smem((const void*)kb_fft_yx<R>, max_smem)});
 }
@@ -208,7 +210,9 @@ cudaError_t batch_enqueue(const BatchLaunch& L, cudaStream_t s0, cudaStream_t s1
     run(true, true, kb_bin_weights<R>, L.bin_weights, (const BinWeightsArgs<R>*)L.bin_weights.tab, s0);
     cudaEventRecord(evFork, s0);
     cudaStreamWaitEvent(s1, evFork, 0);
-    run(false, false, kb_real<R>, L.real, (const RealArgs<R>*)L.real.tab, s1);
+    // four CTAs per SM (64 registers, a small spill) where the blocks fill more than
+    // two (103 registers): 64 systems 946 -> 909 us; 16 systems 214, with four 245
+    run(false, false, L.real.blocks > 2 * kSMs ? kb_real<R, 4> : kb_real<R, 2>, L.real, (const RealArgs<R>*)L.real.tab, s1);
     cudaEventRecord(evJoin, s1);
     for (int i = 0; i < L.nspread; ++i) {
         const BatchKernel& k = L.spread[i];

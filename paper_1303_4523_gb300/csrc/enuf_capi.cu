@@ -23,7 +23,6 @@ namespace {
 constexpr int kMaxTiles = 32768;      // shared-memory histogram limit (128 KB)
 constexpr int kMaxBeads = 1 << 29;    // the kernels index per-bead components as int (3 i + 2, 4 i + 3)
 constexpr int kMaxSmem = 200 * 1024;  // dynamic shared memory the kernels may request
-constexpr int kSMs = 152;
 
 // Kernel attributes (dynamic shared-memory opt-in) belong to the device that
 // was current when they were set: configured once per device and precision.
@@ -459,9 +458,9 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
         // the five passes leave three fields interleaved
         g.h4 = !fs.fused && g.nf == 3 ? 1 : 0;
     }
-    // spreading form (FP32): bricks of whole x rows fused with the x pass where the
-    // two-factor five-pass FFT runs and the brick fits; footprint bricks into the
-    // grid otherwise from n = 128 on; the tile form below
+    // spreading form: reductions by default (k_spread_red); on request (FP32) tiles,
+    // footprint bricks, bricks of whole x rows fused with the x pass where the
+    // two-factor five-pass FFT runs and the brick fits, or regions
     if (P.spread < 0 || P.spread > 4) return fail(plan, ENUF_ERR_INVALID, "spread must be 0..4");
     if (P.pairs < 0 || P.pairs > 2) return fail(plan, ENUF_ERR_INVALID, "pairs must be 0, 1 or 2");
     fs.spread = 1;

@@ -121,6 +121,7 @@ __host__ __device__ constexpr int brick_smem(int T, int BX, int fx_bytes) {
 // Preferred shared-memory split of the two-factor FFT kernels (percent): the plane
 // passes share SMs with the pair kernels, the persistent line passes want three
 // CTAs of 72 KB.
+constexpr int kSMs = 152;
 constexpr int kCarvePlanes = 60, kCarveLines = 100;
 
 // Row length of the real-space kernel table (16-byte aligned rows).
