@@ -119,8 +119,9 @@ typedef struct {
                          cell list (before the charged-bead binning is done), then the
                          real-space pairs; 2 = one launch whose blocks take either role,
                          after both cell structures exist. Automatic (0): 2 in FP32, 1 in
-                         FP64 (measured at the 81000-bead polyelectrolyte, interleaved
-                         steps: FP32 131.0 against 139.4 us, FP64 449.0 against 453.4 us).
+                         FP64 (measured at the 81000-bead polyelectrolyte: FP32 88
+                         against 108 us a step; FP64 453.4 against 449.0 us with the
+                         pair kernels before the present ones).
                          Same result to rounding. */
 } enuf_params;
 
@@ -213,7 +214,7 @@ enuf_status enuf_debug_buffer(enuf_plan_t plan, int which, void* host, size_t by
  * on, the two branches of an evaluation or step (binning -> spreading -> FFT,
  * and the real-space / DPD pairs) run one after the other, so each stage's
  * events time its kernels alone. Stages: */
-enum { ENUF_STAGE_BIN = 0,      /* charged-bead binning (3 kernels) */
+enum { ENUF_STAGE_BIN = 0,      /* charged-bead binning (2 or 3 kernels) */
        ENUF_STAGE_SPREAD = 1,   /* spreading kernel */
        ENUF_STAGE_FFT = 2,      /* the five FFT passes incl. the fused convolution */
        ENUF_STAGE_GATHER = 3,   /* gather kernel */
@@ -324,8 +325,9 @@ typedef struct enuf_batch_s* enuf_batch_t;
 /* One plan per system (params[s], capacity n[s]); all systems share the
  * given stream and are evaluated by one captured CUDA graph.
  * When every system is FP32 and its plan runs the fused-plane two-factor
- * FFT, the column spreading form and the one-kernel binning offsets (the
- * defaults for grids up to n = 112 of n = f1 f2), the graph is one launch
+ * FFT, a tile edge of the column form (spread 0 or 1; the batch spreads by
+ * reductions) and binning offsets formed in the scatter kernel (the defaults
+ * for grids up to n = 112 of n = f1 f2), the graph is one launch
  * sequence for all systems: each kernel of the evaluation (binning, window
  * weights, real space, spreading -- one launch per tile edge present --,
  * the three FFT passes, gather) is launched once over the concatenated grids
@@ -367,8 +369,8 @@ void enuf_batch_destroy(enuf_batch_t batch);
  *   grid   : device real[n_g^3] (n_g = sigma_s * M), OVERWRITTEN,
  *            index (z * n_g + y) * n_g + x
  *   cuda_stream : cudaStream_t to enqueue on (NULL: the legacy default stream)
- * One 16-byte word of the scratch must start at zero, the binning's arrival
- * counter: each call clears it with a memset on cuda_stream before the
+ * The binning's arrival word and tile counters in the scratch must start at
+ * zero: each call clears them with a memset on cuda_stream before the
  * binning (this allocates nothing); every other scratch word is written by
  * the call before it is read. Returns after enqueueing.
  * Limits and rules:

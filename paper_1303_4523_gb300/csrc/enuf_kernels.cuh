@@ -3,11 +3,11 @@
 // sums are always reduced in double.
 //
 // Stages (Table 2 step 4, Eq. 14-25 of the paper):
-//   bin      : charged beads -> tile bins of the oversampled grid (no global atomics)
-//   spread   : transposed NFFT part 1, output-stationary shared-memory tiles
+//   bin      : charged beads -> tile bins of the oversampled grid
+//   spread   : transposed NFFT part 1, by global reductions (or in shared-memory tiles)
 //   fft_x/y  : forward R2C/C2C passes, pruned to |k_t| <= n_c
 //   fft_z    : forward z, influence x deconvolution multiply, FP64 energy and
-//              virial, -i k_a D F for a = x, y, z, inverse z (conjugated NFFT part 1)
+//              virial, -i D F and kz times it, inverse z (conjugated NFFT part 1)
 //   fft_iy/ix: inverse passes to three real fields
 //   gather   : conjugated NFFT part 2, warp per bead, F_i += kappa 2 q_i/L^2 * sum psi h
 //   real     : erfc Ewald + Slater correction pairs (Eq. 31, 27-28) on the tile bins
