@@ -128,13 +128,6 @@ __device__ __forceinline__ double wrap_pos(double x, double L) {
     return w;
 }
 
-template <typename R>
-__device__ __forceinline__ double wrap_to_real(R x, double L) {
-    double w = wrap_pos((double)x, L);
-    if (sizeof(R) == 4) w = (double)__double2float_rn(w);
-    return w;
-}
-
 // Wrapped position in the working precision. Inside [0, L) the value is kept
 // as is (decided in float for float: x <= xmaxf, the largest float below L);
 // outside it goes through the FP64 wrap.
