@@ -128,9 +128,10 @@ __device__ __forceinline__ double wrap_pos(double x, double L) {
     return w;
 }
 
-// Wrapped position in the working precision. Inside [0, L) the value is kept
-// as is (decided in float for float: x <= xmaxf, the largest float below L);
-// outside it goes through the FP64 wrap.
+// Wrapped position in the working precision, in [0, L). Inside [0, L) the value
+// is kept as is (decided in float for float: x <= xmaxf, the largest float
+// below L). FP32: a value within half a unit of L, which only float(L) >= L could
+// hold, is 0, the same point of the periodic box to within its rounding.
 // FP32: x - L q in float arithmetic with error terms, L = Lhi + Llo: the product
 // q Lhi and the difference x - fl(q Lhi) are taken with their exact rounding
 // errors (fused multiply-add; two-sum), which are added back with q Llo before
@@ -149,25 +150,34 @@ __device__ __forceinline__ float wrap_diff(float x, float q, float Lhi, float Ll
 __device__ __forceinline__ float wrap_r(float x, double L, float xmaxf, float Lhi, float Llo) {
     if (x >= 0.0f && x <= xmaxf) return x;
     float q = floorf(__fdiv_rn(x, Lhi));
-    if (!(fabsf(q) < 1048576.0f)) return __double2float_rn(wrap_pos((double)x, L));
-    float w = wrap_diff(x, q, Lhi, Llo);
-    if (w < 0.0f) {
-        q -= 1.0f;
+    float w;
+    if (!(fabsf(q) < 1048576.0f)) {
+        w = __double2float_rn(wrap_pos((double)x, L));
+    } else {
         w = wrap_diff(x, q, Lhi, Llo);
-    } else if (w > xmaxf) {
-        q += 1.0f;
-        const float v = wrap_diff(x, q, Lhi, Llo);
-        if (v >= 0.0f) w = v;   // else x - L (q - 1) lies within half a unit of L: kept as it rounds
+        if (w < 0.0f) {
+            q -= 1.0f;
+            w = wrap_diff(x, q, Lhi, Llo);
+        } else if (w > xmaxf) {
+            q += 1.0f;
+            w = wrap_diff(x, q, Lhi, Llo);
+        }
     }
-    return w < 0.0f ? 0.0f : w;
+    return w < 0.0f || w > xmaxf ? 0.0f : w;   // NaN is kept
 }
 __device__ __forceinline__ double wrap_r(double x, double L, float, float, float) { return wrap_pos(x, L); }
 
 // Grid coordinate u = x_w * (n/L) in [0, n): one FP64 product and one floor
-// (n/L formed once on the host), u >= n wraps to 0.
-__device__ __forceinline__ void grid_coord(double xw, double ratio, int n, int& base, double& frac) {
+// (n/L formed once on the host). Where the product rounds to n, u and the
+// coordinate itself become 0: a bead is stored with the coordinate that its
+// tile (its grid base) holds, because the real-space sweep takes the image
+// shift of a run of candidates from the tiles.
+__device__ __forceinline__ void grid_coord(double& xw, double ratio, int n, int& base, double& frac) {
     double u = __dmul_rn(xw, ratio);
-    if (u >= (double)n) u = __dsub_rn(u, (double)n);
+    if (u >= (double)n) {
+        u = __dsub_rn(u, (double)n);
+        xw = 0.0;
+    }
     const double bb = floor(u);
     base = (int)bb;
     frac = __dsub_rn(u, bb);
@@ -176,24 +186,26 @@ __device__ __forceinline__ void grid_coord(double xw, double ratio, int n, int& 
 // FP32 path: the same floor decided in float on a compensated product. With
 // n/L = rhi + rlo (two floats), p = fl(x rhi) and t = fl(x rlo + (x rhi - p))
 // represent u = p + t to ~1e-13 relative; floor(u) = floor(p), less one when
-// p is an integer and t < 0.
-__device__ __forceinline__ void grid_coord_f(float x, float rhi, float rlo, int n, int& base, float& frac) {
+// p is an integer and t < 0 (u just below n: base n - 1, the coordinate stays).
+__device__ __forceinline__ void grid_coord_f(float& x, float rhi, float rlo, int n, int& base, float& frac) {
     float p = __fmul_rn(x, rhi);
     const float e = __fmaf_rn(x, rhi, -p);
     const float t = __fmaf_rn(x, rlo, e);
-    if (p >= (float)n) p = __fsub_rn(p, (float)n);
+    const bool over = p >= (float)n;
+    if (over) p = __fsub_rn(p, (float)n);
     float b = floorf(p);
     if (p == b && t < 0.0f) b = __fsub_rn(b, 1.0f);
     frac = __fadd_rn(__fsub_rn(p, b), t);
     if (b < 0.0f) b = __fadd_rn(b, (float)n);
+    else if (over) x = 0.0f;
     base = (int)b;
 }
 
 // Grid base and fraction in the working precision.
-__device__ __forceinline__ void grid_coord_r(float xw, const Geo& g, int& base, float& frac) {
+__device__ __forceinline__ void grid_coord_r(float& xw, const Geo& g, int& base, float& frac) {
     grid_coord_f(xw, g.rhi, g.rlo, g.n, base, frac);
 }
-__device__ __forceinline__ void grid_coord_r(double xw, const Geo& g, int& base, double& frac) {
+__device__ __forceinline__ void grid_coord_r(double& xw, const Geo& g, int& base, double& frac) {
     grid_coord(xw, g.ratio, g.n, base, frac);
 }
 
