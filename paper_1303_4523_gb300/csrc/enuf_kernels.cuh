@@ -104,9 +104,10 @@ __device__ __forceinline__ double r_rsqrt(double x) {
 }
 
 // ---------------------------------------------------------------------------
-// Coordinates. Wrapping and grid coordinates are computed in double with the
-// exact operation sequence of the definition (no fused multiply-add), so the
-// integer decisions (grid base, tile, cell) are reproducible.
+// Coordinates. FP64 wraps and grid coordinates follow the exact operation
+// sequence of the definition (no fused multiply-add), FP32 ones are formed in
+// float with error terms, so the integer decisions (grid base, tile, cell) are
+// reproducible.
 // ---------------------------------------------------------------------------
 // q = floor(x / L) comes from a float quotient (off by at most one for
 // |x| < 2^20 L) corrected in double until 0 <= x - L q < L: the same q and w
@@ -135,10 +136,13 @@ __device__ __forceinline__ double wrap_pos(double x, double L) {
 // FP32: x - L q in float arithmetic with error terms, L = Lhi + Llo: the product
 // q Lhi and the difference x - fl(q Lhi) are taken with their exact rounding
 // errors (fused multiply-add; two-sum), which are added back with q Llo before
-// the one rounding that counts. The same value as the FP64 wrap rounded to
-// float but for ties, without its ~8 FP64 instructions per coordinate (16
-// cycles of the SM each; DPD positions drift out of the box, so nearly every
-// warp wraps some bead). Beyond 2^20 boxes the FP64 wrap is taken.
+// the one rounding that counts. The terms added back are below 2^-22 |x| and
+// carry an error below 2^-45 |x|, so a result of at least 2^-16 |x| is the FP64
+// wrap rounded to float but within 1/32 unit of a tie; a smaller one, one at a
+// face and one whose q is off by one take the FP64 wrap. That costs ~8 FP64
+// instructions per coordinate (16 cycles of the SM each), and DPD positions
+// drift out of the box, so nearly every warp wraps some bead, but a bead k boxes
+// away takes it once in 65536 / k times only.
 __device__ __forceinline__ float wrap_diff(float x, float q, float Lhi, float Llo) {
     const float p = __fmul_rn(q, Lhi);
     const float pe = __fmaf_rn(q, Lhi, -p);          // q Lhi = p + pe
@@ -149,21 +153,10 @@ __device__ __forceinline__ float wrap_diff(float x, float q, float Lhi, float Ll
 }
 __device__ __forceinline__ float wrap_r(float x, double L, float xmaxf, float Lhi, float Llo) {
     if (x >= 0.0f && x <= xmaxf) return x;
-    float q = floorf(__fdiv_rn(x, Lhi));
-    float w;
-    if (!(fabsf(q) < 1048576.0f)) {
-        w = __double2float_rn(wrap_pos((double)x, L));
-    } else {
-        w = wrap_diff(x, q, Lhi, Llo);
-        if (w < 0.0f) {
-            q -= 1.0f;
-            w = wrap_diff(x, q, Lhi, Llo);
-        } else if (w > xmaxf) {
-            q += 1.0f;
-            w = wrap_diff(x, q, Lhi, Llo);
-        }
-    }
-    return w < 0.0f || w > xmaxf ? 0.0f : w;   // NaN is kept
+    const float w = wrap_diff(x, floorf(__fdiv_rn(x, Lhi)), Lhi, Llo);
+    if (w >= fabsf(x) * 0x1p-16f && w < xmaxf) return w;
+    const float v = __double2float_rn(wrap_pos((double)x, L));
+    return v > xmaxf ? 0.0f : v;   // NaN is kept
 }
 __device__ __forceinline__ double wrap_r(double x, double L, float, float, float) { return wrap_pos(x, L); }
 
