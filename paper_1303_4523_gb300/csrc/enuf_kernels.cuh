@@ -2601,6 +2601,15 @@ __global__ void __launch_bounds__(kRealThreads, sizeof(R) == 4 ? 4 : 2) k_real(G
 // ---------------------------------------------------------------------------
 // Cells of edge L/ncd > 1 (the plan keeps a relative margin so that rounding
 // of x * ncd/L cannot separate two beads closer than 1 by two cells).
+// The cell of a wrapped coordinate, for the cell list and for the pair sweep that
+// reads it: always inside the list (a coordinate that is not a number converts
+// to 0 from float but to the smallest int from double).
+template <typename R>
+__device__ __forceinline__ int cell_of(R xw, R rinv, int ncd) {
+    const int c = (int)(xw * rinv);
+    return c < 0 ? 0 : (c >= ncd ? ncd - 1 : c);
+}
+
 template <typename R>
 __global__ void k_cell_count(int N, int ncd, double L, R rinv, float xmaxf, float Lhi, float Llo,
                              const R* __restrict__ pos,
@@ -2613,8 +2622,7 @@ __global__ void k_cell_count(int N, int ncd, double L, R rinv, float xmaxf, floa
         int c[3];
 #pragma unroll
         for (int t = 0; t < 3; ++t) {
-            int v = (int)(wrap_r(pos[3 * i + t], L, xmaxf, Lhi, Llo) * rinv);
-            c[t] = v < 0 ? 0 : (v >= ncd ? ncd - 1 : v);
+            c[t] = cell_of(wrap_r(pos[3 * i + t], L, xmaxf, Lhi, Llo), rinv, ncd);
         }
         const int cell = (c[2] * ncd + c[1]) * ncd + c[0];
         ckey[i] = cell;
@@ -2875,9 +2883,9 @@ __device__ __forceinline__ void k_dpd_body(const DpdDev& d, const typename V4<R>
             if constexpr (!F64) vi = sv[s];
             const V pw = sp[s];   // the cell as k_cell_count decided it, in the working precision
             const R ri = dpd_cinv(d, (R)0);
-            cx = min((int)(pw.x * ri), ncd - 1);
-            cy = min((int)(pw.y * ri), ncd - 1);
-            cz = min((int)(pw.z * ri), ncd - 1);
+            cx = cell_of(pw.x, ri, ncd);
+            cy = cell_of(pw.y, ri, ncd);
+            cz = cell_of(pw.z, ri, ncd);
         }
         float fx = 0.f, fy = 0.f, fz = 0.f;
         // the half shell's rows (uniform over the warp), each as its run inside the box

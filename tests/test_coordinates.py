@@ -32,6 +32,12 @@ extern "C" void wrap32(int n, const float* x, double L, float xmaxf, float Lhi, 
         w64[i] = wrap_pos((double)x[i], L);
     }
 }
+extern "C" void cells(int n, const double* x, double rinv, int ncd, int* c64, int* c32) {
+    for (int i = 0; i < n; ++i) {
+        c64[i] = cell_of(x[i], rinv, ncd);
+        c32[i] = cell_of((float)x[i], (float)rinv, ncd);
+    }
+}
 """
 
 
@@ -39,7 +45,7 @@ def _functions(names):
     src = open(SRC).read()
     out = []
     for name in names:
-        found = re.findall(r"^__device__ __forceinline__ \w+ " + name + r"\([^;{]*\{(?:[^\n]*\}$|.*?^\})", src, re.M | re.S)
+        found = re.findall(r"^(?:template <typename R>\n)?__device__ __forceinline__ \w+ " + name + r"\([^;{]*\{(?:[^\n]*\}$|.*?^\})", src, re.M | re.S)
         assert found, name
         out += found
     return "\n".join(out)
@@ -48,7 +54,7 @@ def _functions(names):
 @pytest.fixture(scope="module")
 def host(tmp_path_factory):
     d = tmp_path_factory.mktemp("coords")
-    (d / "c.cpp").write_text(PRELUDE + _functions(["wrap_pos", "wrap_diff", "wrap_r"]) + DRIVER)
+    (d / "c.cpp").write_text(PRELUDE + _functions(["wrap_pos", "wrap_diff", "wrap_r", "cell_of"]) + DRIVER)
     so = str(d / "c.so")
     subprocess.run(["g++", "-std=c++17", "-O1", "-ffp-contract=off", "-shared", "-fPIC", "-o", so, str(d / "c.cpp")],
                    check=True)
@@ -88,3 +94,12 @@ def test_float_wrap_is_the_double_wrap_rounded(host, L):
     err = np.abs(w[~top] - w64[~top])
     bound = np.spacing(w[~top]).astype(np.float64) * (0.5 + 1.0 / 32)
     assert not np.any(err > bound)
+
+
+def test_cells_lie_in_the_list(host):
+    """The cell of every coordinate, numbers or not, is one of the list's."""
+    x = np.array([0.0, 4.999999999999999, 5.0, 30.0, np.nextafter(30.0, 0.0), np.nan, np.inf, -np.inf, -1e-300, 1e300])
+    c64, c32 = np.empty(x.size, np.int32), np.empty(x.size, np.int32)
+    host.cells(x.size, _ptr(x), ctypes.c_double(29.0 / 30.0), 29, _ptr(c64), _ptr(c32))
+    for c in (c64, c32):
+        assert np.all((c >= 0) & (c < 29)) and list(c[[0, 3]]) == [0, 28]
