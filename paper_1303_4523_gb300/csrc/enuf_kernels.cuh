@@ -172,7 +172,7 @@ __device__ __forceinline__ void grid_coord(double& xw, double ratio, int n, int&
         xw = 0.0;
     }
     const double bb = floor(u);
-    base = (int)bb;
+    base = max((int)bb, 0);   // not a number converts to the smallest int: base 0, the fraction stays
     frac = __dsub_rn(u, bb);
 }
 

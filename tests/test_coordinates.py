@@ -23,6 +23,7 @@ static inline float __fmaf_rn(float a, float b, float c) { return fmaf(a, b, c);
 static inline double __dmul_rn(double a, double b) { return a * b; }
 static inline double __dsub_rn(double a, double b) { return a - b; }
 static inline float __double2float_rn(double a) { return (float)a; }
+static inline int max(int a, int b) { return a > b ? a : b; }
 """
 
 DRIVER = """
@@ -31,6 +32,9 @@ extern "C" void wrap32(int n, const float* x, double L, float xmaxf, float Lhi, 
         w[i] = wrap_r(x[i], L, xmaxf, Lhi, Llo);
         w64[i] = wrap_pos((double)x[i], L);
     }
+}
+extern "C" void grid64(int n, double* x, double ratio, int ng, int* base, double* frac) {
+    for (int i = 0; i < n; ++i) grid_coord(x[i], ratio, ng, base[i], frac[i]);
 }
 extern "C" void cells(int n, const double* x, double rinv, int ncd, int* c64, int* c32) {
     for (int i = 0; i < n; ++i) {
@@ -54,7 +58,7 @@ def _functions(names):
 @pytest.fixture(scope="module")
 def host(tmp_path_factory):
     d = tmp_path_factory.mktemp("coords")
-    (d / "c.cpp").write_text(PRELUDE + _functions(["wrap_pos", "wrap_diff", "wrap_r", "cell_of"]) + DRIVER)
+    (d / "c.cpp").write_text(PRELUDE + _functions(["wrap_pos", "wrap_diff", "wrap_r", "grid_coord", "cell_of"]) + DRIVER)
     so = str(d / "c.so")
     subprocess.run(["g++", "-std=c++17", "-O1", "-ffp-contract=off", "-shared", "-fPIC", "-o", so, str(d / "c.cpp")],
                    check=True)
@@ -103,3 +107,16 @@ def test_cells_lie_in_the_list(host):
     host.cells(x.size, _ptr(x), ctypes.c_double(29.0 / 30.0), 29, _ptr(c64), _ptr(c32))
     for c in (c64, c32):
         assert np.all((c >= 0) & (c < 29)) and list(c[[0, 3]]) == [0, 28]
+
+
+def test_grid_base_lies_in_the_grid(host):
+    """FP64 grid base and fraction: inside the grid for every wrapped coordinate and for
+    what is not a number (whose fraction is none either); a coordinate whose product
+    with n/L rounds to n is stored as 0 with base 0."""
+    L, n = 30.0, 96
+    x = np.array([0.0, 1.0, np.nextafter(L, 0.0), np.nan, 29.9, 1e-300])
+    assert x[2] * (n / L) >= n
+    base, frac = np.empty(x.size, np.int32), np.empty(x.size)
+    host.grid64(x.size, _ptr(x), ctypes.c_double(n / L), n, _ptr(base), _ptr(frac))
+    assert list(base) == [0, 3, 0, 0, 95, 0] and x[2] == 0.0 and frac[2] == 0.0
+    assert np.isnan(x[3]) and np.isnan(frac[3]) and np.all((frac[[0, 1, 4, 5]] >= 0) & (frac[[0, 1, 4, 5]] < 1))

@@ -35,3 +35,29 @@ def test_dpd_forces_beside_a_lost_bead(enuf, prec, tol, pairs, bad):
     assert not np.isfinite(p[lost]).all() and np.all(np.isfinite(F[keep]))
     sysm.close()
     plan.close()
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-11), ("fp32", 1e-5)])
+def test_charged_bead_without_a_position(enuf, prec, tol):
+    """A charged bead at NaN makes the reciprocal part of the call NaN (its window has
+    no weights) and nothing else: no error, and the next call on the same plan, with
+    numbers, is the oracle's."""
+    s = W.electrolyte_small("bench")
+    P = dict(L=s.L, M=s.M, **s.params)
+    dt = torch.float32 if prec == "fp32" else torch.float64
+    pos, _, q = _prep(prec, s)
+    charged = np.flatnonzero(q != 0)
+    plan = enuf.Plan(enuf.make_params(prec=prec, **P), s.N)
+    tq = torch.tensor(q, dtype=dt, device="cuda")
+    for bad in (np.nan, np.inf, -np.inf):
+        x = pos.copy()
+        x[charged[3]] = [bad, bad, 1.0]
+        F = torch.empty((s.N, 3), dtype=dt, device="cuda")
+        E, _ = plan.energy_forces(torch.tensor(x, dtype=dt, device="cuda"), tq, F)
+        assert np.isnan(E[1]) and np.isfinite(E[0]) and bool((F[tq == 0] == 0).all())
+    E, _ = plan.energy_forces(torch.tensor(pos, dtype=dt, device="cuda"), tq, F)
+    Fr, Er = orc.real_space(orc.EwaldParams(**P), pos, q)
+    Fk, Ek, _, _ = orc.recip_enuf(orc.EwaldParams(**P), pos, q)
+    assert _rel(F.double().cpu().numpy(), Fr + Fk) < tol
+    assert abs(E[1] - Ek[0]) <= tol * abs(Ek[0])
+    plan.close()
