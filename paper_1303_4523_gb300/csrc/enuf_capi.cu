@@ -1167,7 +1167,7 @@ enuf_status enqueue_force_eval(dpd_system_t sys, cudaStream_t s0, cudaStream_t s
     return enqueue_eval(plan, a, s0, s1, plan->evFork, plan->evJoin, ev, log, false, fuse ? &sys->d : nullptr, step);
 }
 
-enuf_status initial_force(dpd_system_t sys) {
+enuf_status run_initial_force(dpd_system_t sys) {
     enuf_plan_t plan = sys->plan;
     LaunchLog log;
     CU(cudaMemcpyAsync(sys->d.v0, sys->d.vel, (size_t)sys->d.N * 3 * plan->rsz, cudaMemcpyDeviceToDevice,
@@ -1183,6 +1183,25 @@ enuf_status initial_force(dpd_system_t sys) {
     CU(cudaStreamSynchronize(plan->stream));
     CU(cudaGetLastError());
     return ENUF_OK;
+}
+
+// The tile and cell counters are zero between evaluations: the kernel after each
+// count clears them. A captured sequence runs whole or not at all; this one is
+// launched kernel by kernel, so a launch that fails (a kernel that the device
+// has no memory left to load) can leave counts that the next evaluation would
+// add to, beyond the ends of the sorted arrays.
+enuf_status initial_force(dpd_system_t sys) {
+    const enuf_status st = run_initial_force(sys);
+    if (st != ENUF_OK) {
+        enuf_plan_t plan = sys->plan;
+        cudaStreamSynchronize(plan->aux);
+        cudaMemsetAsync(plan->w.tcnt, 0, (size_t)plan->g.ntiles * sizeof(int), plan->stream);
+        cudaMemsetAsync(plan->w.ticket, 0, 4 * sizeof(int), plan->stream);
+        cudaMemsetAsync(sys->d.ccount, 0, (size_t)sys->d.ncells * sizeof(int), plan->stream);
+        cudaStreamSynchronize(plan->stream);
+        cudaGetLastError();
+    }
+    return st;
 }
 
 enuf_status capture_step(dpd_system_t sys) {
