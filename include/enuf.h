@@ -90,9 +90,9 @@ typedef struct {
     int    fft_radix; /* line transforms: 0 = automatic: FP32 grids whose n = f1 f2 with
                          f1, f2 in {4, 5, 6, 8, 10, 12, 16, 20} take the two-factor
                          kernels (both DFTs in registers, one twiddle pass), as do, with radices
-                         9, 15 and 18, grids that only then split (n = 108, 180, 216, 288, 300;
-                         enuf_plan_info reports these as for 2); other grids and FP64 the
-                         Stockham stages as for 2;
+                         9, 15 and 18, grids that only then split (n = 108, 180, 216, 288, 300,
+                         324, 360; enuf_plan_info reports these as for 2, enuf_plan_kernels
+                         their factors); other grids and FP64 the Stockham stages as for 2;
                          1 = Stockham stages over radices 2, 3, 4, 5, 8 only;
                          2 = Stockham stages, the fewest over 2, 3, 4, 5, 8, and for FP32
                          grids from n = 128 on the composite radices 6, 10, 12, 16, 20
@@ -138,8 +138,10 @@ typedef struct {
     int    fft_stages;         /* stages of one length-n line transform (2 for the
                                   two-factor kernels) */
     int    fft_radix[8];       /* their radices in order (two-factor: f1, f2) */
-    int    fft_two_factor;     /* 1: the two-factor kernels (enuf_params.fft_radix) */
-    int    spread;             /* spreading kernel taken (enuf_params.spread: 1 to 4) */
+    int    fft_two_factor;     /* 1: the two-factor kernels with factors of the first set of
+                                  enuf_params.fft_radix (enuf_plan_kernels: every split) */
+    int    spread;             /* spreading form 1 to 4 of enuf_params.spread; for 0 the one that
+                                  the sizes admit (enuf_plan_kernels: the one that runs) */
     int    brick_x;            /* x extent of a spreading brick (forms 2 and 3) */
     int    pairs;              /* DPD pair launches taken (enuf_params.pairs: 1 or 2) */
 } enuf_plan_info;
@@ -173,6 +175,16 @@ enuf_status enuf_get_info(enuf_plan_t plan, enuf_plan_info* info);
  * enuf_get_info gives it), computed on the host: no device, no allocation.
  * Errors: those of enuf_plan's parameter validation. */
 enuf_status enuf_plan_shape(const enuf_params* params, int n_max, enuf_plan_info* info);
+
+/* The kernels that an evaluation with these parameters runs (plans of equal
+ * enuf_plan_info can differ in them), computed on the host. Errors: those of
+ * enuf_plan's parameter validation. */
+typedef struct {
+    int fft_f1, fft_f2;   /* factors of the two-factor line transforms; 0, 0: Stockham stages */
+    int spread;           /* 1 to 4: that form of enuf_params.spread; 5: the reduction form
+                             (a batch that runs as one launch sequence runs it for every value) */
+} enuf_kernel_choice;
+enuf_status enuf_plan_kernels(const enuf_params* params, int n_max, enuf_kernel_choice* out);
 
 /* Electrostatic energy and forces (Eq. 16-25; Table 2 step 4).
  *   n      : number of beads, 0 <= n <= n_max

@@ -17,7 +17,7 @@ is cut, but not what is computed (results agree to rounding):
             from n = 128 on when that saves a stage; 1 keeps radices
             2, 3, 4, 5, 8.
 
-The library's own host logic (enuf_plan_shape) decides which tiles are legal
+The library's own host logic (enuf_plan_shape, enuf_plan_kernels) decides which tiles are legal
 and which choices differ, so the candidates never include a launch shape the
 plan would reject, nor two that run the same kernels.
 Each candidate is timed on the device with CUDA events over repeated
@@ -83,9 +83,12 @@ def _shape(params: enuf.enuf_params, n_max: int):
     """(tile, FFT kernels, radix schedule) of the plan, or None if it is rejected."""
     try:
         info = enuf.plan_shape(params, n_max)
+        run = enuf.plan_kernels(params, n_max)
     except enuf.EnufError:
         return None
-    return info.tile, info.fft_kernels, info.fft_two_factor, tuple(info.fft_radix[:info.fft_stages])
+    # the two-factor kernels have no schedule beside their factors
+    radix = () if run.fft_f1 else tuple(info.fft_radix[:info.fft_stages])
+    return info.tile, info.fft_kernels, run.fft_f1, run.fft_f2, radix
 
 
 def _sequence_ok(params: enuf.enuf_params, n_max: int) -> bool:

@@ -995,6 +995,18 @@ enuf_status enuf_plan_shape(const enuf_params* params, int n_max, enuf_plan_info
     return ENUF_OK;
 }
 
+enuf_status enuf_plan_kernels(const enuf_params* params, int n_max, enuf_kernel_choice* out) {
+    if (!params || !out) return ENUF_ERR_INVALID;
+    std::unique_ptr<enuf_plan_s> tmp(new (std::nothrow) enuf_plan_s());
+    if (!tmp) return ENUF_ERR_OOM;
+    const enuf_status st = derive(tmp.get(), *params, n_max, nullptr);
+    if (st != ENUF_OK) return st;
+    out->fft_f1 = tmp->fs.two ? tmp->fp.f1 : 0;
+    out->fft_f2 = tmp->fs.two ? tmp->fp.f2 : 0;
+    out->spread = tmp->fs.red ? 5 : tmp->fs.spread;
+    return ENUF_OK;
+}
+
 enuf_status enuf_check_word(enuf_plan_t plan, unsigned int* mask, int reset) {
     if (!plan || !mask) return ENUF_ERR_INVALID;
     CU(cudaStreamSynchronize(plan->stream));

@@ -49,6 +49,10 @@ class enuf_plan_info(C.Structure):
                 ("pairs", C.c_int)]
 
 
+class enuf_kernel_choice(C.Structure):
+    _fields_ = [("fft_f1", C.c_int), ("fft_f2", C.c_int), ("spread", C.c_int)]
+
+
 class dpd_params(C.Structure):
     _fields_ = [("ntypes", C.c_int), ("a", C.POINTER(C.c_double)), ("gamma", C.c_double),
                 ("sigma", C.c_double), ("dt", C.c_double), ("lambda_vv", C.c_double),
@@ -67,6 +71,7 @@ def _load():
         "enuf_footprint": (st, [C.POINTER(enuf_params), i, C.POINTER(C.c_size_t)]),
         "enuf_get_info": (st, [vp, C.POINTER(enuf_plan_info)]),
         "enuf_plan_shape": (st, [C.POINTER(enuf_params), i, C.POINTER(enuf_plan_info)]),
+        "enuf_plan_kernels": (st, [C.POINTER(enuf_params), i, C.POINTER(enuf_kernel_choice)]),
         "enuf_accuracy_params": (st, [d, C.POINTER(enuf_params)]),
         "enuf_energy_forces": (st, [vp, i, vp, vp, vp, pd, pd]),
         "enuf_energy_forces_host": (st, [vp, i, vp, vp, vp, pd, pd]),
@@ -106,10 +111,8 @@ def _load():
 
 lib = _load()
 
-EXPORTED = ("enuf_plan", "enuf_footprint", "enuf_get_info", "enuf_plan_shape", "enuf_accuracy_params",
-            "enuf_energy_forces",
-            "enuf_last_energies",
-            "enuf_energy_forces_host", "enuf_debug_buffer", "enuf_enable_timing",
+EXPORTED = ("enuf_plan", "enuf_footprint", "enuf_get_info", "enuf_plan_shape", "enuf_plan_kernels",
+            "enuf_accuracy_params", "enuf_energy_forces", "enuf_last_energies", "enuf_energy_forces_host", "enuf_debug_buffer", "enuf_enable_timing",
             "enuf_stage_time", "enuf_launches_per_eval", "enuf_destroy", "enuf_status_string",
             "enuf_last_error", "dpd_create", "dpd_step", "dpd_copy_energies", "dpd_get_state", "dpd_set_state",
             "dpd_get_forces", "dpd_step_host", "dpd_device_state", "enuf_check_word",
@@ -202,6 +205,14 @@ def plan_shape(params: enuf_params, n_max: int) -> enuf_plan_info:
     info = enuf_plan_info()
     _check(lib.enuf_plan_shape(C.byref(params), int(n_max), C.byref(info)), what="enuf_plan_shape")
     return info
+
+
+def plan_kernels(params: enuf_params, n_max: int) -> enuf_kernel_choice:
+    """The kernels an evaluation with these parameters runs: factors of the
+    two-factor FFT (0, 0: Stockham stages) and spreading form (5: reductions)."""
+    k = enuf_kernel_choice()
+    _check(lib.enuf_plan_kernels(C.byref(params), int(n_max), C.byref(k)), what="enuf_plan_kernels")
+    return k
 
 
 def enuf_footprint(params: enuf_params, n_max: int) -> int:
