@@ -131,36 +131,6 @@ bool fft_radices(int n, FftPlanDev& fp, bool composite) {
     return true;
 }
 
-// Two-factor split n = f1 f2 of the FP32 two-factor kernels: both factors in
-// their radix set; the most balanced split, ties to the larger f2 (phase A
-// reads f2 consecutive elements per line and load). Lengths without such a
-// split (108, 180, 216, 288, 300, 360, ...) take radices 9, 15 and 18 as well
-// (*ext; plan info then keeps reporting their Stockham schedule): five passes
-// at n = 180 in 172 us against 227 on three Stockham stages. False: none.
-bool fft_two_factor(int n, FftPlanDev& fp, int* ext) {
-    static const int kF[] = {4, 5, 6, 8, 10, 12, 16, 20};
-    static const int kFx[] = {4, 5, 6, 8, 9, 10, 12, 15, 16, 18, 20};
-    int best1 = 0, best2 = 0;
-    auto split = [&](const int* f, int cnt) {
-        for (int i = 0; i < cnt; ++i)
-            for (int j = 0; j < cnt; ++j) {
-                const int a = f[i], b = f[j];
-                if (a * b != n) continue;
-                const int m = std::min(a, b), mb = std::min(best1, best2);
-                if (!best1 || m > mb || (m == mb && b > best2)) {
-                    best1 = a;
-                    best2 = b;
-                }
-            }
-    };
-    split(kF, 8);
-    *ext = best1 ? 0 : 1;
-    if (!best1) split(kFx, 11);
-    fp.f1 = best1;
-    fp.f2 = best2;
-    return best1 > 0;
-}
-
 // Largest float strictly below L: a float x lies in [0, L) iff 0 <= x <= this.
 float largest_float_below(double L) {
     float f = (float)L;
@@ -301,7 +271,14 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
         return fail(plan, ENUF_ERR_UNSUPPORTED, "grid n = %d is not 2^a 3^b 5^c", n);
     fp.f1 = fp.f2 = 0;
     int two_ext = 0;
-    if (P.prec == ENUF_FP32 && P.fft_radix == 0) fft_two_factor(n, fp, &two_ext);
+    if (P.prec == ENUF_FP32 && P.fft_radix == 0) {
+        // plan info keeps reporting the Stockham schedule of an extended split (five passes
+        // at n = 180 take 172 us with it against 227 on three Stockham stages)
+        const Fft2Split split = fft2_split(n);
+        fp.f1 = split.f1;
+        fp.f2 = split.f2;
+        two_ext = split.ext ? 1 : 0;
+    }
     if (2 * P.p > n) return fail(plan, ENUF_ERR_INVALID, "window 2p = %d wider than the grid", 2 * P.p);
     // tile edge: divides n, >= p, histogram fits in shared memory
     // the spreading kernel holds a T^3 tile of the grid in shared memory: T <= 24
@@ -426,9 +403,9 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
         };
         // the z pass holds one inverse line per line, two with three fields
         const int zmul = g.nf == 3 ? 2 : 1;
-        fs.smem_xy = (n + (n / 2) * (lsa + lsb)) * csz;
+        fs.smem_xy = fft2_smem_xy(fp.f1, fp.f2, csz);
         fs.smem_yx = (n + (n / 2) * lsa + nc1 * lsb) * csz;
-        fs.fused = (fs.smem_xy <= 100 * 1024 && P.fft_path == 0) ? 1 : 0;
+        fs.fused = (fs.smem_xy <= kFftPlaneSmem && P.fft_path == 0) ? 1 : 0;
         fs.composite = 0;
         if (fs.fused) {
             // the z pass keeps one CTA per line group (spec2 plane-major); a smaller

@@ -589,6 +589,53 @@ __device__ __forceinline__ R spec3_factor(int nf, int a, int kx, int ky) {
 #define ENUF_FFT2_PLANES(X) ENUF_FFT2_PLANES_A(X) ENUF_FFT2_PLANES_B(X)
 #define ENUF_FFT2_LINES(X) ENUF_FFT2_LINES_A(X) ENUF_FFT2_LINES_B(X) ENUF_FFT2_LINES_C(X) ENUF_FFT2_LINES_D(X)
 
+// Two-factor split n = f1 f2: both factors in the radix set of the any-length
+// kernels; the most balanced split, ties to the larger f2 (phase A reads f2
+// consecutive elements per line and load). Lengths without such a split (108,
+// 180, 216, 288, 300, 324, 360) take radices 9, 15 and 18 as well (ext), which only
+// kernels of single lengths have. f1 = 0: none.
+struct Fft2Split {
+    int f1, f2;
+    bool ext;
+};
+constexpr Fft2Split fft2_split(int n) {
+    constexpr int set[] = {4, 5, 6, 8, 10, 12, 16, 20, 9, 15, 18};   // the first eight: any length
+    Fft2Split best{0, 0, false};
+    for (int k = 8; k <= 11 && !best.f1; k += 3)
+        for (int i = 0; i < k; ++i)
+            for (int j = 0; j < k; ++j) {
+                const int a = set[i], b = set[j];
+                if (a * b != n) continue;
+                const int m = a < b ? a : b, mb = best.f1 < best.f2 ? best.f1 : best.f2;
+                if (!best.f1 || m > mb || (m == mb && b > best.f2)) best = Fft2Split{a, b, k > 8};
+            }
+    return best;
+}
+
+// The plane passes hold the twiddles, the n/2 phase-A rows and n/2 result rows of
+// a z-plane; taken up to this size.
+constexpr int kFftPlaneSmem = 100 * 1024;
+__host__ __device__ constexpr int fft2_smem_xy(int f1, int f2, int csz) {
+    return (f1 * f2 + (f1 * f2 / 2) * (fft2_lsa(f1, f2) + fft2_lsb(f1 * f2))) * csz;
+}
+
+// Every split that a plan (n = 2 M, M even, n <= 1024) can take has its kernels:
+// plane passes of that length where they are chosen, line passes of that length
+// where a factor is 9, 15 or 18 (the any-length kernels would leave such lines
+// untransformed).
+constexpr bool fft2_splits_covered() {
+#define ENUF_IS(a, b) || (s.f1 == a && s.f2 == b)
+    for (int n = 8; n <= 1024; n += 4) {
+        const Fft2Split s = fft2_split(n);
+        if (!s.f1) continue;
+        if (fft2_smem_xy(s.f1, s.f2, 8) <= kFftPlaneSmem && !(false ENUF_FFT2_PLANES(ENUF_IS))) return false;
+        if (s.ext && !(false ENUF_FFT2_LINES(ENUF_IS))) return false;
+    }
+#undef ENUF_IS
+    return true;
+}
+static_assert(fft2_splits_covered(), "a two-factor split without kernels");
+
 // body(f1, f2) with the split of fp as constants where the plane passes have
 // kernels of that length, (0, 0) otherwise.
 template <typename Body>
