@@ -1450,7 +1450,7 @@ struct enuf_batch_s {
     std::vector<const void*> g_pos, g_q;
     std::vector<void*> g_F;
     int launches = 0;
-    // one launch sequence over all systems (FP32, see batch_eligible)
+    // one launch sequence over all systems (FP32, see batch_plan_ok)
     bool seq = false;
     cudaStream_t aux = nullptr;
     cudaEvent_t evFork = nullptr, evJoin = nullptr;

@@ -168,18 +168,13 @@ cudaError_t configure_kernels(int max_smem) {
         if (r != cudaSuccess) e = r;
     };
     set((const void*)k_spread<R>);
-    set((const void*)k_spread_col<R, 8, false>);
-    set((const void*)k_spread_col<R, 8, true>);
-    set((const void*)k_spread_col<R, 10, false>);
-    set((const void*)k_spread_col<R, 10, true>);
-    set((const void*)k_spread_col<R, 12, false>);
-    set((const void*)k_spread_col<R, 12, true>);
-    set((const void*)k_spread_col<R, 16, false>);
-    set((const void*)k_spread_col<R, 16, true>);
-    set((const void*)k_spread_col<R, 20, false>);
-    set((const void*)k_spread_col<R, 20, true>);
-    set((const void*)k_spread_col<R, 24, false>);
-    set((const void*)k_spread_col<R, 24, true>);
+    constexpr bool SLAB = sizeof(R) == 8;   // as launch_col
+    set((const void*)k_spread_col<R, 8, SLAB>);
+    set((const void*)k_spread_col<R, 10, SLAB>);
+    set((const void*)k_spread_col<R, 12, SLAB>);
+    set((const void*)k_spread_col<R, 16, SLAB>);
+    set((const void*)k_spread_col<R, 20, SLAB>);
+    set((const void*)k_spread_col<R, 24, SLAB>);
     if constexpr (sizeof(R) == 4) {
         set((const void*)k_spread_brick<R, false>);
         set((const void*)k_spread_brick<R, true>);
@@ -313,7 +308,7 @@ inline void enqueue_spread_sc(const Geo& g, const FftShape& fs, const Work& w, c
 }
 
 // The same passes on the two-factor kernels (FP32 grids with n = f1 f2): the
-// plane passes and the five passes of one length, or of any (<0, 0>). With the
+// plane passes of one length, the five passes of one length or of any (<0, 0>). With the
 // spreading fused with the x pass (spread = 3) the x pass is already done. evZ
 // (or nullptr) is recorded right after the z pass, whose blocks write the
 // reciprocal energy and virial partials (the kernel after it then launches
@@ -384,7 +379,6 @@ void Fft2Lines<F1, F2>::enqueue(const Geo& g, const FftShape& fs, const FftPlanD
     log->kernels += 5;   // the spreading kernel and four passes
 }
 
-extern template struct Fft2Planes<0, 0>;
 extern template struct Fft2Lines<0, 0>;
 #define ENUF_EXTERN(a, b) extern template struct Fft2Planes<a, b>;
 ENUF_FFT2_PLANES(ENUF_EXTERN)
@@ -393,14 +387,14 @@ ENUF_FFT2_PLANES(ENUF_EXTERN)
 ENUF_FFT2_LINES(ENUF_EXTERN)
 #undef ENUF_EXTERN
 
-// f.template operator()<F1, F2>() for the plan's split, <0, 0> without an instance
+// planes or lines with the passes of the plan's split (line passes without an instance: <0, 0>)
 template <typename Planes, typename Lines>
 inline auto fft2_dispatch(const FftShape& fs, const FftPlanDev& fp, Planes&& planes, Lines&& lines) {
 #define ENUF_CASE(a, b) \
     if (fp.f1 == a && fp.f2 == b) return planes(Fft2Planes<a, b>{});
     if (fs.fused) {
         ENUF_FFT2_PLANES(ENUF_CASE)
-        return planes(Fft2Planes<0, 0>{});
+        __builtin_unreachable();   // every split of the plane passes is listed (fft2_splits_covered)
     }
 #undef ENUF_CASE
 #define ENUF_CASE(a, b) \
@@ -557,7 +551,7 @@ cudaError_t enqueue_dpd_forces(const Work& w, const DpdDev& d, cudaStream_t s, E
         launch_carved(w.carve_b, pdl, false, k_scan_mb, (d.ncells + kScanMbSpan - 1) / kScanMbSpan, 1024, 0, s,
                (const int*)d.ccount, d.cstart, d.ncells, d.ccur);
     else
-        launch(pdl, false, k_scan, 1, 1024, 0, s, d.ccount, d.cstart, d.ncells, d.ccur, 0);
+        launch(pdl, false, k_scan, 1, 1024, 0, s, (const int*)d.ccount, d.cstart, d.ncells, d.ccur);
     launch_carved(w.carve_b, pdl, false, k_cell_scatter<R>, blocks, 256, 0, s, d.N, d.L, d.xmaxf, d.Lhi, d.Llo,
            static_cast<const R*>(d.pos),
            static_cast<const R*>(d.v0), (const int*)d.type, d.ckey, d.ccur, static_cast<V*>(d.sp),

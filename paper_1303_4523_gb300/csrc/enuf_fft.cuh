@@ -423,8 +423,8 @@ __host__ __device__ constexpr int fft2_lsb(int n) { return n + 1; }
 // that every offset, quotient and loop bound of a pass is a constant (the
 // runtime form spends two thirds of its instructions on them: ~95 per complex
 // point in the inverse x pass at n = 320, of which ~30 are the transform);
-// FftLen<0, 0>: from the plan, for lengths without an instance of their own and
-// for batches of mixed sizes.
+// FftLen<0, 0>: from the plan, for line passes of lengths without an instance of
+// their own (up to n = 100 with fft_path = 1) and the fused brick spreading.
 template <int F1, int F2>
 struct FftLen {
     static constexpr int kF1 = F1, kF2 = F2;
@@ -636,8 +636,8 @@ constexpr bool fft2_splits_covered() {
 }
 static_assert(fft2_splits_covered(), "a two-factor split without kernels");
 
-// body(f1, f2) with the split of fp as constants where the plane passes have
-// kernels of that length, (0, 0) otherwise.
+// body(f1, f2) with the split of fp as constants: every split of the plane passes is
+// in the list (fft2_splits_covered).
 template <typename Body>
 __device__ __forceinline__ void fft2_by_length(const FftPlanDev& fp, Body body) {
     switch (32 * fp.f1 + fp.f2) {
@@ -645,7 +645,7 @@ __device__ __forceinline__ void fft2_by_length(const FftPlanDev& fp, Body body) 
     case 32 * a + b: body(std::integral_constant<int, a>{}, std::integral_constant<int, b>{}); break;
         ENUF_FFT2_PLANES(ENUF_CASE)
 #undef ENUF_CASE
-        default: body(std::integral_constant<int, 0>{}, std::integral_constant<int, 0>{});
+        default: break;
     }
 }
 

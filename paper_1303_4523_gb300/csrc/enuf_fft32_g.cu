@@ -2,6 +2,5 @@
 #include "enuf_enqueue.cuh"
 
 namespace enuf {
-template struct Fft2Planes<0, 0>;
 template struct Fft2Lines<0, 0>;
 }  // namespace enuf

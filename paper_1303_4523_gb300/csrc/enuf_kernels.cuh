@@ -410,8 +410,6 @@ __device__ __forceinline__ void totals_if_last(const Geo& g, const TotalsArgs& t
 }
 
 
-// Kahan-compensated accumulator (FP64).
-
 // ---------------------------------------------------------------------------
 // a1: binning of the charged beads into tiles of the oversampled grid, a
 // counting sort in two kernels (three with many tiles):
@@ -573,9 +571,9 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(Geo g, int N, const R
 
 // Exclusive scan of in[0, count) into out[0, count], out[count] = total; one
 // CTA of 1024 threads, 16 elements per thread and round (four 16-byte loads).
-// aux, when given, receives a copy of out; zero_in clears the input.
-static __global__ void __launch_bounds__(1024) k_scan(int* __restrict__ in, int* __restrict__ out, int count,
-                                                      int* __restrict__ aux, int zero_in) {
+// aux, when given, receives a copy of out.
+static __global__ void __launch_bounds__(1024) k_scan(const int* __restrict__ in, int* __restrict__ out, int count,
+                                                      int* __restrict__ aux) {
     pdl_enter();
     constexpr int IPT = 16;
     __shared__ int wsum[32];
@@ -627,7 +625,6 @@ static __global__ void __launch_bounds__(1024) k_scan(int* __restrict__ in, int*
                 o4.w = run; run += v[k + 3];
                 *reinterpret_cast<int4*>(out + i0 + k) = o4;
                 if (aux) *reinterpret_cast<int4*>(aux + i0 + k) = o4;
-                if (zero_in) *reinterpret_cast<int4*>(in + i0 + k) = make_int4(0, 0, 0, 0);
             }
         } else {
 #pragma unroll
@@ -636,7 +633,6 @@ static __global__ void __launch_bounds__(1024) k_scan(int* __restrict__ in, int*
                 if (idx < count) {
                     out[idx] = run;
                     if (aux) aux[idx] = run;
-                    if (zero_in) in[idx] = 0;
                 }
                 run += v[k];
             }
