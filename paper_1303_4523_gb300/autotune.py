@@ -3,16 +3,18 @@
 Three plan parameters change which kernels run and how the oversampled grid
 is cut, but not what is computed (results agree to rounding):
 
-  tile      the spreading tile edge T (a divisor of n, p <= T <= 24). It sets
-            the spreading kernel (column form for T in 8, 10, 12, 16, 20, 24,
-            the work-item form otherwise), the binning histogram and the
-            real-space cell list, whose stencil is +-ceil(r_c / (T L / n))
-            tiles per axis.
+  tile      the tile edge T (a divisor of n, p <= T <= 24). It sets the tiles
+            that the charged beads are sorted into, which are the real-space
+            cell list, whose stencil is +-ceil(r_c / (T L / n)) tiles per
+            axis, and where the tile form of the spreading is asked for its
+            kernel (column form for T in 8, 10, 12, 16, 20, 24, the work-item
+            form otherwise).
   fft_path  FP32 grids with n <= 112 run the FFT as whole z-planes in shared
             memory (x and y passes fused); fft_path = 1 forces the five line
             passes instead.
   fft_radix the line transforms: 0 runs FP32 grids whose n = f1 f2 on the
-            two-factor kernels (both DFTs in registers); 2 runs the Stockham
+            two-factor kernels (both DFTs in registers; plan_kernels gives f1
+            and f2); 2 runs the Stockham
             stages, with composite radices (6, 10, 12, 16, 20) for FP32 grids
             from n = 128 on when that saves a stage; 1 keeps radices
             2, 3, 4, 5, 8.
@@ -33,7 +35,7 @@ The cache path is $ENUF_TUNE_CACHE, else ~/.cache/enuf_gb300/tune.json.
 
 For a batch (sequence=True) the FP32 candidates are restricted to the plans
 a batch can run as one launch sequence over all systems (two-factor fused
-FFT planes, the tile spreading form, a column-form tile edge): a faster
+FFT planes, a column-form tile edge): a faster
 single-system choice outside that set takes its system out of the sequence
 and costs the batch more than it saves (measured: the 64-system sweep tuned
 per system ran as 576 graph launches in 1.62 ms, against 1.33 ms for one

@@ -20,7 +20,9 @@ using namespace enuf;
 
 namespace {
 
-constexpr int kMaxTiles = 32768;      // shared-memory histogram limit (128 KB)
+// Tiles of a plan. A rule of the interface: no kernel needs it any more (the tile starts
+// are scanned in global memory from kBinScanTiles on), but what it refuses stays refused.
+constexpr int kMaxTiles = 32768;
 constexpr int kMaxBeads = 1 << 29;    // the kernels index per-bead components as int (3 i + 2, 4 i + 3)
 constexpr int kMaxSmem = 200 * 1024;  // dynamic shared memory the kernels may request
 
@@ -280,9 +282,8 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
         two_ext = split.ext ? 1 : 0;
     }
     if (2 * P.p > n) return fail(plan, ENUF_ERR_INVALID, "window 2p = %d wider than the grid", 2 * P.p);
-    // tile edge: divides n, >= p, histogram fits in shared memory
-    // the spreading kernel holds a T^3 tile of the grid in shared memory: T <= 24
-    // (110 KB in FP64); the binning kernels hold the tile histogram (<= 32768 tiles)
+    // tile edge: divides n, >= p, at most kMaxTiles tiles; the tile form of the spreading
+    // holds a T^3 tile of the grid in shared memory: T <= 24 (110 KB in FP64)
     constexpr int kMaxTile = 24;
     int T = 0;
     if (P.tile > 0) {
@@ -292,7 +293,7 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
                         kMaxTile);
     } else {
         // default: the smallest tile at least r_c wide (the real-space stencil is
-        // then 3^3 tiles) that divides n, is >= p and keeps the histogram in shared memory
+        // then 3^3 tiles) that divides n, is >= p and makes at most kMaxTiles tiles
         const int tmin = std::max(P.p, (int)std::ceil(P.r_cut * n / P.L - 1e-9));
         for (int c = tmin; c <= kMaxTile && !T; ++c)
             if (n % c == 0 && (n / c) * (n / c) * (n / c) <= kMaxTiles) T = c;
@@ -314,7 +315,8 @@ enuf_status derive(enuf_plan_t plan, const enuf_params& P, int n_max, size_t* by
     g.ntiles = g.ntd * g.ntd * g.ntd;
     const double tw = T * P.L / n;
     g.rs = (int)std::ceil(P.r_cut / tw - 1e-12);
-    {   // the real-space kernel stages the stencil of one tile: at most 1024 tiles
+    {   // at most 1024 tiles: a bead walks a row of tiles at a time, and rows with hardly a
+        // bead would cost more than the pairs (a rule of the interface, as kMaxTiles)
         const int hs = std::min(2 * g.rs + 1, n / T);
         if (hs * hs * hs > 1024)
             return fail(plan, ENUF_ERR_UNSUPPORTED, "real-space stencil of %d^3 tiles too large (r_cut/tile)", hs);
@@ -750,7 +752,7 @@ enuf_status upload_tables(enuf_plan_t plan) {
     return ENUF_OK;
 }
 
-// fuse_totals: the gather's last block also reduces the energies (evaluations
+// fuse_totals: one more block of the gather reduces the energies (evaluations
 // outside a DPD step, where nothing follows the gather).
 // step: a DPD step, whose energies but the kinetic one are reduced on the
 // side stream beside the gather (plan->evT then orders the closing kick).

@@ -321,8 +321,8 @@ cudaError_t enqueue_dpd_add(const DpdDev& d, cudaStream_t s, LaunchLog* log, boo
 template <typename R>
 cudaError_t enqueue_spread_only(const Geo& g, const Work& w, const EvalArgs& a, void* grid_out, cudaStream_t s);
 // Batched launch sequence (FP32): a system qualifies when its plan runs the
-// fused-plane two-factor FFT, the column spreading form and the one-kernel
-// binning offsets. batch_bytes: the device tables' size; batch_build writes
+// fused-plane two-factor FFT, has a tile edge of the column form and forms its tile
+// starts in the scatter kernel. batch_bytes: the device tables' size; batch_build writes
 // them (argument tables and block maps) into dbuf and fills the launch
 // parameters; batch_enqueue launches the sequence (fork/join on s1 for the
 // real-space pairs).
