@@ -2568,9 +2568,13 @@ __device__ __forceinline__ void k_real_body(Geo g, const int* __restrict__ tstar
     int* list = reinterpret_cast<int*>(smraw) + warp * 32 * kRealQ + lane;   // FP32: entry k at 32 k
     int2* ring = reinterpret_cast<int2*>(smraw) + warp * kRealRing;          // FP64
     const int nq = tstart[g.ntiles];
-    // lanes per bead: enough to fill the chip, no more (see the plan's real_lanes)
+    // lanes per bead: enough to fill the chip, no more (see the plan's real_lanes). FP32:
+    // two at least, one lane alone walks a bead's whole rows and drains its list more
+    // often; whole calls at one / two lanes: 81,000 beads all charged 2004 / 1287 us (1958
+    // with staged halos), half of 375,000 1229 / 1018, a tenth of 3M 1034 / 1009
+    constexpr int SMIN = real_half<R>() ? 1 : 2;
     int S = 32;
-    while (S > 1 && (long long)nq * S > (S > 8 ? g.real_lanes / 3 * 2 : g.real_lanes)) S >>= 1;
+    while (S > SMIN && (long long)nq * S > (S > 8 ? g.real_lanes / 3 * 2 : g.real_lanes)) S >>= 1;
     RealSum<R> a{(R)0, (R)0, (R)0, (R)0, (R)0};
     if (2 * g.rs + 1 >= g.ntd)
         real_sweep<R, true>(g, nq, S, tstart, sq, sw, sb, spf, list, ring, F, a, blk);
