@@ -2604,11 +2604,10 @@ __global__ void __launch_bounds__(kRealThreads, sizeof(R) == 4 ? 4 : 2) k_real(G
 // of x * ncd/L cannot separate two beads closer than 1 by two cells).
 // The cell of a wrapped coordinate, for the cell list and for the pair sweep that
 // reads it: always inside the list (a coordinate that is not a number converts
-// to 0 from float but to the smallest int from double).
+// to 0 from float, to the smallest int from double: the last cell).
 template <typename R>
 __device__ __forceinline__ int cell_of(R xw, R rinv, int ncd) {
-    const int c = (int)(xw * rinv);
-    return c < 0 ? 0 : (c >= ncd ? ncd - 1 : c);
+    return (int)min((unsigned)(int)(xw * rinv), (unsigned)(ncd - 1));
 }
 
 template <typename R>
