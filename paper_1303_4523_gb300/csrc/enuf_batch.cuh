@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kRealThreads, CTAS) kb_real(const RealArgs<R>*
     pdl_enter();
     const int m = cmap[blockIdx.x];
     const RealArgs<R>& a = tab[m >> kBatchShift];
-    k_real_body<R>(a.g, a.tstart, a.sq, a.sw, a.sb, a.spf, a.F, a.rpart, Blk{m & kBatchLocal, a.nblk});
+    k_real_body<R, true>(a.g, a.tstart, a.sq, a.sw, a.sb, a.spf, a.F, a.rpart, Blk{m & kBatchLocal, a.nblk});
 }
 
 // spreading, reduction form (systems grouped by tile edge; PT: the tap count 2p

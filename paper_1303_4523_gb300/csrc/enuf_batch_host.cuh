@@ -17,12 +17,18 @@ inline void append_blocks(std::vector<int>& cmap, int sys, int nblk) {
 }
 
 // Blocks of one system of a batch in its bead loops. The batch fills the chip,
-// so a system takes few blocks and strides over its beads: real space N / 1024
-// blocks and as many lanes as its beads need (64 systems: 1179 us against 1219
-// with N / 512), gather N / 512 (1171 against 1219 with N / 64), spreading
+// so a system takes few blocks and strides over its beads: real space N / 512
+// blocks and lanes per bead for N / 4 lanes (with a tenth of the beads charged half of
+// the blocks find none and leave at once; with N / 1024 blocks
+// the more charged systems left SMs idle: 40 systems of 3000 to 20,000 beads, a quarter,
+// half and all charged, 654, 2031 and 7780 us against 549, 1498 and 4950; a tenth
+// charged 293 against 290; N / 256: 64 systems, a tenth charged, 895 against 830), gather N / 512 (1171 against 1219 with N / 64), spreading
 // N / 256 (its launches, one per tile edge, follow each other: 40 systems of
 // 3000 to 20,000 beads 345 -> 333 us against N / 512 with the next rule).
-inline int batch_real_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_real, (x.N + 1023) / 1024)); }
+inline int batch_real_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_real, (x.N + 511) / 512)); }
+inline int batch_real_lanes(const BatchSys& x) {
+    return std::max(1, std::min(x.w.nblk_real, (x.N + 1023) / 1024)) * kRealThreads;
+}
 inline int batch_spread_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_gather, (x.N + 255) / 256)); }
 inline int batch_gather_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_gather, (x.N + 511) / 512)); }
 
@@ -106,9 +112,19 @@ cudaError_t batch_build(void* dbuf, const BatchSys* sys, int nsys, BatchLaunch* 
             const int nb = batch_real_blocks(x);
             a[s] = RealArgs<R>{x.g, x.w.tstart, static_cast<const V*>(x.w.sq), static_cast<const V*>(x.w.sw), x.w.sb,
                                x.w.spf, static_cast<R*>(x.F), x.w.part + x.w.off_real, nb};
-            a[s].g.real_lanes = nb * kRealThreads;
-            append_blocks(m, s, nb);
+            a[s].g.real_lanes = batch_real_lanes(x);
         }
+        // small batches: of every system the blocks that have beads with a tenth charged
+        // first, so that the others take no place from them (16 systems 276 us against 286;
+        // 64 systems, several waves either way, 913 against 906 with a system's blocks together)
+        int total = 0;
+        for (int s = 0; s < nsys; ++s) total += batch_real_blocks(sys[s]);
+        const int parts = total <= 8 * kSMs ? 2 : 1;
+        for (int part = 0; part < parts; ++part)
+            for (int s = 0; s < nsys; ++s) {
+                const int nb = batch_real_blocks(sys[s]), h = parts == 1 ? nb : (nb + 1) / 2;
+                for (int b = part ? h : 0; b < (part ? nb : h); ++b) m.push_back((s << kBatchShift) | b);
+            }
         put(L.real, a.data(), a.size() * sizeof(a[0]), m);
         L.real.threads = kRealThreads;
         L.real.smem = real_smem_bytes<R>();
@@ -210,9 +226,10 @@ cudaError_t batch_enqueue(const BatchLaunch& L, cudaStream_t s0, cudaStream_t s1
     run(true, true, kb_bin_weights<R>, L.bin_weights, (const BinWeightsArgs<R>*)L.bin_weights.tab, s0);
     cudaEventRecord(evFork, s0);
     cudaStreamWaitEvent(s1, evFork, 0);
-    // four CTAs per SM (64 registers, a small spill) where the blocks fill more than
-    // two (103 registers): 64 systems 946 -> 909 us; 16 systems 214, with four 245
-    run(false, false, L.real.blocks > 2 * kSMs ? kb_real<R, 4> : kb_real<R, 2>, L.real, (const RealArgs<R>*)L.real.tab, s1);
+    // four CTAs per SM (64 registers, a small spill) where the blocks with beads (half, with
+    // a tenth of the beads charged) fill more than two (103 registers): 64 systems 946 ->
+    // 909 us; 16 systems 214, with four 245
+    run(false, false, L.real.blocks > 4 * kSMs ? kb_real<R, 4> : kb_real<R, 2>, L.real, (const RealArgs<R>*)L.real.tab, s1);
     cudaEventRecord(evJoin, s1);
     for (int i = 0; i < L.nspread; ++i) {
         const BatchKernel& k = L.spread[i];

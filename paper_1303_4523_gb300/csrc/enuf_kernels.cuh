@@ -2556,7 +2556,8 @@ __device__ __forceinline__ void real_sweep(const Geo& g, int nq, int S, const in
 }
 
 // spf: positions of the sorted beads in float (FP32: the sorted array itself).
-template <typename R>
+// LEAVE: a block without beads leaves before the block sum (batches).
+template <typename R, bool LEAVE = false>
 __device__ __forceinline__ void k_real_body(Geo g, const int* __restrict__ tstart,
                                                        const typename V4<R>::T* __restrict__ sq,
                                                        const typename V4<R>::T* __restrict__ sw,
@@ -2575,6 +2576,10 @@ __device__ __forceinline__ void k_real_body(Geo g, const int* __restrict__ tstar
     constexpr int SMIN = real_half<R>() ? 1 : 2;
     int S = 32;
     while (S > SMIN && (long long)nq * S > (S > 8 ? g.real_lanes / 3 * 2 : g.real_lanes)) S >>= 1;
+    if (LEAVE && (long long)blk.id * (kRealThreads / S) >= nq) {
+        if (threadIdx.x == 0) rpart[2 * blk.id] = rpart[2 * blk.id + 1] = 0.0;
+        return;
+    }
     RealSum<R> a{(R)0, (R)0, (R)0, (R)0, (R)0};
     if (2 * g.rs + 1 >= g.ntd)
         real_sweep<R, true>(g, nq, S, tstart, sq, sw, sb, spf, list, ring, F, a, blk);
