@@ -17,14 +17,15 @@ inline void append_blocks(std::vector<int>& cmap, int sys, int nblk) {
 }
 
 // Blocks of one system of a batch in its bead loops. The batch fills the chip,
-// so a system takes few blocks and strides over its beads: real space N / 512
-// blocks and lanes per bead for N / 4 lanes (with a tenth of the beads charged half of
-// the blocks find none and leave at once; with N / 1024 blocks
-// the more charged systems left SMs idle: 40 systems of 3000 to 20,000 beads, a quarter,
-// half and all charged, 654, 2031 and 7780 us against 549, 1498 and 4950; a tenth
-// charged 293 against 290; N / 256: 64 systems, a tenth charged, 895 against 830), gather N / 512 (1171 against 1219 with N / 64), spreading
-// N / 256 (its launches, one per tile edge, follow each other: 40 systems of
-// 3000 to 20,000 beads 345 -> 333 us against N / 512 with the next rule).
+// so a system takes few blocks and strides over its beads.
+// Real space: N / 512 blocks, lanes per bead for N / 4 lanes. With a tenth of the beads
+// charged half of the blocks find none and leave at once. N / 1024 blocks left SMs idle
+// where more are charged: 40 systems of 3000 to 20,000 beads, a tenth, a quarter, half and
+// all charged, 293, 654, 2031 and 7780 us against 290, 549, 1498 and 4950; N / 256: 64
+// systems, a tenth charged, 895 against 830.
+// Gather N / 512 (1171 against 1219 with N / 64), spreading N / 256 (its launches, one per
+// tile edge, follow each other: 40 systems of 3000 to 20,000 beads 345 -> 333 us against
+// N / 512 with the next rule).
 inline int batch_real_blocks(const BatchSys& x) { return std::max(1, std::min(x.w.nblk_real, (x.N + 511) / 512)); }
 inline int batch_real_lanes(const BatchSys& x) {
     return std::max(1, std::min(x.w.nblk_real, (x.N + 1023) / 1024)) * kRealThreads;

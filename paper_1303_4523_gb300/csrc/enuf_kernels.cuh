@@ -2227,7 +2227,7 @@ __global__ void __launch_bounds__(kGatherThreads, gather_ctas<R, PT>()) k_gather
 //     global reductions.
 // The form before it staged the 27-tile halo of every tile in shared memory
 // (27 staged beads per central bead at 3M beads, and as many CTAs as tiles:
-// 8 for a 3000-bead box). Alone: FP32 3M beads 473 -> 259 us, 524k 94 -> 67,
+// 8 for a 3000-bead box). Alone: FP32 3M beads 473 -> 229 us, 524k 94 -> 67,
 // 192k 85 -> 51, 24k 62 -> 22; FP64 375k 264 -> 156, 3000 beads 49 -> 18 us (375k 92
 // alone with more lanes per bead, before the plan's present real_lanes).
 // ---------------------------------------------------------------------------
